@@ -1,8 +1,11 @@
-"""ctypes binding of libjet.so: same names as the C ABI, argument marshalling only.
+"""Binding of libjet.so: same names as the C ABI, argument marshalling only.
 
 Tensors are torch tensors used purely as device-memory handles (``data_ptr()``); every
 step of the path runs inside the library's kernels.  There is no fallback: if the shared
-library is missing the import of any entry point raises.
+library is missing the first call of any entry point raises.
+
+The calls that launch work go through the CPython extension ``_jetcall`` (``csrc/jetcall.cpp``), which turns the
+argument vector into the C call in one native pass; the host-side queries go through ctypes.
 """
 from __future__ import annotations
 
@@ -68,6 +71,7 @@ _SIGNATURES = {
 }
 
 _lib = None
+_ext = None
 
 
 class JetError(RuntimeError):
@@ -96,18 +100,18 @@ def exported_symbols():
     return sorted(_SIGNATURES)
 
 
-def _p(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
-
-
-def _stream(stream):
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    return stream if isinstance(stream, int) else stream.cuda_stream
+def native():
+    """The extension module behind the launching calls (loaded with the library, once)."""
+    global _ext
+    if _ext is None:
+        load()
+        try:
+            from . import _jetcall
+        except ImportError as e:
+            raise RuntimeError("the extension module _jetcall is missing or does not load: build it with "
+                               "`python -m paper_2606_18394_b200.build`; there is no fallback path") from e
+        _ext = _jetcall
+    return _ext
 
 
 def _check(status: int, where: str):
@@ -126,13 +130,8 @@ def jet_tree_build_workspace_bytes(batch, N, V, W) -> int:
 def jet_tree_build(logp, root_token, batch, N, V, W, B, parent, depth, token, score, anc_mask, n_nodes,
                    workspace, workspace_bytes=None, logp_batch_stride=None, logp_depth_stride=None,
                    stream=None, check=True):
-    bs = logp_batch_stride if logp_batch_stride is not None else logp.stride(0)
-    ds = logp_depth_stride if logp_depth_stride is not None else logp.stride(1)
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_build(_p(logp), bs, ds, _p(root_token), batch, N, V, W, B, _p(parent), _p(depth),
-                               _p(token), _p(score), _p(anc_mask), _p(n_nodes), _p(workspace), wb,
-                               _stream(stream))
+    st = native().tree_build(logp, logp_batch_stride, logp_depth_stride, root_token, batch, N, V, W, B, parent, depth, token,
+                             score, anc_mask, n_nodes, workspace, workspace_bytes, stream)
     if check:
         _check(st, "jet_tree_build")
     return st
@@ -149,13 +148,9 @@ def jet_tree_build_scored(logp, root_token, batch, N, V, W, B, score_mode, alpha
                           anc_mask, n_nodes, depth_entropy, workspace, workspace_bytes=None,
                           logp_batch_stride=None, logp_depth_stride=None, stream=None, check=True,
                           node_budget=None):
-    bs = logp_batch_stride if logp_batch_stride is not None else logp.stride(0)
-    ds = logp_depth_stride if logp_depth_stride is not None else logp.stride(1)
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_build_scored(_p(logp), bs, ds, _p(root_token), batch, N, V, W, B, _p(node_budget),
-                                      int(score_mode), float(alpha), _p(parent), _p(depth), _p(token), _p(score), _p(anc_mask),
-                                      _p(n_nodes), _p(depth_entropy), _p(workspace), wb, _stream(stream))
+    st = native().tree_build_scored(logp, logp_batch_stride, logp_depth_stride, root_token, batch, N, V, W, B, node_budget,
+                                    int(score_mode), alpha, parent, depth, token, score, anc_mask, n_nodes, depth_entropy, None,
+                                    False, workspace, workspace_bytes, stream)
     if check:
         _check(st, "jet_tree_build_scored")
     return st
@@ -169,14 +164,9 @@ def jet_tree_build_logits(logits, root_token, batch, N, V, W, B, score_mode, alp
                           anc_mask, n_nodes, depth_entropy, depth_lse, workspace, workspace_bytes=None,
                           logits_batch_stride=None, logits_depth_stride=None, stream=None, check=True,
                           node_budget=None):
-    bs = logits_batch_stride if logits_batch_stride is not None else logits.stride(0)
-    ds = logits_depth_stride if logits_depth_stride is not None else logits.stride(1)
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_build_logits(_p(logits), bs, ds, _p(root_token), batch, N, V, W, B, _p(node_budget),
-                                      int(score_mode), float(alpha), _p(parent), _p(depth), _p(token), _p(score),
-                                      _p(anc_mask), _p(n_nodes), _p(depth_entropy), _p(depth_lse), _p(workspace), wb,
-                                      _stream(stream))
+    st = native().tree_build_scored(logits, logits_batch_stride, logits_depth_stride, root_token, batch, N, V, W, B,
+                                    node_budget, int(score_mode), alpha, parent, depth, token, score, anc_mask, n_nodes,
+                                    depth_entropy, depth_lse, True, workspace, workspace_bytes, stream)
     if check:
         _check(st, "jet_tree_build_logits")
     return st
@@ -203,13 +193,9 @@ def jet_tree_verify_attn(q, k_cache, v_cache, page_table, max_pages_per_seq, pag
                          max_seq_len, tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D,
                          kv_batch_stride, softmax_scale, out, lse, device_status, workspace,
                          workspace_bytes=None, stream=None, check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_verify_attn(_p(q), _p(k_cache), _p(v_cache), _p(page_table), max_pages_per_seq,
-                                     page_size, num_pages, _p(seq_len), max_seq_len, _p(tree_k), _p(tree_v),
-                                     _p(anc_mask), _p(n_nodes), batch, B, Hq, Hkv, D, kv_batch_stride,
-                                     softmax_scale, _p(out), _p(lse), _p(device_status), _p(workspace), wb,
-                                     _stream(stream))
+    st = native().tree_verify_attn(None, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len,
+                                   max_seq_len, tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
+                                   softmax_scale, out, lse, device_status, workspace, workspace_bytes, stream, 0, False)
     if check:
         _check(st, "jet_tree_verify_attn")
     return st
@@ -219,12 +205,9 @@ def jet_tree_verify_attn_tail(q, k_cache, v_cache, page_table, max_pages_per_seq
                               max_seq_len, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
                               softmax_scale, out, lse, device_status, workspace, workspace_bytes=None, stream=None,
                               check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_verify_attn_tail(_p(q), _p(k_cache), _p(v_cache), _p(page_table), max_pages_per_seq,
-                                          page_size, num_pages, _p(seq_len), max_seq_len, _p(anc_mask),
-                                          _p(n_nodes), batch, B, Hq, Hkv, D, kv_batch_stride, softmax_scale,
-                                          _p(out), _p(lse), _p(device_status), _p(workspace), wb, _stream(stream))
+    st = native().tree_verify_attn(None, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len,
+                                   max_seq_len, None, None, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
+                                   softmax_scale, out, lse, device_status, workspace, workspace_bytes, stream, 0, True)
     if check:
         _check(st, "jet_tree_verify_attn_tail")
     return st
@@ -234,13 +217,9 @@ def jet_tree_verify_attn_ex(q, k_cache, v_cache, page_table, max_pages_per_seq, 
                             max_seq_len, tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D,
                             kv_batch_stride, softmax_scale, out, lse, device_status, workspace, flags,
                             workspace_bytes=None, stream=None, check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_verify_attn_ex(_p(q), _p(k_cache), _p(v_cache), _p(page_table), max_pages_per_seq,
-                                        page_size, num_pages, _p(seq_len), max_seq_len, _p(tree_k), _p(tree_v),
-                                        _p(anc_mask), _p(n_nodes), batch, B, Hq, Hkv, D, kv_batch_stride,
-                                        softmax_scale, _p(out), _p(lse), _p(device_status), _p(workspace), wb,
-                                        _stream(stream), int(flags))
+    st = native().tree_verify_attn(None, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len,
+                                   max_seq_len, tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
+                                   softmax_scale, out, lse, device_status, workspace, workspace_bytes, stream, int(flags), False)
     if check:
         _check(st, "jet_tree_verify_attn_ex")
     return st
@@ -250,24 +229,31 @@ def jet_tree_verify_attn_tail_ex(q, k_cache, v_cache, page_table, max_pages_per_
                                  seq_len, max_seq_len, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
                                  softmax_scale, out, lse, device_status, workspace, flags, workspace_bytes=None,
                                  stream=None, check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_verify_attn_tail_ex(_p(q), _p(k_cache), _p(v_cache), _p(page_table), max_pages_per_seq,
-                                             page_size, num_pages, _p(seq_len), max_seq_len, _p(anc_mask),
-                                             _p(n_nodes), batch, B, Hq, Hkv, D, kv_batch_stride, softmax_scale,
-                                             _p(out), _p(lse), _p(device_status), _p(workspace), wb,
-                                             _stream(stream), int(flags))
+    st = native().tree_verify_attn(None, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len,
+                                   max_seq_len, None, None, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
+                                   softmax_scale, out, lse, device_status, workspace, workspace_bytes, stream, int(flags), True)
     if check:
         _check(st, "jet_tree_verify_attn_tail_ex")
     return st
 
 
+def verify_attn_layer(layer, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len, max_seq_len,
+                      tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride, softmax_scale, out, lse,
+                      device_status, workspace, flags, tail, stream=None):
+    """One layer of a stack: q, the caches, tree_k / tree_v and out carry a leading layer dimension and `layer` picks the
+    slice natively (six Python-level tensor slices per call cost more host time than the launch itself)."""
+    st = native().tree_verify_attn(layer, q, k_cache, v_cache, page_table, max_pages_per_seq, page_size, num_pages, seq_len,
+                                   max_seq_len, tree_k, tree_v, anc_mask, n_nodes, batch, B, Hq, Hkv, D, kv_batch_stride,
+                                   softmax_scale, out, lse, device_status, workspace, None, stream, flags, tail)
+    if st != JET_OK:
+        _check(st, "jet_tree_verify_attn_tail_ex" if tail else "jet_tree_verify_attn_ex")
+
+
 def jet_kv_compact_tail(k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table, max_pages_per_seq,
                         page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N, stream=None,
                         check=True):
-    st = load().jet_kv_compact_tail(_p(k_cache), _p(v_cache), cache_layer_stride, kv_batch_stride, _p(page_table),
-                                    max_pages_per_seq, page_size, _p(path), _p(accept_len), _p(seq_len), layers,
-                                    batch, B, Hkv, D, N, _stream(stream))
+    st = native().kv_compact(None, None, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table, max_pages_per_seq,
+                             page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N, stream, True)
     if check:
         _check(st, "jet_kv_compact_tail")
     return st
@@ -280,11 +266,8 @@ def jet_tree_accept_workspace_bytes(batch, B, V) -> int:
 def jet_tree_accept(logits, logits_row_stride, token, parent, depth, anc_mask, n_nodes, batch, B, V, N,
                     tgt_argmax, accept_len, path, out_tokens, workspace, workspace_bytes=None, stream=None,
                     check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_accept(_p(logits), logits_row_stride, _p(token), _p(parent), _p(depth), _p(anc_mask),
-                                _p(n_nodes), batch, B, V, N, _p(tgt_argmax), _p(accept_len), _p(path),
-                                _p(out_tokens), _p(workspace), wb, _stream(stream))
+    st = native().tree_accept(logits, logits_row_stride, token, parent, depth, anc_mask, n_nodes, batch, B, V, N, tgt_argmax,
+                              accept_len, path, out_tokens, workspace, workspace_bytes, stream, False)
     if check:
         _check(st, "jet_tree_accept")
     return st
@@ -298,11 +281,9 @@ def jet_tree_accept_hidden(hidden, lm_head_weight, d, token, parent, depth, anc_
                            tgt_argmax, accept_len, path, out_tokens, device_status, workspace, workspace_bytes=None,
                            stream=None, check=True):
     """Greedy acceptance from the final hidden states: the LM head runs inside the call, only arg-maxima are kept."""
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_accept_hidden(_p(hidden), _p(lm_head_weight), d, _p(token), _p(parent), _p(depth),
-                                       _p(anc_mask), _p(n_nodes), batch, B, V, N, _p(tgt_argmax), _p(accept_len),
-                                       _p(path), _p(out_tokens), _p(device_status), _p(workspace), wb, _stream(stream))
+    st = native().tree_accept_hidden(hidden, lm_head_weight, d, token, parent, depth, anc_mask, n_nodes, batch, B, V, N,
+                                     tgt_argmax, accept_len, path, out_tokens, device_status, workspace, workspace_bytes,
+                                     stream)
     if check:
         _check(st, "jet_tree_accept_hidden")
     return st
@@ -314,9 +295,8 @@ def jet_tree_accept_static(logits, logits_row_stride, token, parent, depth, anc_
     For callers that must not allocate device memory (everything already reserved, or no allocator
     calls allowed on the decode loop).  Problems larger than the built-in array give JET_ERR_WORKSPACE;
     calls that overlap on one GPU race on the shared array."""
-    st = load().jet_tree_accept_static(_p(logits), logits_row_stride, _p(token), _p(parent), _p(depth),
-                                       _p(anc_mask), _p(n_nodes), batch, B, V, N, _p(tgt_argmax),
-                                       _p(accept_len), _p(path), _p(out_tokens), _stream(stream))
+    st = native().tree_accept(logits, logits_row_stride, token, parent, depth, anc_mask, n_nodes, batch, B, V, N, tgt_argmax,
+                              accept_len, path, out_tokens, None, 0, stream, True)
     if check:
         _check(st, "jet_tree_accept_static")
     return st
@@ -330,13 +310,9 @@ def jet_tree_accept_sample(logits, logits_row_stride, temperature, draft_logp, l
                            logp_depth_stride, token, parent, depth, anc_mask, n_nodes, u_accept, u_sample,
                            batch, B, V, N, alpha, accept_len, path, out_tokens, workspace, workspace_bytes=None,
                            stream=None, check=True):
-    wb = workspace_bytes if workspace_bytes is not None else (workspace.numel() * workspace.element_size()
-                                                              if workspace is not None else 0)
-    st = load().jet_tree_accept_sample(_p(logits), logits_row_stride, temperature, _p(draft_logp),
-                                       logp_batch_stride, logp_depth_stride, _p(token), _p(parent), _p(depth),
-                                       _p(anc_mask), _p(n_nodes), _p(u_accept), _p(u_sample), batch, B, V, N,
-                                       _p(alpha), _p(accept_len), _p(path), _p(out_tokens), _p(workspace), wb,
-                                       _stream(stream))
+    st = native().tree_accept_sample(logits, logits_row_stride, temperature, draft_logp, logp_batch_stride, logp_depth_stride,
+                                     token, parent, depth, anc_mask, n_nodes, u_accept, u_sample, batch, B, V, N, alpha,
+                                     accept_len, path, out_tokens, workspace, workspace_bytes, stream)
     if check:
         _check(st, "jet_tree_accept_sample")
     return st
@@ -345,9 +321,8 @@ def jet_tree_accept_sample(logits, logits_row_stride, temperature, draft_logp, l
 def jet_kv_compact(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,
                    max_pages_per_seq, page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N,
                    stream=None, check=True):
-    st = load().jet_kv_compact(_p(tree_k), _p(tree_v), _p(k_cache), _p(v_cache), cache_layer_stride,
-                               kv_batch_stride, _p(page_table), max_pages_per_seq, page_size, _p(path),
-                               _p(accept_len), _p(seq_len), layers, batch, B, Hkv, D, N, _stream(stream))
+    st = native().kv_compact(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,
+                             max_pages_per_seq, page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N, stream, False)
     if check:
         _check(st, "jet_kv_compact")
     return st

@@ -1,14 +1,17 @@
-"""Builds libjet.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libjet.so (the C-ABI library, nvcc for sm_100a) and the binding's CPython extension in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libjet.so")
+# the binding's argument marshalling (a CPython extension linked against libjet.so and torch)
+EXT = os.path.join(PKG, "_jetcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["jet_api.cu", "tree_build.cu", "tree_verify_attn.cu", "tree_accept.cu", "tree_accept_sample.cu",
            "kv_compact.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,15 +28,30 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(EXT):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(EXT))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "jet.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _extension_commands(obj: str) -> tuple[list[str], list[str]]:
+    """Compile and link command of the CPython extension."""
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(troot, "include"),
+           os.path.join(troot, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    compile_cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden",
+                   f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(x for i in inc for x in ("-I", i)),
+                   "-c", os.path.join(CSRC, "jetcall.cpp"), "-o", obj]
+    link_cmd = ["g++", "-shared", "-o", EXT, obj, "-L", PKG, "-l:libjet.so", "-L", os.path.join(troot, "lib"),
+                "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
+    return compile_cmd, link_cmd
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into objects and link libjet.so.  Returns its path."""
+    """Compile everything under csrc/ into objects, link libjet.so and the CPython extension.  Returns libjet.so's path."""
     if not force and not needs_build():
         return LIB
     objdir = os.path.join(PKG, "build")
@@ -48,6 +66,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    ext_obj = os.path.join(objdir, "jetcall.o")
+    ext_compile, ext_link = _extension_commands(ext_obj)
+    procs.append(("jetcall.cpp", subprocess.Popen(ext_compile, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
@@ -55,10 +76,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(f"--- {src}\n{out}\n")
         failed |= p.returncode != 0
     if failed:
-        raise RuntimeError("nvcc failed building libjet.so")
+        raise RuntimeError("compiling libjet.so or its Python binding failed")
     link = [_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
             "-Xcompiler", "-fPIC"]
     subprocess.run(link, check=True)
+    subprocess.run(ext_link, check=True)
     return LIB
 
 

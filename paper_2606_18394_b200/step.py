@@ -156,19 +156,12 @@ class VerifyStep:
         if first_in_stack is None:
             first_in_stack = layer == 0
         flags = jet.JET_ATTN_STABLE_PREFIX if (self.stable_prefix and not first_in_stack) else 0
-        if self.tail:
-            jet.jet_tree_verify_attn_tail_ex(self.q[layer], self.k_cache[layer], self.v_cache[layer],
-                                             self.page_table, self.max_pages, self.page_size, self.num_pages,
-                                             self.seq_len, self.attn_max_len, self.anc_mask, self.n_nodes,
-                                             self.batch, self.B, self.Hq, self.Hkv, self.D, self.kv_batch_stride,
-                                             self.scale, self.out[layer], None, self.status, self.ws_attn, flags)
-            return
-        jet.jet_tree_verify_attn_ex(self.q[layer], self.k_cache[layer], self.v_cache[layer], self.page_table,
-                                    self.max_pages, self.page_size, self.num_pages, self.seq_len,
-                                    self.attn_max_len, self.tree_k[layer], self.tree_v[layer], self.anc_mask,
-                                    self.n_nodes, self.batch, self.B, self.Hq, self.Hkv, self.D,
-                                    self.kv_batch_stride, self.scale, self.out[layer], None, self.status,
-                                    self.ws_attn, flags)
+        tail = self.tail
+        jet.verify_attn_layer(layer, self.q, self.k_cache, self.v_cache, self.page_table, self.max_pages, self.page_size,
+                              self.num_pages, self.seq_len, self.attn_max_len,
+                              None if tail else self.tree_k, None if tail else self.tree_v, self.anc_mask, self.n_nodes,
+                              self.batch, self.B, self.Hq, self.Hkv, self.D, self.kv_batch_stride, self.scale, self.out, None,
+                              self.status, self.ws_attn, flags, tail)
 
     def tree_accept(self):
         jet.jet_tree_accept(self.logits, self.V, self.token, self.parent, self.depth, self.anc_mask, self.n_nodes,
