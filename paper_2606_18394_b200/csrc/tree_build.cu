@@ -2,464 +2,728 @@
 // budgeted tree construction with the accumulated log-probability score).
 // jet_tree_build_scored: the same with the expansion scores of Appendix C (per-depth
 // entropy alone; accumulated log-probability + alpha * per-depth entropy): the scan
-// also leaves per-slice sums of p * log p (fp64), the expansion kernel adds them up
-// per depth and uses the entropy in the queue's priority.
-// jet_tree_build_logits: the same fed with raw draft logits.  One more launch in front
-// (lse_partial_kernel: per-slice maximum and sum of exponentials in fp64); the scan then
-// forms every log-probability on the fly as float(double(z) - lse), so the [N,V]
-// log-probabilities never exist in memory and the second pass over the logits comes
-// out of L2.
+// also leaves per-slice sums of p * log p (fp64), and the expansion kernel uses the
+// per-depth entropy in the queue's priority.
+// jet_tree_build_logits: the same fed with raw draft logits.  The scan leaves per-slice
+// (reference, sum of exponentials) pairs in fp64; a log-probability is float(double(z) - lse),
+// so the [N,V] log-probabilities never exist in memory.
 //
-// Two launches:
-//   topw_partial_kernel  grid (chunks, N, batch): every block scans one slice of one
-//                        vocabulary row and leaves its W best (value, token) keys in
-//                        the workspace -- the only pass over the [N,V] log-probs.
-//   tree_expand_kernel   grid (batch): merges the per-slice candidates, runs the
-//                        sequential pop/expand loop in one warp with the pending
-//                        queue held in shared memory, then emits parent / depth /
-//                        token / score / ancestor bitmask.
+// Launches:
+//   row_scan_kernel      grid (slices, N, batch): the one pass over the [N,V] rows.  It only
+//                        streams: the maximum of every group of 128 entries and the slice's
+//                        fp64 sum go to the workspace.  (Raw logits with an entropy score: a
+//                        second launch of it forms the entropy, which needs the log-sum-exp.)
+//   tree_expand_kernel   grid (batch): per depth, finds the W-th largest group maximum, reads
+//                        the few groups at or above it again and ranks their entries; then runs
+//                        the sequential pop/expand loop in one warp with the pending queue
+//                        in registers and emits parent / depth / token / score / ancestor mask.
+#include "fp64_exp.cuh"
 #include "jet_common.cuh"
 
 namespace jet {
 namespace {
 
-constexpr int kTopThreads = 256;
-constexpr int kTopElems = 16;                        // elements per thread
-constexpr int kTopChunk = kTopThreads * kTopElems;   // vocabulary slice per block
+// ------------------------------------------------------------------------------------------------ scan
+constexpr int kScanThreads = 256;
+constexpr int kScanWarps = kScanThreads / 32;
+constexpr int kRoundElems = 16;                      // elements a thread takes per round (four 16-byte loads)
+constexpr int kRoundChunk = kScanThreads * kRoundElems;
+constexpr int kGroup = 128;                          // entries per group maximum
+constexpr float kTermFloor = 700.0f;                 // exp(-700) is beyond any sum's last place
 
-// One block scans a 4096-element slice of one vocabulary row and leaves its W best keys.  Almost every
-// element is dismissed with one compare: an element among a warp's W best is at least as large as the W-th
-// largest of the 32 per-lane maxima (tau), so only elements >= tau become candidates (as ordered 64-bit keys
-// in shared memory); the block then selects its W best among the few candidates.  Exact for any input: with
-// many equal values all of them become candidates and the key order (value, then lowest index) decides.
-// kEntropy: the block also leaves sum(exp(l) * l) over its slice (fp64; entries of -inf contribute 0) for the
-// per-depth entropy; the reduction order is fixed, so the value does not change from run to run.
-// Loads the 16 elements of a thread: element e has vocabulary index
-//   vec ? base + ((e >> 2) * kTopThreads + tid) * 4 + (e & 3) : base + e * kTopThreads + tid;
-// elements beyond V read as -inf.
-__device__ __forceinline__ void load_slice(const float* __restrict__ row, int base, int V, bool vec, int tid,
-                                           float (&v)[kTopElems]) {
-  if (vec) {
-    const float4* row4 = reinterpret_cast<const float4*>(row + base);
-#pragma unroll
-    for (int i = 0; i < kTopElems / 4; ++i) {
-      const float4 x = __ldg(row4 + i * kTopThreads + tid);
-      v[i * 4 + 0] = x.x; v[i * 4 + 1] = x.y; v[i * 4 + 2] = x.z; v[i * 4 + 3] = x.w;
-    }
+enum ScanMode { kScanMax = 0, kScanEntropy = 1, kScanSum = 2, kScanLogitEntropy = 3 };
+
+// A slice is kRoundChunk * R consecutive entries of one row; float4 number e4 (0 .. 4R - 1) of thread t is
+//   base + (e4 * kScanThreads + t) * 4 .. + 3,
+// read with one 16-byte load, or (unaligned rows) four 4-byte ones; entries beyond V read as -inf.
+__device__ __forceinline__ float4 load4(const float* __restrict__ row, int idx, int V, bool vec) {
+  float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  if (vec && idx + 3 < V) {
+    x = __ldg(reinterpret_cast<const float4*>(row + idx));
   } else {
-#pragma unroll
-    for (int i = 0; i < kTopElems; ++i) {
-      const int idx = base + i * kTopThreads + tid;
-      v[i] = idx < V ? __ldg(row + idx) : -INFINITY;
-    }
+    if (idx < V) x.x = __ldg(row + idx);
+    if (idx + 1 < V) x.y = __ldg(row + idx + 1);
+    if (idx + 2 < V) x.z = __ldg(row + idx + 2);
+    if (idx + 3 < V) x.w = __ldg(row + idx + 3);
   }
+  return x;
 }
 
-// Raw logits: every block leaves (m, z) of its slice, m = the slice's maximum and z = sum(exp(double(x) - m))
-// in fp64 with a fixed reduction order (a slice of -inf only: m = -inf, z = 0).
-__global__ void __launch_bounds__(kTopThreads)
-lse_partial_kernel(const float* __restrict__ logits, int64_t batch_stride, int64_t depth_stride, int V, int nchunks,
-                   bool vec_ok, double* __restrict__ lse_partial) {
-  grid_dependency_wait();
-  const int chunk = blockIdx.x, d = blockIdx.y, b = blockIdx.z;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const float* row = logits + b * batch_stride + d * depth_stride;
-  const int base = chunk * kTopChunk;
-  float v[kTopElems];
-  load_slice(row, base, V, vec_ok && base + kTopChunk <= V, tid, v);
-  float m = -INFINITY;
+__device__ __forceinline__ float warp_max_f32(float x) {
+  const uint32_t u = __reduce_max_sync(0xffffffffu, f32_order(x));
+  return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
+}
+__device__ __forceinline__ double warp_sum_f64(double x) {
 #pragma unroll
-  for (int i = 0; i < kTopElems; ++i) m = fmaxf(m, v[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  __shared__ float s_m[kTopThreads / 32];
-  __shared__ double s_z[kTopThreads / 32];
-  if (lane == 0) s_m[tid >> 5] = m;
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < kTopThreads / 32; ++w) m = fmaxf(m, s_m[w]);
-  double z = 0.0;
-  if (m > -INFINITY) {
-    const double md = static_cast<double>(m);
-#pragma unroll
-    for (int i = 0; i < kTopElems; ++i)
-      if (v[i] > -INFINITY) z += exp(static_cast<double>(v[i]) - md);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-  if (lane == 0) s_z[tid >> 5] = z;
-  __syncthreads();
-  if (tid == 0) {
-    double total = 0.0;
-    for (int w = 0; w < kTopThreads / 32; ++w) total += s_z[w];
-    double* out = lse_partial + ((static_cast<size_t>(b) * gridDim.y + d) * nchunks + chunk) * 2;
-    out[0] = static_cast<double>(m);
-    out[1] = total;
-  }
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
 }
 
-// The row's log-sum-exp from the slices' (m, z): M = max m, lse = M + log(sum z * exp(m - M)), fp64, one warp,
-// fixed order (every block of a row gets the same bits).
-__device__ __forceinline__ double row_lse(const double* __restrict__ part, int nchunks, int lane) {
-  double M = -INFINITY;
-  for (int i = lane; i < nchunks; i += 32) M = fmax(M, part[2 * i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+// The row's log-sum-exp from the slices' (m, z = sum exp(x) * 2^-m), m a whole number: M = the largest m, lse = M ln2 +
+// log(sum z * 2^(m - M)), fp64, one warp, fixed order (every caller gets the same bits).
+__device__ __forceinline__ double row_lse(const double2* __restrict__ part, int slices, int lane) {
+  double M = -INFINITY;                              // this lane's largest m with a finite entry
+  for (int i = lane; i < slices; i += 32) M = fmax(M, part[i].y > 0.0 ? part[i].x : -INFINITY);
+  const uint32_t order = f32_order(static_cast<float>(M));
+  const int holder = __ffs(__ballot_sync(0xffffffffu, order == __reduce_max_sync(0xffffffffu, order))) - 1;
+  M = __shfl_sync(0xffffffffu, M, holder);           // (the largest, up to the rounding of a float: any m near it will do)
   double Z = 0.0;
-  for (int i = lane; i < nchunks; i += 32) {
-    const double m = part[2 * i], z = part[2 * i + 1];
-    if (z > 0.0) Z += z * exp(m - M);
+  for (int i = lane; i < slices; i += 32) {
+    const double2 mz = part[i];
+    const double shift = mz.x - M;                   // beyond -1000 the slice is nothing beside the largest
+    if (mz.y > 0.0 && shift > -1000.0)
+      Z += mz.y * __hiloint2double((1023 + static_cast<int>(shift)) << 20, 0);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
-  return M + log(Z);
+  Z = warp_sum_f64(Z);
+  return fma(M, 0.6931471805599453, log(Z));
 }
 
-// kLogits: the row holds raw logits; lse_partial holds its slices' (m, z) and every element becomes the
-// log-probability float(double(x) - lse) before anything else looks at it (block 0 of the row also leaves
-// float(lse) in depth_lse_out if that is given).
-template <bool kEntropy, bool kLogits>
-__global__ void __launch_bounds__(kTopThreads)
-topw_partial_kernel(const float* __restrict__ logp, int64_t batch_stride, int64_t depth_stride,
-                    int V, int Wc, int nchunks, bool vec_ok,
-                    unsigned long long* __restrict__ cand, double* __restrict__ plogp_partial,
-                    const double* __restrict__ lse_partial, float* __restrict__ depth_lse_out) {
-  grid_dependency_wait();
-  const int chunk = blockIdx.x, d = blockIdx.y, b = blockIdx.z;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const float* row = logp + b * batch_stride + d * depth_stride;
-  const int base = chunk * kTopChunk;
-
-  // element e of this thread has vocabulary index idx_of(e); out-of-range elements are -inf and never candidates
-  float v[kTopElems];
-  const bool vec = vec_ok && base + kTopChunk <= V;
-  auto idx_of = [&](int e) -> int {
-    return vec ? base + ((e >> 2) * kTopThreads + tid) * 4 + (e & 3) : base + e * kTopThreads + tid;
-  };
-  load_slice(row, base, V, vec, tid, v);
-  if constexpr (kLogits) {
-    __shared__ double s_lse;
-    if (tid < 32) {
-      const double lse = row_lse(lse_partial + (static_cast<size_t>(b) * gridDim.y + d) * nchunks * 2, nchunks, lane);
-      if (lane == 0) {
-        s_lse = lse;
-        if (chunk == 0 && depth_lse_out) depth_lse_out[static_cast<size_t>(b) * gridDim.y + d] = static_cast<float>(lse);
+// The same fp64 sums with the general exponential, for slices the table form does not cover (a reference of -inf or beyond
+// its range, entries more than 600 above the reference, log-probabilities above 600): this thread's part, read again.
+// m is the slice's maximum (kScanSum), the lse (kScanLogitEntropy).
+template <int kMode>
+__device__ __noinline__ double slow_sum(const float* __restrict__ row, int base, int rounds, int V, bool vec, double m) {
+  double acc = 0.0;
+  for (int e4 = 0; e4 < 4 * rounds; ++e4) {
+    const float4 q = load4(row, base + (e4 * kScanThreads + static_cast<int>(threadIdx.x)) * 4, V, vec);
+    const float x[4] = {q.x, q.y, q.z, q.w};
+    for (int j = 0; j < 4; ++j) {
+      if (!(x[j] > -INFINITY)) continue;
+      if constexpr (kMode == kScanSum) {
+        acc += exp(static_cast<double>(x[j]) - m);
+      } else {
+        const double l = kMode == kScanLogitEntropy ? static_cast<double>(static_cast<float>(static_cast<double>(x[j]) - m)) : static_cast<double>(x[j]);
+        acc += exp(l) * l;
       }
     }
-    __syncthreads();
-    const double lse = s_lse;
-#pragma unroll
-    for (int i = 0; i < kTopElems; ++i) v[i] = static_cast<float>(static_cast<double>(v[i]) - lse);
   }
+  return acc;
+}
 
-  if constexpr (kEntropy) {
-    double acc = 0.0;
+// One slice of one row per block.  gmax[row][slice * 32 R + g] = maximum of group g (kScanMax / Entropy / Sum); sums[row][slice]:
+//   kScanEntropy       .x = sum(exp(l) * l) of log-probabilities l
+//   kScanSum           (m, sum(exp(z)) * 2^-m) of logits z, m = any whole number that keeps the terms in range
+//   kScanLogitEntropy  .y = sum(exp(l) * l), l = float(double(z) - lse) with the lse of the slices' kScanSum pairs in `pairs`
+// All sums in fp64 in a fixed order: the same value from run to run.  Entries of -inf contribute 0.
+//
+// Bound: HBM without a sum; with one the issue slots and the fp64 pipe (about 25 instructions per entry, 9 of them fp64:
+// 53 us for 32 x 8 rows of 151936 entries, 38 - 42 us of that for the terms alone).  A thread keeps one round of 16 entries in
+// flight while it works on the round before; there is one CTA-wide barrier per slice (two with a sum), so that the blocks of
+// an SM drift apart and one block's loads run under another's arithmetic.  The form before -- 4096 entries per block,
+// every block ranking its own W best, general fp64 exponentials, the logits scanned once for the sum and once for the
+// ranks -- took 107 us for that batch with an entropy and 97 + 103 us from raw logits.
+template <int kMode>
+__global__ void __launch_bounds__(kScanThreads, kMode == kScanMax ? 4 : 3)
+row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t depth_stride, int V, int rounds, bool vec,
+                float* __restrict__ gmax, const double2* __restrict__ pairs, double2* __restrict__ sums) {
+  grid_dependency_wait();
+  const int slice = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float* row = rows + static_cast<int64_t>(blockIdx.z) * batch_stride + static_cast<int64_t>(blockIdx.y) * depth_stride;
+  const size_t row_id = static_cast<size_t>(blockIdx.z) * gridDim.y + blockIdx.y;
+  const int base = slice * kRoundChunk * rounds;
+  __shared__ float s_max[kScanWarps];
+  __shared__ double s_sum[kScanWarps];
+  __shared__ double s_lse;
+
+  float4 cur[4], nxt[4];
+  auto fetch = [&](int r, float4 (&x)[4]) {
 #pragma unroll
-    for (int i = 0; i < kTopElems; ++i)
-      if (v[i] > -INFINITY) acc += exp(static_cast<double>(v[i])) * static_cast<double>(v[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    __shared__ double s_acc[kTopThreads / 32];
-    if (lane == 0) s_acc[tid >> 5] = acc;
+    for (int i = 0; i < 4; ++i) x[i] = load4(row, base + ((r * 4 + i) * kScanThreads + tid) * 4, V, vec);
+  };
+  fetch(0, cur);
+  Exp64Table tab(kMode == kScanMax ? 0 : lane);
+  double ref = 0.0, acc = 0.0;
+  float ref_f = 0.0f, mx = -INFINITY;
+  if constexpr (kMode == kScanLogitEntropy) {
+    if (warp == 0) {
+      const double l = row_lse(pairs + row_id * gridDim.x, gridDim.x, lane);
+      if (lane == 0) s_lse = l;
+    }
     __syncthreads();
+    ref = s_lse;
+  }
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    if (r + 1 < rounds) fetch(r + 1, nxt);
+    float x[kRoundElems];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { x[4 * i] = cur[i].x; x[4 * i + 1] = cur[i].y; x[4 * i + 2] = cur[i].z; x[4 * i + 3] = cur[i].w; }
+#pragma unroll
+    for (int e = 0; e < kRoundElems; ++e) mx = fmaxf(mx, x[e]);
+    if constexpr (kMode == kScanSum) {
+      if (r == 0) {
+        const float mw = warp_max_f32(mx);
+        if (lane == 0) s_max[warp] = mw;
+        __syncthreads();
+        ref_f = s_max[0];
+#pragma unroll
+        for (int w = 1; w < kScanWarps; ++w) ref_f = fmaxf(ref_f, s_max[w]);
+        const int m = __float2int_rn(ref_f * 1.4426950408889634f);     // near the largest entry of the block's first round
+        tab.scale_down(m);
+        ref = static_cast<double>(m);
+      }
+#pragma unroll
+      for (int e = 0; e < kRoundElems; ++e) {
+        const float v = fmaxf(x[e], ref_f - kTermFloor);       // (a term of exp(-700) and one of 0 are the same beside exp(0))
+        const Exp64 t = exp64(v, static_cast<double>(v), tab);
+        acc = fma(t.s, t.p, acc);
+      }
+    } else if constexpr (kMode == kScanEntropy || kMode == kScanLogitEntropy) {
+#pragma unroll
+      for (int e = 0; e < kRoundElems; ++e) {
+        float l = kMode == kScanLogitEntropy ? static_cast<float>(static_cast<double>(x[e]) - ref) : x[e];
+        l = l >= -kTermFloor ? l : 0.0f;               // (entries below it, -inf among them, contribute exactly 0)
+        const double ld = static_cast<double>(l);
+        const Exp64 t = exp64(l, ld, tab);
+        acc = fma(t.s * t.p, ld, acc);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
+  }
+  if constexpr (kMode != kScanLogitEntropy) {
+    // a group: 128 / (16 R) neighbouring threads
+    float g = mx;
+    const int gl = kGroup / (kRoundElems * rounds);
+    for (int o = 1; o < gl; o <<= 1) g = fmaxf(g, __shfl_xor_sync(0xffffffffu, g, o));
+    if ((tid & (gl - 1)) == 0)
+      gmax[(row_id * gridDim.x + slice) * (kScanThreads / gl) + tid / gl] = g;
+  }
+  if constexpr (kMode != kScanMax) {
+    const float mw = warp_max_f32(mx);
+    acc = warp_sum_f64(acc);
+    if constexpr (kMode == kScanSum) __syncthreads();          // s_max of the first round has been read
+    if (lane == 0) { s_max[warp] = mw; s_sum[warp] = acc; }
+    __syncthreads();
+    float m = s_max[0];
+#pragma unroll
+    for (int w = 1; w < kScanWarps; ++w) m = fmaxf(m, s_max[w]);
+    const bool slow = kMode == kScanSum       ? !(fabsf(ref_f) < kExp64Range - 1000.0f) || m > ref_f + 600.0f
+                      : kMode == kScanEntropy ? m > 600.0f : static_cast<double>(m) > ref + 600.0;
+    if (slow) {                                      // (block-uniform)
+      double scale = 1.0;
+      if constexpr (kMode == kScanSum) {
+        ref = rint(static_cast<double>(m) * 1.4426950408889634);
+        scale = exp(static_cast<double>(m) - ref * 0.6931471805599453);
+      }
+      acc = m > -INFINITY ? scale * slow_sum<kMode>(row, base, rounds, V, vec, kMode == kScanSum ? static_cast<double>(m) : ref) : 0.0;
+      acc = warp_sum_f64(acc);
+      __syncthreads();
+      if (lane == 0) s_sum[warp] = acc;
+      __syncthreads();
+    }
     if (tid == 0) {
       double total = 0.0;
-      for (int w = 0; w < kTopThreads / 32; ++w) total += s_acc[w];
-      plogp_partial[(static_cast<size_t>(b) * gridDim.y + d) * nchunks + chunk] = total;
-    }
-  }
-
-  // tau = Wc-th largest of the warp's 32 lane maxima: every lane ranks its maximum (ties by lane) against
-  // the others' with 32 independent shuffles; the lane of rank Wc-1 holds tau
-  float lane_max = -INFINITY;
 #pragma unroll
-  for (int i = 0; i < kTopElems; ++i) lane_max = fmaxf(lane_max, v[i]);
-  int rank = 0;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float other = __shfl_sync(0xffffffffu, lane_max, j);
-    rank += (other > lane_max || (other == lane_max && j < lane)) ? 1 : 0;
-  }
-  const unsigned holder = __ballot_sync(0xffffffffu, rank == Wc - 1);
-  const float tau = __shfl_sync(0xffffffffu, lane_max, __ffs(holder) - 1);
-
-  __shared__ unsigned long long s_cand[kTopChunk];      // worst case: every element of the slice
-  __shared__ int s_count;
-  if (tid == 0) s_count = 0;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < kTopElems; ++i) {
-    const int idx = idx_of(i);
-    if (v[i] >= tau && idx < V) s_cand[atomicAdd(&s_count, 1)] = make_key(v[i], static_cast<uint32_t>(idx));
-  }
-  __syncthreads();
-  const int count = s_count;
-
-  // the block's Wc best candidates, in rank order (keys are unique)
-  unsigned long long* out = cand + ((static_cast<size_t>(b) * gridDim.y + d) * nchunks + chunk) * Wc;
-  if (count <= kTopThreads) {
-    // usual case: one candidate per thread, ranked against all others (broadcast reads, no serial rounds)
-    if (tid < count) {
-      const unsigned long long mine = s_cand[tid];
-      int rank = 0;
-      for (int j = 0; j < count; ++j) rank += s_cand[j] > mine ? 1 : 0;
-      if (rank < Wc) out[rank] = mine;
+      for (int w = 0; w < kScanWarps; ++w) total += s_sum[w];
+      double2* out = sums + row_id * gridDim.x + slice;
+      *out = kMode == kScanSum ? make_double2(ref, total) : make_double2(total, 0.0);
     }
-    if (tid >= count && tid < Wc) out[tid] = 0ull;          // fewer candidates than Wc: no key
-    return;
-  }
-  // many equal values: warp 0 alone walks the candidates in rank order
-  if (tid >= 32) return;
-  // (more than kTopThreads candidates here, too many for registers: every round scans shared memory)
-  unsigned long long prev = ~0ull;
-  for (int r = 0; r < Wc; ++r) {
-    unsigned long long best = 0ull;
-    for (int i = lane; i < count; i += 32) {
-      const unsigned long long k = s_cand[i];
-      if (k < prev && k > best) best = k;
-    }
-    best = warp_max_u64(best);
-    if (lane == 0) out[r] = best;
-    prev = best;
   }
 }
 
-// Algorithm 1 in one warp.  The pending queue lives in registers: node u is kept by lane u % 32 in register
-// u / 32 as a key (score, lowest index first, depth in the low byte), so a pop is a register maximum plus one
-// warp reduction, and the popped node's score and depth come out of the key itself.  kSlots = registers per
-// lane (32 * kSlots >= B); the instruction count of a pop grows with it, hence the template.
+// ------------------------------------------------------------------------------------------------ expansion
+constexpr int kExpThreads = JET_MAX_NODES;
+constexpr int kExpWarps = kExpThreads / 32;
+constexpr int kListCap = 32 + kGroup;                // candidates a warp keeps: the best so far and one group's worth
+
+// The Wc-th largest of the warp's 32 lane values: largest value after largest value until Wc lanes are covered.  (Rolled: this
+// code runs once per launch, from a cold instruction cache, where its length is its cost.)
+__device__ __forceinline__ float warp_nth(float x, int Wc) {
+  uint32_t rest = f32_order(x);                      // 0 = covered (no number has code 0)
+  uint32_t top = 0u;
+#pragma unroll 1
+  for (int covered = 0; covered < Wc;) {
+    top = __reduce_max_sync(0xffffffffu, rest);
+    const bool hit = rest == top;
+    covered += __popc(__ballot_sync(0xffffffffu, hit));
+    if (hit) rest = 0u;
+  }
+  return __uint_as_float((top & 0x80000000u) ? (top & 0x7FFFFFFFu) : ~top);
+}
+
+// Keeps the best Wc of a warp's `count` keys (unique), in rank order, at the front of the list; returns how many that are.
+// kHeld = keys per lane.
+template <int kHeld>
+__device__ __forceinline__ int keep_best(unsigned long long* list, int count, int Wc, int lane) {
+  unsigned long long mine[kHeld];
+  int above[kHeld];
+#pragma unroll
+  for (int i = 0; i < kHeld; ++i) {
+    mine[i] = lane + 32 * i < count ? list[lane + 32 * i] : 0ull;
+    above[i] = 0;
+  }
+#pragma unroll 4
+  for (int j = 0; j < count; ++j) {
+    const unsigned long long other = list[j];
+#pragma unroll
+    for (int i = 0; i < kHeld; ++i) above[i] += other > mine[i] ? 1 : 0;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kHeld; ++i)
+    if (lane + 32 * i < count && above[i] < Wc) list[above[i]] = mine[i];
+  __syncwarp();
+  return min(count, Wc);
+}
+
+// One row of the scan as a warp reads it: lane l's float4 of group g starts at entry base(g) + lane_part.
+struct RowGroups {
+  const float* row;
+  int V, rounds, vec, log_threads, log_gl;           // log2 of groups per slice; of the scan's threads per group
+  int lane_part;
+  __device__ __forceinline__ RowGroups(const float* row, int V, int rounds, int vec, int lane)
+      : row(row), V(V), rounds(rounds), vec(vec) {
+    log_threads = rounds == 1 ? 5 : rounds == 2 ? 6 : 7;
+    log_gl = 8 - log_threads;
+    // thread (lane mod gl) of the group, float4 number lane / gl of that thread
+    lane_part = ((lane >> log_gl) * kScanThreads + (lane & ((1 << log_gl) - 1))) * 4;
+  }
+  __device__ __forceinline__ int base(int g) const {
+    return (g >> log_threads) * (kRoundChunk * rounds) + ((g & ((1 << log_threads) - 1)) << (log_gl + 2));
+  }
+};
+
+// The rows' rank value of an entry: itself, or the log-probability of a raw logit.
+template <bool kLogits>
+__device__ __forceinline__ float rank_value(float x, double lse) {
+  return kLogits ? static_cast<float>(static_cast<double>(x) - lse) : x;
+}
+
+// More groups or entries at or above the threshold than the fast form holds (many nearly equal values): the groups one
+// after the other, in ascending order; an entry is listed only if it beats the worst of the best so far.
+template <bool kLogits>
+__device__ __noinline__ int top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, float cut, int Wc, double lse,
+                                        int lane, unsigned long long* list) {
+  unsigned long long worst = 0ull;                   // keys at or below it cannot be among the best any more
+  int count = 0;
+  for (int g0 = 0; g0 < groups; g0 += 32) {
+    unsigned todo = __ballot_sync(0xffffffffu, __ldg(gm + g0 + lane) >= cut);      // (the number of groups is a multiple of 32)
+    while (todo) {
+      const int g = g0 + __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int idx = rg.base(g) + rg.lane_part;
+      const float4 q = load4(rg.row, idx, rg.V, rg.vec != 0);
+      const float x[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const unsigned long long key = make_key(rank_value<kLogits>(x[j], lse), static_cast<uint32_t>(idx + j));
+        const bool take = x[j] >= cut && idx + j < rg.V && key > worst;
+        const unsigned votes = __ballot_sync(0xffffffffu, take);
+        if (take) list[count + __popc(votes & ((1u << lane) - 1u))] = key;
+        count += __popc(votes);
+      }
+      __syncwarp();
+      if (count > kListCap - kGroup) {
+        count = keep_best<(kListCap + 31) / 32>(list, count, Wc, lane);
+        if (count == Wc) worst = list[Wc - 1];
+        __syncwarp();
+      }
+    }
+  }
+  return keep_best<(kListCap + 31) / 32>(list, count, Wc, lane);
+}
+
+// The row's Wc best (value, token) keys in rank order at the front of w.list, by one warp.  gm = the row's group maxima: at
+// least Wc groups reach the Wc-th largest lane maximum, so the Wc best entries are at or above it, and only groups that
+// reach it are read again (about Wc of them, all at once).  Exact for any input.
+// kLogits: entries are ranked by float(double(z) - lse), which is monotone in z: the threshold is lowered by more than one
+// rounding step of that value, and the keys hold it.  lse() is called while the maxima are on their way.
+// A chain of latencies: maxima (one round trip to L2), threshold, groups (another), ranks.  (With the groups read one
+// after the other and the maxima read twice it took 25 us instead of 3.)
+struct TopScratch {
+  unsigned long long list[kListCap];
+  int groups[32];
+};
+
+template <bool kLogits, typename Lse>
+__device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __restrict__ gm, int groups, int Wc, Lse&& lse_of,
+                                           int lane, TopScratch& w) {
+  constexpr int kQuads = 10;                         // float4 of maxima a lane holds: 1280 groups, 163840 entries
+  constexpr int kBatch = 8;                          // groups whose entries are in flight together
+  float4 h[kQuads];
+  const int quads = groups / 4;                      // (groups is a multiple of 32)
+  const float4* gm4 = reinterpret_cast<const float4*>(gm);
+#pragma unroll
+  for (int i = 0; i < kQuads; ++i)
+    h[i] = i * 32 + lane < quads ? __ldg(gm4 + i * 32 + lane) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  const double lse = lse_of();
+  float best = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < kQuads; ++i) best = fmaxf(best, fmaxf(fmaxf(h[i].x, h[i].y), fmaxf(h[i].z, h[i].w)));
+  for (int i = kQuads * 32 + lane; i < quads; i += 32) {
+    const float4 q = __ldg(gm4 + i);
+    best = fmaxf(best, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
+  }
+  float cut = warp_nth(best, Wc);
+  if constexpr (kLogits)      // 2^-22 of the value: two rounding steps
+    cut = __fsub_rd(cut, fmaxf(fabsf(rank_value<true>(cut, lse)) * 2.384185791015625e-7f, 1e-44f));
+  __syncwarp();
+  // the groups that reach it, up to 32; few lanes have any
+  bool fits = quads <= kQuads * 32;
+  int n = 0;
+  if (fits) {
+    uint32_t bits[2] = {0u, 0u};                     // maximum 4 i + j of this lane reaches the threshold
+#pragma unroll
+    for (int i = 0; i < kQuads; ++i) {
+      const uint32_t m = (h[i].x >= cut ? 1u : 0u) | (h[i].y >= cut ? 2u : 0u) | (h[i].z >= cut ? 4u : 0u) | (h[i].w >= cut ? 8u : 0u);
+      bits[i / 8] |= (i * 32 + lane < quads ? m : 0u) << (4 * (i % 8));
+    }
+#pragma unroll 1
+    for (unsigned todo = __ballot_sync(0xffffffffu, (bits[0] | bits[1]) != 0u); todo && n <= 32;) {
+      // one group of every lane that has one, per step
+      const bool mine = (bits[0] | bits[1]) != 0u;
+      const bool high = bits[0] == 0u;
+      const int bit = __ffs(high ? bits[1] : bits[0]) - 1;
+      const int at = n + __popc(todo & ((1u << lane) - 1u));
+      if (mine && at < 32) w.groups[at] = rg.base((((high ? 8 : 0) + (bit >> 2)) * 32 + lane) * 4 + (bit & 3));
+      n += __popc(todo);
+      if (high) bits[1] &= bits[1] - 1u;
+      else bits[0] &= bits[0] - 1u;
+      todo = __ballot_sync(0xffffffffu, (bits[0] | bits[1]) != 0u);
+    }
+    fits = n <= 32;
+  }
+  __syncwarp();
+  int count = 0;
+  for (int g0 = 0; fits && g0 < n; g0 += kBatch) {
+    float4 q[kBatch];
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
+    uint32_t take = 0u;                              // entry j of float4 i reaches the threshold
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i)
+      take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
+    if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
+#pragma unroll 1
+    for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo;) {
+      // one entry of every lane that has one, per step; read again (L1) rather than picked out of registers by index
+      const int bit = __ffs(take) - 1;
+      const int at = count + __popc(todo & ((1u << lane) - 1u));
+      if (take && at < kListCap) {
+        const int idx = w.groups[g0 + (bit >> 2)] + rg.lane_part + (bit & 3);
+        w.list[at] = idx < rg.V ? make_key(rank_value<kLogits>(__ldg(rg.row + idx), lse), static_cast<uint32_t>(idx)) : 0ull;
+      }
+      count += __popc(todo);
+      take &= take - 1u;
+      todo = __ballot_sync(0xffffffffu, take != 0u);
+    }
+  }
+  __syncwarp();
+  if (!fits || count > kListCap) top_of_many<kLogits>(rg, gm, groups, cut, Wc, lse, lane, w.list);
+  else if (count <= 32) keep_best<1>(w.list, count, Wc, lane);
+  else keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
+}
+
+// Algorithm 1 in one warp.  The children of a node are created together, numbered in rank order, and never gain on
+// each other (scores and priorities do not increase with the rank; ties go to the lower node index), so of every expanded
+// node only its best child not yet taken can be the next one: the pending queue is one entry per EXPANDED node (about B / W
+// of them instead of B), kept in registers -- entry i by lane i % 32 in register i / 32 as a key of two words, (priority,
+// ~index : depth), largest first.  A pop is two warp reductions; the entry then moves on to the next sibling.  The loop
+// only records the nodes it expands; their children are written out by the whole CTA afterwards (child j of expansion e is
+// node 1 + e * Wc + j).  It is one warp's dependent chain, so its length in instructions is its time: about 250 cycles a
+// pop (650 with the children written inside the loop and 64-bit keys; 900 with a queue indexed through local memory).
+// kSlots = registers per lane.
 // kMode: 0 = priority is the accumulated log-probability (the key's value is the node's score); 1 = priority
 // is the entropy of the node's depth; 2 = score + alpha * that entropy, formed as two rounded float operations.
-// depth_h[d] = entropy of the distribution the tokens of depth d + 1 were drawn from.  In modes 1 and 2 the
-// popped node's score is read back from shared memory.
+// depth_h[d] = entropy of the distribution the tokens of depth d + 1 were drawn from.
+struct Expansion { uint32_t lo; float score; };      // the expanded node: (~index : depth) as in the keys, its score
+
+__device__ __forceinline__ int key_node(uint32_t lo) { return static_cast<int>(0xFFFFFFu - (lo >> 8)); }
+
 template <int kSlots, int kMode>
-__device__ __forceinline__ int expand_tree(int lane, int N, int Wc, int B, int root, const float (*top_lp)[JET_MAX_WIDTH],
-                                           const int32_t (*top_tok)[JET_MAX_WIDTH], int32_t* s_parent,
-                                           int32_t* s_depth, int32_t* s_token, float* s_score,
-                                           const float* depth_h, float alpha) {
-  unsigned long long q[kSlots];
+__device__ __forceinline__ int expand_tree(int lane, int N, int Wc, int B, const float (*top_lp)[JET_MAX_WIDTH],
+                                           Expansion* made, const float* depth_h, float alpha) {
+  uint32_t hi[kSlots], lo[kSlots];                   // the entry's best pending child; both 0: none
+  float ps[kSlots];                                  // its parent's score
+  int tl[kSlots];                                    // where the sibling behind it is in the table of log-probabilities (its
+                                                     // rank in the low bits; 0: past the last rank the table has room for)
 #pragma unroll
-  for (int i = 0; i < kSlots; ++i) q[i] = 0ull;
-  auto queue_key = [](float score, int node, int dep) -> unsigned long long {
-    return (static_cast<unsigned long long>(f32_order(score)) << 32) |
-           (static_cast<unsigned long long>(0xFFFFFFu - static_cast<uint32_t>(node)) << 8) |
-           static_cast<unsigned long long>(dep);
-  };
-  if (lane == 0) {
-    s_parent[0] = -1; s_depth[0] = 0; s_token[0] = root; s_score[0] = 0.0f;
-    q[0] = queue_key(0.0f, 0, 0);
+  for (int i = 0; i < kSlots; ++i) {
+    hi[i] = lo[i] = 0u;
+    ps[i] = 0.0f;
+    tl[i] = 0;
   }
-  int n = 1;
-  while (n < B) {
-    unsigned long long best = 0ull;
+  const float* table = top_lp[0];
+  auto priority = [&](float score, int dep) -> uint32_t {      // of a node of depth dep >= 1
+    if constexpr (kMode == 1) return f32_order(depth_h[dep - 1]);
+    if constexpr (kMode == 2) return f32_order(__fadd_rn(score, __fmul_rn(alpha, depth_h[dep - 1])));
+    return f32_order(score);
+  };
+  auto depth_of = [](uint32_t node) { return max(static_cast<int>(node & 0xFFu), 1); };
+  int n = 1, entries = 0;
+  uint32_t node = 0xFFFFFFu << 8;                    // (~index : depth) of the node taken, the root first
+  float score = 0.0f;
+  for (;;) {
+    // the node taken gets its children (its depth is below N: see below)
+    const int d = static_cast<int>(node & 0xFFu);
+    if (lane == 0) made[entries] = {node, score};
+    const int first = n;
+    n += Wc;
+    if (n >= B) break;
+    if (d + 1 < N) {                                 // children at depth N are never expanded: taking one would only drop it
+      // (every lane forms the new entry and its keeper selects it: no indexed register array, which would live in local memory)
+      const uint32_t h = priority(__fadd_rn(score, table[d * JET_MAX_WIDTH]), d + 1);
+      const uint32_t l = ((0xFFFFFFu - static_cast<uint32_t>(first)) << 8) + static_cast<uint32_t>(d + 1);
 #pragma unroll
-    for (int i = 0; i < kSlots; ++i) best = q[i] > best ? q[i] : best;
-    best = warp_max_u64(best);
-    if (best == 0ull) break;                        // nothing pending
-    const int v = static_cast<int>(0xFFFFFFu - (static_cast<uint32_t>(best >> 8) & 0xFFFFFFu));
-    const int d = static_cast<int>(best & 0xFFull);
-    float sv;
-    if constexpr (kMode == 0) sv = key_value(best);
-    else sv = s_score[v];
-#pragma unroll
-    for (int i = 0; i < kSlots; ++i) if (q[i] == best) q[i] = 0ull;      // popped (only its keeper matches)
-    if (d < N) {
-      const int cnt = min(Wc, B - n);
-      const int j = (lane - n) & 31;                // child rank whose node n + j this lane keeps
-      if (j < cnt) {
-        const int u = n + j;
-        const float s = __fadd_rn(sv, top_lp[d][j]);
-        s_parent[u] = v; s_depth[u] = d + 1; s_token[u] = top_tok[d][j]; s_score[u] = s;
-        float prio = s;
-        if constexpr (kMode == 1) prio = depth_h[d];
-        if constexpr (kMode == 2) prio = __fadd_rn(s, __fmul_rn(alpha, depth_h[d]));
-        const unsigned long long key = queue_key(prio, u, d + 1);
-#pragma unroll
-        for (int i = 0; i < kSlots; ++i) if (i == (u >> 5)) q[i] = key;
+      for (int i = 0; i < kSlots; ++i) {
+        const bool here = entries == i * 32 + lane;
+        hi[i] = here ? h : hi[i];
+        lo[i] = here ? l : lo[i];
+        ps[i] = here ? score : ps[i];
+        tl[i] = here ? d * JET_MAX_WIDTH + 1 : tl[i];
       }
-      n += cnt;
-      if constexpr (kMode != 0) __syncwarp();          // the children's scores are read back when they are popped
+    }
+    ++entries;
+    // the priority of the sibling behind every entry's child, off the chain (with many registers only the moved entry's is
+    // worth forming, on it)
+    constexpr bool kAhead = kSlots <= 2;
+    uint32_t ahead[kAhead ? kSlots : 1];
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int i = 0; i < kSlots; ++i) ahead[i] = priority(__fadd_rn(ps[i], table[tl[i]]), depth_of(lo[i]));
+    }
+    uint32_t bh = hi[0], bl = lo[0];
+#pragma unroll
+    for (int i = 1; i < kSlots; ++i) {
+      const bool more = hi[i] > bh || (hi[i] == bh && lo[i] > bl);
+      bh = more ? hi[i] : bh;
+      bl = more ? lo[i] : bl;
+    }
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, bh);
+    node = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
+    if (node == 0u) break;                           // nothing pending
+    float parent_score = 0.0f;
+    int at = 0;
+    if constexpr (kMode != 0 || !kAhead) {
+#pragma unroll
+      for (int i = 0; i < kSlots; ++i) {
+        const bool hit = lo[i] == node;              // (a node is in one entry only)
+        parent_score = hit ? ps[i] : parent_score;
+        at = hit ? tl[i] : at;
+      }
+    }
+    if constexpr (kMode == 0) {
+      score = __uint_as_float((mh & 0x80000000u) ? (mh & 0x7FFFFFFFu) : ~mh);
+    } else {
+      const float own = __fadd_rn(parent_score, table[max(at - 1, 0)]);
+      score = __shfl_sync(0xffffffffu, own, __ffs(__ballot_sync(0xffffffffu, bl == node)) - 1);
+    }
+    // its entry moves on to the next sibling
+    if constexpr (!kAhead) ahead[0] = priority(__fadd_rn(parent_score, table[at]), depth_of(node));
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) {
+      const bool hit = lo[i] == node;
+      const int behind = tl[i] & (JET_MAX_WIDTH - 1);
+      const bool more = behind != 0 && behind < Wc;
+      hi[i] = hit ? (more ? ahead[kAhead ? i : 0] : 0u) : hi[i];
+      lo[i] = hit ? (more ? lo[i] - 256u : 0u) : lo[i];
+      tl[i] += hit ? 1 : 0;
     }
   }
-  return n;
+  return min(n, B);
 }
 
-constexpr int kExpThreads = 256;
+// What the scan left for one call, and how to read it.
+struct ScanView {
+  const float* rows;
+  int64_t batch_stride, depth_stride;
+  const float* gmax;                                 // [batch * N][slices * 32 R]
+  const double2* pairs;                              // [batch * N][slices] (reference, sum) of raw logits, or null
+  const double2* plogp;                              // [batch * N][slices] .x = sum(p * log p) with an entropy score, or null
+  int slices, rounds, vec;
+};
 
 template <int kMode>
 __global__ void __launch_bounds__(kExpThreads)
-tree_expand_kernel(const float* __restrict__ logp, int64_t batch_stride, int64_t depth_stride,
-                   const int32_t* __restrict__ root_token, int N, int Wc, int B, int nchunks,
-                   const unsigned long long* __restrict__ cand,
+tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, int N, int V, int Wc, int B, float alpha,
                    int32_t* __restrict__ parent_out, int32_t* __restrict__ depth_out,
                    int32_t* __restrict__ token_out, float* __restrict__ score_out,
                    uint32_t* __restrict__ anc_out, int32_t* __restrict__ n_nodes_out,
-                   const double* __restrict__ plogp_partial, float alpha, float* __restrict__ depth_entropy_out,
-                   const int32_t* __restrict__ node_budget) {
+                   float* __restrict__ depth_entropy_out, float* __restrict__ depth_lse_out,
+                   const int32_t* __restrict__ node_budget, const int32_t* __restrict__ len_src, int32_t* __restrict__ len_dst) {
   grid_dependency_wait();
   __shared__ int32_t s_top_tok[JET_MAX_DEPTH][JET_MAX_WIDTH];
-  __shared__ float s_top_lp[JET_MAX_DEPTH][JET_MAX_WIDTH];
-  __shared__ int32_t s_parent[JET_MAX_NODES], s_depth[JET_MAX_NODES], s_token[JET_MAX_NODES];
-  __shared__ float s_score[JET_MAX_NODES];
+  __shared__ float s_top_lp[JET_MAX_DEPTH + 1][JET_MAX_WIDTH];      // (one row more: the entry behind a row's last is read, not used)
+  __shared__ union {
+    TopScratch top[kExpWarps];
+    struct {
+      Expansion made[JET_MAX_NODES];
+      int32_t parent[JET_MAX_NODES];
+    } tree;
+  } sh;
   __shared__ float s_depth_h[JET_MAX_DEPTH];
   __shared__ int s_n;
 
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // this sequence's budget: B, or its own smaller one (the arrays are padded to B either way)
+  const int Bb = node_budget ? max(1, min(B, node_budget[b])) : B;
+  const int root = root_token[b];
+  if (len_dst && tid == kExpThreads - 1) len_dst[b] = len_src[b];
 
-  // ---- merge the per-slice candidates: depth d's W best of nchunks*Wc keys (keys are unique,
-  //      so "largest key below the previous winner" walks them in rank order)
-  for (int d = warp; d < N; d += kExpThreads / 32) {
+  // ---- per depth: log-sum-exp, entropy, the W best entries; one warp per row
+  for (int d = warp; d < N; d += kExpWarps) {
+    const size_t row_id = static_cast<size_t>(b) * N + d;
     if constexpr (kMode != 0) {
-      // entropy of row d: minus the sum of the slices' partial sums (fp64, fixed order), rounded once
-      const double* part = plogp_partial + (static_cast<size_t>(b) * N + d) * nchunks;
+      // entropy: minus the sum of the slices' partial sums (fp64, fixed order), rounded once
+      const double2* part = scan.plogp + row_id * scan.slices;
       double acc = 0.0;
-      for (int i = lane; i < nchunks; i += 32) acc += part[i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      for (int i = lane; i < scan.slices; i += 32) acc += part[i].x;
+      acc = warp_sum_f64(acc);
       if (lane == 0) {
         const float h = static_cast<float>(-acc);
         s_depth_h[d] = h;
-        if (depth_entropy_out) depth_entropy_out[static_cast<size_t>(b) * N + d] = h;
+        if (depth_entropy_out) depth_entropy_out[row_id] = h;
       }
     }
-    const unsigned long long* c = cand + (static_cast<size_t>(b) * N + d) * nchunks * Wc;
-    const int total = nchunks * Wc;
-    constexpr int kHeld = 16;                 // candidates a lane can keep in registers
-    unsigned long long held[kHeld];
-    const bool in_regs = total <= 32 * kHeld; // usual case: one pass over global memory, rounds on registers
-    if (in_regs) {
-#pragma unroll
-      for (int i = 0; i < kHeld; ++i) held[i] = lane + 32 * i < total ? c[lane + 32 * i] : 0ull;
+    const int groups = scan.slices * 32 * scan.rounds;
+    const RowGroups rg(scan.rows + b * scan.batch_stride + d * scan.depth_stride, V, scan.rounds, scan.vec, lane);
+    const float* gm = scan.gmax + row_id * groups;
+    TopScratch& w = sh.top[warp];
+    if (scan.pairs) {
+      top_of_row<true>(rg, gm, groups, Wc, [&] {
+        const double lse = row_lse(scan.pairs + row_id * scan.slices, scan.slices, lane);
+        if (lane == 0 && depth_lse_out) depth_lse_out[row_id] = static_cast<float>(lse);
+        return lse;
+      }, lane, w);
+    } else {
+      top_of_row<false>(rg, gm, groups, Wc, [] { return 0.0; }, lane, w);
     }
-    unsigned long long prev = ~0ull;
-    for (int r = 0; r < Wc; ++r) {
-      unsigned long long best = 0ull;
-      if (in_regs) {
-#pragma unroll
-        for (int i = 0; i < kHeld; ++i) if (held[i] < prev && held[i] > best) best = held[i];
-      } else {
-        for (int i = lane; i < total; i += 32) {
-          const unsigned long long k = c[i];
-          if (k < prev && k > best) best = k;
-        }
-      }
-      best = warp_max_u64(best);
-      if (lane == 0) {
-        const uint32_t t = key_index(best);
-        s_top_tok[d][r] = static_cast<int32_t>(t);
-        s_top_lp[d][r] = key_value(best);            // the key holds the value itself: no second look-up
-      }
-      prev = best;
+    if (lane < Wc) {
+      const unsigned long long k = w.list[lane];
+      s_top_tok[d][lane] = static_cast<int32_t>(key_index(k));
+      s_top_lp[d][lane] = key_value(k);              // the key holds the value itself: no second look-up
     }
+    __syncwarp();
   }
   __syncthreads();
 
-  // ---- Algorithm 1: one warp, queue in registers (as many per lane as the budget needs)
-  // this sequence's budget: B, or its own smaller one (the arrays are padded to B either way)
-  const int Bmax = B;
-  if (node_budget) B = max(1, min(B, node_budget[b]));
-  if (warp == 0) {
-    const int root = root_token[b];
+  // ---- Algorithm 1: one warp, as many queue registers per lane as the expanded nodes need
+  if (warp == 0 && Bb == 1) {
+    if (lane == 0) s_n = 1;
+  } else if (warp == 0) {
+    const int slots = ((Bb - 1 + Wc - 1) / Wc + 31) / 32;      // every expansion but the last adds Wc nodes
+    Expansion* made = sh.tree.made;
     int n;
-    if (B <= 32) n = expand_tree<1, kMode>(lane, N, Wc, B, root, s_top_lp, s_top_tok, s_parent, s_depth, s_token, s_score, s_depth_h, alpha);
-    else if (B <= 64) n = expand_tree<2, kMode>(lane, N, Wc, B, root, s_top_lp, s_top_tok, s_parent, s_depth, s_token, s_score, s_depth_h, alpha);
-    else if (B <= 128) n = expand_tree<4, kMode>(lane, N, Wc, B, root, s_top_lp, s_top_tok, s_parent, s_depth, s_token, s_score, s_depth_h, alpha);
-    else if (B <= 256) n = expand_tree<8, kMode>(lane, N, Wc, B, root, s_top_lp, s_top_tok, s_parent, s_depth, s_token, s_score, s_depth_h, alpha);
-    else n = expand_tree<JET_MAX_NODES / 32, kMode>(lane, N, Wc, B, root, s_top_lp, s_top_tok, s_parent, s_depth, s_token, s_score, s_depth_h, alpha);
+    if (slots <= 1) n = expand_tree<1, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    else if (slots <= 2) n = expand_tree<2, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    else if (slots <= 4) n = expand_tree<4, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    else n = expand_tree<JET_MAX_NODES / 32, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     if (lane == 0) s_n = n;
   }
   __syncthreads();
 
-  // ---- emit
-  const int n = s_n;
-  B = Bmax;
+  // ---- emit: one thread per node; its ancestors have descending indices, so its mask row is written word by word from
+  //      the last one down
+  static_assert(kExpThreads >= JET_MAX_NODES, "one thread per node");
+  const int n = s_n, v = tid;
+  const int words = (B + 31) / 32;
   const size_t o = static_cast<size_t>(b) * B;
-  for (int v = tid; v < B; v += kExpThreads) {
-    const bool live = v < n;
-    parent_out[o + v] = live ? s_parent[v] : -1;
-    depth_out[o + v] = live ? s_depth[v] : -1;
-    token_out[o + v] = live ? s_token[v] : -1;
-    if (score_out) score_out[o + v] = live ? s_score[v] : 0.0f;
+  int par = -1, dep = -1, tok = -1;
+  float sc = 0.0f;
+  if (v == 0) {
+    dep = 0;
+    tok = root;
+  } else if (v < n) {
+    const int e = (v - 1) / Wc, j = v - 1 - e * Wc;
+    const Expansion x = sh.tree.made[e];
+    par = key_node(x.lo);
+    dep = static_cast<int>(x.lo & 0xFFu) + 1;
+    tok = s_top_tok[dep - 1][j];
+    sc = __fadd_rn(x.score, s_top_lp[dep - 1][j]);
+  }
+  sh.tree.parent[v] = par;
+  if (v < B) {
+    parent_out[o + v] = par;
+    depth_out[o + v] = dep;
+    token_out[o + v] = tok;
+    if (score_out) score_out[o + v] = sc;
+  }
+  __syncthreads();
+  if (v < B) {
+    uint32_t* mask = anc_out + (o + v) * words;
+    int u = v < n ? v : -1;
+    for (int w = words - 1; w >= 0; --w) {
+      uint32_t bits = 0u;
+      while (u >= 0 && (u >> 5) == w) {
+        bits |= 1u << (u & 31);
+        u = sh.tree.parent[u];
+      }
+      mask[w] = bits;
+    }
   }
   if (tid == 0) n_nodes_out[b] = n;
-  const int words = (B + 31) / 32;
-  for (int i = tid; i < B * words; i += kExpThreads) {
-    const int v = i / words, w = i - v * words;
-    uint32_t bits = 0u;
-    if (v < n) {
-      for (int u = v; u >= 0; u = s_parent[u])
-        if ((u >> 5) == w) bits |= 1u << (u & 31);
-    }
-    anc_out[o * words + i] = bits;
+}
+
+// How the rows are cut: rounds of 4096 entries per block.  More rounds keep loads in flight under arithmetic, fewer give
+// more blocks: the most (up to 4) that still leave about six blocks per SM.
+struct ScanPlan { int rounds, slices, groups; };
+ScanPlan scan_plan(int batch, int N, int V) {
+  ScanPlan p{1, 0, 0};
+  const int64_t rows = static_cast<int64_t>(batch) * N;
+  for (int r = 4; r >= 1; r /= 2) {
+    p.rounds = r;
+    p.slices = static_cast<int>((static_cast<int64_t>(V) + kRoundChunk * r - 1) / (kRoundChunk * r));
+    if (rows * p.slices >= 888) break;
   }
+  p.groups = p.slices * 32 * p.rounds;
+  return p;
 }
 
-int chunks_for(int V) { return (V + kTopChunk - 1) / kTopChunk; }
-
-size_t cand_bytes(int batch, int N, int V, int W) {
-  const size_t Wc = static_cast<size_t>(W < V ? W : V);
-  return round_up(static_cast<size_t>(batch) * N * chunks_for(V) * Wc * sizeof(unsigned long long), 256);
+// Workspace: group maxima, then (raw logits) the log-sum-exp pairs, then (entropy scores) the p * log p sums.
+size_t gmax_bytes(int batch, int N, int V) {
+  return round_up(static_cast<size_t>(batch) * N * scan_plan(batch, N, V).groups * sizeof(float), 256);
+}
+size_t sums_bytes(int batch, int N, int V) {
+  return round_up(static_cast<size_t>(batch) * N * scan_plan(batch, N, V).slices * sizeof(double2), 256);
 }
 
-// Checks and launches shared by the two entry points (score_mode: JET_SCORE_*).
-jet_status tree_build_launch(const float* logp, int64_t logp_batch_stride, int64_t logp_depth_stride,
+// Checks and launches shared by the entry points (score_mode: JET_SCORE_*).
+jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t depth_stride,
                              const int32_t* root_token, int batch, int N, int V, int W, int B, int score_mode,
                              float alpha, int32_t* parent, int32_t* depth, int32_t* token, float* score,
                              uint32_t* anc_mask, int32_t* n_nodes, float* depth_entropy,
                              const int32_t* node_budget, void* workspace, size_t workspace_bytes, size_t need,
-                             void* stream, bool from_logits = false, float* depth_lse = nullptr) {
-  if (!logp || !root_token || !parent || !depth || !token || !anc_mask || !n_nodes)
+                             void* stream, bool from_logits = false, float* depth_lse = nullptr,
+                             const int32_t* len_src = nullptr, int32_t* len_dst = nullptr) {
+  if (!rows || !root_token || !parent || !depth || !token || !anc_mask || !n_nodes)
     return JET_ERR_INVALID_ARG;
   if (batch < 1 || batch > 65535 || N < 1 || N > JET_MAX_DEPTH || W < 1 || W > JET_MAX_WIDTH || V < 1 ||
-      B < 1 || B > JET_MAX_NODES || logp_depth_stride < V || logp_batch_stride < 0)
+      B < 1 || B > JET_MAX_NODES || depth_stride < V || batch_stride < 0)
     return JET_ERR_INVALID_ARG;
   if (score_mode < JET_SCORE_ACCUM_LOGP || score_mode > JET_SCORE_HYBRID) return JET_ERR_INVALID_ARG;
   if (score_mode == JET_SCORE_HYBRID && !(alpha == alpha && alpha > -INFINITY && alpha < INFINITY)) return JET_ERR_INVALID_ARG;
-  if (!aligned(logp, 4)) return JET_ERR_INVALID_ARG;
+  if (!aligned(rows, 4)) return JET_ERR_INVALID_ARG;
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
 
   const int Wc = W < V ? W : V;
-  const int nchunks = chunks_for(V);
-  const bool vec_ok = aligned(logp, 16) && logp_batch_stride % 4 == 0 && logp_depth_stride % 4 == 0;
+  const ScanPlan plan = scan_plan(batch, N, V);
+  const bool vec = aligned(rows, 16) && batch_stride % 4 == 0 && depth_stride % 4 == 0;
+  const bool scored = score_mode != JET_SCORE_ACCUM_LOGP;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  auto* cand = static_cast<unsigned long long*>(workspace);
-  auto* plogp = reinterpret_cast<double*>(static_cast<uint8_t*>(workspace) + cand_bytes(batch, N, V, W));
-  const double* no_lse = nullptr;
-  float* no_out = nullptr;
+  auto* ws = static_cast<uint8_t*>(workspace);
+  auto* gmax = reinterpret_cast<float*>(ws);
+  ws += gmax_bytes(batch, N, V);
+  auto* pairs = from_logits ? reinterpret_cast<double2*>(ws) : nullptr;
+  if (from_logits) ws += sums_bytes(batch, N, V);
+  auto* plogp = scored ? reinterpret_cast<double2*>(ws) : nullptr;
+  const dim3 grid(plan.slices, N, batch);
+  auto scan = [&](auto kernel, double2* sums) {
+    launch_dependent(kernel, grid, dim3(kScanThreads), st, rows, batch_stride, depth_stride, V, plan.rounds, vec, gmax, pairs, sums);
+  };
   if (from_logits) {
-    double* lse_part = plogp + round_up(static_cast<size_t>(batch) * N * nchunks * sizeof(double), 256) / sizeof(double);
-    launch_dependent(lse_partial_kernel, dim3(nchunks, N, batch), dim3(kTopThreads), st,
-        logp, logp_batch_stride, logp_depth_stride, V, nchunks, vec_ok, lse_part);
-    const double* lse_in = lse_part;
-    if (score_mode == JET_SCORE_ACCUM_LOGP)
-      launch_dependent(topw_partial_kernel<false, true>, dim3(nchunks, N, batch), dim3(kTopThreads), st,
-          logp, logp_batch_stride, logp_depth_stride, V, Wc, nchunks, vec_ok, cand, static_cast<double*>(nullptr),
-          lse_in, depth_lse);
-    else
-      launch_dependent(topw_partial_kernel<true, true>, dim3(nchunks, N, batch), dim3(kTopThreads), st,
-          logp, logp_batch_stride, logp_depth_stride, V, Wc, nchunks, vec_ok, cand, plogp, lse_in, depth_lse);
-  } else if (score_mode == JET_SCORE_ACCUM_LOGP) {
-    launch_dependent(topw_partial_kernel<false, false>, dim3(nchunks, N, batch), dim3(kTopThreads), st,
-        logp, logp_batch_stride, logp_depth_stride, V, Wc, nchunks, vec_ok, cand, static_cast<double*>(nullptr),
-        no_lse, no_out);
+    scan(row_scan_kernel<kScanSum>, pairs);
+    if (scored) scan(row_scan_kernel<kScanLogitEntropy>, plogp);
+  } else if (scored) {
+    scan(row_scan_kernel<kScanEntropy>, plogp);
   } else {
-    launch_dependent(topw_partial_kernel<true, false>, dim3(nchunks, N, batch), dim3(kTopThreads), st,
-        logp, logp_batch_stride, logp_depth_stride, V, Wc, nchunks, vec_ok, cand, plogp, no_lse, no_out);
+    scan(row_scan_kernel<kScanMax>, nullptr);
   }
-  if (score_mode == JET_SCORE_ACCUM_LOGP) {
-    launch_dependent(tree_expand_kernel<0>, dim3(batch), dim3(kExpThreads), st, logp, logp_batch_stride, logp_depth_stride,
-        root_token, N, Wc, B, nchunks, cand, parent, depth, token, score, anc_mask, n_nodes,
-        static_cast<const double*>(nullptr), 0.0f, static_cast<float*>(nullptr), node_budget);
-    return launch_status();
-  }
-  if (score_mode == JET_SCORE_ENTROPY)
-    launch_dependent(tree_expand_kernel<1>, dim3(batch), dim3(kExpThreads), st, logp, logp_batch_stride, logp_depth_stride,
-        root_token, N, Wc, B, nchunks, cand, parent, depth, token, score, anc_mask, n_nodes,
-        static_cast<const double*>(plogp), 0.0f, depth_entropy, node_budget);
-  else
-    launch_dependent(tree_expand_kernel<2>, dim3(batch), dim3(kExpThreads), st, logp, logp_batch_stride, logp_depth_stride,
-        root_token, N, Wc, B, nchunks, cand, parent, depth, token, score, anc_mask, n_nodes,
-        static_cast<const double*>(plogp), alpha, depth_entropy, node_budget);
+  const ScanView view{rows, batch_stride, depth_stride, gmax, pairs, plogp, plan.slices, plan.rounds, vec ? 1 : 0};
+  auto expand = score_mode == JET_SCORE_ACCUM_LOGP ? tree_expand_kernel<0>
+                : score_mode == JET_SCORE_ENTROPY  ? tree_expand_kernel<1> : tree_expand_kernel<2>;
+  launch_dependent(expand, dim3(batch), dim3(kExpThreads), st, view, root_token, N, V, Wc, B, alpha, parent, depth, token,
+                   score, anc_mask, n_nodes, depth_entropy, depth_lse, node_budget, len_src, len_dst);
   return launch_status();
 }
 
@@ -468,7 +732,17 @@ jet_status tree_build_launch(const float* logp, int64_t logp_batch_stride, int64
 
 extern "C" size_t jet_tree_build_workspace_bytes(int batch, int N, int V, int W) {
   if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
-  return jet::cand_bytes(batch, N, V, W);
+  return jet::gmax_bytes(batch, N, V);
+}
+
+extern "C" size_t jet_tree_build_scored_workspace_bytes(int batch, int N, int V, int W) {
+  if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
+  return jet::gmax_bytes(batch, N, V) + jet::sums_bytes(batch, N, V);
+}
+
+extern "C" size_t jet_tree_build_logits_workspace_bytes(int batch, int N, int V, int W) {
+  if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
+  return jet::gmax_bytes(batch, N, V) + 2 * jet::sums_bytes(batch, N, V);
 }
 
 extern "C" jet_status jet_tree_build(const float* logp, int64_t logp_batch_stride,
@@ -477,16 +751,10 @@ extern "C" jet_status jet_tree_build(const float* logp, int64_t logp_batch_strid
                                      int32_t* depth, int32_t* token, float* score,
                                      uint32_t* anc_mask, int32_t* n_nodes, void* workspace,
                                      size_t workspace_bytes, void* stream) {
-  const size_t need = (batch >= 1 && N >= 1 && V >= 1 && W >= 1) ? jet::cand_bytes(batch, N, V, W) : 0;
+  const size_t need = jet_tree_build_workspace_bytes(batch, N, V, W);
   return jet::tree_build_launch(logp, logp_batch_stride, logp_depth_stride, root_token, batch, N, V, W, B,
                                 JET_SCORE_ACCUM_LOGP, 0.0f, parent, depth, token, score, anc_mask, n_nodes, nullptr,
                                 nullptr, workspace, workspace_bytes, need, stream);
-}
-
-extern "C" size_t jet_tree_build_scored_workspace_bytes(int batch, int N, int V, int W) {
-  if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
-  return jet::cand_bytes(batch, N, V, W) +
-         jet::round_up(static_cast<size_t>(batch) * N * jet::chunks_for(V) * sizeof(double), 256);
 }
 
 extern "C" jet_status jet_tree_build_scored(const float* logp, int64_t logp_batch_stride,
@@ -500,12 +768,6 @@ extern "C" jet_status jet_tree_build_scored(const float* logp, int64_t logp_batc
   return jet::tree_build_launch(logp, logp_batch_stride, logp_depth_stride, root_token, batch, N, V, W, B, score_mode,
                                 alpha, parent, depth, token, score, anc_mask, n_nodes, depth_entropy, node_budget,
                                 workspace, workspace_bytes, need, stream);
-}
-
-extern "C" size_t jet_tree_build_logits_workspace_bytes(int batch, int N, int V, int W) {
-  if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
-  return jet_tree_build_scored_workspace_bytes(batch, N, V, W) +
-         jet::round_up(static_cast<size_t>(batch) * N * jet::chunks_for(V) * 2 * sizeof(double), 256);
 }
 
 extern "C" jet_status jet_tree_build_logits(const float* logits, int64_t logits_batch_stride,
