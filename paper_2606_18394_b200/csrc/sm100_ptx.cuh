@@ -171,6 +171,15 @@ __device__ __forceinline__ void umma_commit2(uint32_t bar, uint16_t cta_mask) {
                ::"r"(bar), "h"(cta_mask) : "memory");
 }
 
+// TMA load into this CTA's shared memory whose bytes may be credited to the barrier of either CTA of the pair
+// (bar = a cluster address, see map_to_rank).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+
 // CTA-wide barrier as an explicit instruction.  Unlike __syncthreads() the compiler can neither drop one of
 // two adjacent barriers nor merge them, so code paths that are compiled separately for different warps of
 // a CTA (and contain different work between the barriers) stay in step barrier for barrier.

@@ -171,7 +171,7 @@ accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks,
 
 // ------------------------------------------------------------------------------------------------
 // lm_head_argmax_kernel: the target's greedy prediction straight from the final hidden states -- the logits
-// never exist in memory.  One CTA computes a tile of 128 vocabulary entries for MT * 128 rows:
+// never exist in memory.  One CTA computes a tile of 128 vocabulary entries for up to 128 rows:
 //   D[row, token] = sum_k X[row, k] * W[token, k]      (bf16 operands, fp32 accumulation in TMEM)
 // with the LM-head weights streamed once through a ring of shared-memory stages by TMA (the hidden states come
 // along per 64-wide K chunk, out of L2), tcgen05.mma issued by one thread, and an epilogue in which the thread
@@ -184,15 +184,10 @@ constexpr int kLmThreads = 192;
 constexpr uint32_t kLmWaitRounds = 1u << 17;        // bounded waits: about a second in total
 constexpr uint32_t kLmWaitHintNs = 8192;
 
-template <int MT>
-struct LmCfg {
-  // (two stages with two row groups: 98 KB, so that two CTAs share an SM -- with 256 TMEM columns each -- and one
-  //  CTA's epilogue runs under the other's weight stream: 335 -> 319 us at 256 rows against four stages and one CTA)
-  static constexpr int kStages = MT == 1 ? 3 : 2;
-  static constexpr int kStageBytes = (1 + MT) * kLmBlockBytes;
-  static constexpr int kSmemBytes = kStages * kStageBytes + 2048;
-  static constexpr int kTmemCols = 128 * MT;
-};
+// (three stages: 98 KB, two CTAs per SM, so that one CTA's epilogue runs under the other's weight stream)
+constexpr int kLmStages = 3;
+constexpr int kLmStageBytes = 2 * kLmBlockBytes;
+constexpr int kLmSmemBytes = kLmStages * kLmStageBytes + 2048;
 
 __device__ __forceinline__ bool lm_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
   for (uint32_t i = 0; i < kLmWaitRounds; ++i) {
@@ -203,17 +198,15 @@ __device__ __forceinline__ bool lm_wait(uint32_t bar, uint32_t parity, volatile 
   return false;
 }
 
-template <int MT>
 __global__ void __launch_bounds__(kLmThreads)
 lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w, int rows, int V,
                       int d, unsigned long long* __restrict__ keys, int32_t* __restrict__ status) {
-  using C = LmCfg<MT>;
-  constexpr int S = C::kStages;
+  constexpr int S = kLmStages;
   extern __shared__ uint8_t lm_smem_raw[];
   const uint32_t base = (ptx::smem_u32(lm_smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = lm_smem_raw + (base - ptx::smem_u32(lm_smem_raw));
-  const uint32_t sBar = base + S * C::kStageBytes;
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + S * C::kStageBytes + 256);
+  const uint32_t sBar = base + S * kLmStageBytes;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + S * kLmStageBytes + 256);
   volatile uint32_t* abort_flag = tmem_slot + 1;
   auto full = [&](int s) { return sBar + 8u * s; };
   auto empty = [&](int s) { return sBar + 8u * (S + s); };
@@ -231,7 +224,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     ptx::prefetch_tmap(&tm_x);
     ptx::prefetch_tmap(&tm_w);
   } else if (warp == 1) {
-    ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), C::kTmemCols);
+    ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), kLmBN);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -241,7 +234,6 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   grid_dependency_wait();
 
   const int n0 = blockIdx.x * kLmBN;                  // first vocabulary entry of this tile
-  const int row0 = blockIdx.y * (kLmBM * MT);         // first row of this CTA's row group
   const int KC = d / kLmBK;
 
   if (warp == 0) {
@@ -249,11 +241,10 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       for (int kc = 0; kc < KC; ++kc) {
         const int s = kc % S;
         if (kc >= S && !lm_wait(empty(s), ((kc / S) - 1) & 1, abort_flag)) break;
-        const uint32_t dst = base + s * C::kStageBytes;
-        ptx::mbar_arrive_expect_tx(full(s), C::kStageBytes);
+        const uint32_t dst = base + s * kLmStageBytes;
+        ptx::mbar_arrive_expect_tx(full(s), kLmStageBytes);
         ptx::tma_load_2d(dst, &tm_w, full(s), kc * kLmBK, n0);
-        for (int mt = 0; mt < MT; ++mt)
-          ptx::tma_load_2d(dst + (1 + mt) * kLmBlockBytes, &tm_x, full(s), kc * kLmBK, row0 + mt * kLmBM);
+        ptx::tma_load_2d(dst + kLmBlockBytes, &tm_x, full(s), kc * kLmBK, 0);
       }
     }
   } else if (warp == 1) {
@@ -265,16 +256,13 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       ptx::tc_fence_after();
-      const uint64_t desc_w = ptx::smem_desc_sw128(base + s * C::kStageBytes, 0);
+      const uint64_t desc_w = ptx::smem_desc_sw128(base + s * kLmStageBytes, 0);
+      const uint64_t desc_x = ptx::smem_desc_sw128(base + s * kLmStageBytes + kLmBlockBytes, 0);
       if (ptx::elect_one()) {
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          const uint64_t desc_x = ptx::smem_desc_sw128(base + s * C::kStageBytes + (1 + mt) * kLmBlockBytes, 0);
-#pragma unroll
-          for (int k4 = 0; k4 < kLmBK / 16; ++k4)
-            ptx::umma_ss(tmem_base + mt * kLmBN, desc_x + static_cast<uint64_t>((k4 * 32) >> 4),
-                         desc_w + static_cast<uint64_t>((k4 * 32) >> 4), idesc, (kc > 0 || k4 > 0) ? 1u : 0u);
-        }
+        for (int k4 = 0; k4 < kLmBK / 16; ++k4)
+          ptx::umma_ss(tmem_base, desc_x + static_cast<uint64_t>((k4 * 32) >> 4), desc_w + static_cast<uint64_t>((k4 * 32) >> 4),
+                       idesc, (kc > 0 || k4 > 0) ? 1u : 0u);
         ptx::umma_commit(empty(s));
         if (kc == KC - 1) ptx::umma_commit(tmem_full);
       }
@@ -285,61 +273,300 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     if (__all_sync(0xffffffffu, ok)) {
       ptx::tc_fence_after();
       const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+      const int row = (warp & 3) * 32 + lane;
+      float best = 0.0f;
+      uint32_t best_idx = 0xFFFFFFFFu;
 #pragma unroll 1
-      for (int mt = 0; mt < MT; ++mt) {
-        const int row = row0 + mt * kLmBM + (warp & 3) * 32 + lane;
-        float best = 0.0f;
-        uint32_t best_idx = 0xFFFFFFFFu;
-#pragma unroll 1
-        for (int c = 0; c < kLmBN / 32; ++c) {
-          uint32_t x[32];
-          ptx::tmem_ld32(t_lane + mt * kLmBN + c * 32, x);
-          ptx::tmem_wait_ld();
+      for (int c = 0; c < kLmBN / 32; ++c) {
+        uint32_t x[32];
+        ptx::tmem_ld32(t_lane + c * 32, x);
+        ptx::tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const uint32_t col = static_cast<uint32_t>(n0 + c * 32 + j);       // ascending: ties keep the lowest id
-            const float vj = __uint_as_float(x[j]);
-            if (col < static_cast<uint32_t>(V) && (best_idx == 0xFFFFFFFFu || vj > best)) { best = vj; best_idx = col; }
-          }
+        for (int j = 0; j < 32; ++j) {
+          const uint32_t col = static_cast<uint32_t>(n0 + c * 32 + j);       // ascending: ties keep the lowest id
+          const float vj = __uint_as_float(x[j]);
+          if (col < static_cast<uint32_t>(V) && (best_idx == 0xFFFFFFFFu || vj > best)) { best = vj; best_idx = col; }
         }
-        if (row < rows && best_idx != 0xFFFFFFFFu) atomicMax(keys + row, make_key(best, best_idx));
       }
+      if (row < rows && best_idx != 0xFFFFFFFFu) atomicMax(keys + row, make_key(best, best_idx));
     }
   }
   ptx::tc_fence_before();
   ptx::cta_sync();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, C::kTmemCols);
+    ptx::tmem_dealloc(tmem_base, kLmBN);
   }
   if (tid == 0 && *abort_flag && status) *status = JET_ERR_TIMEOUT;
 }
 
-template <int MT>
 jet_status launch_lm_head(const CUtensorMap& tx, const CUtensorMap& tw, int rows, int V, int d, unsigned long long* keys,
                           int32_t* status, cudaStream_t st) {
-  using C = LmCfg<MT>;
   static std::atomic<int> configured[64];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return JET_ERR_CUDA;
   if (configured[dev].load(std::memory_order_acquire) == 0) {
-    if (cudaFuncSetAttribute(lm_head_argmax_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
+    if (cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLmSmemBytes) != cudaSuccess) {
       cudaGetLastError();
       return JET_ERR_CUDA;
     }
     configured[dev].store(1, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((V + kLmBN - 1) / kLmBN, (rows + kLmBM * MT - 1) / (kLmBM * MT));
+  cfg.gridDim = dim3((V + kLmBN - 1) / kLmBN);
   cfg.blockDim = dim3(kLmThreads);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cfg.dynamicSmemBytes = kLmSmemBytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, lm_head_argmax_kernel<MT>, tx, tw, rows, V, d, keys, status) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, lm_head_argmax_kernel, tx, tw, rows, V, d, keys, status) != cudaSuccess) {
+    cudaGetLastError();
+    return JET_ERR_CUDA;
+  }
+  return JET_OK;
+}
+
+// ------------------------------------------------------------------------------------------------
+// lm_head_argmax_pair_kernel: the same for more than 128 rows, where one pass over the weights is enough arithmetic to make
+// the tensor cores the bound.  Persistent CTA pairs (clusters of two, tcgen05 cta_group::2): every product is one M = 256
+// instruction -- 128 rows in each CTA, the weight rows of the tile split between the two -- and a pair keeps TWO
+// accumulators of up to 256 columns in TMEM, fed from the same ring stage:
+//   kRows2 = false  256 rows against two weight blocks side by side (129 .. 256 rows)
+//   kRows2 = true   two blocks of 256 rows against one weight block (more rows, in groups of 512)
+// so a stage of 48 KB per CTA carries 2 x 4 instructions, about 50 bytes of L2 -> SM traffic per SM and clock (a 256 x 256 tile
+// needs 62, two or four 128-row groups on one CTA as before needed 80 - 96 and re-read the weight block from shared memory for
+// each).  The host picks the block width so that the tiles divide evenly over the pairs.  One warpgroup per
+// accumulator scans it for (largest value, lowest token id) while the other accumulator's last products and the next
+// tile's first loads run.  256 rows x 4096 x 151936: 319 -> 244 us (1305 TFLOP/s, 5.1 TB/s); 512 rows:
+// 712 -> 437 us (1459 TFLOP/s).
+// Warp roles per CTA: 0 = TMA producer (its own rows and its half of the weight block; the bytes of both CTAs are credited to
+// the even CTA's barrier), 1 = MMA issue (even CTA only), 2 = TMEM allocation, 4 .. 11 = epilogue.
+constexpr int kLpThreads = 384;
+constexpr int kLpStages = 4;
+constexpr int kLpStageBytes = 3 * kLmBlockBytes;
+constexpr int kLpSmemBytes = kLpStages * kLpStageBytes + 1024 + 1024;
+
+struct LpBars { enum { kFull = 0, kEmpty = kLpStages, kAccFull = 2 * kLpStages, kAccEmpty = kAccFull + 2, kCount = kAccEmpty + 2 }; };
+
+template <bool kRows2>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLpThreads, 1)
+lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w, int rows, int V,
+                           int d, int bn, int tiles, unsigned long long* __restrict__ keys, int32_t* __restrict__ status) {
+  constexpr int S = kLpStages;
+  constexpr int kXBlocks = kRows2 ? 2 : 1, kWBlocks = kRows2 ? 1 : 2;
+  extern __shared__ uint8_t lm_smem_raw[];
+  const uint32_t base = (ptx::smem_u32(lm_smem_raw) + 1023u) & ~1023u;
+  uint8_t* gen = lm_smem_raw + (base - ptx::smem_u32(lm_smem_raw));
+  const uint32_t sBar = base + S * kLpStageBytes;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + S * kLpStageBytes + 256);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+  auto bar = [&](int i) { return sBar + 8u * i; };
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = ptx::cluster_ctarank();
+
+  if (warp == 0 && lane == 0) {
+    for (int s = 0; s < S; ++s) {
+      ptx::mbar_init(bar(LpBars::kFull + s), 1);
+      ptx::mbar_init(bar(LpBars::kEmpty + s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      ptx::mbar_init(bar(LpBars::kAccFull + a), 1);
+      ptx::mbar_init(bar(LpBars::kAccEmpty + a), 8);          // the four warps of an accumulator's warpgroup, both CTAs
+    }
+    ptx::fence_mbar_init();
+    *abort_flag = 0u;
+    ptx::prefetch_tmap(&tm_x);
+    ptx::prefetch_tmap(&tm_w);
+  } else if (warp == 2) {
+    ptx::tmem_alloc2(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+    ptx::tmem_relinquish2();
+  }
+  ptx::tc_fence_before();
+  ptx::cta_sync();
+  ptx::cluster_sync_all();                           // both CTAs' barriers exist
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();
+
+  const int KC = d / kLmBK;
+  const int pairs = gridDim.x / 2, pair = blockIdx.x / 2;
+  const int group_rows = kRows2 ? 512 : 256;
+  const int groups = (rows + group_rows - 1) / group_rows;
+  const int half = bn / 2;                           // weight rows of a block that each CTA loads
+  const uint32_t stage_tx = static_cast<uint32_t>(kXBlocks * kLmBlockBytes + kWBlocks * half * 128);
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      for (int t = pair; t < tiles && ok; t += pairs) {
+        for (int g = 0; g < groups && ok; ++g) {
+          const int row0 = g * group_rows + static_cast<int>(rank) * kLmBM;
+          const int w0 = t * (kWBlocks * bn) + static_cast<int>(rank) * half;
+          for (int kc = 0; kc < KC; ++kc, ++it) {
+            const int s = it % S;
+            if (it >= S && !lm_wait(bar(LpBars::kEmpty + s), ((it / S) - 1) & 1, abort_flag)) { ok = false; break; }
+            const uint32_t dst = base + s * kLpStageBytes;
+            const uint32_t full = ptx::map_to_rank(bar(LpBars::kFull + s), 0);
+            if (rank == 0) ptx::mbar_arrive_expect_tx(bar(LpBars::kFull + s), 2 * stage_tx);
+            for (int x = 0; x < kXBlocks; ++x)
+              ptx::tma_load_2d_pair(dst + x * kLmBlockBytes, &tm_x, full, kc * kLmBK, row0 + x * 256);
+            for (int w = 0; w < kWBlocks; ++w)
+              ptx::tma_load_2d_pair(dst + (kXBlocks + w) * kLmBlockBytes, &tm_w, full, kc * kLmBK, w0 + w * bn);
+          }
+        }
+      }
+      // after a wait that gave up: copies in flight land within microseconds; stay until they surely have
+      if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+    }
+  } else if (warp == 1 && rank == 0) {
+    const uint32_t idesc = ptx::umma_idesc_bf16(2 * kLmBM, bn, false);
+    int it = 0, item = 0;
+    bool ok = true;
+    for (int t = pair; t < tiles && ok; t += pairs) {
+      for (int g = 0; g < groups && ok; ++g, ++item) {
+        for (int kc = 0; kc < KC && ok; ++kc, ++it) {
+          const int s = it % S;
+          ok = __all_sync(0xffffffffu, lm_wait(bar(LpBars::kFull + s), (it / S) & 1, abort_flag));
+          if (!ok) break;
+          const uint32_t stage = base + s * kLpStageBytes;
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            if (kc == 0 && item > 0) {               // the tile before has been read out of this accumulator
+              ok = __all_sync(0xffffffffu, lm_wait(bar(LpBars::kAccEmpty + a), (item - 1) & 1, abort_flag));
+              if (!ok) break;
+            }
+            ptx::tc_fence_after();
+            const uint64_t desc_x = ptx::smem_desc_sw128(stage + (kRows2 ? a : 0) * kLmBlockBytes, 0);
+            const uint64_t desc_w = ptx::smem_desc_sw128(stage + (kXBlocks + (kRows2 ? 0 : a)) * kLmBlockBytes, 0);
+            if (ptx::elect_one()) {
+#pragma unroll
+              for (int k4 = 0; k4 < kLmBK / 16; ++k4)
+                ptx::umma_ss2(tmem_base + a * 256, desc_x + static_cast<uint64_t>((k4 * 32) >> 4),
+                              desc_w + static_cast<uint64_t>((k4 * 32) >> 4), idesc, (kc > 0 || k4 > 0) ? 1u : 0u);
+              if (a == 1) ptx::umma_commit2(bar(LpBars::kEmpty + s), 3);
+              if (kc == KC - 1) ptx::umma_commit2(bar(LpBars::kAccFull + a), 3);
+            }
+            __syncwarp();
+          }
+        }
+      }
+    }
+  } else if (warp >= 4) {
+    const int a = (warp - 4) >> 2;                   // this warpgroup's accumulator
+    const uint32_t t_acc = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + a * 256;
+    const uint32_t acc_empty = ptx::map_to_rank(bar(LpBars::kAccEmpty + a), 0);
+    float best = -INFINITY;
+    uint32_t best_idx = 0xFFFFFFFFu;                 // none yet
+    int row = 0, item = 0;
+    bool ok = true;
+    for (int t = pair; t < tiles && ok; t += pairs) {
+      const int n0 = t * (kWBlocks * bn) + (kRows2 ? 0 : a * bn);      // first token of this accumulator's columns
+      const int cols = max(0, min(bn, V - n0));
+      for (int g = 0; g < groups && ok; ++g, ++item) {
+        row = g * group_rows + (kRows2 ? a * 256 : 0) + static_cast<int>(rank) * kLmBM + (warp & 3) * 32 + lane;
+        ok = __all_sync(0xffffffffu, lm_wait(bar(LpBars::kAccFull + a), item & 1, abort_flag));
+        if (!ok) break;
+        ptx::tc_fence_after();
+        if (groups > 1) { best = -INFINITY; best_idx = 0xFFFFFFFFu; }
+#pragma unroll 1
+        for (int c = 0; c < cols; c += 32) {
+          uint32_t x[32];
+          ptx::tmem_ld32(t_acc + c, x);
+          ptx::tmem_wait_ld();
+          if (c + 32 > cols) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) if (c + j >= cols) x[j] = 0xFF800000u;
+          }
+          float m = __uint_as_float(x[0]);
+#pragma unroll
+          for (int j = 1; j < 32; ++j) m = fmaxf(m, __uint_as_float(x[j]));
+          if (m > best || (best_idx == 0xFFFFFFFFu && m == best)) {      // (ascending tokens: a tie keeps the lower id)
+            best = m;
+            int at = 0;
+#pragma unroll
+            for (int j = 31; j >= 0; --j) at = __uint_as_float(x[j]) == m ? j : at;
+            best_idx = static_cast<uint32_t>(n0 + c + at);
+          }
+        }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive_peer(acc_empty);
+        if (groups > 1 && row < rows && best_idx != 0xFFFFFFFFu) atomicMax(keys + row, make_key(best, best_idx));
+      }
+    }
+    // one group of rows: a row keeps its best over all of the pair's tiles
+    if (groups == 1 && row < rows && best_idx != 0xFFFFFFFFu) atomicMax(keys + row, make_key(best, best_idx));
+  }
+  ptx::tc_fence_before();
+  ptx::cta_sync();
+  ptx::cluster_sync_all();                           // neither CTA's barriers or TMEM go before both are done
+  if (warp == 2) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc2(tmem_base, 512);
+  }
+  if (tid == 0 && *abort_flag && status) *status = JET_ERR_TIMEOUT;
+}
+
+// Width of a weight block: the multiple of 16 up to 256 for which the pair with the most tiles does the least work (a tile
+// costs its width and, for its first loads and last scan, about as much as 8 more columns).
+int lm_block_width(int V, int pairs, int w_blocks) {
+  int best = 256;
+  double best_cost = -1.0;
+  for (int bn = 96; bn <= 256; bn += 16) {
+    const int tiles = (V + w_blocks * bn - 1) / (w_blocks * bn);
+    const double cost = static_cast<double>((tiles + pairs - 1) / pairs) * (w_blocks * bn + 8);
+    if (best_cost < 0.0 || cost <= best_cost) { best = bn; best_cost = cost; }
+  }
+  return best;
+}
+
+template <bool kRows2>
+jet_status launch_lm_head_pair(const CUtensorMap& tx, const void* weight, int rows, int V, int d, unsigned long long* keys,
+                               int32_t* status, cudaStream_t st) {
+  static std::atomic<int> pairs_of[64];              // per device: CTA pairs that fit at once
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return JET_ERR_CUDA;
+  auto kernel = lm_head_argmax_pair_kernel<kRows2>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kLpThreads);
+  cfg.dynamicSmemBytes = kLpSmemBytes;
+  cfg.stream = st;
+  int pairs = pairs_of[dev].load(std::memory_order_acquire);
+  if (pairs == 0) {
+    cudaLaunchAttribute cluster[1];
+    cluster[0].id = cudaLaunchAttributeClusterDimension;
+    cluster[0].val.clusterDim.x = 2;
+    cluster[0].val.clusterDim.y = 1;
+    cluster[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(256);
+    cfg.attrs = cluster;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLpSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&pairs, kernel, &cfg) != cudaSuccess || pairs < 1) {
+      cudaGetLastError();
+      return JET_ERR_CUDA;
+    }
+    pairs_of[dev].store(pairs, std::memory_order_release);
+  }
+  const int w_blocks = kRows2 ? 1 : 2;
+  const int bn = lm_block_width(V, pairs, w_blocks);
+  const int tiles = (V + w_blocks * bn - 1) / (w_blocks * bn);
+  CUtensorMap tw;
+  const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(V)};
+  const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
+  const uint32_t box[2] = {64, static_cast<uint32_t>(bn / 2)};
+  if (!tma_make_map_bf16(&tw, weight, 2, dims, str, box)) return JET_ERR_CUDA;
+  cfg.gridDim = dim3(2 * (tiles < pairs ? tiles : pairs));
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, tx, tw, rows, V, d, bn, tiles, keys, status) != cudaSuccess) {
     cudaGetLastError();
     return JET_ERR_CUDA;
   }
@@ -451,18 +678,12 @@ extern "C" jet_status jet_tree_accept_hidden(const void* hidden, const void* lm_
   const size_t need = jet_tree_accept_hidden_workspace_bytes(batch, B);
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
   const int rows = batch * B;
-  CUtensorMap tx, tw;
+  CUtensorMap tx;
   {
     const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(rows)};
     const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
     const uint32_t box[2] = {64, 128};
     if (!tma_make_map_bf16(&tx, hidden, 2, dims, str, box)) return JET_ERR_CUDA;
-  }
-  {
-    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(V)};
-    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
-    const uint32_t box[2] = {64, 128};
-    if (!tma_make_map_bf16(&tw, lm_head_weight, 2, dims, str, box)) return JET_ERR_CUDA;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto* keys = static_cast<unsigned long long*>(workspace);
@@ -471,12 +692,21 @@ extern "C" jet_status jet_tree_accept_hidden(const void* hidden, const void* lm_
     cudaGetLastError();
     return JET_ERR_CUDA;
   }
-  // rows per CTA: every row group of a CTA shares the weight tile it streams, so more rows per CTA means the
-  // weights cross HBM fewer times (once for up to 512 rows)
+  // Up to 128 rows the call is a weight stream and one 128-row CTA per weight tile keeps HBM busy; above, it is bound by the
+  // tensor cores and runs on CTA pairs (the weights cross HBM once per 512 rows).
   jet_status r;
-  if (rows <= 128) r = launch_lm_head<1>(tx, tw, rows, V, d, keys, device_status, st);
-  else if (rows <= 256) r = launch_lm_head<2>(tx, tw, rows, V, d, keys, device_status, st);
-  else r = launch_lm_head<4>(tx, tw, rows, V, d, keys, device_status, st);
+  if (rows <= kLmBM) {
+    CUtensorMap tw;
+    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(V)};
+    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
+    const uint32_t box[2] = {64, 128};
+    if (!tma_make_map_bf16(&tw, lm_head_weight, 2, dims, str, box)) return JET_ERR_CUDA;
+    r = launch_lm_head(tx, tw, rows, V, d, keys, device_status, st);
+  } else if (rows <= 2 * kLmBM) {
+    r = launch_lm_head_pair<false>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
+  } else {
+    r = launch_lm_head_pair<true>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
+  }
   if (r != JET_OK) return r;
   const int threads = (B + 31) / 32 * 32;
   launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, keys, 1, token, parent, depth, anc_mask, n_nodes, B, N,
