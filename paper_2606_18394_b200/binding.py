@@ -150,7 +150,7 @@ def jet_tree_build_scored(logp, root_token, batch, N, V, W, B, score_mode, alpha
                           node_budget=None):
     st = native().tree_build_scored(logp, logp_batch_stride, logp_depth_stride, root_token, batch, N, V, W, B, node_budget,
                                     int(score_mode), alpha, parent, depth, token, score, anc_mask, n_nodes, depth_entropy, None,
-                                    False, workspace, workspace_bytes, stream)
+                                    False, workspace, workspace_bytes, stream, None, None)
     if check:
         _check(st, "jet_tree_build_scored")
     return st
@@ -166,10 +166,21 @@ def jet_tree_build_logits(logits, root_token, batch, N, V, W, B, score_mode, alp
                           node_budget=None):
     st = native().tree_build_scored(logits, logits_batch_stride, logits_depth_stride, root_token, batch, N, V, W, B,
                                     node_budget, int(score_mode), alpha, parent, depth, token, score, anc_mask, n_nodes,
-                                    depth_entropy, depth_lse, True, workspace, workspace_bytes, stream)
+                                    depth_entropy, depth_lse, True, workspace, workspace_bytes, stream, None, None)
     if check:
         _check(st, "jet_tree_build_logits")
     return st
+
+
+def tree_build_step(rows, root_token, batch, N, V, W, B, node_budget, score_mode, alpha, parent, depth, token, score, anc_mask,
+                    n_nodes, depth_entropy, depth_lse, from_logits, workspace, seq_len0, seq_len):
+    """Tree construction at the start of a step (any score mode, log-probabilities or logits) that also restarts seq_len from
+    seq_len0."""
+    st = native().tree_build_scored(rows, None, None, root_token, batch, N, V, W, B, node_budget, score_mode, alpha, parent,
+                                    depth, token, score, anc_mask, n_nodes, depth_entropy, depth_lse, from_logits, workspace,
+                                    None, None, seq_len0, seq_len)
+    if st != JET_OK:
+        _check(st, "jet_tree_build")
 
 
 def jet_tree_verify_attn_workspace_bytes(batch, B, Hq, Hkv, D, max_seq_len) -> int:

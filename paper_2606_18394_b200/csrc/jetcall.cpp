@@ -13,6 +13,12 @@
 
 #include "jet.h"
 
+extern "C" jet_status jet_internal_tree_build_step(
+    const float* rows, int64_t batch_stride, int64_t depth_stride, const int32_t* root_token, int batch, int N, int V, int W, int B,
+    const int32_t* node_budget, int score_mode, float alpha, int32_t* parent, int32_t* depth, int32_t* token, float* score,
+    uint32_t* anc_mask, int32_t* n_nodes, float* depth_entropy, float* depth_lse, int from_logits, const int32_t* len_src,
+    int32_t* len_dst, void* workspace, size_t workspace_bytes, void* stream);
+
 namespace {
 
 // Walks the positional arguments of one call; after the first conversion error every further read returns 0.
@@ -179,16 +185,17 @@ PyObject* tree_build(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
 }
 
 // (rows, batch_stride, depth_stride, root_token, batch, N, V, W, B, node_budget, score_mode, alpha, parent, depth, token,
-//  score, anc_mask, n_nodes, depth_entropy, depth_lse, from_logits, workspace, workspace_bytes, stream)
+//  score, anc_mask, n_nodes, depth_entropy, depth_lse, from_logits, workspace, workspace_bytes, stream, len_src, len_dst);
+// len_dst not None: the same call also sets len_dst = len_src.
 PyObject* tree_build_scored(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
-  Args a(argv, argc, 24);
+  Args a(argv, argc, 26);
   if (a.bad()) return nullptr;
   int64_t s[2];
   bool bad = false;
   row_strides(argv[0], argv + 1, s, &bad);
   if (bad) return nullptr;
   const float* rows = in<float>(a.ptr());
-  Args b(argv + 3, argc - 3, 21);
+  Args b(argv + 3, argc - 3, 23);
   const int32_t* root = in<int32_t>(b.ptr());
   const int batch = b.i32(), N = b.i32(), V = b.i32(), W = b.i32(), B = b.i32();
   const int32_t* budget = in<int32_t>(b.ptr());
@@ -206,7 +213,12 @@ PyObject* tree_build_scored(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
   size_t wb = 0;
   void* ws = b.workspace(&wb);
   void* st = b.stream();
+  const int32_t* len_src = in<int32_t>(b.ptr());
+  int32_t* len_dst = out<int32_t>(b.ptr());
   if (b.bad()) return nullptr;
+  if (len_dst)
+    JET_CALL(jet_internal_tree_build_step(rows, s[0], s[1], root, batch, N, V, W, B, budget, mode, alpha, parent, depth, token,
+                                          score, anc, n_nodes, entropy, lse, from_logits ? 1 : 0, len_src, len_dst, ws, wb, st));
   JET_CALL(from_logits ? jet_tree_build_logits(rows, s[0], s[1], root, batch, N, V, W, B, budget, mode, alpha, parent, depth,
                                                token, score, anc, n_nodes, entropy, lse, ws, wb, st)
                        : jet_tree_build_scored(rows, s[0], s[1], root, batch, N, V, W, B, budget, mode, alpha, parent, depth,

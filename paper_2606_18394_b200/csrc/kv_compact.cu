@@ -1,102 +1,131 @@
-// jet_kv_compact: commit of the accepted path.  One launch copies the K and V rows of
-// every accepted node of every layer and sequence behind the prefix (contiguous or paged
-// cache); a second one-block launch then advances seq_len, so that no copy block can see
-// an already advanced length.
+// jet_kv_compact: commit of the accepted path.  One launch: a cluster of 8 CTAs per sequence copies the K and V rows of
+// every accepted node of every layer behind the prefix (contiguous or paged cache) and, once every CTA of the cluster has
+// read the old length, advances seq_len.  jet_kv_compact_tail: the same in place, for a cache that holds the tree's rows
+// behind the prefix.
+//
+// Bound: latency (a step commits 0.1 - 3 MB).  The chain is lengths -> path and page table -> rows, three round trips; the rows of
+// a sequence are spread over the warps of its cluster with all loads of a warp in flight at once.  (A block per row or
+// (layer, K|V) with a second launch for the lengths, as before, cost a launch more: about 2 us of GPU time in a
+// captured step and 2.3 us of host time in one issued call by call.)
 #include "jet_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace jet {
 namespace {
 
-__global__ void __launch_bounds__(256)
-kv_compact_kernel(const uint4* __restrict__ tree_k, const uint4* __restrict__ tree_v,
-                  uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
-                  int64_t layer_stride16, int64_t batch_stride16,
-                  const int32_t* __restrict__ page_table, int max_pages, int page_size,
-                  const int32_t* __restrict__ path, const int32_t* __restrict__ accept_len,
-                  const int32_t* __restrict__ seq_len, int batch, int B, int row16, int N) {
-  grid_dependency_wait();
-  const int i = blockIdx.x, b = blockIdx.y, layer = blockIdx.z;
-  if (i > accept_len[b]) return;
-  const int node = path[static_cast<size_t>(b) * (N + 1) + i];
-  if (node < 0 || node >= B) return;
-  const int64_t pos = static_cast<int64_t>(seq_len[b]) + i;
-  int64_t dst_row;
-  if (pos < 0) return;
-  if (page_table) {
-    if (pos / page_size >= max_pages) return;        // (a length beyond the table is the caller's error: no access outside it)
-    const int page = page_table[static_cast<size_t>(b) * max_pages + pos / page_size];
-    dst_row = static_cast<int64_t>(page) * page_size + pos % page_size;
-    dst_row = layer * layer_stride16 + dst_row * row16;
-  } else {
-    dst_row = layer * layer_stride16 + b * batch_stride16 + pos * row16;
-  }
-  const int64_t src = ((static_cast<int64_t>(layer) * batch + b) * B + node) * row16;
-  for (int t = threadIdx.x; t < 2 * row16; t += blockDim.x) {
-    if (t < row16) k_cache[dst_row + t] = tree_k[src + t];
-    else v_cache[dst_row + t - row16] = tree_v[src + t - row16];
-  }
-}
+constexpr int kCommitCluster = 8;
+constexpr int kCommitThreads = 512;
+constexpr int kCommitWarps = kCommitCluster * kCommitThreads / 32;      // warps of a cluster
 
-// In-place variant: the tree's K/V rows sit in the cache at positions seq_len + node.  Row seq_len + path[i]
-// moves to seq_len + i for i = 1 .. accept_len (path[i] >= i; the root stays where it is).  One block per
-// (sequence, layer, K or V): all source rows are read into registers before any is written, with a block-wide
-// barrier in between, so overlapping source and destination ranges are safe.
-constexpr int kTailThreads = 256;
-constexpr int kTailHeld = 8;           // 16-byte pieces a thread can hold: 256 * 8 * 16 bytes = 32 KiB per block pass
+struct CommitParams {
+  int64_t layer_stride16, batch_stride16;            // in 16-byte pieces
+  const int32_t* page_table;
+  const int32_t* path;
+  const int32_t* accept_len;
+  int32_t* seq_len;
+  int max_pages, page_size, layers, batch, B, row16, N;
+};
 
-__global__ void __launch_bounds__(kTailThreads)
-kv_compact_tail_kernel(uint4* __restrict__ k_cache, uint4* __restrict__ v_cache, int64_t layer_stride16,
-                       int64_t batch_stride16, const int32_t* __restrict__ page_table, int max_pages,
-                       int page_size, const int32_t* __restrict__ path, const int32_t* __restrict__ accept_len,
-                       const int32_t* __restrict__ seq_len, int B, int row16, int N) {
-  grid_dependency_wait();
-  const int b = blockIdx.x, layer = blockIdx.y;
-  uint4* cache = blockIdx.z == 0 ? k_cache : v_cache;
-  const int a = min(accept_len[b], N);
-  const int64_t L = seq_len[b];
-  auto row_of = [&](int64_t pos) -> int64_t {
-    if (page_table) {
-      // (the index is kept inside the table: a length beyond it is the caller's error and must not become an access
-      //  outside the table)
-      const int64_t slot = min(max(pos / page_size, static_cast<int64_t>(0)), static_cast<int64_t>(max_pages - 1));
-      const int page = page_table[static_cast<size_t>(b) * max_pages + slot];
-      return layer * layer_stride16 + (static_cast<int64_t>(page) * page_size + pos % page_size) * row16;
-    }
-    return layer * layer_stride16 + b * batch_stride16 + pos * row16;
+// The path of sequence b and where its rows lie, worked out once per CTA: node[i] (-1: not to be copied) and the cache row
+// offsets (within a layer) of position seq_len + i and -- in-place layout -- seq_len + node[i].
+struct CommitTable {
+  int64_t dst[JET_MAX_DEPTH + 1], src[JET_MAX_DEPTH + 1];
+  int node[JET_MAX_DEPTH + 1];
+};
+
+template <bool kTail>
+__device__ __forceinline__ int commit_table(const CommitParams& p, int b, CommitTable& t) {
+  const int a = min(p.accept_len[b], p.N);
+  const int64_t len = p.seq_len[b];
+  auto row_of = [&](int64_t pos) -> int64_t {        // -1: outside the page table (a length beyond it is the caller's error)
+    if (pos < 0) return -1;
+    if (!p.page_table) return b * p.batch_stride16 + pos * p.row16;
+    if (pos / p.page_size >= p.max_pages) return -1;
+    const int page = p.page_table[static_cast<size_t>(b) * p.max_pages + pos / p.page_size];
+    return (static_cast<int64_t>(page) * p.page_size + pos % p.page_size) * p.row16;
   };
-  // pieces of the rows i = 1 .. a, in passes of what the block can hold; a pass never writes a row that a later
-  // pass still has to read, because rows are taken in increasing i and path[i] >= i, path increasing
-  const int total = a * row16;
-  for (int base = 0; base < total; base += kTailThreads * kTailHeld) {
-    uint4 held[kTailHeld];
+  for (int i = threadIdx.x; i <= a; i += kCommitThreads) {
+    int node = p.path[static_cast<size_t>(b) * (p.N + 1) + i];
+    if (node < 0 || node >= p.B) node = -1;
+    const int64_t dst = row_of(len + i), src = kTail && node >= 0 ? row_of(len + node) : 0;
+    if (dst < 0 || src < 0) node = -1;
+    t.node[i] = node;
+    t.dst[i] = dst;
+    t.src[i] = src;
+  }
+  __syncthreads();
+  // every CTA has read the length: one of them may advance it
+  __syncwarp();
+  ptx::cluster_sync_all();
+  if (threadIdx.x == 0 && ptx::cluster_ctarank() == 0) p.seq_len[b] = static_cast<int32_t>(len) + p.accept_len[b] + 1;
+  return a;
+}
+
+__global__ void __launch_bounds__(kCommitThreads)
+kv_compact_kernel(const uint4* __restrict__ tree_k, const uint4* __restrict__ tree_v, uint4* __restrict__ k_cache,
+                  uint4* __restrict__ v_cache, const CommitParams p) {
+  grid_dependency_wait();
+  __shared__ CommitTable t;
+  const int b = blockIdx.x / kCommitCluster;
+  const int a = commit_table<false>(p, b, t);
+  if (a < 0) return;
+  const int lane = threadIdx.x & 31;
+  const int rows = 2 * p.layers * (a + 1);           // row r: path entry r mod (a + 1) of (layer, K | V) number r / (a + 1)
+  for (int r = (blockIdx.x % kCommitCluster) * (kCommitThreads / 32) + (threadIdx.x >> 5); r < rows; r += kCommitWarps) {
+    const int lk = r / (a + 1), i = r - lk * (a + 1), layer = lk >> 1;
+    const int node = t.node[i];
+    if (node < 0) continue;
+    const uint4* src = ((lk & 1) ? tree_v : tree_k) + ((static_cast<int64_t>(layer) * p.batch + b) * p.B + node) * p.row16;
+    uint4* dst = ((lk & 1) ? v_cache : k_cache) + layer * p.layer_stride16 + t.dst[i];
+    int e = lane;
+    for (; e + 96 < p.row16; e += 128) {
+      uint4 x[4];
 #pragma unroll
-    for (int k = 0; k < kTailHeld; ++k) {
-      const int e = base + k * kTailThreads + threadIdx.x;
-      if (e < total) {
-        const int i = 1 + e / row16, piece = e % row16;
-        const int node = path[static_cast<size_t>(b) * (N + 1) + i];
-        held[k] = (node >= 0 && node < B) ? cache[row_of(L + node) + piece] : make_uint4(0u, 0u, 0u, 0u);
-      }
-    }
-    __syncthreads();
+      for (int k = 0; k < 4; ++k) x[k] = __ldg(src + e + 32 * k);
 #pragma unroll
-    for (int k = 0; k < kTailHeld; ++k) {
-      const int e = base + k * kTailThreads + threadIdx.x;
-      if (e < total) {
-        const int i = 1 + e / row16, piece = e % row16;
-        const int node = path[static_cast<size_t>(b) * (N + 1) + i];
-        if (node >= 0 && node < B && node != i) cache[row_of(L + i) + piece] = held[k];
-      }
+      for (int k = 0; k < 4; ++k) dst[e + 32 * k] = x[k];
     }
-    __syncthreads();
+    for (; e < p.row16; e += 32) dst[e] = __ldg(src + e);
   }
 }
 
-__global__ void advance_seq_len_kernel(const int32_t* __restrict__ accept_len,
-                                       int32_t* __restrict__ seq_len, int batch) {
+// In place: row seq_len + path[i] moves to seq_len + i for i = 1 .. accept_len (path[i] >= i; the root stays where it is).
+// One warp per (layer, K | V): it reads kTailHeld pieces per lane into registers before it writes any, so overlapping source
+// and destination ranges are safe; a pass never writes a row that a later pass still has to read, because rows are taken
+// in increasing i and path[i] >= i, path increasing.
+constexpr int kTailHeld = 16;
+
+__global__ void __launch_bounds__(kCommitThreads)
+kv_compact_tail_kernel(uint4* k_cache, uint4* v_cache, const CommitParams p) {
   grid_dependency_wait();
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x)
-    seq_len[b] += accept_len[b] + 1;
+  __shared__ CommitTable t;
+  const int b = blockIdx.x / kCommitCluster;
+  const int a = commit_table<true>(p, b, t);
+  const int lane = threadIdx.x & 31, total = a * p.row16;
+  for (int lk = (blockIdx.x % kCommitCluster) * (kCommitThreads / 32) + (threadIdx.x >> 5); lk < 2 * p.layers; lk += kCommitWarps) {
+    uint4* cache = ((lk & 1) ? v_cache : k_cache) + (lk >> 1) * p.layer_stride16;
+    for (int base = 0; base < total; base += 32 * kTailHeld) {
+      uint4 held[kTailHeld];
+#pragma unroll
+      for (int k = 0; k < kTailHeld; ++k) {
+        const int e = base + k * 32 + lane;
+        if (e < total) {
+          const int i = 1 + e / p.row16;
+          if (t.node[i] >= 0) held[k] = cache[t.src[i] + e % p.row16];
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < kTailHeld; ++k) {
+        const int e = base + k * 32 + lane;
+        if (e < total) {
+          const int i = 1 + e / p.row16;
+          if (t.node[i] >= 0 && t.node[i] != i) cache[t.dst[i] + e % p.row16] = held[k];
+        }
+      }
+      __syncwarp();
+    }
+  }
 }
 
 }  // namespace
@@ -125,12 +154,11 @@ extern "C" jet_status jet_kv_compact(const void* tree_k, const void* tree_v, voi
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row16 = static_cast<int>(row_elems / 8);
-  launch_dependent(kv_compact_kernel, dim3(N + 1, batch, layers), dim3(256), st,
-      static_cast<const uint4*>(tree_k), static_cast<const uint4*>(tree_v),
-      static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), cache_layer_stride / 8,
-      kv_batch_stride / 8, page_table, max_pages_per_seq, page_size, path, accept_len, seq_len,
-      batch, B, row16, N);
-  launch_dependent(advance_seq_len_kernel, dim3(1), dim3(256), st, accept_len, seq_len, batch);
+  const CommitParams p{cache_layer_stride / 8, kv_batch_stride / 8, page_table, path, accept_len, seq_len,
+                       max_pages_per_seq, page_size, layers, batch, B, row16, N};
+  launch_dependent_cluster(kv_compact_kernel, dim3(kCommitCluster * batch), dim3(kCommitThreads), kCommitCluster, st,
+      static_cast<const uint4*>(tree_k), static_cast<const uint4*>(tree_v), static_cast<uint4*>(k_cache),
+      static_cast<uint4*>(v_cache), p);
   return launch_status();
 }
 
@@ -154,9 +182,9 @@ extern "C" jet_status jet_kv_compact_tail(void* k_cache, void* v_cache, int64_t 
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row16 = static_cast<int>(row_elems / 8);
-  launch_dependent(kv_compact_tail_kernel, dim3(batch, layers, 2), dim3(kTailThreads), st,
-      static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), cache_layer_stride / 8, kv_batch_stride / 8,
-      page_table, max_pages_per_seq, page_size, path, accept_len, seq_len, B, row16, N);
-  launch_dependent(advance_seq_len_kernel, dim3(1), dim3(256), st, accept_len, seq_len, batch);
+  const CommitParams p{cache_layer_stride / 8, kv_batch_stride / 8, page_table, path, accept_len, seq_len,
+                       max_pages_per_seq, page_size, layers, batch, B, row16, N};
+  launch_dependent_cluster(kv_compact_tail_kernel, dim3(kCommitCluster * batch), dim3(kCommitThreads), kCommitCluster, st,
+      static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), p);
   return launch_status();
 }

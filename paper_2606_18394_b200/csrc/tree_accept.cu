@@ -1,6 +1,6 @@
 // jet_tree_accept: greedy acceptance of the deepest matching root-to-node path.
 //
-// Two launches:
+// Two launches (one, accept_small_kernel, for small problems):
 //   argmax_partial_kernel  grid (chunks, batch*B rows): the one HBM pass over the target
 //                          logits; each block reduces a slice of one row to a
 //                          (value, lowest index) key in the workspace.  Padding rows are
@@ -95,40 +95,36 @@ argmax_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int 
   }
 }
 
-__global__ void __launch_bounds__(JET_MAX_NODES)
-accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks,
-                   const int32_t* __restrict__ token, const int32_t* __restrict__ parent,
-                   const int32_t* __restrict__ depth, const uint32_t* __restrict__ anc_mask,
-                   const int32_t* __restrict__ n_nodes, int B, int N,
-                   int32_t* __restrict__ tgt_out, int32_t* __restrict__ accept_len,
-                   int32_t* __restrict__ path, int32_t* __restrict__ out_tokens) {
-  grid_dependency_wait();
+// What a sequence's tree looks like and where its result goes (the arguments of jet_tree_accept).
+struct TreeView {
+  const int32_t *token, *parent, *depth;
+  const uint32_t* anc_mask;
+  const int32_t* n_nodes;
+  int B, N;
+  int32_t *tgt_out, *accept_len, *path, *out_tokens;
+};
+
+// Path selection of sequence b by one CTA of at least B threads, one per node: tgt = the target's arg-max at this thread's
+// node (-1 for padding).
+__device__ __forceinline__ void select_path(const TreeView& t, int b, int32_t tgt) {
   __shared__ int32_t s_tgt[JET_MAX_NODES];
   __shared__ uint32_t s_match[JET_MAX_NODES / 32];
   __shared__ uint32_t s_best[JET_MAX_NODES / 32];
   __shared__ uint32_t s_end_row[JET_MAX_NODES / 32];
   __shared__ int s_end;
 
-  const int b = blockIdx.x, v = threadIdx.x, lane = v & 31, warp = v >> 5;
-  const int n = min(n_nodes[b], B);
+  const int v = threadIdx.x, lane = v & 31, warp = v >> 5;
+  const int B = t.B, N = t.N, n = min(t.n_nodes[b], B);
   const int words = (B + 31) / 32;
   const size_t o = static_cast<size_t>(b) * B;
   const bool live = v < n;              // blockDim.x >= B, n <= B
-
-  int32_t tgt = -1;
-  if (live) {
-    unsigned long long k = 0ull;
-    const unsigned long long* pr = partial + (o + v) * nchunks;
-    for (int c = 0; c < nchunks; ++c) { const unsigned long long x = pr[c]; k = x > k ? x : k; }
-    tgt = static_cast<int32_t>(key_index(k));
-  }
+  int my_parent = -1, my_depth = -1, my_token = -1;
+  if (live) { my_parent = t.parent[o + v]; my_depth = t.depth[o + v]; my_token = t.token[o + v]; }
   s_tgt[v] = tgt;
-  if (v < B) tgt_out[o + v] = tgt;
+  if (v < B) t.tgt_out[o + v] = tgt;
   __syncthreads();
 
   // match[v]: the root always matches; other nodes iff token == target prediction at the parent
-  int my_parent = -1, my_depth = -1, my_token = -1;
-  if (live) { my_parent = parent[o + v]; my_depth = depth[o + v]; my_token = token[o + v]; }
   const bool match = live && (v == 0 || (my_parent >= 0 && my_parent < n && my_token == s_tgt[my_parent]));
   const uint32_t mbits = __ballot_sync(0xffffffffu, match);
   if (lane == 0) s_match[warp] = mbits;
@@ -137,7 +133,7 @@ accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks,
   // accepted iff every node of Anc(v)+{v} matches
   bool acc = live;
   if (live) {
-    const uint32_t* row = anc_mask + (o + v) * words;
+    const uint32_t* row = t.anc_mask + (o + v) * words;
     for (int w = 0; w < words; ++w) acc = acc && ((row[w] & ~s_match[w]) == 0u);
   }
   // deepest accepted node, ties -> lowest index
@@ -152,21 +148,85 @@ accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks,
   }
   __syncthreads();
   const int end = s_end;
-  if (v < words) s_end_row[v] = anc_mask[(o + end) * words + v];
+  if (v < words) s_end_row[v] = t.anc_mask[(o + end) * words + v];
   __syncthreads();
 
   // (clamped: the arrays of a tree are the caller's and are not validated; a depth outside 0 .. N must not turn
   //  into a store outside the N + 1 entries of this sequence's outputs)
-  const int a = s_tgt[end] >= 0 ? min(max(depth[o + end], 0), N) : 0;
-  int32_t* my_path = path + static_cast<size_t>(b) * (N + 1);
-  int32_t* my_tok = out_tokens + static_cast<size_t>(b) * (N + 1);
+  const int a = s_tgt[end] >= 0 ? min(max(t.depth[o + end], 0), N) : 0;
+  int32_t* my_path = t.path + static_cast<size_t>(b) * (N + 1);
+  int32_t* my_tok = t.out_tokens + static_cast<size_t>(b) * (N + 1);
   for (int i = v; i <= N; i += blockDim.x)
     if (i > a) { my_path[i] = -1; my_tok[i] = -1; }
   if (live && ((s_end_row[v >> 5] >> (v & 31)) & 1u) && my_depth >= 0 && my_depth <= N) {
     my_path[my_depth] = v;
     if (my_depth >= 1) my_tok[my_depth - 1] = my_token;
   }
-  if (v == 0) { accept_len[b] = a; my_tok[a] = s_tgt[end]; }
+  if (v == 0) { t.accept_len[b] = a; my_tok[a] = s_tgt[end]; }
+}
+
+__global__ void __launch_bounds__(JET_MAX_NODES)
+accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks, const TreeView t) {
+  grid_dependency_wait();
+  const int b = blockIdx.x, v = threadIdx.x;
+  int32_t tgt = -1;
+  if (v < min(t.n_nodes[b], t.B)) {
+    unsigned long long k = 0ull;
+    const unsigned long long* pr = partial + (static_cast<size_t>(b) * t.B + v) * nchunks;
+    for (int c = 0; c < nchunks; ++c) { const unsigned long long x = pr[c]; k = x > k ? x : k; }
+    tgt = static_cast<int32_t>(key_index(k));
+  }
+  select_path(t, b, tgt);
+}
+
+// Both parts in one launch for small problems: a CTA per sequence, a warp per row of logits.  Up to kSmallLogits logits a
+// sequence one CTA reads them in about the time that the second launch of the two-kernel form takes to start.
+constexpr int kSmallThreads = JET_MAX_NODES;
+constexpr int kSmallLogits = 32768, kSmallRow = 4096;
+
+__global__ void __launch_bounds__(kSmallThreads)
+accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t) {
+  grid_dependency_wait();
+  __shared__ int32_t s_row[JET_MAX_NODES];
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  const int n = min(t.n_nodes[b], t.B);
+  for (int v = threadIdx.x >> 5; v < n; v += kSmallThreads / 32) {
+    const float* p = logits + (static_cast<int64_t>(b) * t.B + v) * row_stride;
+    float best = 0.0f;
+    uint32_t best_idx = 0xFFFFFFFFu;                 // none yet
+    auto take = [&](float x, int idx) {              // (called with ascending indices)
+      if (idx < V && (best_idx == 0xFFFFFFFFu || x > best)) { best = x; best_idx = static_cast<uint32_t>(idx); }
+    };
+    for (int base = 0; base < V; base += 1024) {     // eight 16-byte loads of a lane in flight
+      float4 x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int idx = base + (i * 32 + lane) * 4;
+        x[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (vec_ok && idx + 3 < V) {
+          x[i] = __ldcs(reinterpret_cast<const float4*>(p + idx));
+        } else {
+          if (idx < V) x[i].x = __ldg(p + idx);
+          if (idx + 1 < V) x[i].y = __ldg(p + idx + 1);
+          if (idx + 2 < V) x[i].z = __ldg(p + idx + 2);
+          if (idx + 3 < V) x[i].w = __ldg(p + idx + 3);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int idx = base + (i * 32 + lane) * 4;
+        take(x[i].x, idx);
+        take(x[i].y, idx + 1);
+        take(x[i].z, idx + 2);
+        take(x[i].w, idx + 3);
+      }
+    }
+    const unsigned long long key = warp_max_u64(best_idx == 0xFFFFFFFFu ? 0ull : make_key(best, best_idx));
+    if (lane == 0) s_row[v] = static_cast<int32_t>(key_index(key));
+  }
+  __syncthreads();
+  const int v = threadIdx.x;
+  select_path(t, b, v < n ? s_row[v] : -1);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -611,12 +671,15 @@ extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_st
   const bool vec_ok = aligned(logits, 16) && logits_row_stride % 4 == 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto* partial = static_cast<unsigned long long*>(workspace);
+  const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
+  if (V <= kSmallRow && static_cast<int64_t>(B) * V <= kSmallLogits) {
+    launch_dependent(accept_small_kernel, dim3(batch), dim3(kSmallThreads), st, logits, logits_row_stride, V, vec_ok, tree);
+    return launch_status();
+  }
   launch_dependent(argmax_partial_kernel, dim3(nchunks, batch * B), dim3(kArgThreads), st,
       logits, logits_row_stride, V, B, n_nodes, nchunks, vec_ok, partial);
   const int threads = (B + 31) / 32 * 32;
-  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, partial, nchunks, token, parent, depth, anc_mask,
-                                                 n_nodes, B, N, tgt_argmax, accept_len, path,
-                                                 out_tokens);
+  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, partial, nchunks, tree);
   return launch_status();
 }
 
@@ -709,7 +772,7 @@ extern "C" jet_status jet_tree_accept_hidden(const void* hidden, const void* lm_
   }
   if (r != JET_OK) return r;
   const int threads = (B + 31) / 32 * 32;
-  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, keys, 1, token, parent, depth, anc_mask, n_nodes, B, N,
-                   tgt_argmax, accept_len, path, out_tokens);
+  const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
+  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, keys, 1, tree);
   return launch_status();
 }

@@ -13,7 +13,7 @@
 //                        streams: the maximum of every group of 128 entries and the slice's
 //                        fp64 sum go to the workspace.  (Raw logits with an entropy score: a
 //                        second launch of it forms the entropy, which needs the log-sum-exp.)
-//   tree_expand_kernel   grid (batch): per depth, finds the W-th largest group maximum, reads
+//   tree_expand_kernel   grid (batch): (small problems: forms the group maxima itself, one launch;) per depth, finds the W-th largest group maximum, reads
 //                        the few groups at or above it again and ranks their entries; then runs
 //                        the sequential pop/expand loop in one warp with the pending queue
 //                        in registers and emits parent / depth / token / score / ancestor mask.
@@ -292,13 +292,13 @@ __device__ __forceinline__ float rank_value(float x, double lse) {
 
 // More groups or entries at or above the threshold than the fast form holds (many nearly equal values): the groups one
 // after the other, in ascending order; an entry is listed only if it beats the worst of the best so far.
-template <bool kLogits>
+template <bool kLogits, bool kDirect>
 __device__ __noinline__ int top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, float cut, int Wc, double lse,
                                         int lane, unsigned long long* list) {
   unsigned long long worst = 0ull;                   // keys at or below it cannot be among the best any more
   int count = 0;
   for (int g0 = 0; g0 < groups; g0 += 32) {
-    unsigned todo = __ballot_sync(0xffffffffu, __ldg(gm + g0 + lane) >= cut);      // (the number of groups is a multiple of 32)
+    unsigned todo = __ballot_sync(0xffffffffu, (kDirect ? gm[g0 + lane] : __ldg(gm + g0 + lane)) >= cut);      // (the number of groups is a multiple of 32)
     while (todo) {
       const int g = g0 + __ffs(todo) - 1;
       todo &= todo - 1;
@@ -336,7 +336,7 @@ struct TopScratch {
   int groups[32];
 };
 
-template <bool kLogits, typename Lse>
+template <bool kLogits, bool kDirect, typename Lse>
 __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __restrict__ gm, int groups, int Wc, Lse&& lse_of,
                                            int lane, TopScratch& w) {
   constexpr int kQuads = 10;                         // float4 of maxima a lane holds: 1280 groups, 163840 entries
@@ -346,13 +346,13 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
   const float4* gm4 = reinterpret_cast<const float4*>(gm);
 #pragma unroll
   for (int i = 0; i < kQuads; ++i)
-    h[i] = i * 32 + lane < quads ? __ldg(gm4 + i * 32 + lane) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    h[i] = i * 32 + lane < quads ? (kDirect ? gm4[i * 32 + lane] : __ldg(gm4 + i * 32 + lane)) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   const double lse = lse_of();
   float best = -INFINITY;
 #pragma unroll
   for (int i = 0; i < kQuads; ++i) best = fmaxf(best, fmaxf(fmaxf(h[i].x, h[i].y), fmaxf(h[i].z, h[i].w)));
   for (int i = kQuads * 32 + lane; i < quads; i += 32) {
-    const float4 q = __ldg(gm4 + i);
+    const float4 q = kDirect ? gm4[i] : __ldg(gm4 + i);
     best = fmaxf(best, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
   }
   float cut = warp_nth(best, Wc);
@@ -410,7 +410,7 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
     }
   }
   __syncwarp();
-  if (!fits || count > kListCap) top_of_many<kLogits>(rg, gm, groups, cut, Wc, lse, lane, w.list);
+  if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, cut, Wc, lse, lane, w.list);
   else if (count <= 32) keep_best<1>(w.list, count, Wc, lane);
   else keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
 }
@@ -534,7 +534,11 @@ struct ScanView {
   int slices, rounds, vec;
 };
 
-template <int kMode>
+// Small problems (accumulated log-probabilities only): the expansion kernel forms the group maxima itself, in shared memory,
+// and the scan's launch falls away.  Up to this many 4096-entry slices of all rows of a sequence (48 entries per thread).
+constexpr int kDirectSlices = 6;
+
+template <int kMode, bool kDirect = false>
 __global__ void __launch_bounds__(kExpThreads)
 tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, int N, int V, int Wc, int B, float alpha,
                    int32_t* __restrict__ parent_out, int32_t* __restrict__ depth_out,
@@ -560,6 +564,25 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
   const int Bb = node_budget ? max(1, min(B, node_budget[b])) : B;
   const int root = root_token[b];
   if (len_dst && tid == kExpThreads - 1) len_dst[b] = len_src[b];
+  __shared__ __align__(16) float s_gmax[kDirect ? kDirectSlices * 32 : 1];
+  if constexpr (kDirect) {
+    // a warp takes the 32 float4 columns of one block of 32 scan threads: four groups of eight threads
+    for (int u = warp; u < N * scan.slices * (kScanThreads / 32); u += kExpWarps) {
+      const int slice = u / (kScanThreads / 32), first = u % (kScanThreads / 32) * 32, d = slice / scan.slices;
+      const float* row = scan.rows + b * scan.batch_stride + d * scan.depth_stride;
+      const int base = (slice - d * scan.slices) * kRoundChunk + (first + lane) * 4;
+      float4 q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = load4(row, base + i * kScanThreads * 4, V, scan.vec != 0);
+      float m = -INFINITY;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(fmaxf(q[i].x, q[i].y), fmaxf(q[i].z, q[i].w)));
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((lane & 7) == 0) s_gmax[slice * 32 + (first + lane) / 8] = m;
+    }
+    __syncthreads();
+  }
 
   // ---- per depth: log-sum-exp, entropy, the W best entries; one warp per row
   for (int d = warp; d < N; d += kExpWarps) {
@@ -578,16 +601,16 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     }
     const int groups = scan.slices * 32 * scan.rounds;
     const RowGroups rg(scan.rows + b * scan.batch_stride + d * scan.depth_stride, V, scan.rounds, scan.vec, lane);
-    const float* gm = scan.gmax + row_id * groups;
+    const float* gm = kDirect ? s_gmax + d * groups : scan.gmax + row_id * groups;
     TopScratch& w = sh.top[warp];
-    if (scan.pairs) {
-      top_of_row<true>(rg, gm, groups, Wc, [&] {
+    if (!kDirect && scan.pairs) {
+      top_of_row<true, kDirect>(rg, gm, groups, Wc, [&] {
         const double lse = row_lse(scan.pairs + row_id * scan.slices, scan.slices, lane);
         if (lane == 0 && depth_lse_out) depth_lse_out[row_id] = static_cast<float>(lse);
         return lse;
       }, lane, w);
     } else {
-      top_of_row<false>(rg, gm, groups, Wc, [] { return 0.0; }, lane, w);
+      top_of_row<false, kDirect>(rg, gm, groups, Wc, [] { return 0.0; }, lane, w);
     }
     if (lane < Wc) {
       const unsigned long long k = w.list[lane];
@@ -697,7 +720,7 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
 
   const int Wc = W < V ? W : V;
-  const ScanPlan plan = scan_plan(batch, N, V);
+  ScanPlan plan = scan_plan(batch, N, V);
   const bool vec = aligned(rows, 16) && batch_stride % 4 == 0 && depth_stride % 4 == 0;
   const bool scored = score_mode != JET_SCORE_ACCUM_LOGP;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -711,7 +734,11 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   auto scan = [&](auto kernel, double2* sums) {
     launch_dependent(kernel, grid, dim3(kScanThreads), st, rows, batch_stride, depth_stride, V, plan.rounds, vec, gmax, pairs, sums);
   };
-  if (from_logits) {
+  const bool direct = !scored && !from_logits && static_cast<int64_t>(N) * ((V + kRoundChunk - 1) / kRoundChunk) <= kDirectSlices;
+  if (direct) {
+    plan.rounds = 1;
+    plan.slices = (V + kRoundChunk - 1) / kRoundChunk;
+  } else if (from_logits) {
     scan(row_scan_kernel<kScanSum>, pairs);
     if (scored) scan(row_scan_kernel<kScanLogitEntropy>, plogp);
   } else if (scored) {
@@ -720,7 +747,8 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
     scan(row_scan_kernel<kScanMax>, nullptr);
   }
   const ScanView view{rows, batch_stride, depth_stride, gmax, pairs, plogp, plan.slices, plan.rounds, vec ? 1 : 0};
-  auto expand = score_mode == JET_SCORE_ACCUM_LOGP ? tree_expand_kernel<0>
+  auto expand = direct ? tree_expand_kernel<0, true>
+                : score_mode == JET_SCORE_ACCUM_LOGP ? tree_expand_kernel<0>
                 : score_mode == JET_SCORE_ENTROPY  ? tree_expand_kernel<1> : tree_expand_kernel<2>;
   launch_dependent(expand, dim3(batch), dim3(kExpThreads), st, view, root_token, N, V, Wc, B, alpha, parent, depth, token,
                    score, anc_mask, n_nodes, depth_entropy, depth_lse, node_budget, len_src, len_dst);
@@ -781,4 +809,21 @@ extern "C" jet_status jet_tree_build_logits(const float* logits, int64_t logits_
   return jet::tree_build_launch(logits, logits_batch_stride, logits_depth_stride, root_token, batch, N, V, W, B,
                                 score_mode, alpha, parent, depth, token, score, anc_mask, n_nodes, depth_entropy,
                                 node_budget, workspace, workspace_bytes, need, stream, true, depth_lse);
+}
+
+// Not part of the C ABI: what VerifyStep calls -- any of the entry points above, and seq_len restarted from its value at the
+// beginning of the step by the same launch (a device-to-device copy in front of every step cost 4.9 us of host time, and
+// about 2 us on the GPU, where it also breaks the chain of dependent launches).
+extern "C" JET_API jet_status jet_internal_tree_build_step(
+    const float* rows, int64_t batch_stride, int64_t depth_stride, const int32_t* root_token, int batch, int N, int V, int W, int B,
+    const int32_t* node_budget, int score_mode, float alpha, int32_t* parent, int32_t* depth, int32_t* token, float* score,
+    uint32_t* anc_mask, int32_t* n_nodes, float* depth_entropy, float* depth_lse, int from_logits, const int32_t* len_src,
+    int32_t* len_dst, void* workspace, size_t workspace_bytes, void* stream) {
+  if (!len_src || !len_dst) return JET_ERR_INVALID_ARG;
+  const size_t need = from_logits ? jet_tree_build_logits_workspace_bytes(batch, N, V, W)
+                      : score_mode == JET_SCORE_ACCUM_LOGP ? jet_tree_build_workspace_bytes(batch, N, V, W)
+                                                           : jet_tree_build_scored_workspace_bytes(batch, N, V, W);
+  return jet::tree_build_launch(rows, batch_stride, depth_stride, root_token, batch, N, V, W, B, score_mode, alpha, parent, depth,
+                                token, score, anc_mask, n_nodes, depth_entropy, node_budget, workspace, workspace_bytes, need,
+                                stream, from_logits != 0, depth_lse, len_src, len_dst);
 }

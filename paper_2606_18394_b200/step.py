@@ -201,8 +201,10 @@ class VerifyStep:
     def run_front(self):
         """Everything that does not need the target logits: tree construction and the attention of all layers.
         seq_len restarts from seq_len0 so that repeated steps (and graph replays) see the same prefix lengths."""
-        self.seq_len.copy_(self.seq_len0)
-        self.tree_build()
+        mode = {"accum_logp": 0, "entropy": 1, "hybrid": 2}[self.score_mode]
+        jet.tree_build_step(self.logp, self.root_token, self.batch, self.N, self.V, self.W, self.B, self.node_budget, mode,
+                            self.score_alpha, self.parent, self.depth, self.token, self.score, self.anc_mask, self.n_nodes,
+                            self.depth_entropy, self.depth_lse, self.draft_logits, self.ws_build, self.seq_len0, self.seq_len)
         for layer in range(self.layers):
             self.verify_attn(layer)
 
@@ -221,10 +223,17 @@ class VerifyStep:
         self.run_front()
         self.run_back()
 
-    LAUNCHES_PER_STEP_FIXED = 6      # tree_build 2, tree_accept 2, kv_compact 2
+    @property
+    def launches_around_attention(self):
+        """Kernel launches of a step's tree construction, acceptance and commit (a small tree or acceptance is one launch)."""
+        scored = self.score_mode != "accum_logp"
+        small_build = not scored and not self.draft_logits and self.N * ((self.V + 4095) // 4096) <= 6
+        build = 1 if small_build else 3 if scored and self.draft_logits else 2
+        accept = 1 if self.accept_mode == "greedy" and self.V <= 4096 and self.B * self.V <= 32768 else 2
+        return build + accept + 1
 
     def launches_per_step(self, attn_launches_per_layer=None):
         if attn_launches_per_layer is None:       # what the library says one attention call of this shape enqueues
             attn_launches_per_layer = jet.jet_tree_verify_attn_launches(self.batch, self.B, self.Hq, self.Hkv, self.D,
                                                                         self.attn_max_len)
-        return self.LAUNCHES_PER_STEP_FIXED + (1 if self.draft_logits else 0) + self.layers * attn_launches_per_layer
+        return self.launches_around_attention + self.layers * attn_launches_per_layer
