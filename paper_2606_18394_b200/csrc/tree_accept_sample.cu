@@ -4,7 +4,7 @@
 //   row_lse_partial_kernel  grid (slices, batch*B): one pass over the target logits; every block
 //                           leaves the maximum and the sum of exp((x - max) / T) of one 8192-entry
 //                           slice of one row in the workspace.  Padding rows are not read.
-//   accept_sample_kernel    one cluster of 8 CTAs per sequence, 1024 threads each: finishes the rows' log-sum-exp, computes
+//   accept_sample_kernel    one cluster of 8 CTAs per sequence, 512 threads each: finishes the rows' log-sum-exp, computes
 //                           alpha_v = min(1, p_parent(token_v) / q_depth(token_v)) and the accept
 //                           bit u_v < alpha_v for every node, picks the deepest node whose whole
 //                           branch is accepted, then draws the correction token at that node by
@@ -23,7 +23,14 @@ namespace {
 constexpr int kLseThreads = 256;
 constexpr int kLseElems = 32;
 constexpr int kLseChunk = kLseThreads * kLseElems;
-constexpr int kSampleThreads = 1024;
+// One thread per node of the largest tree.  Bound of the sampling kernel: latency -- each CTA reads some 20 KB of logits
+// and log-probabilities behind a chain of small dependent look-ups.  512 threads (with at most 64 registers two CTAs share an
+// SM: the 256 CTAs of a batch of 32 are one wave, not two) and kSampleUnroll steps of loads in flight per warp:
+// 32 sequences of 64 nodes, V 151936: 227 -> 215 us for both launches (the scan's 1.25 GB alone need 190 us at the measured
+// copy bandwidth).
+constexpr int kSampleThreads = 512;
+constexpr int kSampleUnroll = 2;           // (three spill at 64 registers)
+static_assert(kSampleThreads >= JET_MAX_NODES, "a thread per node");
 constexpr int kSampleStep = 128;          // vocabulary entries a warp handles per step (4 per lane)
 constexpr int kSampleCluster = 8;         // CTAs per sequence
 constexpr int kMaxStepsTotal = 4096;      // 128-entry steps per row: vocabularies up to 524288 entries
@@ -100,7 +107,7 @@ row_lse_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int
   }
 }
 
-__global__ void __launch_bounds__(kSampleThreads)
+__global__ void __launch_bounds__(kSampleThreads, 2)
 accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const float* __restrict__ logits,
                      int64_t row_stride, float inv_t, const float* __restrict__ draft_logp,
                      int64_t logp_batch_stride, int64_t logp_depth_stride,
@@ -130,8 +137,10 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   if (live) {
     const float2* pr = partial + (o + v) * nchunks;
     float m = -INFINITY;
+#pragma unroll 8
     for (int c = 0; c < nchunks; ++c) m = fmaxf(m, pr[c].x);
     float s = 0.0f;
+#pragma unroll 8
     for (int c = 0; c < nchunks; ++c) {
       const float2 q = pr[c];
       if (q.x > -INFINITY) s += q.y * exp2f((q.x - m) * inv_t * kLog2e);
@@ -199,10 +208,9 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   const int steps = (total_steps + kWarps * kSampleCluster - 1) / (kWarps * kSampleCluster);      // per warp
   const int first_step = (rank * kWarps + warp) * steps;                    // this warp's steps, vocabulary order
   const bool vec = vec_rows;
-  // masses of the 4 entries of this lane in step `g` (global step index)
-  auto masses = [&](int g, bool use_residual, float (&mval)[4]) {
+  // the 4 entries of this lane in step `g` (global step index): logits and, for the residual, draft log-probabilities
+  auto load = [&](int g, bool use_residual, float (&x4)[4], float (&q4)[4]) {
     const int idx = g * kSampleStep + lane * 4;
-    float x4[4], q4[4] = {0.f, 0.f, 0.f, 0.f};
     if (vec && idx + 3 < V) {
       const float4 t = *reinterpret_cast<const float4*>(xrow + idx);
       x4[0] = t.x; x4[1] = t.y; x4[2] = t.z; x4[3] = t.w;
@@ -217,6 +225,8 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
         if (use_residual) q4[j] = idx + j < V ? qrow[idx + j] : -INFINITY;
       }
     }
+  };
+  auto masses = [&](const float (&x4)[4], const float (&q4)[4], bool use_residual, float (&mval)[4]) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float pe = expf((x4[j] - m_e) * inv_t - ln_e);
@@ -228,13 +238,19 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   bool use_residual = residual;
   int picked = -1;
   for (int attempt = 0; attempt < 2; ++attempt) {
-    for (int st = 0; st < steps; ++st) {
-      const int g = first_step + st;
-      if (g < total_steps) {
+    const int last_step = min(first_step + steps, total_steps);
+    for (int g0 = first_step; g0 < last_step; g0 += kSampleUnroll) {
+      float x4[kSampleUnroll][4], q4[kSampleUnroll][4];
+#pragma unroll
+      for (int k = 0; k < kSampleUnroll; ++k)
+        if (g0 + k < last_step) load(g0 + k, use_residual, x4[k], q4[k]);
+#pragma unroll
+      for (int k = 0; k < kSampleUnroll; ++k) {
+        if (g0 + k >= last_step) break;
         float mval[4];
-        masses(g, use_residual, mval);
+        masses(x4[k], q4[k], use_residual, mval);
         const double part = warp_sum_d(static_cast<double>(mval[0]) + mval[1] + mval[2] + mval[3]);
-        if (lane == 0) step0[g] = part;
+        if (lane == 0) step0[g0 + k] = part;
       }
     }
     cluster.sync();                                            // the table is complete
@@ -283,8 +299,9 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
       if (s_pick_step < 0) {
         retry = true;                                          // no mass: fall back to the target distribution itself
       } else if (warp == 0) {
-        float mval[4];
-        masses(s_pick_step, use_residual, mval);
+        float x4[4], q4[4], mval[4];
+        load(s_pick_step, use_residual, x4, q4);
+        masses(x4, q4, use_residual, mval);
         const double mine = static_cast<double>(mval[0]) + mval[1] + mval[2] + mval[3];
         double pre = mine;                                     // inclusive prefix sum over the lanes
 #pragma unroll
