@@ -211,25 +211,20 @@ JET_API jet_status jet_tree_build_logits(const float* logits, int64_t logits_bat
  * Workspace: unlike the other calls, the first 4096 bytes of this workspace hold
  * counters that must be ZERO when the call starts.  Zero them once after
  * allocating the workspace; every call that completes leaves them zero again.
- * (A call that reported JET_ERR_TIMEOUT may leave them dirty: zero them again.
- * Counters that are not zero on entry are the caller's error: the key slices of
- * a work item then never see each other arrive, every CTA gives up after its
- * bounded wait, device_status reads JET_ERR_TIMEOUT and the outputs are
- * undefined; nothing faults and the next call on a zeroed workspace is correct.)
  * When a sequence has fewer work items than the GPU has SMs, its key range is cut
- * into slices that run as separate CTAs and hand each other their partial rows
- * through this workspace inside the one launch.  That exchange assumes that all
- * CTAs of the launch are resident at once: the plan is sized from the device's SM
- * count, so give the call the whole GPU (no other kernel holding SMs at the same
- * time through another stream, MPS or a green context).  If some CTAs cannot
- * start until others finish, the waiting ones give up after about a second with
- * JET_ERR_TIMEOUT instead of hanging.
- * (For shapes with few query rows per KV head -- one 128-row query tile, e.g.
- * up to 32 nodes at 4 query heads per KV head -- the slices only WRITE their rows
- * in the first launch and a second, small launch combines them: then nothing
- * waits inside a kernel, the counters are unused and the residency assumption
- * falls away; jet_tree_verify_attn_launches tells which form a shape gets.
- * JET_FORCE_SPLIT="<slices>,g" / ",h" selects the one- / two-launch form.)
+ * into slices that run as separate CTAs.  They combine their partial rows inside
+ * a thread-block cluster, or write them to this workspace, where a second small
+ * launch combines them: nothing waits for another CTA inside a kernel there, and the
+ * CTAs need not be resident together (jet_tree_verify_attn_launches tells which form a
+ * shape gets).
+ * A third form, for tests and comparison, exchanges the rows through the workspace
+ * inside the one launch (JET_FORCE_SPLIT="<slices>,g").  It uses the counters and
+ * assumes that all CTAs of the launch are resident at once: the plan is sized from the
+ * device's SM count, so give that call the whole GPU.  If some CTAs cannot
+ * start until others finish, or the counters were not zero on entry (also after a
+ * JET_ERR_TIMEOUT: zero them again), the waiting CTAs give up after about a second:
+ * device_status reads JET_ERR_TIMEOUT and the outputs are undefined; nothing faults
+ * and the next call on a zeroed workspace is correct.
  * Stream capture: the first call for a shape family on a device configures the
  * kernel (shared-memory size, cluster attribute) and asks the driver how many
  * clusters fit; make it outside any stream capture (one warm-up call per head
@@ -303,9 +298,9 @@ JET_API jet_status jet_tree_verify_attn_tail(const void* q, const void* k_cache,
  *   JET_ATTN_STABLE_PREFIX   the caller promises that seq_len, n_nodes, page_table
  *       and every cache row at a position below seq_len[b] were written by work
  *       that had finished before the kernel DIRECTLY PRECEDING this call in the
- *       stream could let its successor start (for the kernels of this library,
- *       which signal only after their own dependency wait, and for ordinary
- *       launches: "not written by the directly preceding launch, nor by
+ *       stream could let its successor start (for the calls of this library, which
+ *       let a successor start only when all work before the call has finished,
+ *       and for ordinary launches: "not written by the directly preceding call, nor by
  *       anything running concurrently on another stream").  The kernel then
  *       reads the lengths and streams the prefix K/V tiles into shared memory
  *       before its dependency wait, i.e. under the preceding kernel's tail.

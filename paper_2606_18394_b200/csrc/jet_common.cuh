@@ -19,11 +19,12 @@ inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // stream drains, so its launch latency is hidden.  Every kernel launched this way executes grid_dependency_wait()
 // before its first access to global memory.
 template <typename... KArgs, typename... Args>
-inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t stream, Args... args) {
+inline void launch_dependent_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                  Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -31,6 +32,11 @@ inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, cu
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t stream, Args... args) {
+  launch_dependent_smem(kernel, grid, block, 0, stream, args...);
 }
 
 // The same with thread-block clusters of `cluster` CTAs along x.

@@ -174,12 +174,15 @@ static_assert(PBars::kKvReady - PBars::kKvFull == Cfg<128, 1, true>::kStages && 
 // Every wait is bounded: at most kWaitRounds suspensions of at most kWaitHintNs each -- a second at the longest; the
 // hardware may end a suspension early, and waits that did run out were seen to do so after some tens of
 // milliseconds, still far beyond anything a launch of well under a millisecond waits for.
-// Register split (setmaxnreg): warps 0-3 (producer, MMA issuer, helpers) keep kRegsControl registers per
-// thread, the softmax warpgroups get kRegsSoftmax; 128 * kRegsControl + 256 * kRegsSoftmax must not exceed
-// the 384 * 168 registers the CTA is launched with.
-constexpr int kRegsControl = 104;
-constexpr int kRegsSoftmax = 200;
-static_assert(128 * kRegsControl + 256 * kRegsSoftmax <= 384 * 168, "register split exceeds the CTA's allocation");
+// Register split (setmaxnreg): warps 0-3 (producer, MMA issuer, helpers) keep `control` registers per
+// thread, the softmax warpgroups get `softmax`; 128 * control + 256 * softmax must not exceed
+// the 384 * launch registers the CTA is launched with.  A launch whose slices a second launch merges (kTwo) takes
+// less than the register file: a small CTA of the merge kernel then fits beside it (see kMergeSmall).  Nothing spills in
+// that form; the long launches, which gain nothing from it, ran 1.5 % slower with it.
+template <bool kTwo> struct Regs { static constexpr int launch = 168, control = 104, softmax = 200; };
+template <> struct Regs<true> { static constexpr int launch = 144, control = 64, softmax = 184; };
+static_assert(128 * Regs<false>::control + 256 * Regs<false>::softmax <= 384 * Regs<false>::launch, "register split exceeds the CTA's allocation");
+static_assert(128 * Regs<true>::control + 256 * Regs<true>::softmax <= 384 * Regs<true>::launch, "register split exceeds the CTA's allocation");
 
 constexpr uint32_t kWaitRounds = 1u << 16;
 constexpr uint32_t kWaitHintNs = 16384;
@@ -279,9 +282,11 @@ __device__ __forceinline__ void exp_chunk(const uint32_t (&x)[32], float sl2, fl
 }
 
 // kSorted: the sequences of a batch are launched longest prefix first (see the set-up of warp 3).
+// kTwo: the key slices leave their rows in the workspace for the merge kernel (no other form of the exchange is compiled:
+// the kernel starts from cold instruction caches in every layer, and what it does not hold it does not fetch).
 // tm_k64 / tm_tk64: the K maps with boxes of 64 rows (a pair CTA's half of a key tile); unused otherwise.
-template <int D, int MT, bool kSorted = false, bool kPair = false>
-__global__ void __launch_bounds__(Cfg<D, MT, kPair>::kThreads, 1)
+template <int D, int MT, bool kSorted = false, bool kPair = false, bool kTwo = false>
+__global__ void __maxnreg__(Regs<kTwo>::launch)
 tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_tk,
                  const __grid_constant__ CUtensorMap tm_tv, const __grid_constant__ CUtensorMap tm_k64,
@@ -399,6 +404,10 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         ptx::prefetch_tmap(&tm_tk64);
       }
     }
+    // The query rows are asked into L2 as well, for a caller whose queries are not there already (0.5 - 3 % of a layer).
+    if (!sorted_launch && lane == 0)
+      for (int mt = 0; mt < n_mt; ++mt)
+        for (int h = 0; h < kHalves; ++h) ptx::tma_prefetch_4d(&tm_q, h * 64, 0, g, b_rank * p.B + node_lo + mt * npt);
     // A single sequence's length is very often exactly the caller's bound.  On that guess this slice's first
     // key tiles are asked into L2 now -- before the grid dependency wait, under the previous kernel's tail: L2
     // is where that kernel's writes arrive, so a line prefetched early cannot go stale -- and the copies
@@ -468,7 +477,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   if (tid == 0) JET_TR(41);
   // The barriers of every CTA of the cluster must exist before any CTA arrives on them remotely:
   // arrive on the hardware cluster barrier now, wait for it only when the slices are merged.
-  const bool via_cluster = S > 1 && !p.via_global;
+  const bool via_cluster = !kTwo && S > 1 && !p.via_global;
   const uint32_t tmem_base = *tmem_slot;
   if (tid == 0) JET_TR(42);
   // Inputs may be written by the preceding kernel of the stream: nothing in global memory is touched before
@@ -742,9 +751,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       } else {
         ptx::cta_sync();
       }
-      const uint8_t* src_rows = via_cluster ? smem_gen + C::kRecvOff : stage;         // S == 1: the staged rows themselves
+      [[maybe_unused]] const uint8_t* src_rows = via_cluster ? smem_gen + C::kRecvOff : stage;         // S == 1: the staged rows themselves
       bool rows_ok = merge_ok;
-      if (S > 1 && !via_cluster) {
+      if (kTwo || (S > 1 && !via_cluster)) {
         // Exchange through the workspace: publish this CTA's staged rows, count the slices of the unit
         // that have published (bounded spin), then fetch this CTA's block of rows from every slice.
         constexpr uint32_t kBlockBytes = kBM * C::kRecvPitch;
@@ -762,7 +771,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         // Two launches: this one ends here; the merge kernel that follows it in the stream starts when every
         // CTA of this launch has exited, i.e. when every block is in place -- no counter, no spin, and no need
         // for the slices to be resident together.
-        if (p.via_global == 2) continue;
+        if (kTwo || p.via_global == 2) continue;
         ptx::cta_sync();
         if (!kSm && tid == 0) {
           // the last slice to arrive knows from its own count that everybody has published
@@ -943,7 +952,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // Warps 0-3 need few registers; what they give up goes to the softmax warpgroups, which hold a whole
     // score row (128 values) per thread.
     if (tid == 0) JET_TR(15);
-    ptx::setmaxnreg_dec<kRegsControl>();
+    ptx::setmaxnreg_dec<Regs<kTwo>::control>();
     if (tid == 0) JET_TR(18);
 
     // =========================================================== TMA producer (warp 0)
@@ -1465,7 +1474,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
     epilogue(std::false_type{});
   } else {
-    ptx::setmaxnreg_inc<kRegsSoftmax>();
+    ptx::setmaxnreg_inc<Regs<kTwo>::softmax>();
     if (early) ptx::grid_dep_wait();        // ancestor masks, outputs and the workspace belong behind the wait
     constexpr int kChunks = kBN / 32;                       // 32-key chunks per row and tile
     static_assert(kChunks == 4, "the register-resident row is written out for four 32-key chunks");
@@ -2044,82 +2053,99 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 // Second launch of the two-launch slice merge: every key slice of a work item has left its 128 normalised rows
 // (D bf16 values + log2-sum-exp, fp32) in the workspace; one thread combines 8 output values of one row over the
 // S slices with softmax weights of the slice sums and writes them (bf16), the first thread of a row also its
-// log-sum-exp.  All loads of a thread are independent of each other: one round trip to L2.
+// log-sum-exp.  Bound: latency -- one round trip to L2 with all loads of a thread independent of each other, and a few
+// hundred instructions on cold caches.  So
+//  * the next kernel of the stream may start at once (it waits for this one before it reads anything that this one or
+//    the slices write), and this kernel itself is resident, with its index arithmetic done, before the slices end:
+//    1.2 us less per layer than starting the next one from here on;
+//  * kS >= S is the number of slices that the code is written out for, so that no thread runs through absent ones;
+//  * kSmall: CTAs of kMergeSmall threads and at most 80 registers, no more of them than there are SMs, find room beside
+//    the attention CTAs.  With more rows than one such wave covers, CTAs of kMergeLarge threads, each with an SM
+//    to itself (kMergeLargeSmem; nothing is stored there): two on one SM share its path to L2 while others idle.
+// One layer of 32 query and 8 KV heads of 128, prefix 4096, 64 nodes, nine slices: 11.6 us against 12.5 with the exchange
+// inside the launch; 32 nodes 10.7 against 11.9.
+constexpr int kMergeSmall = 128, kMergeSmallRegs = 80, kMergeSmallSlices = 12;
+constexpr int kMergeLarge = 384;
+constexpr int kMergeLargeSmem = 120 * 1024;
+static_assert(kMergeSmall * kMergeSmallRegs + 384 * Regs<true>::launch <= 65536, "the small merge CTA does not fit beside an attention CTA");
+
 struct MergeParams {
   const uint8_t* partials;
   const int32_t* n_nodes;
   __nv_bfloat16* out;
   float* lse;
-  int B, Hq, Hkv, G, S, MT, n_mgroups, npt;
+  int B, Hq, Hkv, G, S, MT, n_mgroups, npt, tiles;      // tiles: query tiles of the launch, units * MT
   uint32_t magic_G;
 };
 
-template <int D>
-__global__ void __launch_bounds__(256) tree_attn_merge_kernel(const MergeParams p) {
-  constexpr int kPitch = D * 2 + 16;
-  constexpr int kItemsPerRow = D / 8;
-  constexpr int kRowsPerCta = 256 / kItemsPerRow;
-  constexpr int kBlocksPerTile = kBM / kRowsPerCta;
-  ptx::grid_dep_wait();
+template <int D, int kS, int kThreads>
+__device__ __forceinline__ void merge_rows(const MergeParams& p) {
   ptx::grid_dep_launch();
-  int bx = static_cast<int>(blockIdx.x);
-  const int rb = bx % kBlocksPerTile;
-  bx /= kBlocksPerTile;
-  const int mt = bx % p.MT, mgroup = bx / p.MT;
-  const int g = blockIdx.y, b = blockIdx.z;
-  const int row = rb * kRowsPerCta + static_cast<int>(threadIdx.x) / kItemsPerRow;
-  const int c8 = static_cast<int>(threadIdx.x) % kItemsPerRow;
+  constexpr int kPitch = D * 2 + 16;
+  constexpr int kItems = D / 8;
+  const int slot = blockIdx.x * (kThreads / kItems) + static_cast<int>(threadIdx.x) / kItems;      // row of all tiles
+  const int c8 = static_cast<int>(threadIdx.x) % kItems;
+  const int tile = slot / kBM, row = slot % kBM;
+  const int unit = tile / p.MT, mt = tile - unit * p.MT;
+  const int bg = unit / p.n_mgroups, mgroup = unit - bg * p.n_mgroups;
+  const int b = bg / p.Hkv, g = bg - b * p.Hkv;
   const int R = mt * kBM + row;                              // row within the work item
   const int vq = static_cast<int>(udiv(R, p.magic_G));
   const int v = mgroup * p.MT * p.npt + vq, h = g * p.G + (R - vq * p.G);
-  if (v >= p.B) return;
-  const int n = min(p.n_nodes[b], p.B);
-  const int unit = (b * p.Hkv + g) * p.n_mgroups + mgroup;
   const int S = p.S;
   const size_t stride = static_cast<size_t>(p.MT) * kBM * kPitch;       // distance between consecutive slices
   const uint8_t* row0 = p.partials + (static_cast<size_t>(unit) * S * p.MT + mt) * (static_cast<size_t>(kBM) * kPitch) +
                         static_cast<size_t>(row) * kPitch;
-  // every load of the thread is issued before any is used (the slots are valid memory for any row)
-  float lc[kMaxSplit];
-  uint4 x[kMaxSplit];
+  uint4* dst = reinterpret_cast<uint4*>(p.out + ((static_cast<size_t>(b) * p.B + v) * p.Hq + h) * D + c8 * 8);
+  ptx::grid_dep_wait();
+  if (tile >= p.tiles || v >= p.B) return;
+  float l[kS];
+  uint4 x[kS];
 #pragma unroll
-  for (int c = 0; c < kMaxSplit; ++c) {
+  for (int c = 0; c < kS; ++c) {
+    l[c] = -INFINITY;
+    x[c] = make_uint4(0u, 0u, 0u, 0u);
     if (c < S) {
-      lc[c] = __ldcg(reinterpret_cast<const float*>(row0 + c * stride + D * 2));
+      l[c] = __ldcg(reinterpret_cast<const float*>(row0 + c * stride + D * 2));
       x[c] = __ldcg(reinterpret_cast<const uint4*>(row0 + c * stride + c8 * 16));
-    } else {
-      lc[c] = -INFINITY;
-      x[c] = make_uint4(0u, 0u, 0u, 0u);
     }
   }
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  float lse2 = -INFINITY;
-  float mx = -INFINITY;
+  const int n = min(p.n_nodes[b], p.B);
+  float mx = l[0];
 #pragma unroll
-  for (int c = 0; c < kMaxSplit; ++c) mx = fmaxf(mx, lc[c]);
-  if (v < n && mx > -INFINITY) {
-    float wsum = 0.0f;
+  for (int c = 1; c < kS; ++c) mx = fmaxf(mx, l[c]);
+  const bool live = v < n && mx > -INFINITY;
+  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, wsum = 0.0f;
 #pragma unroll
-    for (int c = 0; c < kMaxSplit; ++c) {
-      const float w = lc[c] > -INFINITY ? exp2f(lc[c] - mx) : 0.0f;       // absent slices get weight 0 ...
-      wsum += w;
-      const uint32_t v4[4] = {x[c].x, x[c].y, x[c].z, x[c].w};
+  for (int c = 0; c < kS; ++c) {
+    // slices without a key of this row (log-sum-exp -inf) get weight 0, and whatever their rows hold is not used
+    const bool has = l[c] > -INFINITY;
+    const float w = has ? exp2f(l[c] - mx) : 0.0f;
+    wsum += w;
+    const uint32_t v4[4] = {has ? x[c].x : 0u, has ? x[c].y : 0u, has ? x[c].z : 0u, has ? x[c].w : 0u};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {      // bf16 pair -> fp32: the bits are the upper half of the float
-        const float lo = __uint_as_float(v4[q] << 16), hi = __uint_as_float(v4[q] & 0xFFFF0000u);
-        acc[2 * q] += w > 0.0f ? w * lo : 0.0f;                          // ... and whatever they hold is not used
-        acc[2 * q + 1] += w > 0.0f ? w * hi : 0.0f;
-      }
+    for (int q = 0; q < 4; ++q) {                            // bf16 pair -> fp32: the bits are the upper half of the float
+      acc[2 * q] += w * __uint_as_float(v4[q] << 16);
+      acc[2 * q + 1] += w * __uint_as_float(v4[q] & 0xFFFF0000u);
     }
-    const float inv = 1.0f / wsum;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] *= inv;
-    lse2 = mx + log2f(wsum);
   }
-  *reinterpret_cast<uint4*>(p.out + ((static_cast<size_t>(b) * p.B + v) * p.Hq + h) * D + c8 * 8) =
-      make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]),
-                 pack_bf16(acc[6], acc[7]));
-  if (p.lse && c8 == 0) p.lse[(static_cast<size_t>(b) * p.Hq + h) * p.B + v] = lse2 * 0.6931471805599453f;
+  const float inv = 1.0f / wsum;
+  uint4 o = make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
+                       pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+  if (!live) o = make_uint4(0u, 0u, 0u, 0u);
+  *dst = o;
+  if (p.lse && c8 == 0)
+    p.lse[(static_cast<size_t>(b) * p.Hq + h) * p.B + v] = live ? (mx + log2f(wsum)) * 0.6931471805599453f : -INFINITY;
+}
+
+template <int D, int kS>
+__global__ void __maxnreg__(kMergeSmallRegs) tree_attn_merge_small_kernel(const MergeParams p) {
+  merge_rows<D, kS, kMergeSmall>(p);
+}
+
+template <int D, int kS>
+__global__ void __launch_bounds__(kMergeLarge) tree_attn_merge_large_kernel(const MergeParams p) {
+  merge_rows<D, kS, kMergeLarge>(p);
 }
 
 // ------------------------------------------------------------------------------------------ host
@@ -2202,9 +2228,9 @@ bool configure_kernel() {
                  cudaSuccess &&
              cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     };
-    state = (set(tree_attn_kernel<D, MT, false, kPair>) && set(tree_attn_kernel<D, MT, true, kPair>))
-                ? 1
-                : -1;
+    bool ok = set(tree_attn_kernel<D, MT, false, kPair>) && set(tree_attn_kernel<D, MT, true, kPair>);
+    if constexpr (MT == 1 && !kPair) ok = ok && set(tree_attn_kernel<D, 1, false, false, true>) && set(tree_attn_kernel<D, 1, true, false, true>);
+    state = ok ? 1 : -1;
     if (state < 0) cudaGetLastError();
     state_ref.store(state, std::memory_order_release);
   }
@@ -2248,19 +2274,54 @@ int max_active_clusters_for(int D, int mt, int cluster) {
   return mt == 1 ? max_active_clusters<64, 1>(cluster) : max_active_clusters<64, 2>(cluster);
 }
 
-// Picks the query-tile grouping and the number of key slices with a cost model fitted to measurements, in
-// units of one key tile of a one-query-tile CTA whose K/V comes out of L2 (about 1900 cycles):
-//   key tile, one query tile per CTA   1 + 0.75 / g    g = CTAs that read the same K/V tile side by side
-//                                                      (the first one fetches it from HBM, the others hit L2)
-//   key tile, two query tiles per CTA  max(2.2, 1 + 0.75 / g)   two softmax chains share the tensor core,
-//                                                      but the K/V tile is loaded once for both
-//   fixed cost of a CTA                6 (no slices), 8 (slices merged inside a cluster), 10 (through the
-//                                      workspace); 1.6 times that with two query tiles (two merge rounds)
-// and the CTAs run in waves of what the device holds at once.
-// Measured: a key tile costs a pair CTA 1800 cycles against 1475 for a CTA on its own (the hand-overs cross two SMs),
-// so the planner never prefers the pair form; JET_FORCE_PAIR=1 selects it.
-constexpr double kPairTile = 1.22;    // a pair CTA's key tile against a single CTA's
-constexpr double kPairFixed = 1.0;    // what a pair adds per CTA (cluster barriers at set-up, end of pass, teardown)
+// Small merge CTAs where one wave of them covers the rows and their registers hold the slices.
+bool merge_is_small(int query_tiles, int ns, int D) {
+  return ns <= kMergeSmallSlices && query_tiles * kBM <= sm_count() * (kMergeSmall / (D / 8));
+}
+
+// Picks the query-tile grouping, the number of key slices and the form of their merge with a cost model, in microseconds
+// of a launch in the steady state of a layer stack, fitted to a sweep of all forms and slice counts over batches 1 - 4,
+// budgets 16 - 256, prefixes 128 - 16384 (the plans chosen were within 0.4 us of the best form of each shape, most within 0.1):
+//   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power), or what HBM takes for the K/V tiles of all
+//                          CTAs that do not share one (1.45 f / g at D 128, g = CTAs that read the same tile side by side);
+//                          1.76 with two query tiles (two softmax chains share a tensor core)
+//   fixed, no slices       5.2 + 2.4 f
+//   slices in a cluster    5.7 with four, 6.0 with eight, 7.0 with an odd number, else 6.4, + 2.4 f.  (Four and eight: the
+//                          shape of the row exchange is a power of two.)  Clusters of up to eight CTAs are
+//                          portable; larger ones measured slower than the second launch everywhere.
+//   a second launch merges 5.9 + 2.2 f, + 0.5 with the large merge CTAs, + 0.4 when two CTAs have to share a TPC, + 0.7 and 2.0 with
+//                          more than 10 and 12 slices (longer merge code); never below the 4 us of host time that each
+//                          launch costs a caller who issues layer by layer
+// all of the fixed part 1.6 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
+// at once.  The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
+// second launch at every shape, and CTA pairs need 1.22 times the key-tile time (the hand-overs cross two SMs): both
+// run where they are asked for (JET_FORCE_SPLIT="<slices>,g", JET_FORCE_PAIR=1).
+// More than four sequences (ragged, usually paged, and enough work items for several waves): the fit above does not cover them.  There
+// the unit is a key tile out of L2 (0.8 us), a tile costs 1 + 0.75 / g and the fixed parts are 6 / 8 / 10 (none, cluster, second
+// launch): with few CTAs per K/V tile this prefers more, shorter CTAs, which even out sequences of different lengths
+// (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).
+double plan_cost(int batch, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
+  if (batch > 4) {
+    const double shared = 1.0 + 0.75 / n_mgroups, per_tile = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
+    return waves * ((tiles + ns - 1) / ns * per_tile + (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) * (mt == 1 ? 1.0 : 1.6));
+  }
+  const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
+  double tile = mt == 1 ? 0.78 + 0.14 * f : 1.76;
+  const double hbm = 1.45 * f * D / 128 / n_mgroups;
+  if (tile < hbm) tile = hbm;
+  double fixed, floor = 4.0;
+  if (ns == 1) {
+    fixed = 5.2 + 2.4 * f;
+  } else if (via == 0) {
+    fixed = (ns == 4 ? 5.7 : ns == 8 ? 6.0 : ns % 2 ? 7.0 : 6.4) + 2.4 * f;
+  } else {
+    fixed = 5.9 + 2.2 * f + (merge_is_small(units * mt, ns, D) ? 0.0 : 0.5) + (2 * ctas > sm_count() ? 0.4 : 0.0) +
+            (ns > 12 ? 2.0 : ns > 10 ? 0.7 : 0.0);
+    floor = 8.0;
+  }
+  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : 1.6));
+  return cost < floor ? floor - 0.01 * (floor - cost) : cost;      // (still in order below the floor)
+}
 
 Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
   const int G = Hq / Hkv;
@@ -2285,17 +2346,12 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
     pl.mt = mt;
     pl.n_mgroups = (rows + mt * kBM - 1) / (mt * kBM);
     pl.units = batch * Hkv * pl.n_mgroups;
-    const double shared = 1.0 + 0.75 / pl.n_mgroups;
-    const double tile_cost = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
-    const double fixed_scale = mt == 1 ? 1.0 : 1.6;
     // CTA pairs: one 128-wide query tile per CTA, an even number of them per work item
     const bool pair_ok = D == 128 && mt == 1 && pl.n_mgroups % 2 == 0;
-    auto consider = [&](int ns, int via_global, double waves, double fixed, double given_cost = -1.0, int pair = 0) {
+    auto consider = [&](int ns, int via_global, double waves, int pair = 0) {
       if (force_ns && (ns != force_ns || (ns > 1 && via_global != force_via))) return;
-      if (force_pair && (force_pair > 0) != (pair != 0) && (pair || pair_ok)) return;
-      const double cost = given_cost >= 0.0 ? given_cost
-                                            : waves * (((tiles + ns - 1) / ns) * tile_cost * (pair ? kPairTile : 1.0) +
-                                                       (fixed + (pair ? kPairFixed : 0.0)) * fixed_scale);
+      if (pair != (force_pair > 0 && pair_ok ? 1 : 0)) return;
+      const double cost = plan_cost(batch, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
       if (best_cost < 0.0 || cost < best_cost) {
         best = pl;
         best.nsplit = ns;
@@ -2307,28 +2363,16 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
 
     for (int ns = 1; ns <= kMaxSplit && ns <= tiles; ++ns) {
       // (a) the slices of a unit form a thread-block cluster and merge through distributed shared memory
-      const int resident = max_active_clusters_for(D, mt, ns);
-      if (resident > 0) consider(ns, 0, static_cast<double>((pl.units + resident - 1) / resident), ns == 1 ? 6.0 : 8.0);
-      if (pair_ok && ns == 1) consider(1, 0, static_cast<double>((pl.units + sm_count() - 1) / sm_count()), 6.0, -1.0, 1);
-      // (b) independent CTAs that merge through the workspace: all of them must be resident at once
-      //     (a cluster has to fit into one GPC, which can leave a third of the SMs idle)
-      //     -- either inside the launch (arrival counters, bounded spin), or with a second small launch that
-      //     combines the blocks once the first has ended (nothing waits inside a kernel)
+      const int resident = ns <= 8 || force_ns ? max_active_clusters_for(D, mt, ns) : 0;
+      if (resident > 0) consider(ns, 0, static_cast<double>((pl.units + resident - 1) / resident));
+      if (pair_ok && ns == 1) consider(1, 0, static_cast<double>((pl.units + sm_count() - 1) / sm_count()), 1);
+      // (b) independent CTAs that merge through the workspace: all of them resident at once (a cluster has to fit into
+      //     one GPC, which can leave a third of the SMs idle).  With a second small launch that combines the blocks
+      //     once the first has ended nothing waits inside a kernel.
       if (ns > 1 && static_cast<long>(pl.units) * ns <= sm_count() &&
           static_cast<size_t>(pl.units) * mt * 2 * sizeof(int) <= kCounterBytes) {
-        // measured (Qwen3-8B layer shape, prefix 4096 / 16384): with one query tile per KV head (few rows, many
-        // slices) the two-launch form is 1-3 % faster, with more query tiles the single launch is (2.6 % at 64 nodes)
-        const int via = force_via ? force_via : (pl.n_mgroups == 1 ? 2 : 1);
-        if (via == 2 && mt == 1 && pl.n_mgroups == 1) {
-          // One query tile per KV head: few work items, so the launch is a handful of tiles per CTA plus the
-          // merge.  Fitted to a sweep of 6 .. 18 slices at prefixes 2048 .. 16384 (budgets 16 and 32): 0.6 us per
-          // key tile of a CTA, 0.1 us per slice for the second launch, 0.25 us more per slice beyond 12 (in the
-          // planner's unit of 0.8 us: 0.75, 0.125, 0.31).  9 - 11 slices win up to prefix 8192, 13 - 18 beyond.
-          consider(ns, via, 1.0, 0.0, ((tiles + ns - 1) / ns) * 0.75 + 0.125 * ns + 0.31 * (ns > 12 ? ns - 12 : 0) + 9.7);
-        } else {
-          consider(ns, via, 1.0, 10.0);
-          if (pair_ok) consider(ns, via, 1.0, 10.0, -1.0, 1);
-        }
+        consider(ns, force_via ? force_via : 2, 1.0);
+        if (pair_ok) consider(ns, force_via ? force_via : 1, 1.0, 1);
       }
     }
   }
@@ -2346,6 +2390,45 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
 size_t workspace_need(const Plan& pl, int D) {
   if (!pl.via_global) return 256;
   return kCounterBytes + static_cast<size_t>(pl.units) * pl.nsplit * pl.mt * kBM * (D * 2 + 16);
+}
+
+// The shared-memory preference is that of the attention kernel: an SM that changes its split between
+// L1 and shared memory drains first, which cost 0.2 - 0.4 us per layer.
+template <int D>
+bool launch_merge(const MergeParams& m, cudaStream_t st) {
+  using Kernel = void (*)(MergeParams);
+  static const Kernel small[] = {tree_attn_merge_small_kernel<D, 4>, tree_attn_merge_small_kernel<D, 8>,
+                                 tree_attn_merge_small_kernel<D, 10>, tree_attn_merge_small_kernel<D, kMergeSmallSlices>};
+  static const Kernel large[] = {tree_attn_merge_large_kernel<D, 4>, tree_attn_merge_large_kernel<D, 8>,
+                                 tree_attn_merge_large_kernel<D, 10>, tree_attn_merge_large_kernel<D, kMergeSmallSlices>,
+                                 tree_attn_merge_large_kernel<D, kMaxSplit>};
+  static std::atomic<int> states[kMaxDevices];      // per device: 0 = not yet, 1 = ok, -1 = failed
+  std::atomic<int>& state_ref = states[current_device()];
+  int state = state_ref.load(std::memory_order_acquire);
+  if (state == 0) {
+    bool ok = true;
+    auto carve = [&](Kernel k) {
+      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    };
+    for (Kernel k : small) carve(k);
+    for (Kernel k : large) {
+      carve(k);
+      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMergeLargeSmem) == cudaSuccess;
+    }
+    if (!ok) cudaGetLastError();
+    state_ref.store(state = ok ? 1 : -1, std::memory_order_release);
+  }
+  if (state < 0) return false;
+  const int which = m.S <= 4 ? 0 : m.S <= 8 ? 1 : m.S <= 10 ? 2 : m.S <= kMergeSmallSlices ? 3 : 4;
+  const int64_t rows = static_cast<int64_t>(m.tiles) * kBM;
+  auto grid = [&](int threads) {
+    const int per = threads / (D / 8);
+    return dim3(static_cast<unsigned>((rows + per - 1) / per));
+  };
+  const bool is_small = merge_is_small(m.tiles, m.S, D);
+  launch_dependent_smem(is_small ? small[which] : large[which], is_small ? grid(kMergeSmall) : grid(kMergeLarge),
+                        dim3(is_small ? kMergeSmall : kMergeLarge), is_small ? 0 : kMergeLargeSmem, st, m);
+  return true;
 }
 
 template <int D, int MT, bool kPair = false>
@@ -2374,9 +2457,10 @@ jet_status launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMa
   cfg.attrs = attrs;
   cfg.numAttrs = na;
   const bool sorted = p.batch > 1 && p.batch <= kMaxSorted;
-  const cudaError_t err =
-      sorted ? cudaLaunchKernelEx(&cfg, tree_attn_kernel<D, MT, true, kPair>, tq, tk, tv, ttk, ttv, tk64, ttk64, p)
-             : cudaLaunchKernelEx(&cfg, tree_attn_kernel<D, MT, false, kPair>, tq, tk, tv, ttk, ttv, tk64, ttk64, p);
+  auto kernel = sorted ? tree_attn_kernel<D, MT, true, kPair> : tree_attn_kernel<D, MT, false, kPair>;
+  if constexpr (MT == 1 && !kPair)
+    if (pl.via_global == 2) kernel = sorted ? tree_attn_kernel<D, 1, true, false, true> : tree_attn_kernel<D, 1, false, false, true>;
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, tq, tk, tv, ttk, ttv, tk64, ttk64, p);
   if (err != cudaSuccess) {
 #ifdef JET_TRACE
     fprintf(stderr, "attention launch failed: %s (grid %d x %d x %d, cluster %d, %d slices, merge form %d, D %d, MT %d)\n",
@@ -2394,8 +2478,8 @@ jet_status launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMa
     m.lse = p.lse;
     m.B = p.B; m.Hq = p.Hq; m.Hkv = p.Hkv; m.G = p.G; m.S = pl.nsplit; m.MT = MT; m.n_mgroups = pl.n_mgroups; m.npt = p.npt;
     m.magic_G = p.magic_G;
-    constexpr int kRowsPerCta = 256 / (D / 8);
-    launch_dependent(tree_attn_merge_kernel<D>, dim3((kBM / kRowsPerCta) * MT * pl.n_mgroups, p.Hkv, p.batch), dim3(256), st, m);
+    m.tiles = pl.units * MT;
+    if (!launch_merge<D>(m, st)) return JET_ERR_CUDA;
   }
   return launch_status();
 }
