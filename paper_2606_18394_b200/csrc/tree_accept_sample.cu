@@ -4,7 +4,7 @@
 //   row_lse_partial_kernel  grid (slices, batch*B): one pass over the target logits; every block
 //                           leaves the maximum and the sum of exp((x - max) / T) of one 8192-entry
 //                           slice of one row in the workspace.  Padding rows are not read.
-//   accept_sample_kernel    one cluster of 8 CTAs per sequence, 512 threads each: finishes the rows' log-sum-exp, computes
+//   accept_sample_kernel    one cluster of 8 CTAs per sequence, 512 or 1024 threads each: finishes the rows' log-sum-exp, computes
 //                           alpha_v = min(1, p_parent(token_v) / q_depth(token_v)) and the accept
 //                           bit u_v < alpha_v for every node, picks the deepest node whose whole
 //                           branch is accepted, then draws the correction token at that node by
@@ -23,14 +23,15 @@ namespace {
 constexpr int kLseThreads = 256;
 constexpr int kLseElems = 32;
 constexpr int kLseChunk = kLseThreads * kLseElems;
-// One thread per node of the largest tree.  Bound of the sampling kernel: latency -- each CTA reads some 20 KB of logits
-// and log-probabilities behind a chain of small dependent look-ups.  512 threads (with at most 64 registers two CTAs share an
-// SM: the 256 CTAs of a batch of 32 are one wave, not two) and kSampleUnroll steps of loads in flight per warp:
-// 32 sequences of 64 nodes, V 151936: 227 -> 215 us for both launches (the scan's 1.25 GB alone need 190 us at the measured
-// copy bandwidth).
-constexpr int kSampleThreads = 512;
+// Bound of the sampling kernel: latency -- a CTA reads some 20 KB of logits and log-probabilities behind a chain of small
+// dependent look-ups, kSampleUnroll steps of loads in flight per warp.  While the device holds all clusters with one CTA
+// per SM (15 of them: a cluster of eight has to fit into one GPC) it takes 1024 threads; beyond that 512 (a thread per node of the largest tree; at most 64 registers), so that two share an
+// SM: the 256 CTAs of a batch of 32 are one wave, not two.  32 sequences of 64 nodes, V 151936: 217 -> 205 us for both
+// launches (reading the 1.25 GB of logits alone takes 190 us at the measured copy bandwidth).
+constexpr int kSampleThreadsFew = 1024, kSampleThreadsMany = 512;
+constexpr int kSampleFewBatch = 15;
 constexpr int kSampleUnroll = 2;           // (three spill at 64 registers)
-static_assert(kSampleThreads >= JET_MAX_NODES, "a thread per node");
+static_assert(kSampleThreadsMany >= JET_MAX_NODES, "a thread per node");
 constexpr int kSampleStep = 128;          // vocabulary entries a warp handles per step (4 per lane)
 constexpr int kSampleCluster = 8;         // CTAs per sequence
 constexpr int kMaxStepsTotal = 4096;      // 128-entry steps per row: vocabularies up to 524288 entries
@@ -73,6 +74,21 @@ row_lse_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int
       const float4 q = __ldcs(p4 + i * kLseThreads + tid);
       x[i * 4 + 0] = q.x; x[i * 4 + 1] = q.y; x[i * 4 + 2] = q.z; x[i * 4 + 3] = q.w;
     }
+  } else if (vec_ok) {
+    // the row's last, partial slice: still 16-byte loads wherever four entries are in range
+#pragma unroll
+    for (int i = 0; i < kLseElems / 4; ++i) {
+      const int idx = base + (i * kLseThreads + tid) * 4;
+      float4 q = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      if (idx + 3 < V) {
+        q = __ldcs(reinterpret_cast<const float4*>(p + idx));
+      } else {
+        if (idx < V) q.x = __ldcs(p + idx);
+        if (idx + 1 < V) q.y = __ldcs(p + idx + 1);
+        if (idx + 2 < V) q.z = __ldcs(p + idx + 2);
+      }
+      x[i * 4 + 0] = q.x; x[i * 4 + 1] = q.y; x[i * 4 + 2] = q.z; x[i * 4 + 3] = q.w;
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < kLseElems; ++i) {
@@ -107,7 +123,8 @@ row_lse_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int
   }
 }
 
-__global__ void __launch_bounds__(kSampleThreads, 2)
+template <int kSampleThreads>
+__global__ void __launch_bounds__(kSampleThreads, 1024 / kSampleThreads)
 accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const float* __restrict__ logits,
                      int64_t row_stride, float inv_t, const float* __restrict__ draft_logp,
                      int64_t logp_batch_stride, int64_t logp_depth_stride,
@@ -402,7 +419,8 @@ extern "C" jet_status jet_tree_accept_sample(const float* logits, int64_t logits
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch * kSampleCluster);
-    cfg.blockDim = dim3(kSampleThreads);
+    const bool few = batch <= kSampleFewBatch;
+    cfg.blockDim = dim3(few ? kSampleThreadsFew : kSampleThreadsMany);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -414,7 +432,8 @@ extern "C" jet_status jet_tree_accept_sample(const float* logits, int64_t logits
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, accept_sample_kernel, static_cast<const float2*>(partial), nchunks, logits,
+    auto kernel = few ? accept_sample_kernel<kSampleThreadsFew> : accept_sample_kernel<kSampleThreadsMany>;
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<const float2*>(partial), nchunks, logits,
                            logits_row_stride, inv_t, draft_logp, logp_batch_stride, logp_depth_stride, token, parent,
                            depth, anc_mask, n_nodes, u_accept, u_sample, B, V, N, vec_rows, alpha, accept_len, path,
                            out_tokens) != cudaSuccess) {
