@@ -25,9 +25,10 @@ constexpr int kLseElems = 32;
 constexpr int kLseChunk = kLseThreads * kLseElems;
 // Bound of the sampling kernel: latency -- a CTA reads some 20 KB of logits and log-probabilities behind a chain of small
 // dependent look-ups, kSampleUnroll steps of loads in flight per warp.  While the device holds all clusters with one CTA
-// per SM (15 of them: a cluster of eight has to fit into one GPC) it takes 1024 threads; beyond that 512 (a thread per node of the largest tree; at most 64 registers), so that two share an
-// SM: the 256 CTAs of a batch of 32 are one wave, not two.  32 sequences of 64 nodes, V 151936: 217 -> 205 us for both
-// launches (reading the 1.25 GB of logits alone takes 190 us at the measured copy bandwidth).
+// per SM (15 of them: a cluster of eight has to fit into one GPC) it takes 1024 threads; beyond that 512 (a thread per node
+// of the largest tree; at most 64 registers), so that two share an SM: the 256 CTAs of a batch of 32 are one wave, not
+// two.  32 sequences of 64 nodes, V 151936: 217 -> 205 us for both launches (reading the 1.25 GB of logits alone takes
+// 190 us at the measured copy bandwidth).
 constexpr int kSampleThreadsFew = 1024, kSampleThreadsMany = 512;
 constexpr int kSampleFewBatch = 15;
 constexpr int kSampleUnroll = 2;           // (three spill at 64 registers)
