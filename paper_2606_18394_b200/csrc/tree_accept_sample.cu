@@ -29,6 +29,9 @@ constexpr int kLseChunk = kLseThreads * kLseElems;
 // of the largest tree; at most 64 registers), so that two share an SM: the 256 CTAs of a batch of 32 are one wave, not
 // two.  32 sequences of 64 nodes, V 151936: 217 -> 205 us for both launches (reading the 1.25 GB of logits alone takes
 // 190 us at the measured copy bandwidth).
+// One sequence of 61 nodes, V 151936, inside a step: 27.8 -> 24.0 us for both launches with the look-ups that do not need the
+// scan in front of the dependency wait, the rows' later steps prefetched, the step table read eight entries at a time
+// and one cluster barrier fewer.
 constexpr int kSampleThreadsFew = 1024, kSampleThreadsMany = 512;
 constexpr int kSampleFewBatch = 15;
 constexpr int kSampleUnroll = 2;           // (three spill at 64 registers)
@@ -135,10 +138,9 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
                      const float* __restrict__ u_sample, int B, int V, int N, bool vec_rows, float* __restrict__ alpha_out,
                      int32_t* __restrict__ accept_len, int32_t* __restrict__ path,
                      int32_t* __restrict__ out_tokens) {
-  grid_dependency_wait();
   __shared__ float s_max[JET_MAX_NODES], s_lnsum[JET_MAX_NODES];      // per row: max, ln sum exp((x - max) / T)
   __shared__ uint32_t s_ok[JET_MAX_NODES / 32], s_best[kSampleThreads / 32], s_end_row[JET_MAX_NODES / 32];
-  __shared__ int s_end, s_has_child, s_pick_warp, s_pick_step, s_token;
+  __shared__ int s_end, s_has_child, s_retry, s_pick_step, s_token;
   __shared__ double s_step[kMaxStepsTotal], s_before, s_target;      // CTA 0: mass of every 128-entry step, vocabulary order
 
   namespace cg = cooperative_groups;
@@ -150,6 +152,19 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   const size_t o = static_cast<size_t>(b) * B;
   const bool live = v < n;
   const float* lp = draft_logp + b * logp_batch_stride;
+
+  // The launch before this one is the scan, which lets its successor start only once everything before IT has finished, and
+  // which writes nothing but the slices' statistics: the tree, its draft log-probabilities and the target's logits at its
+  // tokens -- two dependent look-ups, usually from DRAM -- are read here, under the scan's tail.
+  int my_parent = -1, my_depth = -1, my_token = -1;
+  float my_u = 0.0f, lq = -INFINITY, my_x = 0.0f;
+  if (live) { my_parent = parent[o + v]; my_depth = depth[o + v]; my_token = token[o + v]; my_u = u_accept[o + v]; }
+  const bool rated = live && v > 0 && my_parent >= 0 && my_parent < n && my_token >= 0 && my_token < V && my_depth >= 1 && my_depth <= N;
+  if (rated) {
+    lq = lp[static_cast<int64_t>(my_depth - 1) * logp_depth_stride + my_token];
+    my_x = logits[static_cast<int64_t>(o + my_parent) * row_stride + my_token];
+  }
+  grid_dependency_wait();
 
   // ---- row statistics
   if (live) {
@@ -170,18 +185,14 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   __syncthreads();
 
   // ---- alpha_v = min(1, p_parent(token) / q_depth(parent)(token)); accepted iff u_v < alpha_v
-  int my_parent = -1, my_depth = -1, my_token = -1;
   float alpha = 1.0f;
   bool ok = live && v == 0;
-  if (live) { my_parent = parent[o + v]; my_depth = depth[o + v]; my_token = token[o + v]; }
-  if (live && v > 0 && my_parent >= 0 && my_parent < n && my_token >= 0 && my_token < V && my_depth >= 1 && my_depth <= N) {
-    const float lq = lp[static_cast<int64_t>(my_depth - 1) * logp_depth_stride + my_token];
+  if (rated) {
     if (lq > -INFINITY) {
-      const float x = logits[static_cast<int64_t>(o + my_parent) * row_stride + my_token];
-      const float lr = (x - s_max[my_parent]) * inv_t - s_lnsum[my_parent] - lq;      // ln(p / q)
+      const float lr = (my_x - s_max[my_parent]) * inv_t - s_lnsum[my_parent] - lq;      // ln(p / q)
       alpha = lr >= 0.0f ? 1.0f : expf(lr);
     }
-    ok = u_accept[o + v] < alpha;
+    ok = my_u < alpha;
   }
   if (alpha_out && v < B) alpha_out[o + v] = live ? alpha : 0.0f;
   const uint32_t okbits = __ballot_sync(0xffffffffu, ok);
@@ -257,6 +268,12 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   int picked = -1;
   for (int attempt = 0; attempt < 2; ++attempt) {
     const int last_step = min(first_step + steps, total_steps);
+    if (lane < 4)                                              // (a step is four lines of 128 bytes; the draft's row is cold)
+      for (int g = first_step + kSampleUnroll; g < last_step; ++g) {
+        const int idx = min(g * kSampleStep + lane * 32, V - 1);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(xrow + idx));
+        if (use_residual) asm volatile("prefetch.global.L2 [%0];" ::"l"(qrow + idx));
+      }
     for (int g0 = first_step; g0 < last_step; g0 += kSampleUnroll) {
       float x4[kSampleUnroll][4], q4[kSampleUnroll][4];
 #pragma unroll
@@ -279,6 +296,7 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
         const int per_lane = (total_steps + 31) / 32;
         const int s_lo = lane * per_lane, s_hi = min(total_steps, s_lo + per_lane);
         double tot_l = 0.0;
+#pragma unroll 8
         for (int g = s_lo; g < s_hi; ++g) tot_l += s_step[g];
         double cum_l = tot_l;
 #pragma unroll
@@ -298,13 +316,18 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
           double run = cum_l - tot_l;
           int last_step = -1;
           double last_before = 0.0;
-          for (int g = s_lo; g < s_hi; ++g) {
-            const double m = s_step[g];
-            if (m > 0.0) {
-              last_step = g; last_before = run;
-              if (run + m > target) { ps = g; before = run; break; }
+          for (int g0 = s_lo; g0 < s_hi && ps < 0; g0 += 8) {  // (eight entries read at once, then added in order)
+            double m8[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m8[k] = g0 + k < s_hi ? s_step[g0 + k] : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              if (ps < 0 && m8[k] > 0.0) {
+                last_step = g0 + k; last_before = run;
+                if (run + m8[k] > target) { ps = g0 + k; before = run; }
+              }
+              run += m8[k];
             }
-            run += m;
           }
           if (ps < 0) { ps = last_step; before = last_before; }
           s_pick_step = ps;
@@ -353,13 +376,11 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
       __syncthreads();
       picked = s_token;
     }
-    // the whole cluster learns whether the pass has to be repeated with p itself (only when the residual is empty)
-    int* retry_flag = cluster.map_shared_rank(&s_pick_warp, 0);
-    if (rank == 0 && v == 0) s_pick_warp = retry ? 1 : 0;
+    // the whole cluster learns whether the pass has to be repeated with p itself (only when the residual is empty): CTA 0
+    // leaves the verdict in every CTA's own shared memory (written again, if at all, behind the next pass's barrier)
+    if (rank == 0 && v < kSampleCluster) *cluster.map_shared_rank(&s_retry, v) = retry ? 1 : 0;
     cluster.sync();
-    const bool again = *retry_flag != 0 && use_residual;
-    cluster.sync();                                            // everybody has read the flag before it changes again
-    if (!again) break;
+    if (s_retry == 0 || !use_residual) break;
     use_residual = false;
   }
   if (rank != 0) return;                                       // CTA 0 alone writes the results
