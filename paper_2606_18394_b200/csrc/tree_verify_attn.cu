@@ -2284,7 +2284,7 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // budgets 16 - 256, prefixes 128 - 16384 (the plans chosen were within 0.4 us of the best form of each shape, most within 0.1):
 //   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power), or what HBM takes for the K/V tiles of all
 //                          CTAs that do not share one (1.45 f / g at D 128, g = CTAs that read the same tile side by side);
-//                          1.76 with two query tiles (two softmax chains share a tensor core)
+//                          1.65 with two query tiles (two softmax chains share a tensor core)
 //   fixed, no slices       5.2 + 2.4 f
 //   slices in a cluster    5.7 with four, 6.0 with eight, 7.0 with an odd number, else 6.4, + 2.4 f.  (Four and eight: the
 //                          shape of the row exchange is a power of two.)  Clusters of up to eight CTAs are
@@ -2292,21 +2292,21 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 //   a second launch merges 5.9 + 2.2 f, + 0.5 with the large merge CTAs, + 0.4 when two CTAs have to share a TPC, + 0.7 and 2.0 with
 //                          more than 10 and 12 slices (longer merge code); never below the 4 us of host time that each
 //                          launch costs a caller who issues layer by layer
-// all of the fixed part 1.6 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
+// all of the fixed part 1.45 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
 // at once.  The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
 // second launch at every shape, and CTA pairs need 1.22 times the key-tile time (the hand-overs cross two SMs): both
 // run where they are asked for (JET_FORCE_SPLIT="<slices>,g", JET_FORCE_PAIR=1).
-// More than four sequences (ragged, usually paged, and enough work items for several waves): the fit above does not cover them.  There
+// More than four sequences (ragged, usually paged) or more than 64 query tiles: the fit above does not cover them.  There
 // the unit is a key tile out of L2 (0.8 us), a tile costs 1 + 0.75 / g and the fixed parts are 6 / 8 / 10 (none, cluster, second
 // launch): with few CTAs per K/V tile this prefers more, shorter CTAs, which even out sequences of different lengths
 // (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).
-double plan_cost(int batch, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
-  if (batch > 4) {
+double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
+  if (!fitted) {
     const double shared = 1.0 + 0.75 / n_mgroups, per_tile = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
     return waves * ((tiles + ns - 1) / ns * per_tile + (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) * (mt == 1 ? 1.0 : 1.6));
   }
   const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
-  double tile = mt == 1 ? 0.78 + 0.14 * f : 1.76;
+  double tile = mt == 1 ? 0.78 + 0.14 * f : 1.65;
   const double hbm = 1.45 * f * D / 128 / n_mgroups;
   if (tile < hbm) tile = hbm;
   double fixed, floor = 4.0;
@@ -2319,7 +2319,7 @@ double plan_cost(int batch, int mt, int ns, int via, double waves, int ctas, int
             (ns > 12 ? 2.0 : ns > 10 ? 0.7 : 0.0);
     floor = 8.0;
   }
-  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : 1.6));
+  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : 1.45));
   return cost < floor ? floor - 0.01 * (floor - cost) : cost;      // (still in order below the floor)
 }
 
@@ -2327,6 +2327,7 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
   const int G = Hq / Hkv;
   const int rows = B * G;
   const int tiles = (max_seq_len + kBN - 1) / kBN + (B + kBN - 1) / kBN;
+  const bool fitted = batch <= 4 && batch * Hkv * ((rows + kBM - 1) / kBM) <= 64;      // the range plan_cost was fitted over
   Plan best{};
   double best_cost = -1.0;
   // Test hooks (read once per process): JET_FORCE_MT = query tiles per CTA, JET_FORCE_SPLIT = "slices" or
@@ -2351,7 +2352,7 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
     auto consider = [&](int ns, int via_global, double waves, int pair = 0) {
       if (force_ns && (ns != force_ns || (ns > 1 && via_global != force_via))) return;
       if (pair != (force_pair > 0 && pair_ok ? 1 : 0)) return;
-      const double cost = plan_cost(batch, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
+      const double cost = plan_cost(fitted, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
       if (best_cost < 0.0 || cost < best_cost) {
         best = pl;
         best.nsplit = ns;
