@@ -60,3 +60,11 @@ def test_logits_beyond_the_table_form(offset, spread):
     z[0, 1, :4096] = -np.inf                         # a slice without a finite entry
     compare_logits(z, [2], 3, 6, 30, "accum_logp", 0.0)
     compare_logits(z, [2], 3, 6, 30, "hybrid", 0.5)
+
+
+@pytest.mark.parametrize("V,W", [(9, 9), (1150, 9), (1350, 9), (4096, 32), (4097, 32), (12160, 5), (16384, 9), (16385, 10)])
+def test_rows_of_few_groups(V, W):
+    rng = np.random.default_rng(V + W)
+    compare_logits(np.stack([make_draft_logits(rng, 4, V, 3.0) for _ in range(2)]), [7, 8], 4, W, 163, "hybrid", 0.5)
+    compare_scored(np.stack([make_logp(rng, 1, V, 3.0, peaked_p=0.6)]), [7], 1, W, 20, "accum_logp", 0.0)
+    compare_logits(np.zeros((1, 2, V), np.float32), [7], 2, W, 50, "accum_logp", 0.0)
