@@ -2284,7 +2284,7 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // budgets 16 - 256, prefixes 128 - 16384 (the plans chosen were within 0.4 us of the best form of each shape, most within 0.1):
 //   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power), or what HBM takes for the K/V tiles of all
 //                          CTAs that do not share one (1.45 f / g at D 128, g = CTAs that read the same tile side by side);
-//                          1.65 with two query tiles (two softmax chains share a tensor core)
+//                          1.65 (second launch) or 1.75 with two query tiles (two softmax chains share a tensor core)
 //   fixed, no slices       5.2 + 2.4 f
 //   slices in a cluster    5.7 with four, 6.0 with eight, 7.0 with an odd number, else 6.4, + 2.4 f.  (Four and eight: the
 //                          shape of the row exchange is a power of two.)  Clusters of up to eight CTAs are
@@ -2292,7 +2292,7 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 //   a second launch merges 5.9 + 2.2 f, + 0.5 with the large merge CTAs, + 0.4 when two CTAs have to share a TPC, + 0.7 and 2.0 with
 //                          more than 10 and 12 slices (longer merge code); never below the 4 us of host time that each
 //                          launch costs a caller who issues layer by layer
-// all of the fixed part 1.45 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
+// all of the fixed part 1.45 or 1.6 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
 // at once.  The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
 // second launch at every shape, and CTA pairs need 1.22 times the key-tile time (the hand-overs cross two SMs): both
 // run where they are asked for (JET_FORCE_SPLIT="<slices>,g", JET_FORCE_PAIR=1).
@@ -2306,7 +2306,7 @@ double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, i
     return waves * ((tiles + ns - 1) / ns * per_tile + (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) * (mt == 1 ? 1.0 : 1.6));
   }
   const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
-  double tile = mt == 1 ? 0.78 + 0.14 * f : 1.65;
+  double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.65 : 1.75;
   const double hbm = 1.45 * f * D / 128 / n_mgroups;
   if (tile < hbm) tile = hbm;
   double fixed, floor = 4.0;
@@ -2319,7 +2319,7 @@ double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, i
             (ns > 12 ? 2.0 : ns > 10 ? 0.7 : 0.0);
     floor = 8.0;
   }
-  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : 1.45));
+  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : via == 2 ? 1.45 : 1.6));
   return cost < floor ? floor - 0.01 * (floor - cost) : cost;      // (still in order below the floor)
 }
 
