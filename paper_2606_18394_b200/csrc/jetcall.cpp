@@ -6,9 +6,13 @@
 // library's own host work (attention call as a whole 19.6 -> 5 us).  Only argument marshalling lives here: every
 // function calls the C function of the same name in libjet.so with the GIL released and returns its status.
 //
-// A device pointer is None, an int, a torch tensor, or anything with a data_ptr() method.
+// A device pointer is None, an int, a torch tensor, or anything with a data_ptr() method.  Plain tensors (and Parameters) are
+// read natively; a subclass is asked through its own Python methods, which it may override.  A tensor without an address
+// (sparse, wrapped by a transform) makes at::Tensor throw: the entry points below turn that into the Python exception
+// that the tensor's own method raises (see guarded).
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "jet.h"
@@ -41,6 +45,15 @@ class Args {
     PyObject* o = next();
     if (!o) return nullptr;
     if (!THPVariable_Check(o)) return address(o);
+    if (!THPVariable_CheckExact(o)) {
+      PyObject* index = PyLong_FromLongLong(layer);
+      PyObject* slice = index ? PyObject_GetItem(o, index) : nullptr;
+      if (!slice) bad_ = true;
+      void* p = slice ? address(slice) : nullptr;
+      Py_XDECREF(slice);
+      Py_XDECREF(index);
+      return p;
+    }
     const at::Tensor& t = THPVariable_Unpack(o);
     const int64_t n = t.dim() > 0 ? t.size(0) : 0;
     if (layer < -n || layer >= n) {
@@ -93,15 +106,7 @@ class Args {
   void* stream() {
     PyObject* o = next();
     if (!o) return nullptr;
-    if (o == Py_None) {
-      try {
-        return c10::cuda::getCurrentCUDAStream().stream();
-      } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        bad_ = true;
-        return nullptr;
-      }
-    }
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
     if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
     PyObject* s = PyObject_GetAttrString(o, "cuda_stream");
     void* p = s ? PyLong_AsVoidPtr(s) : nullptr;
@@ -119,7 +124,7 @@ class Args {
   }
   void* address(PyObject* o) {
     if (o == Py_None) return nullptr;
-    if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+    if (THPVariable_CheckExact(o)) return THPVariable_Unpack(o).data_ptr();
     PyObject* v = PyLong_Check(o) ? Py_NewRef(o) : PyObject_CallMethod(o, "data_ptr", nullptr);
     void* p = v ? PyLong_AsVoidPtr(v) : nullptr;
     Py_XDECREF(v);
@@ -136,21 +141,46 @@ const T* in(void* p) { return static_cast<const T*>(p); }
 template <typename T>
 T* out(void* p) { return static_cast<T*>(p); }
 
+class WithoutGil {
+ public:
+  WithoutGil() : state_(PyEval_SaveThread()) {}
+  ~WithoutGil() { PyEval_RestoreThread(state_); }
+
+ private:
+  PyThreadState* state_;
+};
+
 #define JET_CALL(expr)                       \
   do {                                       \
     if (a.bad()) return nullptr;             \
     jet_status status;                       \
-    Py_BEGIN_ALLOW_THREADS;                  \
-    status = (expr);                         \
-    Py_END_ALLOW_THREADS;                    \
+    {                                        \
+      WithoutGil no_gil;                     \
+      status = (expr);                       \
+    }                                        \
     return PyLong_FromLong(status);          \
   } while (0)
+
+using Entry = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
+
+// An exception that leaves a function the interpreter calls ends the process; here it becomes a Python exception.
+template <Entry kEntry>
+PyObject* guarded(PyObject* self, PyObject* const* argv, Py_ssize_t argc) {
+  HANDLE_TH_ERRORS
+  return kEntry(self, argv, argc);
+  END_HANDLE_TH_ERRORS
+}
 
 // Strides of [batch, N, V] rows: given, or None = those of the tensor itself.
 void row_strides(PyObject* rows, PyObject* const* given, int64_t (&s)[2], bool* bad) {
   for (int d = 0; d < 2; ++d) {
-    if (given[d] == Py_None && THPVariable_Check(rows) && THPVariable_Unpack(rows).dim() > d) {
+    if (given[d] == Py_None && THPVariable_CheckExact(rows) && THPVariable_Unpack(rows).dim() > d) {
       s[d] = THPVariable_Unpack(rows).stride(d);
+    } else if (given[d] == Py_None && THPVariable_Check(rows)) {
+      PyObject* v = PyObject_CallMethod(rows, "stride", "i", d);
+      s[d] = v ? PyLong_AsLongLong(v) : -1;
+      Py_XDECREF(v);
+      if (s[d] == -1 && PyErr_Occurred()) { *bad = true; return; }
     } else {
       s[d] = PyLong_AsLongLong(given[d]);
       if (s[d] == -1 && PyErr_Occurred()) { *bad = true; return; }
@@ -367,7 +397,7 @@ PyObject* kv_compact(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
                                  D, N, st));
 }
 
-#define JET_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+#define JET_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {JET_METHOD(tree_build),         JET_METHOD(tree_build_scored),  JET_METHOD(tree_verify_attn),
                          JET_METHOD(tree_accept),        JET_METHOD(tree_accept_hidden), JET_METHOD(tree_accept_sample),
                          JET_METHOD(kv_compact),         {nullptr, nullptr, 0, nullptr}};
