@@ -110,6 +110,9 @@ def native():
         except ImportError as e:
             raise RuntimeError("the extension module _jetcall is missing or does not load: build it with "
                                "`python -m paper_2606_18394_b200.build`; there is no fallback path") from e
+        if _jetcall.torch_version != str(torch.__version__):
+            raise RuntimeError(f"the extension module _jetcall was built for torch {_jetcall.torch_version}, this is "
+                               f"{torch.__version__}: build it again with `python -m paper_2606_18394_b200.build`")
         _ext = _jetcall
     return _ext
 

@@ -1,6 +1,7 @@
 """Builds libjet.so (the C-ABI library, nvcc for sm_100a) and the binding's CPython extension in-tree."""
 from __future__ import annotations
 
+import json
 import os
 import subprocess
 import sys
@@ -12,6 +13,8 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libjet.so")
 # the binding's argument marshalling (a CPython extension linked against libjet.so and torch)
 EXT = os.path.join(PKG, "_jetcall" + sysconfig.get_config_var("EXT_SUFFIX"))
+# what the extension was built for: it links torch's libraries, whose C++ interface changes between versions
+STAMP = os.path.join(PKG, "build", "jetcall.json")
 SOURCES = ["jet_api.cu", "tree_build.cu", "tree_verify_attn.cu", "tree_accept.cu", "tree_accept_sample.cu",
            "kv_compact.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -27,8 +30,19 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def _environment() -> dict:
+    import torch
+    return {"torch": str(torch.__version__), "cxx11_abi": int(torch._C._GLIBCXX_USE_CXX11_ABI), "python": sys.version.split()[0]}
+
+
 def needs_build() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(EXT):
+        return True
+    try:
+        with open(STAMP) as f:
+            if json.load(f) != _environment():
+                return True
+    except (OSError, ValueError):
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(EXT))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "jet.h")]
@@ -43,7 +57,8 @@ def _extension_commands(obj: str) -> tuple[list[str], list[str]]:
     inc = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(troot, "include"),
            os.path.join(troot, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
     compile_cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden",
-                   f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(x for i in inc for x in ("-I", i)),
+                   f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                   f'-DJET_TORCH_VERSION="{torch.__version__}"', *(x for i in inc for x in ("-I", i)),
                    "-c", os.path.join(CSRC, "jetcall.cpp"), "-o", obj]
     link_cmd = ["g++", "-shared", "-o", EXT, obj, "-L", PKG, "-l:libjet.so", "-L", os.path.join(troot, "lib"),
                 "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
@@ -81,6 +96,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             "-Xcompiler", "-fPIC"]
     subprocess.run(link, check=True)
     subprocess.run(ext_link, check=True)
+    with open(STAMP, "w") as f:
+        json.dump(_environment(), f)
     return LIB
 
 

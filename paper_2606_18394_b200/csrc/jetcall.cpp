@@ -406,4 +406,8 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_jetcall", "argument marshalli
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__jetcall() { return PyModule_Create(&module_def); }
+PyMODINIT_FUNC PyInit__jetcall() {
+  PyObject* m = PyModule_Create(&module_def);
+  if (m && PyModule_AddStringConstant(m, "torch_version", JET_TORCH_VERSION) != 0) Py_CLEAR(m);
+  return m;
+}
