@@ -2280,10 +2280,8 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 }
 
 // Picks the query-tile grouping, the number of key slices and the form of their merge with a cost model, in microseconds
-// of a launch in the steady state of a layer stack, fitted to a sweep of all forms and slice counts over batches 1 - 4,
-// budgets 16 - 256, prefixes 128 - 16384 (the plans chosen were within 0.4 us of the best form of each shape, most within 0.1):
-//   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power), or what HBM takes for the K/V tiles of all
-//                          CTAs that do not share one (1.45 f / g at D 128, g = CTAs that read the same tile side by side);
+// of a launch in the steady state of a layer stack:
+//   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power);
 //                          1.65 (second launch) or 1.75 with two query tiles (two softmax chains share a tensor core)
 //   fixed, no slices       5.2 + 2.4 f
 //   slices in a cluster    5.7 with four, 6.0 with eight, 7.0 with an odd number, else 6.4, + 2.4 f.  (Four and eight: the
@@ -2293,22 +2291,30 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 //                          more than 10 and 12 slices (longer merge code); never below the 4 us of host time that each
 //                          launch costs a caller who issues layer by layer
 // all of the fixed part 1.45 or 1.6 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
-// at once.  The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
+// at once.  There is no term for what HBM delivers: where it binds it binds every form alike, and the host knows only the
+// longest sequence.  (A term that charged 1.45 f / g per tile as if all sequences had that length kept ragged batches on
+// fewer slices: three sequences of 4548 - 19896 keys, 15 nodes, 32 / 8 heads, paged: 52.4 us with four slices of 24 work items
+// against 41.5 with six.)
+// The range this holds for, `fitted`: up to four sequences and 64 query tiles.  Measured against all forms of 1003 shapes there
+// (budgets 4 - 512, prefixes 64 - 100000, D 64 and 128, contiguous and paged, lengths of a batch spread from 20 to 100 % of
+// the longest): the plans chosen take 1.9 % more than the best form of each shape on average, more than 5 % at 139 of them,
+// 31 % at worst; with the HBM term 2.5 %, 182, 38 %.
+// Beyond it -- more than four sequences or 64 query tiles -- the unit is a key tile out of L2 (0.8 us), a tile costs
+// 1 + 0.75 / g (g = CTAs that read the same tile side by side) and the fixed parts are 6 / 8 / 10 (none, cluster, second
+// launch): with few CTAs per K/V tile this prefers more, shorter CTAs, which even out sequences of different lengths
+// (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).  There the
+// plans take 4.2 % more than the best form on average (735 shapes), and waves are whole numbers, so that two forms whose
+// costs are a per cent apart change places by chance.
+// The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
 // second launch at every shape, and CTA pairs need 1.22 times the key-tile time (the hand-overs cross two SMs): both
 // run where they are asked for (JET_FORCE_SPLIT="<slices>,g", JET_FORCE_PAIR=1).
-// More than four sequences (ragged, usually paged) or more than 64 query tiles: the fit above does not cover them.  There
-// the unit is a key tile out of L2 (0.8 us), a tile costs 1 + 0.75 / g and the fixed parts are 6 / 8 / 10 (none, cluster, second
-// launch): with few CTAs per K/V tile this prefers more, shorter CTAs, which even out sequences of different lengths
-// (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).
 double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
   if (!fitted) {
     const double shared = 1.0 + 0.75 / n_mgroups, per_tile = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
     return waves * ((tiles + ns - 1) / ns * per_tile + (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) * (mt == 1 ? 1.0 : 1.6));
   }
   const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
-  double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.65 : 1.75;
-  const double hbm = 1.45 * f * D / 128 / n_mgroups;
-  if (tile < hbm) tile = hbm;
+  const double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.65 : 1.75;
   double fixed, floor = 4.0;
   if (ns == 1) {
     fixed = 5.2 + 2.4 * f;
@@ -2327,7 +2333,7 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
   const int G = Hq / Hkv;
   const int rows = B * G;
   const int tiles = (max_seq_len + kBN - 1) / kBN + (B + kBN - 1) / kBN;
-  const bool fitted = batch <= 4 && batch * Hkv * ((rows + kBM - 1) / kBM) <= 64;      // the range plan_cost was fitted over
+  const bool fitted = batch <= 4 && batch * Hkv * ((rows + kBM - 1) / kBM) <= 64;      // (see plan_cost)
   Plan best{};
   double best_cost = -1.0;
   // Test hooks (read once per process): JET_FORCE_MT = query tiles per CTA, JET_FORCE_SPLIT = "slices" or
