@@ -227,17 +227,26 @@ constexpr int kExpThreads = JET_MAX_NODES;
 constexpr int kExpWarps = kExpThreads / 32;
 constexpr int kListCap = 32 + kGroup;                // candidates a warp keeps: the best so far and one group's worth
 
-// The Wc-th largest of the warp's 32 lane values: largest value after largest value until Wc lanes are covered.  (Rolled: this
-// code runs once per launch, from a cold instruction cache, where its length is its cost.)
-__device__ __forceinline__ float warp_nth(float x, int Wc) {
-  uint32_t rest = f32_order(x);                      // 0 = covered (no number has code 0)
+// The Wc-th largest of the warp's 32 kPer values, kPer of them in every lane: largest value after largest value until Wc are
+// covered.  (Rolled: this code runs once per launch, from a cold instruction cache, where its length is its cost.)
+template <int kPer>
+__device__ __forceinline__ float warp_nth(const float (&x)[kPer], int Wc) {
+  uint32_t rest[kPer];                               // 0 = covered (no number has code 0)
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) rest[i] = f32_order(x[i]);
   uint32_t top = 0u;
 #pragma unroll 1
   for (int covered = 0; covered < Wc;) {
-    top = __reduce_max_sync(0xffffffffu, rest);
-    const bool hit = rest == top;
-    covered += __popc(__ballot_sync(0xffffffffu, hit));
-    if (hit) rest = 0u;
+    uint32_t mine = rest[0];
+#pragma unroll
+    for (int i = 1; i < kPer; ++i) mine = max(mine, rest[i]);
+    top = __reduce_max_sync(0xffffffffu, mine);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const bool hit = rest[i] == top;
+      covered += __popc(__ballot_sync(0xffffffffu, hit));
+      if (hit) rest[i] = 0u;
+    }
   }
   return __uint_as_float((top & 0x80000000u) ? (top & 0x7FFFFFFFu) : ~top);
 }
@@ -290,15 +299,27 @@ __device__ __forceinline__ float rank_value(float x, double lse) {
   return kLogits ? static_cast<float>(static_cast<double>(x) - lse) : x;
 }
 
-// More groups or entries at or above the threshold than the fast form holds (many nearly equal values): the groups one
-// after the other, in ascending order; an entry is listed only if it beats the worst of the best so far.
+constexpr int kBatch = 8;                            // groups whose entries are in flight together
+constexpr int kTopGroups = 64;                       // qualifying groups the fast form lists
+
+struct TopScratch {
+  unsigned long long list[kListCap];
+  int groups[kTopGroups];
+};
+
+// More groups or entries at or above the threshold than the fast form holds (equal or nearly equal values, rows with few
+// finite entries): the groups one after the other, in ascending order.  Once there are Wc candidates, an entry is listed only
+// if it beats the worst of them, and a group is read only if its maximum at its lowest index would.  (8 rows of 151936
+// equal entries, W 7: 16 us a call, 464 when every group was read.)
 template <bool kLogits, bool kDirect>
-__device__ __noinline__ int top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, float cut, int Wc, double lse,
-                                        int lane, unsigned long long* list) {
+__device__ __noinline__ void top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, float cut, int Wc, double lse,
+                                         int lane, TopScratch& w) {
   unsigned long long worst = 0ull;                   // keys at or below it cannot be among the best any more
   int count = 0;
-  for (int g0 = 0; g0 < groups; g0 += 32) {
-    unsigned todo = __ballot_sync(0xffffffffu, (kDirect ? gm[g0 + lane] : __ldg(gm + g0 + lane)) >= cut);      // (the number of groups is a multiple of 32)
+  for (int g0 = 0; g0 < groups; g0 += 32) {          // (the number of groups is a multiple of 32)
+    const float most = kDirect ? gm[g0 + lane] : __ldg(gm + g0 + lane);
+    const unsigned long long bound = make_key(rank_value<kLogits>(most, lse), static_cast<uint32_t>(rg.base(g0 + lane)));
+    unsigned todo = __ballot_sync(0xffffffffu, most >= cut && bound > worst);
     while (todo) {
       const int g = g0 + __ffs(todo) - 1;
       todo &= todo - 1;
@@ -310,118 +331,176 @@ __device__ __noinline__ int top_of_many(const RowGroups rg, const float* __restr
         const unsigned long long key = make_key(rank_value<kLogits>(x[j], lse), static_cast<uint32_t>(idx + j));
         const bool take = x[j] >= cut && idx + j < rg.V && key > worst;
         const unsigned votes = __ballot_sync(0xffffffffu, take);
-        if (take) list[count + __popc(votes & ((1u << lane) - 1u))] = key;
+        if (take) w.list[count + __popc(votes & ((1u << lane) - 1u))] = key;
         count += __popc(votes);
       }
       __syncwarp();
       if (count > kListCap - kGroup) {
-        count = keep_best<(kListCap + 31) / 32>(list, count, Wc, lane);
-        if (count == Wc) worst = list[Wc - 1];
+        count = keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
+        if (count == Wc) {
+          worst = w.list[Wc - 1];
+          todo &= __ballot_sync(0xffffffffu, bound > worst);
+        }
         __syncwarp();
       }
     }
   }
-  return keep_best<(kListCap + 31) / 32>(list, count, Wc, lane);
+  keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
 }
 
-// The row's Wc best (value, token) keys in rank order at the front of w.list, by one warp.  gm = the row's group maxima: at
-// least Wc groups reach the Wc-th largest lane maximum, so the Wc best entries are at or above it, and only groups that
-// reach it are read again (about Wc of them, all at once).  Exact for any input.
+// The row's Wc best (value, token) keys in rank order at the front of w.list, by one warp.  gm = the row's group maxima.  The
+// groups are dealt out to buckets; at least Wc groups reach the Wc-th largest bucket maximum, so the Wc best entries are
+// at or above it, and only groups that reach it are read again, eight at a time.  Exact for any input.
 // kLogits: entries are ranked by float(double(z) - lse), which is monotone in z: the threshold is lowered by more than one
 // rounding step of that value, and the keys hold it.  lse() is called while the maxima are on their way.
 // A chain of latencies: maxima (one round trip to L2), threshold, groups (another), ranks.  (With the groups read one
 // after the other and the maxima read twice it took 25 us instead of 3.)
-struct TopScratch {
-  unsigned long long list[kListCap];
-  int groups[32];
-};
-
+//  * Up to kFewWidth candidates 32 buckets do, one per lane: about 32 ln(32 / (32 - W)) groups qualify (8 of 7, 15 of 12 of any
+//    number of groups).  Beyond, 31 at W = 20 and 110 at W = 32, so there the four maxima of a lane's float4 stay apart: 128
+//    buckets, 37 groups at W = 32, for a longer threshold loop.
+//  * A lane holds the maxima of kQuads float4, 1280 groups (163840 entries) of the warp, in registers; longer rows take them
+//    in passes of that many, twice.
+// (8 rows of 151936 entries, W 32, 256 nodes: 121 -> 16 us a call, W 20 26 -> 14, W 7 as before; 200003 entries, W 7, 64 nodes: 15.5 -> 10.4.
+// Such rows fell to top_of_many before, and the kernels before this one took 114, 65 and 10.7.)
 template <bool kLogits, bool kDirect, typename Lse>
 __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __restrict__ gm, int groups, int Wc, Lse&& lse_of,
                                            int lane, TopScratch& w) {
-  constexpr int kQuads = 10;                         // float4 of maxima a lane holds: 1280 groups, 163840 entries
-  constexpr int kBatch = 8;                          // groups whose entries are in flight together
+  constexpr int kQuads = 10;
+  constexpr int kFewWidth = 12;
   float4 h[kQuads];
   const int quads = groups / 4;                      // (groups is a multiple of 32)
   const float4* gm4 = reinterpret_cast<const float4*>(gm);
+  auto fetch = [&](int first) {                      // float4 number first + 32 i + lane
 #pragma unroll
-  for (int i = 0; i < kQuads; ++i)
-    h[i] = i * 32 + lane < quads ? (kDirect ? gm4[i * 32 + lane] : __ldg(gm4 + i * 32 + lane)) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    for (int i = 0; i < kQuads; ++i) {
+      const int at = first + i * 32 + lane;
+      h[i] = at < quads ? (kDirect ? gm4[at] : __ldg(gm4 + at)) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    }
+  };
+  fetch(0);
   // Fewer than 128 groups leave lanes without a float4, and the W-th largest of the lanes' maxima would be -inf, i.e. no
   // threshold at all: there a lane takes every 32nd group instead (4 rows of 1350 entries, W 9, entropy score: 41 -> 19 us
-  // for the whole construction).
-  float best = -INFINITY;
-  if (groups < 128) {
+  // for the whole construction), or with many candidates, for which the groups are too few buckets (8 rows of 4096
+  // entries, W 32: 37 -> 14 us), the entries themselves.
+  float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  if (groups < 128 && Wc > kFewWidth) {
+#pragma unroll 1
+    for (int e0 = lane * 4; e0 < rg.V; e0 += kBatch * 128) {
+      float4 q[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, e0 + i * 128, rg.V, rg.vec != 0);
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        best[0] = fmaxf(best[0], q[i].x);
+        best[1] = fmaxf(best[1], q[i].y);
+        best[2] = fmaxf(best[2], q[i].z);
+        best[3] = fmaxf(best[3], q[i].w);
+      }
+    }
+  } else if (groups < 128) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const int g = i * 32 + lane;
-      if (g < groups) best = fmaxf(best, kDirect ? gm[g] : __ldg(gm + g));
+      if (g < groups) best[i] = kDirect ? gm[g] : __ldg(gm + g);
     }
   }
   const double lse = lse_of();
+#pragma unroll 1
+  for (int first = 0; groups >= 128;) {
 #pragma unroll
-  for (int i = 0; i < kQuads && groups >= 128; ++i) best = fmaxf(best, fmaxf(fmaxf(h[i].x, h[i].y), fmaxf(h[i].z, h[i].w)));
-  for (int i = kQuads * 32 + lane; i < quads; i += 32) {
-    const float4 q = kDirect ? gm4[i] : __ldg(gm4 + i);
-    best = fmaxf(best, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
+    for (int i = 0; i < kQuads; ++i) {
+      best[0] = fmaxf(best[0], h[i].x);
+      best[1] = fmaxf(best[1], h[i].y);
+      best[2] = fmaxf(best[2], h[i].z);
+      best[3] = fmaxf(best[3], h[i].w);
+    }
+    first += kQuads * 32;
+    if (first >= quads) break;
+    fetch(first);
   }
-  float cut = warp_nth(best, Wc);
-  if constexpr (kLogits)      // 2^-22 of the value: two rounding steps
-    cut = __fsub_rd(cut, fmaxf(fabsf(rank_value<true>(cut, lse)) * 2.384185791015625e-7f, 1e-44f));
+  auto threshold = [&](float nth) {
+    if constexpr (kLogits)    // 2^-22 of the value: two rounding steps
+      nth = __fsub_rd(nth, fmaxf(fabsf(rank_value<true>(nth, lse)) * 2.384185791015625e-7f, 1e-44f));
+    return nth;
+  };
+  float cut;
+  if (Wc <= kFewWidth) {
+    const float lane_best[1] = {fmaxf(fmaxf(best[0], best[1]), fmaxf(best[2], best[3]))};
+    cut = threshold(warp_nth<1>(lane_best, Wc));
+  } else {
+    cut = threshold(warp_nth<4>(best, Wc));
+  }
   __syncwarp();
-  // the groups that reach it, up to 32; few lanes have any
-  bool fits = quads <= kQuads * 32;
+  // the groups that reach it, up to kTopGroups; few lanes have any
   int n = 0;
-  if (fits) {
+#pragma unroll 1
+  for (int first = 0; first < quads && n <= kTopGroups; first += kQuads * 32) {
+    if (quads > kQuads * 32) fetch(first);
     uint32_t bits[2] = {0u, 0u};                     // maximum 4 i + j of this lane reaches the threshold
 #pragma unroll
     for (int i = 0; i < kQuads; ++i) {
       const uint32_t m = (h[i].x >= cut ? 1u : 0u) | (h[i].y >= cut ? 2u : 0u) | (h[i].z >= cut ? 4u : 0u) | (h[i].w >= cut ? 8u : 0u);
-      bits[i / 8] |= (i * 32 + lane < quads ? m : 0u) << (4 * (i % 8));
+      bits[i / 8] |= (first + i * 32 + lane < quads ? m : 0u) << (4 * (i % 8));
     }
 #pragma unroll 1
-    for (unsigned todo = __ballot_sync(0xffffffffu, (bits[0] | bits[1]) != 0u); todo && n <= 32;) {
+    for (unsigned todo = __ballot_sync(0xffffffffu, (bits[0] | bits[1]) != 0u); todo && n <= kTopGroups;) {
       // one group of every lane that has one, per step
       const bool mine = (bits[0] | bits[1]) != 0u;
       const bool high = bits[0] == 0u;
       const int bit = __ffs(high ? bits[1] : bits[0]) - 1;
       const int at = n + __popc(todo & ((1u << lane) - 1u));
-      if (mine && at < 32) w.groups[at] = rg.base((((high ? 8 : 0) + (bit >> 2)) * 32 + lane) * 4 + (bit & 3));
+      if (mine && at < kTopGroups) w.groups[at] = rg.base((first + ((high ? 8 : 0) + (bit >> 2)) * 32 + lane) * 4 + (bit & 3));
       n += __popc(todo);
       if (high) bits[1] &= bits[1] - 1u;
       else bits[0] &= bits[0] - 1u;
       todo = __ballot_sync(0xffffffffu, (bits[0] | bits[1]) != 0u);
     }
-    fits = n <= 32;
   }
+  const bool fits = n <= kTopGroups;
   __syncwarp();
+  // their entries that reach it, up to kListCap; if there are more, once again with a threshold from the entries themselves
+  // (a row that rises or falls over its groups has whole groups above the first one)
   int count = 0;
-  for (int g0 = 0; fits && g0 < n; g0 += kBatch) {
-    float4 q[kBatch];
-#pragma unroll
-    for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
-    uint32_t take = 0u;                              // entry j of float4 i reaches the threshold
-#pragma unroll
-    for (int i = 0; i < kBatch; ++i)
-      take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
-    if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
 #pragma unroll 1
-    for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo;) {
-      // one entry of every lane that has one, per step; read again (L1) rather than picked out of registers by index
-      const int bit = __ffs(take) - 1;
-      const int at = count + __popc(todo & ((1u << lane) - 1u));
-      if (take && at < kListCap) {
-        const int idx = w.groups[g0 + (bit >> 2)] + rg.lane_part + (bit & 3);
-        w.list[at] = idx < rg.V ? make_key(rank_value<kLogits>(__ldg(rg.row + idx), lse), static_cast<uint32_t>(idx)) : 0ull;
+  for (int attempt = 0; fits && attempt < 2; ++attempt) {
+    count = 0;
+    best[0] = best[1] = best[2] = best[3] = -INFINITY;
+#pragma unroll 1
+    for (int g0 = 0; g0 < n; g0 += kBatch) {
+      float4 q[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
+      uint32_t take = 0u;                            // entry j of float4 i reaches the threshold
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
+        best[0] = fmaxf(best[0], q[i].x);
+        best[1] = fmaxf(best[1], q[i].y);
+        best[2] = fmaxf(best[2], q[i].z);
+        best[3] = fmaxf(best[3], q[i].w);
       }
-      count += __popc(todo);
-      take &= take - 1u;
-      todo = __ballot_sync(0xffffffffu, take != 0u);
+      if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
+#pragma unroll 1
+      for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo && count <= kListCap;) {
+        // one entry of every lane that has one, per step; read again (L1) rather than picked out of registers by index
+        const int bit = __ffs(take) - 1;
+        const int at = count + __popc(todo & ((1u << lane) - 1u));
+        if (take && at < kListCap) {
+          const int idx = w.groups[g0 + (bit >> 2)] + rg.lane_part + (bit & 3);
+          w.list[at] = idx < rg.V ? make_key(rank_value<kLogits>(__ldg(rg.row + idx), lse), static_cast<uint32_t>(idx)) : 0ull;
+        }
+        count += __popc(todo);
+        take &= take - 1u;
+        todo = __ballot_sync(0xffffffffu, take != 0u);
+      }
     }
+    if (count <= kListCap) break;
+    cut = fmaxf(cut, threshold(warp_nth<4>(best, Wc)));
   }
   __syncwarp();
-  if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, cut, Wc, lse, lane, w.list);
+  if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, cut, Wc, lse, lane, w);
   else if (count <= 32) keep_best<1>(w.list, count, Wc, lane);
+  else if (count <= 64) keep_best<2>(w.list, count, Wc, lane);
   else keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
 }
 
@@ -635,12 +714,14 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
   if (warp == 0 && Bb == 1) {
     if (lane == 0) s_n = 1;
   } else if (warp == 0) {
-    const int slots = ((Bb - 1 + Wc - 1) / Wc + 31) / 32;      // every expansion but the last adds Wc nodes
+    // every expansion but the last adds Wc nodes; a chain (Wc 1) has at most N
+    const int slots = ((Wc == 1 ? min(Bb - 1, N) : (Bb - 1 + Wc - 1) / Wc) + 31) / 32;
     Expansion* made = sh.tree.made;
     int n;
     if (slots <= 1) n = expand_tree<1, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     else if (slots <= 2) n = expand_tree<2, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     else if (slots <= 4) n = expand_tree<4, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    else if (slots <= 8) n = expand_tree<8, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     else n = expand_tree<JET_MAX_NODES / 32, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     if (lane == 0) s_n = n;
   }

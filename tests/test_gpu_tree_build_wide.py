@@ -1,0 +1,99 @@
+"""Tree construction of wide trees and large vocabularies: more groups than a warp holds in registers, thresholds from 32 and from
+128 buckets, more qualifying groups or entries than the lists hold, every size of the pending queue; and no width or
+vocabulary at which the selection falls to a form many times slower."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2606_18394_b200 as jet
+from jet_inputs import make_draft_logits, make_logp
+from test_gpu_tree_build_logits import _compare as compare_logits
+from test_gpu_tree_build_scored import _compare as compare_scored
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("V", [163840, 163841, 262144, 327680, 327681])      # one, two and three passes of 1280 groups
+@pytest.mark.parametrize("W", [7, 32])
+def test_passes_over_the_group_maxima(V, W):
+    rng = np.random.default_rng(V + W)
+    compare_scored(np.stack([make_logp(rng, 2, V, 3.0)]), [7], 2, W, 60, "accum_logp", 0.0)
+    compare_logits(np.stack([make_draft_logits(rng, 2, V, 3.0)]), [7], 2, W, 60, "hybrid", 0.5)
+
+
+@pytest.mark.parametrize("W", [12, 13, 20, 31, 32])
+@pytest.mark.parametrize("V", [31, 33, 1024, 4096 * 4, 4096 * 4 + 1, 50257])
+def test_thresholds_from_many_buckets(V, W):
+    rng = np.random.default_rng(V * 100 + W)
+    compare_scored(np.stack([make_logp(rng, 3, V, 2.0)]), [7], 3, W, 200, "hybrid", 0.5)
+    compare_logits(np.stack([make_draft_logits(rng, 3, V, 2.0)]), [7], 3, W, 200, "accum_logp", 0.0)
+
+
+@pytest.mark.parametrize("groups", [63, 64, 65, 130])
+@pytest.mark.parametrize("per_group", [1, 2, 3])
+def test_list_limits(groups, per_group):
+    """`groups` of the scan's groups with `per_group` equal entries each at the top: both limits of the lists (64 groups, 160
+    entries), on either side.  (A group of one round: 32 entries of each of a slice's four blocks of 1024.)"""
+    rng = np.random.default_rng(groups * 10 + per_group)
+    V = 4096 * 6 + 8
+    z = rng.standard_normal((1, 2, V)).astype(np.float32)
+    g = np.arange(groups)
+    first = g // 32 * 4096 + g % 32 * 32 + 3
+    z[:, :, (first[:, None] + 1024 * np.arange(per_group)[None, :]).reshape(-1)] = 20.0
+    for W in (7, 32):
+        compare_logits(z, [3], 2, W, 60, "accum_logp", 0.0)
+
+
+@pytest.mark.parametrize("V", [1024, 4100, 20000, 151936])
+@pytest.mark.parametrize("kind", ["equal", "steps", "masked", "rising", "falling", "rising_steps"])
+def test_ties_and_slopes(V, kind):
+    rng = np.random.default_rng(V)
+    z = np.zeros((1, 2, V), np.float32)
+    slope = np.arange(V, dtype=np.float32) * np.float32(1e-4)
+    if kind == "steps":
+        z += rng.integers(0, 3, z.shape).astype(np.float32)
+    elif kind == "masked":
+        z[:, :, 40:] = -np.inf
+        z[:, :, :40] += rng.standard_normal((1, 2, 40)).astype(np.float32)
+        z[:, :, V // 2] = 0.5
+    elif kind == "rising_steps":
+        z += np.floor(slope * np.float32(20.0))
+    elif kind != "equal":
+        z += slope if kind == "rising" else -slope
+    for W in (7, 32):
+        compare_logits(z, [3], 2, W, 60, "accum_logp", 0.0)
+        compare_scored(z, [3], 2, W, 60, "accum_logp", 0.0)
+
+
+@pytest.mark.parametrize("N,W,B", [(64, 1, 512), (32, 1, 40), (33, 1, 40), (16, 2, 511), (16, 2, 512), (16, 3, 386), (16, 3, 387), (16, 2, 130)])
+def test_queue_registers(N, W, B):
+    rng = np.random.default_rng(N + W + B)
+    compare_scored(np.stack([make_logp(rng, N, 300, 2.0)]), [1], N, W, B, "accum_logp", 0.0)
+    compare_scored(np.stack([make_logp(rng, N, 300, 2.0)]), [1], N, W, B, "entropy", 0.0)
+
+
+def _time(V, W, B=64, spread=3.0):
+    N, dev = 8, "cuda:0"
+    i32 = dict(dtype=torch.int32, device=dev)
+    rows = torch.log_softmax(torch.randn((1, N, V), generator=torch.Generator(dev).manual_seed(1), device=dev) * spread, -1)
+    tree = [torch.empty((1, B), **i32) for _ in range(3)] + [torch.empty((1, B), device=dev),
+            torch.empty((1, B, (B + 31) // 32), **i32), torch.empty(1, **i32)]
+    ws = torch.empty(max(256, jet.jet_tree_build_workspace_bytes(1, N, V, W)), dtype=torch.uint8, device=dev)
+    root, times = torch.zeros(1, **i32), []
+    for _ in range(12):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        for _ in range(20):
+            jet.jet_tree_build(rows, root, 1, N, V, W, B, *tree, ws)
+        end.record()
+        torch.cuda.synchronize()
+        times.append(start.elapsed_time(end))
+    return min(times)
+
+
+def test_no_cliff():
+    """32 candidates instead of 10 (and fewer expansions), and rows of equal entries: 12 and 46 times the time while such rows were
+    read group by group, 1.5 and 2 times now; the bounds leave room for noise and clocks."""
+    base = _time(128256, 10)
+    assert _time(128256, 32) < 4 * base
+    assert _time(128256, 10, spread=0.0) < 8 * base
