@@ -98,6 +98,11 @@ JET_API const char* jet_status_string(jet_status s);
  */
 JET_API size_t jet_tree_build_workspace_bytes(int batch, int N, int V, int W);
 
+/* Kernel launches that one tree-construction call enqueues (score_mode as for jet_tree_build_scored; from_logits nonzero:
+ * jet_tree_build_logits), 0 for invalid arguments.  Host-only, for callers that count launches.
+ */
+JET_API int jet_tree_build_launches(int N, int V, int score_mode, int from_logits);
+
 JET_API jet_status jet_tree_build(const float* logp, int64_t logp_batch_stride, int64_t logp_depth_stride,
                           const int32_t* root_token, int batch, int N, int V, int W, int B,
                           int32_t* parent, int32_t* depth, int32_t* token, float* score,
@@ -355,6 +360,11 @@ JET_API jet_status jet_tree_verify_attn_tail_ex(const void* q, const void* k_cac
  *                correction token tgt_argmax[v*], then -1
  */
 JET_API size_t jet_tree_accept_workspace_bytes(int batch, int B, int V);
+
+/* Kernel launches that one jet_tree_accept call enqueues (0 for invalid arguments); jet_tree_accept_sample and
+ * jet_tree_accept_hidden take two, the latter behind a memset of its workspace.  Host-only.
+ */
+JET_API int jet_tree_accept_launches(int B, int V);
 
 JET_API jet_status jet_tree_accept(const float* logits, int64_t logits_row_stride, const int32_t* token,
                            const int32_t* parent, const int32_t* depth, const uint32_t* anc_mask,

@@ -22,9 +22,11 @@ from .binding import (  # noqa: F401
     jet_tree_accept_hidden_workspace_bytes,
     jet_tree_accept_sample,
     jet_tree_accept_sample_workspace_bytes,
+    jet_tree_accept_launches,
     jet_tree_accept_static,
     jet_tree_accept_workspace_bytes,
     jet_tree_build,
+    jet_tree_build_launches,
     jet_tree_build_logits,
     jet_tree_build_logits_workspace_bytes,
     jet_tree_build_scored,

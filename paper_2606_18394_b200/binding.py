@@ -32,6 +32,7 @@ _vp, _i, _i64, _f, _sz = _c.c_void_p, _c.c_int, _c.c_int64, _c.c_float, _c.c_siz
 _SIGNATURES = {
     "jet_status_string": (_c.c_char_p, [_c.c_int32]),
     "jet_tree_build_workspace_bytes": (_sz, [_i, _i, _i, _i]),
+    "jet_tree_build_launches": (_i, [_i, _i, _i, _i]),
     "jet_tree_build": (_c.c_int32, [_vp, _i64, _i64, _vp, _i, _i, _i, _i, _i, _vp, _vp, _vp, _vp, _vp,
                                     _vp, _vp, _sz, _vp]),
     "jet_tree_build_scored_workspace_bytes": (_sz, [_i, _i, _i, _i]),
@@ -56,6 +57,7 @@ _SIGNATURES = {
     "jet_kv_compact_tail": (_c.c_int32, [_vp, _vp, _i64, _i64, _vp, _i, _i, _vp, _vp, _vp, _i, _i, _i, _i,
                                          _i, _i, _vp]),
     "jet_tree_accept_workspace_bytes": (_sz, [_i, _i, _i]),
+    "jet_tree_accept_launches": (_i, [_i, _i]),
     "jet_tree_accept": (_c.c_int32, [_vp, _i64, _vp, _vp, _vp, _vp, _vp, _i, _i, _i, _i, _vp, _vp, _vp,
                                      _vp, _vp, _sz, _vp]),
     "jet_tree_accept_hidden_workspace_bytes": (_sz, [_i, _i]),
@@ -128,6 +130,10 @@ def status_string(status: int) -> str:
 
 def jet_tree_build_workspace_bytes(batch, N, V, W) -> int:
     return load().jet_tree_build_workspace_bytes(batch, N, V, W)
+
+
+def jet_tree_build_launches(N, V, score_mode=0, from_logits=False) -> int:
+    return load().jet_tree_build_launches(N, V, int(score_mode), int(from_logits))
 
 
 def jet_tree_build(logp, root_token, batch, N, V, W, B, parent, depth, token, score, anc_mask, n_nodes,
@@ -275,6 +281,10 @@ def jet_kv_compact_tail(k_cache, v_cache, cache_layer_stride, kv_batch_stride, p
 
 def jet_tree_accept_workspace_bytes(batch, B, V) -> int:
     return load().jet_tree_accept_workspace_bytes(batch, B, V)
+
+
+def jet_tree_accept_launches(B, V) -> int:
+    return load().jet_tree_accept_launches(B, V)
 
 
 def jet_tree_accept(logits, logits_row_stride, token, parent, depth, anc_mask, n_nodes, batch, B, V, N,

@@ -183,6 +183,7 @@ accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks, 
 // sequence one CTA reads them in about the time that the second launch of the two-kernel form takes to start.
 constexpr int kSmallThreads = JET_MAX_NODES;
 constexpr int kSmallLogits = 32768, kSmallRow = 4096;
+bool accept_is_small(int B, int V) { return V <= kSmallRow && static_cast<int64_t>(B) * V <= kSmallLogits; }
 
 __global__ void __launch_bounds__(kSmallThreads)
 accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t) {
@@ -649,6 +650,11 @@ extern "C" size_t jet_tree_accept_workspace_bytes(int batch, int B, int V) {
   return jet::round_up(static_cast<size_t>(batch) * B * jet::chunks_for(V) * sizeof(unsigned long long), 256);
 }
 
+extern "C" int jet_tree_accept_launches(int B, int V) {
+  if (B < 1 || B > JET_MAX_NODES || V < 1) return 0;
+  return jet::accept_is_small(B, V) ? 1 : 2;
+}
+
 extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_stride,
                                       const int32_t* token, const int32_t* parent,
                                       const int32_t* depth, const uint32_t* anc_mask,
@@ -672,7 +678,7 @@ extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_st
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto* partial = static_cast<unsigned long long*>(workspace);
   const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
-  if (V <= kSmallRow && static_cast<int64_t>(B) * V <= kSmallLogits) {
+  if (accept_is_small(B, V)) {
     launch_dependent(accept_small_kernel, dim3(batch), dim3(kSmallThreads), st, logits, logits_row_stride, V, vec_ok, tree);
     return launch_status();
   }

@@ -784,6 +784,11 @@ ScanPlan scan_plan(int batch, int N, int V) {
   return p;
 }
 
+// The group maxima are formed inside the expansion kernel: no launch in front of it.
+bool build_direct(int N, int V, bool scored, bool from_logits) {
+  return !scored && !from_logits && static_cast<int64_t>(N) * ((static_cast<int64_t>(V) + kRoundChunk - 1) / kRoundChunk) <= kDirectSlices;
+}
+
 // Workspace: group maxima, then (raw logits) the log-sum-exp pairs, then (entropy scores) the p * log p sums.
 size_t gmax_bytes(int batch, int N, int V) {
   return round_up(static_cast<size_t>(batch) * N * scan_plan(batch, N, V).groups * sizeof(float), 256);
@@ -825,7 +830,7 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   auto scan = [&](auto kernel, double2* sums) {
     launch_dependent(kernel, grid, dim3(kScanThreads), st, rows, batch_stride, depth_stride, V, plan.rounds, vec, gmax, pairs, sums);
   };
-  const bool direct = !scored && !from_logits && static_cast<int64_t>(N) * ((V + kRoundChunk - 1) / kRoundChunk) <= kDirectSlices;
+  const bool direct = build_direct(N, V, scored, from_logits);
   if (direct) {
     plan.rounds = 1;
     plan.slices = (V + kRoundChunk - 1) / kRoundChunk;
@@ -862,6 +867,12 @@ extern "C" size_t jet_tree_build_scored_workspace_bytes(int batch, int N, int V,
 extern "C" size_t jet_tree_build_logits_workspace_bytes(int batch, int N, int V, int W) {
   if (batch < 1 || N < 1 || V < 1 || W < 1) return 0;
   return jet::gmax_bytes(batch, N, V) + 2 * jet::sums_bytes(batch, N, V);
+}
+
+extern "C" int jet_tree_build_launches(int N, int V, int score_mode, int from_logits) {
+  if (N < 1 || N > JET_MAX_DEPTH || V < 1 || score_mode < JET_SCORE_ACCUM_LOGP || score_mode > JET_SCORE_HYBRID) return 0;
+  const bool scored = score_mode != JET_SCORE_ACCUM_LOGP;
+  return jet::build_direct(N, V, scored, from_logits != 0) ? 1 : scored && from_logits ? 3 : 2;
 }
 
 extern "C" jet_status jet_tree_build(const float* logp, int64_t logp_batch_stride,

@@ -226,10 +226,9 @@ class VerifyStep:
     @property
     def launches_around_attention(self):
         """Kernel launches of a step's tree construction, acceptance and commit (a small tree or acceptance is one launch)."""
-        scored = self.score_mode != "accum_logp"
-        small_build = not scored and not self.draft_logits and self.N * ((self.V + 4095) // 4096) <= 6
-        build = 1 if small_build else 3 if scored and self.draft_logits else 2
-        accept = 1 if self.accept_mode == "greedy" and self.V <= 4096 and self.B * self.V <= 32768 else 2
+        mode = {"accum_logp": 0, "entropy": 1, "hybrid": 2}[self.score_mode]
+        build = jet.jet_tree_build_launches(self.N, self.V, mode, self.draft_logits)
+        accept = jet.jet_tree_accept_launches(self.B, self.V) if self.accept_mode == "greedy" else 2
         return build + accept + 1
 
     def launches_per_step(self, attn_launches_per_layer=None):

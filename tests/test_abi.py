@@ -34,3 +34,10 @@ def test_status_strings_and_workspace_queries():
     assert jet.jet_tree_build_workspace_bytes(1, 8, 151936, 7) % 256 == 0
     assert jet.jet_tree_accept_workspace_bytes(32, 64, 151936) >= 32 * 64 * 8
     assert jet.jet_tree_build_workspace_bytes(0, 8, 10, 7) == 0
+
+
+def test_launch_queries():
+    assert [jet.jet_tree_build_launches(N, V) for N, V in ((1, 1), (6, 4096), (6, 4097), (3, 8192), (4, 8192), (1, 24577))] == [1, 1, 2, 1, 2, 2]
+    assert [jet.jet_tree_build_launches(2, 100, mode, raw) for mode, raw in ((0, True), (1, False), (2, True))] == [2, 2, 3]
+    assert [jet.jet_tree_accept_launches(B, V) for B, V in ((8, 4096), (9, 4096), (1, 4097), (512, 64))] == [1, 2, 2, 1]
+    assert jet.jet_tree_build_launches(0, 10) == jet.jet_tree_build_launches(1, 10, 3) == jet.jet_tree_accept_launches(0, 10) == 0
