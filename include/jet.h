@@ -503,6 +503,11 @@ JET_API jet_status jet_tree_accept_sample(const float* logits, int64_t logits_ro
  *   seq_len      i32 [batch], read and then updated in place
  * Every cache byte outside the written rows is left untouched.
  */
+/* Kernel launches that one commit call enqueues on the calling thread's current device (tail nonzero: jet_kv_compact_tail),
+ * 0 for invalid arguments.  Host-only.
+ */
+JET_API int jet_kv_compact_launches(int layers, int batch, int Hkv, int D, int N, int tail);
+
 JET_API jet_status jet_kv_compact(const void* tree_k, const void* tree_v, void* k_cache, void* v_cache,
                           int64_t cache_layer_stride, int64_t kv_batch_stride,
                           const int32_t* page_table, int max_pages_per_seq, int page_size,

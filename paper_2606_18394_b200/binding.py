@@ -68,6 +68,7 @@ _SIGNATURES = {
     "jet_tree_accept_sample_workspace_bytes": (_sz, [_i, _i, _i]),
     "jet_tree_accept_sample": (_c.c_int32, [_vp, _i64, _f, _vp, _i64, _i64, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                             _i, _i, _i, _i, _vp, _vp, _vp, _vp, _vp, _sz, _vp]),
+    "jet_kv_compact_launches": (_i, [_i, _i, _i, _i, _i, _i]),
     "jet_kv_compact": (_c.c_int32, [_vp, _vp, _vp, _vp, _i64, _i64, _vp, _i, _i, _vp, _vp, _vp, _i, _i,
                                     _i, _i, _i, _i, _vp]),
 }
@@ -340,6 +341,10 @@ def jet_tree_accept_sample(logits, logits_row_stride, temperature, draft_logp, l
     if check:
         _check(st, "jet_tree_accept_sample")
     return st
+
+
+def jet_kv_compact_launches(layers, batch, Hkv, D, N, tail=False) -> int:
+    return load().jet_kv_compact_launches(layers, batch, Hkv, D, N, int(tail))
 
 
 def jet_kv_compact(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,

@@ -1,21 +1,23 @@
-// jet_kv_compact: commit of the accepted path.  One launch: a cluster of 8 CTAs per sequence copies the K and V rows of
-// every accepted node of every layer behind the prefix (contiguous or paged cache) and, once every CTA of the cluster has
-// read the old length, advances seq_len.  jet_kv_compact_tail: the same in place, for a cache that holds the tree's rows
-// behind the prefix.
+// jet_kv_compact: commit of the accepted path: the K and V rows of every accepted node of every layer are copied behind the
+// prefix (contiguous or paged cache), then seq_len advances.  jet_kv_compact_tail: the same in place, for a cache that
+// holds the tree's rows behind the prefix.
 //
-// Bound: latency (a step commits 0.1 - 3 MB).  The chain is lengths -> path and page table -> rows, three round trips; the rows of
-// a sequence are spread over the warps of its cluster with all loads of a warp in flight at once.  (A block per row or
-// (layer, K|V) with a second launch for the lengths, as before, cost a launch more: about 2 us of GPU time in a
-// captured step and 2.3 us of host time in one issued call by call.)
+// Bound: latency (a step commits 0.1 - 3 MB).  The chain is lengths and path -> page table -> rows; the rows of all
+// sequences are spread over the GPU, a warp per row, and a CTA works the path of its sequence out once.  No CTA may see an
+// advanced length, so seq_len is advanced by a second launch, or, where one CTA per sequence is enough (kAloneRows), by that
+// CTA: the second launch costs 1.7 us of host time and, started under the first, no GPU time that shows.
+// us per call in a captured stream (a cluster of eight CTAs per sequence before; page size 16, 8 heads of 128 and 36 layers
+// where not said otherwise; in place in brackets):
+//   1 sequence, 6 rows                  6.3 -> 4.8   [8.9 -> 5.8]      1 sequence, 65 rows    29 -> 6.3  [48 -> 17]
+//   32 sequences, 6 rows                10.2 -> 10.3 [20.1 -> 12.7]    128, one layer, 5 rows  11.2 -> 4.3 [23.5 -> 4.8]
+//   8 sequences, 48 layers, 4 heads     6.8 -> 6.1   [8.1 -> 6.3]      128, 5 rows            40 -> 37.9 [61.6 -> 30.6]
 #include "jet_common.cuh"
-#include "sm100_ptx.cuh"
 
 namespace jet {
 namespace {
 
-constexpr int kCommitCluster = 8;
-constexpr int kCommitThreads = 512;
-constexpr int kCommitWarps = kCommitCluster * kCommitThreads / 32;      // warps of a cluster
+constexpr int kCommitThreads = 256, kCommitThreadsAlone = 512;      // of a CTA; of one that has its sequence to itself
+constexpr int kTailHeld = 16;                        // rows a lane of the in-place form has in flight
 
 struct CommitParams {
   int64_t layer_stride16, batch_stride16;            // in 16-byte pieces
@@ -24,19 +26,24 @@ struct CommitParams {
   const int32_t* accept_len;
   int32_t* seq_len;
   int max_pages, page_size, layers, batch, B, row16, N;
+  int ctas;                                          // per sequence
 };
 
-// The path of sequence b and where its rows lie, worked out once per CTA: node[i] (-1: not to be copied) and the cache row
-// offsets (within a layer) of position seq_len + i and -- in-place layout -- seq_len + node[i].
+// The path of sequence b and where its rows lie: node[i] (-1: not to be copied) and the cache row offsets (within a layer) of
+// position seq_len + i and -- in-place layout -- seq_len + node[i].
 struct CommitTable {
   int64_t dst[JET_MAX_DEPTH + 1], src[JET_MAX_DEPTH + 1];
   int node[JET_MAX_DEPTH + 1];
 };
 
+// Fills the table and returns a: entries 0 .. a of the path are committed.  A CTA that has its sequence to itself advances
+// seq_len once all its threads have the length.
 template <bool kTail>
 __device__ __forceinline__ int commit_table(const CommitParams& p, int b, CommitTable& t) {
-  const int a = min(p.accept_len[b], p.N);
-  const int64_t len = p.seq_len[b];
+  const int i = threadIdx.x;
+  const int accepted = p.accept_len[b], len = p.seq_len[b];
+  int node = i <= p.N ? p.path[static_cast<size_t>(b) * (p.N + 1) + i] : -1;      // (in flight with the lengths)
+  const int a = min(accepted, p.N);
   auto row_of = [&](int64_t pos) -> int64_t {        // -1: outside the page table (a length beyond it is the caller's error)
     if (pos < 0) return -1;
     if (!p.page_table) return b * p.batch_stride16 + pos * p.row16;
@@ -44,83 +51,142 @@ __device__ __forceinline__ int commit_table(const CommitParams& p, int b, Commit
     const int page = p.page_table[static_cast<size_t>(b) * p.max_pages + pos / p.page_size];
     return (static_cast<int64_t>(page) * p.page_size + pos % p.page_size) * p.row16;
   };
-  for (int i = threadIdx.x; i <= a; i += kCommitThreads) {
-    int node = p.path[static_cast<size_t>(b) * (p.N + 1) + i];
+  if (i <= a) {
     if (node < 0 || node >= p.B) node = -1;
-    const int64_t dst = row_of(len + i), src = kTail && node >= 0 ? row_of(len + node) : 0;
+    const int64_t dst = row_of(static_cast<int64_t>(len) + i), src = kTail && node >= 0 ? row_of(static_cast<int64_t>(len) + node) : 0;
     if (dst < 0 || src < 0) node = -1;
     t.node[i] = node;
     t.dst[i] = dst;
     t.src[i] = src;
   }
   __syncthreads();
-  // every CTA has read the length: one of them may advance it
-  __syncwarp();
-  ptx::cluster_sync_all();
-  if (threadIdx.x == 0 && ptx::cluster_ctarank() == 0) p.seq_len[b] = static_cast<int32_t>(len) + p.accept_len[b] + 1;
+  if (p.ctas == 1 && threadIdx.x == 0) p.seq_len[b] = len + accepted + 1;
   return a;
 }
 
-__global__ void __launch_bounds__(kCommitThreads)
+// A warp per row, two rows in flight.  Row r: path entry r mod (a + 1) of (layer, K | V) number r / (a + 1).
+__global__ void __launch_bounds__(kCommitThreadsAlone)
 kv_compact_kernel(const uint4* __restrict__ tree_k, const uint4* __restrict__ tree_v, uint4* __restrict__ k_cache,
                   uint4* __restrict__ v_cache, const CommitParams p) {
   grid_dependency_wait();
   __shared__ CommitTable t;
-  const int b = blockIdx.x / kCommitCluster;
+  const int b = blockIdx.x / p.ctas;
   const int a = commit_table<false>(p, b, t);
-  if (a < 0) return;
-  const int lane = threadIdx.x & 31;
-  const int rows = 2 * p.layers * (a + 1);           // row r: path entry r mod (a + 1) of (layer, K | V) number r / (a + 1)
-  for (int r = (blockIdx.x % kCommitCluster) * (kCommitThreads / 32) + (threadIdx.x >> 5); r < rows; r += kCommitWarps) {
-    const int lk = r / (a + 1), i = r - lk * (a + 1), layer = lk >> 1;
-    const int node = t.node[i];
-    if (node < 0) continue;
-    const uint4* src = ((lk & 1) ? tree_v : tree_k) + ((static_cast<int64_t>(layer) * p.batch + b) * p.B + node) * p.row16;
-    uint4* dst = ((lk & 1) ? v_cache : k_cache) + layer * p.layer_stride16 + t.dst[i];
-    int e = lane;
-    for (; e + 96 < p.row16; e += 128) {
-      uint4 x[4];
+  const int lane = threadIdx.x & 31, warps = p.ctas * (blockDim.x >> 5);
+  const int rows = 2 * p.layers * (a + 1);           // (a below 0: none)
+  for (int r0 = (blockIdx.x % p.ctas) * (blockDim.x >> 5) + (threadIdx.x >> 5); r0 < rows; r0 += 2 * warps) {
+    const uint4* src[2];
+    uint4* dst[2];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) x[k] = __ldg(src + e + 32 * k);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) dst[e + 32 * k] = x[k];
+    for (int k = 0; k < 2; ++k) {
+      const int r = r0 + k * warps, lk = r / (a + 1), i = r - lk * (a + 1), layer = lk >> 1;
+      const int node = r < rows ? t.node[i] : -1;
+      src[k] = node < 0 ? nullptr : ((lk & 1) ? tree_v : tree_k) + ((static_cast<int64_t>(layer) * p.batch + b) * p.B + node) * p.row16;
+      dst[k] = ((lk & 1) ? v_cache : k_cache) + layer * p.layer_stride16 + t.dst[i];
     }
-    for (; e < p.row16; e += 32) dst[e] = __ldg(src + e);
+    for (int e0 = 0; e0 < p.row16; e0 += 128) {
+      uint4 x[2][4];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = e0 + j * 32 + lane;
+          if (src[k] && e < p.row16) x[k][j] = __ldg(src[k] + e);
+        }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = e0 + j * 32 + lane;
+          if (src[k] && e < p.row16) dst[k][e] = x[k][j];
+        }
+    }
   }
 }
 
 // In place: row seq_len + path[i] moves to seq_len + i for i = 1 .. accept_len (path[i] >= i; the root stays where it is).
-// One warp per (layer, K | V, 32 of the row's 16-byte columns); columns do not meet, so a lane's own order is all that
-// counts: it reads kTailHeld rows into registers before it writes any, and never writes a row that it still has to read,
-// because rows are taken in increasing i and path[i] >= i, path increasing.  (With a warp per (layer, K | V) few layers
-// left most of the cluster idle: 36 layers of 8 heads of 128, four rows: 9.7 -> 7.0 us.)
-constexpr int kTailHeld = 16;
-
-__global__ void __launch_bounds__(kCommitThreads)
+// A unit is (layer, K | V, 32 of the row's 16-byte columns); columns do not meet, so a lane's own order is all that
+// counts: it reads kTailHeld rows of a unit into registers before it writes any, and never writes a row that it still has to
+// read, because rows are taken in increasing i and path[i] >= i, path increasing.  With few rows a warp holds several
+// units at once, if there are more units than warps.
+__global__ void __launch_bounds__(kCommitThreadsAlone, 1)
 kv_compact_tail_kernel(uint4* k_cache, uint4* v_cache, const CommitParams p) {
   grid_dependency_wait();
   __shared__ CommitTable t;
-  const int b = blockIdx.x / kCommitCluster;
+  const int b = blockIdx.x / p.ctas;
   const int a = commit_table<true>(p, b, t);
-  const int lane = threadIdx.x & 31, blocks = (p.row16 + 31) / 32;
-  for (int u = (blockIdx.x % kCommitCluster) * (kCommitThreads / 32) + (threadIdx.x >> 5); u < 2 * p.layers * blocks; u += kCommitWarps) {
-    const int lk = u / blocks, column = (u - lk * blocks) * 32 + lane;
-    if (column >= p.row16) continue;
-    uint4* cache = ((lk & 1) ? v_cache : k_cache) + (lk >> 1) * p.layer_stride16 + column;
-    for (int i0 = 1; i0 <= a; i0 += kTailHeld) {
+  if (a < 1) return;
+  const int lane = threadIdx.x & 31, warp = (blockIdx.x % p.ctas) * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = p.ctas * (blockDim.x >> 5);
+  const int columns = (p.row16 + 31) / 32, units = 2 * p.layers * columns;
+  const int rows = min(a, kTailHeld);                // of a unit that are held at once
+  const int per = max(1, min(kTailHeld / rows, (units + warps - 1) / warps));
+  for (int first = warp * per; first < units; first += warps * per) {
+    const int lk0 = first / columns, column0 = first - lk0 * columns;
+    for (int i0 = 1; i0 <= a; i0 += kTailHeld) {     // (one pass unless per is 1)
+      auto each = [&](auto&& piece) {
+        int lk = lk0, column = column0, i = i0;
+#pragma unroll
+        for (int k = 0; k < kTailHeld; ++k) {
+          if (k >= rows * per || lk >= 2 * p.layers || i > a) break;      // (warp-uniform)
+          const int e = column * 32 + lane;
+          if (t.node[i] >= 0 && t.node[i] != i && e < p.row16)
+            piece(k, ((lk & 1) ? v_cache : k_cache) + (lk >> 1) * p.layer_stride16 + e, i);
+          if (++i == i0 + rows && per > 1) {
+            i = 1;
+            if (++column == columns) { column = 0; ++lk; }
+          }
+        }
+      };
       uint4 held[kTailHeld];
-#pragma unroll
-      for (int k = 0; k < kTailHeld; ++k)
-        if (i0 + k <= a && t.node[i0 + k] >= 0) held[k] = cache[t.src[i0 + k]];
-#pragma unroll
-      for (int k = 0; k < kTailHeld; ++k)
-        if (i0 + k <= a && t.node[i0 + k] >= 0 && t.node[i0 + k] != i0 + k) cache[t.dst[i0 + k]] = held[k];
+      each([&](int k, uint4* cache, int i) { held[k] = cache[t.src[i]]; });
+      each([&](int k, uint4* cache, int i) { cache[t.dst[i]] = held[k]; });
     }
   }
 }
 
+__global__ void advance_seq_len_kernel(const int32_t* __restrict__ accept_len, int32_t* __restrict__ seq_len, int batch) {
+  grid_dependency_wait();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < batch) seq_len[b] += accept_len[b] + 1;
+}
+
+// Sequences of at most this many rows get one CTA: 8 layers of 9 positions, 144 rows, 7.4 us that way instead of 4.3.
+constexpr int kAloneRows = 64;
+// CTAs of kCommitThreads that an SM holds: more rows than their warps cover are taken in turns, not in waves.
+constexpr int kCopyResident = 3, kTailResident = 2;
+
+struct CommitPlan {
+  int ctas, threads;                                 // per sequence; of a CTA
+  int launches() const { return ctas > 1 ? 2 : 1; }
+};
+
+// A warp per row of every layer, or, in place, per unit.
+CommitPlan commit_plan(int layers, int batch, int row16, int N, bool tail) {
+  const int64_t rows = static_cast<int64_t>(2 * layers) * (N + 1);
+  if (rows <= kAloneRows) return {1, kCommitThreadsAlone};
+  const int64_t work = tail ? static_cast<int64_t>(2 * layers) * ((row16 + 31) / 32) : rows;
+  const int64_t fill = (work + kCommitThreads / 32 - 1) / (kCommitThreads / 32);
+  const int64_t spread = (tail ? kTailResident : kCopyResident) * sm_count() / batch;
+  return {static_cast<int>(fill < spread ? fill : spread > 1 ? spread : 1), kCommitThreads};
+}
+
+template <typename Kernel, typename... Args>
+jet_status commit_launch(Kernel kernel, bool tail, CommitParams p, cudaStream_t st, Args... args) {
+  const CommitPlan plan = commit_plan(p.layers, p.batch, p.row16, p.N, tail);
+  p.ctas = plan.ctas;
+  launch_dependent(kernel, dim3(static_cast<unsigned>(p.ctas) * p.batch), dim3(plan.threads), st, args..., p);
+  if (plan.launches() > 1)
+    launch_dependent(advance_seq_len_kernel, dim3((p.batch + 255) / 256), dim3(256), st, p.accept_len, p.seq_len, p.batch);
+  return launch_status();
+}
+
 }  // namespace
 }  // namespace jet
+
+extern "C" int jet_kv_compact_launches(int layers, int batch, int Hkv, int D, int N, int tail) {
+  if (layers < 1 || layers > 65535 || batch < 1 || Hkv < 1 || D < 1 || N < 1 || N > JET_MAX_DEPTH) return 0;
+  return jet::commit_plan(layers, batch, static_cast<int>(static_cast<int64_t>(Hkv) * D / 8), N, tail != 0).launches();
+}
 
 extern "C" jet_status jet_kv_compact(const void* tree_k, const void* tree_v, void* k_cache,
                                      void* v_cache, int64_t cache_layer_stride,
@@ -146,11 +212,9 @@ extern "C" jet_status jet_kv_compact(const void* tree_k, const void* tree_v, voi
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row16 = static_cast<int>(row_elems / 8);
   const CommitParams p{cache_layer_stride / 8, kv_batch_stride / 8, page_table, path, accept_len, seq_len,
-                       max_pages_per_seq, page_size, layers, batch, B, row16, N};
-  launch_dependent_cluster(kv_compact_kernel, dim3(kCommitCluster * batch), dim3(kCommitThreads), kCommitCluster, st,
-      static_cast<const uint4*>(tree_k), static_cast<const uint4*>(tree_v), static_cast<uint4*>(k_cache),
-      static_cast<uint4*>(v_cache), p);
-  return launch_status();
+                       max_pages_per_seq, page_size, layers, batch, B, row16, N, 1};
+  return commit_launch(kv_compact_kernel, false, p, st, static_cast<const uint4*>(tree_k), static_cast<const uint4*>(tree_v),
+                       static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache));
 }
 
 extern "C" jet_status jet_kv_compact_tail(void* k_cache, void* v_cache, int64_t cache_layer_stride,
@@ -174,8 +238,6 @@ extern "C" jet_status jet_kv_compact_tail(void* k_cache, void* v_cache, int64_t 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row16 = static_cast<int>(row_elems / 8);
   const CommitParams p{cache_layer_stride / 8, kv_batch_stride / 8, page_table, path, accept_len, seq_len,
-                       max_pages_per_seq, page_size, layers, batch, B, row16, N};
-  launch_dependent_cluster(kv_compact_tail_kernel, dim3(kCommitCluster * batch), dim3(kCommitThreads), kCommitCluster, st,
-      static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache), p);
-  return launch_status();
+                       max_pages_per_seq, page_size, layers, batch, B, row16, N, 1};
+  return commit_launch(kv_compact_tail_kernel, true, p, st, static_cast<uint4*>(k_cache), static_cast<uint4*>(v_cache));
 }

@@ -640,7 +640,6 @@ int chunks_for(int V) { return (V + kArgChunk - 1) / kArgChunk; }
 // slice).  It lives in every device context that loads the library (1 MiB) until the process exits.
 constexpr size_t kStaticKeys = JET_STATIC_ACCEPT_SCRATCH_BYTES / sizeof(unsigned long long);
 static __device__ __align__(256) unsigned long long g_accept_scratch[kStaticKeys];
-constexpr int kMaxDevices = 64;
 
 }  // namespace
 }  // namespace jet

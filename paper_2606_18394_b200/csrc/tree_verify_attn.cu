@@ -2179,33 +2179,6 @@ bool make_map(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Everything the host side caches about the GPU is kept per device (a process may drive several).
-constexpr int kMaxDevices = 64;
-int current_device() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-    cudaGetLastError();
-    return 0;
-  }
-  return dev;
-}
-
-int sm_count() {
-  static std::atomic<int> cache[kMaxDevices];
-  const int dev = current_device();
-  int n = cache[dev].load(std::memory_order_relaxed);
-  if (n == 0) {
-    int v = 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
-      cudaGetLastError();
-      v = 148;
-    }
-    n = v;
-    cache[dev].store(n, std::memory_order_relaxed);
-  }
-  return n;
-}
-
 struct Plan {
   int mt;          // query tiles per CTA (1 or 2)
   int n_mgroups;   // groups of mt query tiles per (sequence, KV head)

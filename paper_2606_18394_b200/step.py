@@ -225,11 +225,11 @@ class VerifyStep:
 
     @property
     def launches_around_attention(self):
-        """Kernel launches of a step's tree construction, acceptance and commit (a small tree or acceptance is one launch)."""
+        """Kernel launches of a step's tree construction, acceptance and commit (small ones take fewer)."""
         mode = {"accum_logp": 0, "entropy": 1, "hybrid": 2}[self.score_mode]
         build = jet.jet_tree_build_launches(self.N, self.V, mode, self.draft_logits)
         accept = jet.jet_tree_accept_launches(self.B, self.V) if self.accept_mode == "greedy" else 2
-        return build + accept + 1
+        return build + accept + jet.jet_kv_compact_launches(self.layers, self.batch, self.Hkv, self.D, self.N, self.tail)
 
     def launches_per_step(self, attn_launches_per_layer=None):
         if attn_launches_per_layer is None:       # what the library says one attention call of this shape enqueues
