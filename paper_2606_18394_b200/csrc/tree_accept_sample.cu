@@ -25,7 +25,7 @@ constexpr int kLseElems = 32;
 constexpr int kLseChunk = kLseThreads * kLseElems;
 // Bound of the sampling kernel: latency -- a CTA reads some 20 KB of logits and log-probabilities behind a chain of small
 // dependent look-ups, kSampleUnroll steps of loads in flight per warp.  While the device holds all clusters with one CTA
-// per SM (15 of them: a cluster of eight has to fit into one GPC) it takes 1024 threads; beyond that 512 (a thread per node
+// per SM (15 of them on a B200: a cluster of eight has to fit into one GPC) it takes 1024 threads; beyond that 512 (a thread per node
 // of the largest tree; at most 64 registers), so that two share an SM: the 256 CTAs of a batch of 32 are one wave, not
 // two.  32 sequences of 64 nodes, V 151936: 217 -> 205 us for both launches (reading the 1.25 GB of logits alone takes
 // 190 us at the measured copy bandwidth).
@@ -33,7 +33,6 @@ constexpr int kLseChunk = kLseThreads * kLseElems;
 // scan in front of the dependency wait, the rows' later steps prefetched, the step table read eight entries at a time
 // and one cluster barrier fewer.
 constexpr int kSampleThreadsFew = 1024, kSampleThreadsMany = 512;
-constexpr int kSampleFewBatch = 15;
 constexpr int kSampleUnroll = 2;           // (three spill at 64 registers)
 static_assert(kSampleThreadsMany >= JET_MAX_NODES, "a thread per node");
 constexpr int kSampleStep = 128;          // vocabulary entries a warp handles per step (4 per lane)
@@ -397,6 +396,36 @@ accept_sample_kernel(const float2* __restrict__ partial, int nchunks, const floa
   if (v == 0) { accept_len[b] = a; my_tok[a] = picked; }
 }
 
+cudaLaunchAttribute sample_cluster_attribute() {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kSampleCluster;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  return at;
+}
+
+// How many clusters of 1024-thread CTAs the device holds at once (asked once per device; 0 if it cannot be told).
+int resident_sample_clusters() {
+  static std::atomic<int> cache[kMaxDevices];        // 0 = not asked, else the count plus 1
+  std::atomic<int>& known = cache[current_device()];
+  if (known.load(std::memory_order_relaxed) == 0) {
+    cudaLaunchAttribute at[1] = {sample_cluster_attribute()};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(64 * kSampleCluster);
+    cfg.blockDim = dim3(kSampleThreadsFew);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, accept_sample_kernel<kSampleThreadsFew>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    known.store(n + 1, std::memory_order_relaxed);
+  }
+  return known.load(std::memory_order_relaxed) - 1;
+}
+
 int lse_chunks_for(int V) { return (V + kLseChunk - 1) / kLseChunk; }
 
 }  // namespace
@@ -441,15 +470,12 @@ extern "C" jet_status jet_tree_accept_sample(const float* logits, int64_t logits
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch * kSampleCluster);
-    const bool few = batch <= kSampleFewBatch;
+    const bool few = batch <= resident_sample_clusters();
     cfg.blockDim = dim3(few ? kSampleThreadsFew : kSampleThreadsMany);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kSampleCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    attr[0] = sample_cluster_attribute();
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
