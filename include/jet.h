@@ -364,7 +364,7 @@ JET_API size_t jet_tree_accept_workspace_bytes(int batch, int B, int V);
 /* Kernel launches that one jet_tree_accept call enqueues (0 for invalid arguments); jet_tree_accept_sample and
  * jet_tree_accept_hidden take two, the latter behind a memset of its workspace.  Host-only.
  */
-JET_API int jet_tree_accept_launches(int B, int V);
+JET_API int jet_tree_accept_launches(int batch, int B, int V);
 
 JET_API jet_status jet_tree_accept(const float* logits, int64_t logits_row_stride, const int32_t* token,
                            const int32_t* parent, const int32_t* depth, const uint32_t* anc_mask,

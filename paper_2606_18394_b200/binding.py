@@ -57,7 +57,7 @@ _SIGNATURES = {
     "jet_kv_compact_tail": (_c.c_int32, [_vp, _vp, _i64, _i64, _vp, _i, _i, _vp, _vp, _vp, _i, _i, _i, _i,
                                          _i, _i, _vp]),
     "jet_tree_accept_workspace_bytes": (_sz, [_i, _i, _i]),
-    "jet_tree_accept_launches": (_i, [_i, _i]),
+    "jet_tree_accept_launches": (_i, [_i, _i, _i]),
     "jet_tree_accept": (_c.c_int32, [_vp, _i64, _vp, _vp, _vp, _vp, _vp, _i, _i, _i, _i, _vp, _vp, _vp,
                                      _vp, _vp, _sz, _vp]),
     "jet_tree_accept_hidden_workspace_bytes": (_sz, [_i, _i]),
@@ -284,8 +284,8 @@ def jet_tree_accept_workspace_bytes(batch, B, V) -> int:
     return load().jet_tree_accept_workspace_bytes(batch, B, V)
 
 
-def jet_tree_accept_launches(B, V) -> int:
-    return load().jet_tree_accept_launches(B, V)
+def jet_tree_accept_launches(batch, B, V) -> int:
+    return load().jet_tree_accept_launches(batch, B, V)
 
 
 def jet_tree_accept(logits, logits_row_stride, token, parent, depth, anc_mask, n_nodes, batch, B, V, N,

@@ -179,11 +179,17 @@ accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks, 
   select_path(t, b, tgt);
 }
 
-// Both parts in one launch for small problems: a CTA per sequence, a warp per row of logits.  Up to kSmallLogits logits a
-// sequence one CTA reads them in about the time that the second launch of the two-kernel form takes to start.
+// Both parts in one launch for small problems: a CTA per sequence, a warp per row of logits.  One turn of its 16 warps takes
+// about 1.3 us, the two-kernel form 4.3 us and 4 us more for every 1000 rows of the batch, so the one launch is for a tree
+// of one turn (16 x 1024 logits: 3.8 us against 4.3) and for batches (32 x 64 x 512: 7.4 against 12.9); rows
+// longer than kSmallRow are too long for a warp (4 x 4096: 5.1 against 4.1), and a large tree alone takes its turns one
+// after the other (512 x 64: 42.7 against 7.6).
 constexpr int kSmallThreads = JET_MAX_NODES;
-constexpr int kSmallLogits = 32768, kSmallRow = 4096;
-bool accept_is_small(int B, int V) { return V <= kSmallRow && static_cast<int64_t>(B) * V <= kSmallLogits; }
+constexpr int kSmallRow = 2048, kSmallLogits = 16384, kSmallBatch = 20, kSmallBatchLogits = 32768;
+bool accept_is_small(int batch, int B, int V) {
+  const int64_t logits = static_cast<int64_t>(B) * V;
+  return V <= kSmallRow && ((B <= kSmallThreads / 32 && logits <= kSmallLogits) || (batch >= kSmallBatch && logits <= kSmallBatchLogits));
+}
 
 __global__ void __launch_bounds__(kSmallThreads)
 accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t) {
@@ -649,9 +655,9 @@ extern "C" size_t jet_tree_accept_workspace_bytes(int batch, int B, int V) {
   return jet::round_up(static_cast<size_t>(batch) * B * jet::chunks_for(V) * sizeof(unsigned long long), 256);
 }
 
-extern "C" int jet_tree_accept_launches(int B, int V) {
-  if (B < 1 || B > JET_MAX_NODES || V < 1) return 0;
-  return jet::accept_is_small(B, V) ? 1 : 2;
+extern "C" int jet_tree_accept_launches(int batch, int B, int V) {
+  if (batch < 1 || B < 1 || B > JET_MAX_NODES || V < 1) return 0;
+  return jet::accept_is_small(batch, B, V) ? 1 : 2;
 }
 
 extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_stride,
@@ -677,7 +683,7 @@ extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_st
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto* partial = static_cast<unsigned long long*>(workspace);
   const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
-  if (accept_is_small(B, V)) {
+  if (accept_is_small(batch, B, V)) {
     launch_dependent(accept_small_kernel, dim3(batch), dim3(kSmallThreads), st, logits, logits_row_stride, V, vec_ok, tree);
     return launch_status();
   }

@@ -228,7 +228,7 @@ class VerifyStep:
         """Kernel launches of a step's tree construction, acceptance and commit (small ones take fewer)."""
         mode = {"accum_logp": 0, "entropy": 1, "hybrid": 2}[self.score_mode]
         build = jet.jet_tree_build_launches(self.N, self.V, mode, self.draft_logits)
-        accept = jet.jet_tree_accept_launches(self.B, self.V) if self.accept_mode == "greedy" else 2
+        accept = jet.jet_tree_accept_launches(self.batch, self.B, self.V) if self.accept_mode == "greedy" else 2
         return build + accept + jet.jet_kv_compact_launches(self.layers, self.batch, self.Hkv, self.D, self.N, self.tail)
 
     def launches_per_step(self, attn_launches_per_layer=None):

@@ -39,8 +39,9 @@ def test_status_strings_and_workspace_queries():
 def test_launch_queries():
     assert [jet.jet_tree_build_launches(N, V) for N, V in ((1, 1), (6, 4096), (6, 4097), (3, 8192), (4, 8192), (1, 24577))] == [1, 1, 2, 1, 2, 2]
     assert [jet.jet_tree_build_launches(2, 100, mode, raw) for mode, raw in ((0, True), (1, False), (2, True))] == [2, 2, 3]
-    assert [jet.jet_tree_accept_launches(B, V) for B, V in ((8, 4096), (9, 4096), (1, 4097), (512, 64))] == [1, 2, 2, 1]
+    assert [jet.jet_tree_accept_launches(*a) for a in ((1, 16, 1024), (1, 16, 1025), (1, 17, 64), (1, 4, 2049), (20, 64, 512), (20, 64, 513),
+                                                      (19, 64, 512), (20, 512, 64))] == [1, 2, 2, 2, 1, 2, 2, 1]
     assert [jet.jet_kv_compact_launches(*a, tail) for tail in (False, True) for a in
             ((1, 1, 8, 128, 31), (1, 1, 8, 128, 32), (36, 4, 8, 128, 8), (36, 2000, 8, 128, 8))] == [1, 2, 2, 1] + [1, 1, 2, 1]
     assert jet.jet_kv_compact_launches(1, 1, 8, 128, 0) == 0
-    assert jet.jet_tree_build_launches(0, 10) == jet.jet_tree_build_launches(1, 10, 3) == jet.jet_tree_accept_launches(0, 10) == 0
+    assert jet.jet_tree_build_launches(0, 10) == jet.jet_tree_build_launches(1, 10, 3) == jet.jet_tree_accept_launches(1, 0, 10) == 0
