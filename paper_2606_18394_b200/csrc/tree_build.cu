@@ -13,10 +13,11 @@
 //                        streams: the maximum of every group of 128 entries and the slice's
 //                        fp64 sum go to the workspace.  (Raw logits with an entropy score: a
 //                        second launch of it forms the entropy, which needs the log-sum-exp.)
-//   tree_expand_kernel   grid (batch): (small problems: forms the group maxima itself, one launch;) per depth, finds the W-th largest group maximum, reads
-//                        the few groups at or above it again and ranks their entries; then runs
-//                        the sequential pop/expand loop in one warp with the pending queue
-//                        in registers and emits parent / depth / token / score / ancestor mask.
+//   tree_expand_kernel   grid (batch): per depth, finds a threshold that W groups reach, reads the
+//                        groups at or above it again and ranks their entries; then runs the
+//                        sequential pop/expand loop in one warp with the pending queue in
+//                        registers and emits parent / depth / token / score / ancestor mask.
+//                        (Small problems: it forms the group maxima itself, one launch.)
 #include "fp64_exp.cuh"
 #include "jet_common.cuh"
 
@@ -463,8 +464,19 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
   int count = 0;
 #pragma unroll 1
   for (int attempt = 0; fits && attempt < 2; ++attempt) {
+    if (attempt != 0) {
+      best[0] = best[1] = best[2] = best[3] = -INFINITY;
+#pragma unroll 1
+      for (int g = 0; g < n; ++g) {
+        const float4 q = load4(rg.row, w.groups[g] + rg.lane_part, rg.V, rg.vec != 0);
+        best[0] = fmaxf(best[0], q.x);
+        best[1] = fmaxf(best[1], q.y);
+        best[2] = fmaxf(best[2], q.z);
+        best[3] = fmaxf(best[3], q.w);
+      }
+      cut = fmaxf(cut, threshold(warp_nth<4>(best, Wc)));
+    }
     count = 0;
-    best[0] = best[1] = best[2] = best[3] = -INFINITY;
 #pragma unroll 1
     for (int g0 = 0; g0 < n; g0 += kBatch) {
       float4 q[kBatch];
@@ -472,13 +484,8 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
       for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
       uint32_t take = 0u;                            // entry j of float4 i reaches the threshold
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
+      for (int i = 0; i < kBatch; ++i)
         take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
-        best[0] = fmaxf(best[0], q[i].x);
-        best[1] = fmaxf(best[1], q[i].y);
-        best[2] = fmaxf(best[2], q[i].z);
-        best[3] = fmaxf(best[3], q[i].w);
-      }
       if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
 #pragma unroll 1
       for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo && count <= kListCap;) {
@@ -495,7 +502,6 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
       }
     }
     if (count <= kListCap) break;
-    cut = fmaxf(cut, threshold(warp_nth<4>(best, Wc)));
   }
   __syncwarp();
   if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, cut, Wc, lse, lane, w);
