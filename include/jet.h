@@ -94,7 +94,10 @@ JET_API const char* jet_status_string(jet_status s);
  *   score        fp32 [batch, B] out, may be NULL
  *   anc_mask     u32 [batch, B, ceil(B/32)] out
  *   n_nodes      i32 [batch] out
- * Limits: 1 <= N <= JET_MAX_DEPTH, 1 <= W <= JET_MAX_WIDTH, V >= 1.
+ * Limits: 1 <= N <= JET_MAX_DEPTH, 1 <= W <= JET_MAX_WIDTH, V >= 1.  Cost: one pass
+ * over the rows and a selection per row whose time grows slowly with W and V; rows
+ * in which very many entries tie for a place among the W largest take longer (1024
+ * equal entries about 2.5 times).
  */
 JET_API size_t jet_tree_build_workspace_bytes(int batch, int N, int V, int W);
 
@@ -158,11 +161,13 @@ JET_API jet_status jet_tree_build_scored(const float* logp, int64_t logp_batch_s
  *   logp[b,d,t] = fl32(double(z[b,d,t]) - lse[b,d])   (one rounding);
  * candidates are ranked by these fp32 log-probabilities (two logits that round
  * to the same log-probability tie -> lowest token id), entropies are taken of
- * them, scores add them.  The fp64 sums are formed in a fixed order (per 4096-
- * entry slice, then over the slices), so results do not change from run to run;
- * against another summation order lse can differ in its last bits, which moves
- * a log-probability only if it sits within ~1e-15 (relative) of a rounding
- * boundary.
+ * them, scores add them.  The fp64 sums are formed in an order fixed by batch, N
+ * and V (a row is cut into slices of 4096, 8192 or 16384 entries, the longer ones
+ * for larger batches), so results do not change from run to run; against another
+ * summation order -- the same row in a batch of another size among them -- lse can
+ * differ in its last bits, which moves a log-probability only if it sits within
+ * ~1e-15 (relative) of a rounding boundary.  The same holds for the entropies of
+ * jet_tree_build_scored.
  *
  *   logits       fp32 [batch, N, V], strides as for logp.  No NaN, no +inf; a
  *                row must hold at least one finite entry (-inf = probability 0)
@@ -213,8 +218,15 @@ JET_API jet_status jet_tree_build_logits(const float* logits, int64_t logits_bat
  * at most 65535 (they are grid dimensions).  max_seq_len is a bound, but a call
  * with one sequence whose seq_len equals it exactly starts a little faster (the
  * first key tiles are prefetched on that guess).
+ * Reproducibility: a call gives the same bits every time.  Which bits depends on the
+ * launch plan: the rows of every key slice are rounded to bf16 before the slices are
+ * combined, so another plan -- another batch, budget, max_seq_len, device or version
+ * of this library -- moves outputs by up to the bf16 rounding of a partial row (2^-9
+ * of the slice's values, 0.3 % of the output's norm with four or five slices of few
+ * keys).  jet_tree_verify_attn_plan tells the plan.
  * Workspace: unlike the other calls, the first 4096 bytes of this workspace hold
- * counters that must be ZERO when the call starts.  Zero them once after
+ * counters that must be ZERO when the call starts (only the third form below, which
+ * the planner does not choose, reads them).  Zero them once after
  * allocating the workspace; every call that completes leaves them zero again.
  * When a sequence has fewer work items than the GPU has SMs, its key range is cut
  * into slices that run as separate CTAs.  They combine their partial rows inside
@@ -393,7 +405,8 @@ JET_API jet_status jet_tree_accept(const float* logits, int64_t logits_row_strid
  *   d               hidden size, a multiple of 64
  *   every other argument as for jet_tree_accept; device_status as for the attention call
  * Cost: one pass over the weights (V * d * 2 bytes from HBM) for up to 512 rows; more
- * rows stream them once per group of 512.
+ * rows stream them once per group of 512.  Rows are computed in groups: 128, 256, then
+ * whole groups of 512 (513 rows cost about what 1024 cost).
  * Workspace: jet_tree_accept_hidden_workspace_bytes (one 64-bit key per row; need not
  * be initialised).
  */

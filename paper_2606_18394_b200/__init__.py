@@ -1,7 +1,8 @@
 """B200-native tree-verification kernels (tree build, tree attention, acceptance, KV commit).
 
 The product is ``libjet.so`` (C ABI declared in ``include/jet.h``); this package is the
-thin ctypes binding with the same names.  Importing the package does not need a GPU;
+thin binding with the same names (launching calls are marshalled in C++, queries by ctypes).
+Importing the package does not need a GPU;
 calling an entry point needs the built library and fails loudly without it.
 """
 from .binding import (  # noqa: F401

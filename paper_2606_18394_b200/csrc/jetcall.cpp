@@ -1,10 +1,11 @@
 // _jetcall: the Python side of the C ABI's call path, in C++.
 //
 // An entry point takes up to thirty arguments, ten of them tensors.  Marshalled by ctypes from Python a call cost
-// 12 - 20 us of host time (data_ptr() of every tensor, the current stream, one conversion object per argument), more
-// than the kernels of a small call take; here it is one pass over the argument vector: 1 - 2 us in front of the
-// library's own host work (attention call as a whole 19.6 -> 5 us).  Only argument marshalling lives here: every
-// function calls the C function of the same name in libjet.so with the GIL released and returns its status.
+// 11 - 20 us of host time (data_ptr() of every tensor, the current stream, one conversion object per argument), more
+// than the kernels of a small call take; here it is one pass over the argument vector, 0.5 us for the twenty-nine
+// arguments of an attention call.  (A commit of one launch as a whole: 11.3 -> 3.0 us, a step of four: 64 -> 14 - 22 us, by host.)
+// Only argument marshalling lives here: every function calls the C function of the same name in libjet.so with the GIL
+// released and returns its status.
 //
 // A device pointer is None, an int, a torch tensor, or anything with a data_ptr() method.  Plain tensors (and Parameters) are
 // read natively; a subclass is asked through its own Python methods, which it may override.  A tensor without an address
