@@ -2278,9 +2278,12 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).  There the
 // plans take 4.2 % more than the best form on average (735 shapes), and waves are whole numbers, so that two forms whose
 // costs are a per cent apart change places by chance.
-// The exchange inside one launch through the workspace (arrival counters, bounded spin) is 0.3 - 1 us slower than a
-// second launch at every shape, and CTA pairs need 1.22 times the key-tile time (the hand-overs cross two SMs): both
-// run where they are asked for (JET_FORCE_SPLIT="<slices>,g", JET_FORCE_PAIR=1).
+// Not planned, only run where they are asked for: CTA pairs (JET_FORCE_PAIR=1), which need 1.22 times the key-tile time (the
+// hand-overs cross two SMs), and the exchange inside one launch through the workspace (JET_FORCE_SPLIT="<slices>,g"; arrival
+// counters, bounded spin, all CTAs resident at once).  Against a second launch that is 0.2 - 2 us slower at D 128 up to
+// 9000 keys (32 / 8 heads, prefix 4096: 64 nodes 12.5 against 11.8 us, 16 nodes 12.3 against 10.7), within 2 % of it for long
+// sequences, and 0.2 - 0.8 us (2 - 6 %) faster at D 64 or with 18 slices of two query tiles: not enough for kernels that wait
+// for one another.
 double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
   if (!fitted) {
     const double shared = 1.0 + 0.75 / n_mgroups, per_tile = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
