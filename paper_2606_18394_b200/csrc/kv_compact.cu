@@ -5,18 +5,22 @@
 // Bound: latency (a step commits 0.1 - 3 MB).  The chain is lengths and path -> page table -> rows; the rows of all
 // sequences are spread over the GPU, a warp per row, and a CTA works the path of its sequence out once.  No CTA may see an
 // advanced length, so seq_len is advanced by a second launch, or, where one CTA per sequence is enough (kAloneRows), by that
-// CTA: the second launch costs 1.7 us of host time and, started under the first, no GPU time that shows.
+// CTA: the second launch costs 1.7 us of host time.  It starts once all CTAs hold their lengths and runs beside the copies.  (While it
+// waited for them before its load and store, a commit of several layers took 0.2 - 0.4 us more: acceptance and commit of 36 layers, 4
+// rows, paged: 8.2 against 7.9 us; 32 sequences, 4 layers: 12.9 against 12.6.)
 // us per call in a captured stream (a cluster of eight CTAs per sequence before; page size 16, 8 heads of 128 and 36 layers
 // where not said otherwise; in place in brackets):
 //   1 sequence, 6 rows                  6.3 -> 4.8   [8.9 -> 5.8]      1 sequence, 65 rows    29 -> 6.3  [48 -> 17]
 //   32 sequences, 6 rows                10.2 -> 10.3 [20.1 -> 12.7]    128, one layer, 5 rows  11.2 -> 4.3 [23.5 -> 4.8]
 //   8 sequences, 48 layers, 4 heads     6.8 -> 6.1   [8.1 -> 6.3]      128, 5 rows            40 -> 37.9 [61.6 -> 30.6]
 #include "jet_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace jet {
 namespace {
 
-constexpr int kCommitThreads = 256, kCommitThreadsAlone = 512;      // of a CTA; of one that has its sequence to itself
+// Threads of a CTA; of one that has its sequence to itself.  (With 1024 the copy spills: 52 rows 0.5 us slower.)
+constexpr int kCommitThreads = 256, kCommitThreadsAlone = 512;
 constexpr int kTailHeld = 16;                        // rows a lane of the in-place form has in flight
 
 struct CommitParams {
@@ -36,11 +40,14 @@ struct CommitTable {
   int node[JET_MAX_DEPTH + 1];
 };
 
-// Fills the table and returns a: entries 0 .. a of the path are committed.  A CTA that has its sequence to itself advances
-// seq_len once all its threads have the length.
+// Waits for the kernels before this one, fills the table and returns a: entries 0 .. a of the path are committed.  A CTA that
+// has its sequence to itself advances seq_len once all its threads have the length; else the launch behind this one does, and
+// is let go only now: it starts when every CTA has got here, so that no CTA can read a length that it has advanced.
 template <bool kTail>
 __device__ __forceinline__ int commit_table(const CommitParams& p, int b, CommitTable& t) {
   const int i = threadIdx.x;
+  if (p.ctas == 1) grid_dependency_wait();
+  else ptx::grid_dep_wait();
   const int accepted = p.accept_len[b], len = p.seq_len[b];
   int node = i <= p.N ? p.path[static_cast<size_t>(b) * (p.N + 1) + i] : -1;      // (in flight with the lengths)
   const int a = min(accepted, p.N);
@@ -59,8 +66,9 @@ __device__ __forceinline__ int commit_table(const CommitParams& p, int b, Commit
     t.dst[i] = dst;
     t.src[i] = src;
   }
-  __syncthreads();
-  if (p.ctas == 1 && threadIdx.x == 0) p.seq_len[b] = len + accepted + 1;
+  __syncthreads();                                   // (the lengths have arrived: they went into the table and a)
+  if (p.ctas != 1) ptx::grid_dep_launch();
+  else if (threadIdx.x == 0) p.seq_len[b] = len + accepted + 1;
   return a;
 }
 
@@ -68,7 +76,6 @@ __device__ __forceinline__ int commit_table(const CommitParams& p, int b, Commit
 __global__ void __launch_bounds__(kCommitThreadsAlone)
 kv_compact_kernel(const uint4* __restrict__ tree_k, const uint4* __restrict__ tree_v, uint4* __restrict__ k_cache,
                   uint4* __restrict__ v_cache, const CommitParams p) {
-  grid_dependency_wait();
   __shared__ CommitTable t;
   const int b = blockIdx.x / p.ctas;
   const int a = commit_table<false>(p, b, t);
@@ -111,7 +118,6 @@ kv_compact_kernel(const uint4* __restrict__ tree_k, const uint4* __restrict__ tr
 // units at once, if there are more units than warps.
 __global__ void __launch_bounds__(kCommitThreadsAlone, 1)
 kv_compact_tail_kernel(uint4* k_cache, uint4* v_cache, const CommitParams p) {
-  grid_dependency_wait();
   __shared__ CommitTable t;
   const int b = blockIdx.x / p.ctas;
   const int a = commit_table<true>(p, b, t);
@@ -144,10 +150,15 @@ kv_compact_tail_kernel(uint4* k_cache, uint4* v_cache, const CommitParams p) {
   }
 }
 
-__global__ void advance_seq_len_kernel(const int32_t* __restrict__ accept_len, int32_t* __restrict__ seq_len, int batch) {
-  grid_dependency_wait();
+// Runs beside the copies: by the time it starts (see commit_table) whatever wrote the two inputs has completed and every
+// copying CTA has its length.  The stream's next kernel may be scheduled beside it at once, and, as this one ends behind the
+// copies, finds both done when its own wait returns.  (Reads from L2: the kernel that wrote the inputs may have ended after
+// this SM last cached the lines.)
+__global__ void advance_seq_len_kernel(const int32_t* accept_len, int32_t* seq_len, int batch) {
+  ptx::grid_dep_launch();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < batch) seq_len[b] += accept_len[b] + 1;
+  if (b < batch) seq_len[b] = __ldcg(seq_len + b) + __ldcg(accept_len + b) + 1;
+  ptx::grid_dep_wait();
 }
 
 // Sequences of at most this many rows get one CTA: 8 layers of 9 positions, 144 rows, 7.4 us that way instead of 4.3.

@@ -61,6 +61,49 @@ def test_in_place(shape, paged):
     assert np.array_equal(gk.reshape(kc.shape), rk) and np.array_equal(gv.reshape(vc.shape), rv)
 
 
+@pytest.mark.parametrize("layers,batch,D", [(2, 1, 64), (9, 1, 64), (6, 40, 64), (3, 150, 8)])
+def test_commits_in_a_row(layers, batch, D):
+    """Each commit takes the length that the one before it left, with no kernel between them: a copy that saw a length too early
+    or too late, or a commit that began before the last one's copies ended, leaves other rows."""
+    B, N, commits, dev = 16, 8, 24, "cuda:0"
+    rng = np.random.default_rng(layers + batch)
+    paths, accepts = [], []
+    for _ in range(commits):
+        accepts.append(rng.integers(0, N + 1, size=batch))
+        paths.append(_random_paths(rng, batch, B, N, accepts[-1]))
+    rows = commits * (N + 1)
+    tk, tv = _rand_bits(rng, (layers, batch, B, 1, D)), _rand_bits(rng, (layers, batch, B, 1, D))
+    rk, rv = _rand_bits(rng, (layers, batch, rows, 1, D)), _rand_bits(rng, (layers, batch, rows, 1, D))
+    rs = np.zeros(batch, np.int32)
+    on_gpu = lambda x: torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).to(dev)
+    gtk, gtv, gk, gv = on_gpu(tk), on_gpu(tv), on_gpu(rk), on_gpu(rv)
+    seq = torch.zeros(batch, dtype=torch.int32, device=dev)
+    gp = [torch.from_numpy(np.asarray(p, np.int32)).to(dev) for p in paths]
+    ga = [torch.from_numpy(np.asarray(a, np.int32)).to(dev) for a in accepts]
+    torch.cuda.synchronize()
+
+    def run():
+        for p, a in zip(gp, ga):
+            jet.jet_kv_compact(gtk, gtv, gk, gv, gk.stride(0), gk.stride(1), None, 0, 0, p, a, seq, layers, batch, B, 1, D, N)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    graph.replay()
+    for p, a in zip(paths, accepts):
+        rk, rv, rs = kv_compact_ref(tk, tv, rk, rv, None, p, a, rs)
+    assert np.array_equal(seq.cpu().numpy(), rs)
+    for got, want in ((gk, rk), (gv, rv)):
+        assert np.array_equal(got.cpu().numpy(), np.ascontiguousarray(want).view(np.int16))
+    with_graph = gk.clone(), gv.clone()
+    gk.zero_(), gv.zero_(), seq.zero_()
+    run()                                            # and issued one by one
+    assert np.array_equal(seq.cpu().numpy(), rs)
+    for b in range(batch):
+        n = int(rs[b])
+        assert torch.equal(gk[:, b, :n], with_graph[0][:, b, :n]) and torch.equal(gv[:, b, :n], with_graph[1][:, b, :n])
+
+
 def _time(layers, N, a):
     B, Hkv, D, dev = 256, 8, 128, "cuda:0"
     i32 = dict(dtype=torch.int32, device=dev)
