@@ -308,15 +308,70 @@ struct TopScratch {
   int groups[kTopGroups];
 };
 
-// More groups or entries at or above the threshold than the fast form holds (equal or nearly equal values, rows with few
-// finite entries): the groups one after the other, in ascending order.  Once there are Wc candidates, an entry is listed only
-// if it beats the worst of them, and a group is read only if its maximum at its lowest index would.  (8 rows of 151936
-// equal entries, W 7: 16 us a call, 464 when every group was read.)
+// A threshold of entries from the Wc-th largest maximum (or entry).  Raw logits: their rank values are rounded, so it is
+// lowered by 2^-22 of the rank value, two rounding steps.
+template <bool kLogits>
+__device__ __forceinline__ float threshold_of(float nth, double lse) {
+  if constexpr (kLogits) nth = __fsub_rd(nth, fmaxf(fabsf(rank_value<true>(nth, lse)) * 2.384185791015625e-7f, 1e-44f));
+  return nth;
+}
+
+// More groups or entries at or above the threshold than the fast form holds.
+//  * n <= kTopGroups: the groups are listed, but hold too many entries (a row that rises or falls over its groups has whole
+//    groups above the first threshold): once again with a threshold from those entries themselves.
+//  * More groups, or still too many entries (equal or nearly equal values, rows with few finite entries): the groups one after the
+//    other, in ascending order.  Once there are Wc candidates, an entry is listed only if it beats the worst of them,
+//    and a group is read only if its maximum at its lowest index would.  (8 rows of 151936 equal entries, W 7: 16 us a
+//    call, 464 when every group was read.)
 template <bool kLogits, bool kDirect>
-__device__ __noinline__ void top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, float cut, int Wc, double lse,
+__device__ __noinline__ void top_of_many(const RowGroups rg, const float* __restrict__ gm, int groups, int n, float cut, int Wc, double lse,
                                          int lane, TopScratch& w) {
-  unsigned long long worst = 0ull;                   // keys at or below it cannot be among the best any more
   int count = 0;
+  if (n <= kTopGroups) {
+    auto load = [&](int g0, float4 (&q)[kBatch]) {
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
+    };
+    float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+    for (int g0 = 0; g0 < n; g0 += kBatch) {
+      float4 q[kBatch];
+      load(g0, q);
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        best[0] = fmaxf(best[0], q[i].x);
+        best[1] = fmaxf(best[1], q[i].y);
+        best[2] = fmaxf(best[2], q[i].z);
+        best[3] = fmaxf(best[3], q[i].w);
+      }
+    }
+    cut = fmaxf(cut, threshold_of<kLogits>(warp_nth<4>(best, Wc), lse));
+#pragma unroll 1
+    for (int g0 = 0; g0 < n && count <= kListCap; g0 += kBatch) {
+      float4 q[kBatch];
+      load(g0, q);
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int idx = g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V;
+        const float x[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool take = x[j] >= cut && idx + j < rg.V;
+          const unsigned votes = __ballot_sync(0xffffffffu, take);
+          const int at = count + __popc(votes & ((1u << lane) - 1u));
+          if (take && at < kListCap) w.list[at] = make_key(rank_value<kLogits>(x[j], lse), static_cast<uint32_t>(idx + j));
+          count += __popc(votes);
+        }
+      }
+    }
+    __syncwarp();
+    if (count <= kListCap) {
+      keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
+      return;
+    }
+    count = 0;
+  }
+  unsigned long long worst = 0ull;                   // keys at or below it cannot be among the best any more
   for (int g0 = 0; g0 < groups; g0 += 32) {          // (the number of groups is a multiple of 32)
     const float most = kDirect ? gm[g0 + lane] : __ldg(gm + g0 + lane);
     const unsigned long long bound = make_key(rank_value<kLogits>(most, lse), static_cast<uint32_t>(rg.base(g0 + lane)));
@@ -361,13 +416,18 @@ __device__ __noinline__ void top_of_many(const RowGroups rg, const float* __rest
 //    buckets, 37 groups at W = 32, for a longer threshold loop.
 //  * A lane holds the maxima of kQuads float4, 1280 groups (163840 entries) of the warp, in registers; longer rows take them
 //    in passes of that many, twice.
-// (8 rows of 151936 entries, W 32, 256 nodes: 121 -> 16 us a call, W 20 26 -> 14, W 7 as before; 200003 entries, W 7, 64 nodes: 15.5 -> 10.4.
+// (8 rows of 151936 entries, W 32, 256 nodes: 137 -> 15 us a call, W 20 24 -> 10, W 7 7.4 -> 7.5; 200003 entries, W 7, 64 nodes: 14.8 -> 9.3.
 // Such rows fell to top_of_many before, and the kernels before this one took 114, 65 and 10.7.)
-template <bool kLogits, bool kDirect, typename Lse>
+// kWide: more than kFewWidth candidates or longer rows than one pass.  The usual form is compiled without their code, and what
+// overflowing lists need is all in top_of_many: a step runs this once, from a cold instruction cache, where code that is only
+// jumped over counts too.  (Construction behind other kernels, as in a step: 0.5 - 1.1 us less than with one form for all, e.g. 7 sequences
+// of 301 nodes, 14 depths, step 330.3 -> 327.7 us; called over and over, 0.1 us less.  The kernel before the wide forms: 328.2.)
+constexpr int kQuads = 10;
+constexpr int kFewWidth = 12;
+
+template <bool kLogits, bool kDirect, bool kWide, typename Lse>
 __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __restrict__ gm, int groups, int Wc, Lse&& lse_of,
                                            int lane, TopScratch& w) {
-  constexpr int kQuads = 10;
-  constexpr int kFewWidth = 12;
   float4 h[kQuads];
   const int quads = groups / 4;                      // (groups is a multiple of 32)
   const float4* gm4 = reinterpret_cast<const float4*>(gm);
@@ -384,7 +444,7 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
   // for the whole construction), or with many candidates, for which the groups are too few buckets (8 rows of 4096
   // entries, W 32: 37 -> 14 us), the entries themselves.
   float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  if (groups < 128 && Wc > kFewWidth) {
+  if (kWide && groups < 128 && Wc > kFewWidth) {
 #pragma unroll 1
     for (int e0 = lane * 4; e0 < rg.V; e0 += kBatch * 128) {
       float4 q[kBatch];
@@ -416,27 +476,23 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
       best[3] = fmaxf(best[3], h[i].w);
     }
     first += kQuads * 32;
-    if (first >= quads) break;
+    if (!kWide || first >= quads) break;
     fetch(first);
   }
-  auto threshold = [&](float nth) {
-    if constexpr (kLogits)    // 2^-22 of the value: two rounding steps
-      nth = __fsub_rd(nth, fmaxf(fabsf(rank_value<true>(nth, lse)) * 2.384185791015625e-7f, 1e-44f));
-    return nth;
-  };
   float cut;
-  if (Wc <= kFewWidth) {
+  if (!kWide || Wc <= kFewWidth) {
     const float lane_best[1] = {fmaxf(fmaxf(best[0], best[1]), fmaxf(best[2], best[3]))};
-    cut = threshold(warp_nth<1>(lane_best, Wc));
+    cut = warp_nth<1>(lane_best, Wc);
   } else {
-    cut = threshold(warp_nth<4>(best, Wc));
+    cut = warp_nth<4>(best, Wc);
   }
+  cut = threshold_of<kLogits>(cut, lse);
   __syncwarp();
   // the groups that reach it, up to kTopGroups; few lanes have any
   int n = 0;
 #pragma unroll 1
   for (int first = 0; first < quads && n <= kTopGroups; first += kQuads * 32) {
-    if (quads > kQuads * 32) fetch(first);
+    if (kWide && quads > kQuads * 32) fetch(first);
     uint32_t bits[2] = {0u, 0u};                     // maximum 4 i + j of this lane reaches the threshold
 #pragma unroll
     for (int i = 0; i < kQuads; ++i) {
@@ -459,52 +515,34 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
   }
   const bool fits = n <= kTopGroups;
   __syncwarp();
-  // their entries that reach it, up to kListCap; if there are more, once again with a threshold from the entries themselves
-  // (a row that rises or falls over its groups has whole groups above the first one)
+  // their entries that reach it, up to kListCap
   int count = 0;
 #pragma unroll 1
-  for (int attempt = 0; fits && attempt < 2; ++attempt) {
-    if (attempt != 0) {
-      best[0] = best[1] = best[2] = best[3] = -INFINITY;
-#pragma unroll 1
-      for (int g = 0; g < n; ++g) {
-        const float4 q = load4(rg.row, w.groups[g] + rg.lane_part, rg.V, rg.vec != 0);
-        best[0] = fmaxf(best[0], q.x);
-        best[1] = fmaxf(best[1], q.y);
-        best[2] = fmaxf(best[2], q.z);
-        best[3] = fmaxf(best[3], q.w);
-      }
-      cut = fmaxf(cut, threshold(warp_nth<4>(best, Wc)));
-    }
-    count = 0;
-#pragma unroll 1
-    for (int g0 = 0; g0 < n; g0 += kBatch) {
-      float4 q[kBatch];
+  for (int g0 = 0; fits && g0 < n; g0 += kBatch) {
+    float4 q[kBatch];
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
-      uint32_t take = 0u;                            // entry j of float4 i reaches the threshold
+    for (int i = 0; i < kBatch; ++i) q[i] = load4(rg.row, g0 + i < n ? w.groups[g0 + i] + rg.lane_part : rg.V, rg.V, rg.vec != 0);
+    uint32_t take = 0u;                              // entry j of float4 i reaches the threshold
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i)
-        take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
-      if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
+    for (int i = 0; i < kBatch; ++i)
+      take |= ((q[i].x >= cut ? 1u : 0u) | (q[i].y >= cut ? 2u : 0u) | (q[i].z >= cut ? 4u : 0u) | (q[i].w >= cut ? 8u : 0u)) << (4 * i);
+    if (cut == -INFINITY) take = g0 + kBatch <= n ? take : take & ((1u << (4 * (n - g0))) - 1u);      // (absent groups read as -inf)
 #pragma unroll 1
-      for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo && count <= kListCap;) {
-        // one entry of every lane that has one, per step; read again (L1) rather than picked out of registers by index
-        const int bit = __ffs(take) - 1;
-        const int at = count + __popc(todo & ((1u << lane) - 1u));
-        if (take && at < kListCap) {
-          const int idx = w.groups[g0 + (bit >> 2)] + rg.lane_part + (bit & 3);
-          w.list[at] = idx < rg.V ? make_key(rank_value<kLogits>(__ldg(rg.row + idx), lse), static_cast<uint32_t>(idx)) : 0ull;
-        }
-        count += __popc(todo);
-        take &= take - 1u;
-        todo = __ballot_sync(0xffffffffu, take != 0u);
+    for (unsigned todo = __ballot_sync(0xffffffffu, take != 0u); todo && count <= kListCap;) {
+      // one entry of every lane that has one, per step; read again (L1) rather than picked out of registers by index
+      const int bit = __ffs(take) - 1;
+      const int at = count + __popc(todo & ((1u << lane) - 1u));
+      if (take && at < kListCap) {
+        const int idx = w.groups[g0 + (bit >> 2)] + rg.lane_part + (bit & 3);
+        w.list[at] = idx < rg.V ? make_key(rank_value<kLogits>(__ldg(rg.row + idx), lse), static_cast<uint32_t>(idx)) : 0ull;
       }
+      count += __popc(todo);
+      take &= take - 1u;
+      todo = __ballot_sync(0xffffffffu, take != 0u);
     }
-    if (count <= kListCap) break;
   }
   __syncwarp();
-  if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, cut, Wc, lse, lane, w);
+  if (!fits || count > kListCap) top_of_many<kLogits, kDirect>(rg, gm, groups, n, cut, Wc, lse, lane, w);
   else if (count <= 32) keep_best<1>(w.list, count, Wc, lane);
   else if (count <= 64) keep_best<2>(w.list, count, Wc, lane);
   else keep_best<(kListCap + 31) / 32>(w.list, count, Wc, lane);
@@ -633,7 +671,7 @@ struct ScanView {
 // and the scan's launch falls away.  Up to this many 4096-entry slices of all rows of a sequence (48 entries per thread).
 constexpr int kDirectSlices = 6;
 
-template <int kMode, bool kDirect = false>
+template <int kMode, bool kDirect, bool kWide>
 __global__ void __launch_bounds__(kExpThreads)
 tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, int N, int V, int Wc, int B, float alpha,
                    int32_t* __restrict__ parent_out, int32_t* __restrict__ depth_out,
@@ -699,13 +737,13 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     const float* gm = kDirect ? s_gmax + d * groups : scan.gmax + row_id * groups;
     TopScratch& w = sh.top[warp];
     if (!kDirect && scan.pairs) {
-      top_of_row<true, kDirect>(rg, gm, groups, Wc, [&] {
+      top_of_row<true, kDirect, kWide>(rg, gm, groups, Wc, [&] {
         const double lse = row_lse(scan.pairs + row_id * scan.slices, scan.slices, lane);
         if (lane == 0 && depth_lse_out) depth_lse_out[row_id] = static_cast<float>(lse);
         return lse;
       }, lane, w);
     } else {
-      top_of_row<false, kDirect>(rg, gm, groups, Wc, [] { return 0.0; }, lane, w);
+      top_of_row<false, kDirect, kWide>(rg, gm, groups, Wc, [] { return 0.0; }, lane, w);
     }
     if (lane < Wc) {
       const unsigned long long k = w.list[lane];
@@ -849,9 +887,12 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
     scan(row_scan_kernel<kScanMax>, nullptr);
   }
   const ScanView view{rows, batch_stride, depth_stride, gmax, pairs, plogp, plan.slices, plan.rounds, vec ? 1 : 0};
-  auto expand = direct ? tree_expand_kernel<0, true>
-                : score_mode == JET_SCORE_ACCUM_LOGP ? tree_expand_kernel<0>
-                : score_mode == JET_SCORE_ENTROPY  ? tree_expand_kernel<1> : tree_expand_kernel<2>;
+  const bool wide = Wc > kFewWidth || plan.slices * 32 * plan.rounds > kQuads * 128;
+  auto pick = [&](auto narrow_form, auto wide_form) { return wide ? wide_form : narrow_form; };
+  auto expand = direct ? pick(tree_expand_kernel<0, true, false>, tree_expand_kernel<0, true, true>)
+                : score_mode == JET_SCORE_ACCUM_LOGP ? pick(tree_expand_kernel<0, false, false>, tree_expand_kernel<0, false, true>)
+                : score_mode == JET_SCORE_ENTROPY  ? pick(tree_expand_kernel<1, false, false>, tree_expand_kernel<1, false, true>)
+                                                   : pick(tree_expand_kernel<2, false, false>, tree_expand_kernel<2, false, true>);
   launch_dependent(expand, dim3(batch), dim3(kExpThreads), st, view, root_token, N, V, Wc, B, alpha, parent, depth, token,
                    score, anc_mask, n_nodes, depth_entropy, depth_lse, node_budget, len_src, len_dst);
   return launch_status();
