@@ -10,9 +10,11 @@
 // rows, paged: 8.2 against 7.9 us; 32 sequences, 4 layers: 12.9 against 12.6.)
 // us per call in a captured stream (a cluster of eight CTAs per sequence before; page size 16, 8 heads of 128 and 36 layers
 // where not said otherwise; in place in brackets):
-//   1 sequence, 6 rows                  6.3 -> 4.8   [8.9 -> 5.8]      1 sequence, 65 rows    29 -> 6.3  [48 -> 17]
-//   32 sequences, 6 rows                10.2 -> 10.3 [20.1 -> 12.7]    128, one layer, 5 rows  11.2 -> 4.3 [23.5 -> 4.8]
-//   8 sequences, 48 layers, 4 heads     6.8 -> 6.1   [8.1 -> 6.3]      128, 5 rows            40 -> 37.9 [61.6 -> 30.6]
+//   1 sequence, 6 rows                  5.3 -> 3.5   [8.1 -> 4.8]      1 sequence, 65 rows    28 -> 5.3  [50 -> 17]
+//   32 sequences, 6 rows                11.6 -> 9.9  [22.4 -> 15.0]    128, one layer, 5 rows  10.2 -> 3.3 [23.5 -> 4.8]
+//   8 sequences, 48 layers, 4 heads     5.3 -> 4.2   [7.4 -> 5.6]      128, 5 rows            39 -> 37  [61 -> 33]
+// Left behind the clusters: 33 - 64 rows of 2 KB in one CTA, 0.4 us (two turns of its warps; a second launch costs a caller
+// who issues call by call more than that).
 #include "jet_common.cuh"
 #include "sm100_ptx.cuh"
 
