@@ -31,6 +31,7 @@ constexpr int kRoundElems = 16;                      // elements a thread takes 
 constexpr int kRoundChunk = kScanThreads * kRoundElems;
 constexpr int kGroup = 128;                          // entries per group maximum
 constexpr float kTermFloor = 700.0f;                 // exp(-700) is beyond any sum's last place
+constexpr double kNothing = 1e-290;                  // an entropy sum below it has no term of its own (the smallest would be 1e-45)
 
 enum ScanMode { kScanMax = 0, kScanEntropy = 1, kScanSum = 2, kScanLogitEntropy = 3 };
 
@@ -107,8 +108,8 @@ __device__ __noinline__ double slow_sum(const float* __restrict__ row, int base,
 //   kScanLogitEntropy  .y = sum(exp(l) * l), l = float(double(z) - lse) with the lse of the slices' kScanSum pairs in `pairs`
 // All sums in fp64 in a fixed order: the same value from run to run.  Entries of -inf contribute 0.
 //
-// Bound: HBM without a sum; with one the issue slots and the fp64 pipe (about 25 instructions per entry, 9 of them fp64:
-// 53 us for 32 x 8 rows of 151936 entries, 38 - 42 us of that for the terms alone).  A thread keeps one round of 16 entries in
+// Bound: HBM without a sum; with one the issue slots (31.6 instructions per entry, 10.9 of them fp64, which take two slots: 94 % of
+// the slots in 53 us for 32 x 8 rows of 151936 entries; row_share_kernel takes calls of that size).  A thread keeps one round of 16 entries in
 // flight while it works on the round before; there is one CTA-wide barrier per slice (two with a sum), so that the blocks of
 // an SM drift apart and one block's loads run under another's arithmetic.  The form before -- 4096 entries per block,
 // every block ranking its own W best, general fp64 exponentials, the logits scanned once for the sum and once for the
@@ -132,7 +133,7 @@ row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t de
     for (int i = 0; i < 4; ++i) x[i] = load4(row, base + ((r * 4 + i) * kScanThreads + tid) * 4, V, vec);
   };
   fetch(0, cur);
-  Exp64Table tab(kMode == kScanMax ? 0 : lane);
+  LaneExp64 exp64(kMode == kScanMax ? 0 : lane);
   double ref = 0.0, acc = 0.0;
   float ref_f = 0.0f, mx = -INFINITY;
   if constexpr (kMode == kScanLogitEntropy) {
@@ -160,13 +161,13 @@ row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t de
 #pragma unroll
         for (int w = 1; w < kScanWarps; ++w) ref_f = fmaxf(ref_f, s_max[w]);
         const int m = __float2int_rn(ref_f * 1.4426950408889634f);     // near the largest entry of the block's first round
-        tab.scale_down(m);
+        exp64.scale_down(m);
         ref = static_cast<double>(m);
       }
 #pragma unroll
       for (int e = 0; e < kRoundElems; ++e) {
         const float v = fmaxf(x[e], ref_f - kTermFloor);       // (a term of exp(-700) and one of 0 are the same beside exp(0))
-        const Exp64 t = exp64(v, static_cast<double>(v), tab);
+        const Exp64 t = exp64(v, static_cast<double>(v));
         acc = fma(t.s, t.p, acc);
       }
     } else if constexpr (kMode == kScanEntropy || kMode == kScanLogitEntropy) {
@@ -175,7 +176,7 @@ row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t de
         float l = kMode == kScanLogitEntropy ? static_cast<float>(static_cast<double>(x[e]) - ref) : x[e];
         l = l >= -kTermFloor ? l : 0.0f;               // (entries below it, -inf among them, contribute exactly 0)
         const double ld = static_cast<double>(l);
-        const Exp64 t = exp64(l, ld, tab);
+        const Exp64 t = exp64(l, ld);
         acc = fma(t.s * t.p, ld, acc);
       }
     }
@@ -199,7 +200,7 @@ row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t de
     float m = s_max[0];
 #pragma unroll
     for (int w = 1; w < kScanWarps; ++w) m = fmaxf(m, s_max[w]);
-    const bool slow = kMode == kScanSum       ? !(fabsf(ref_f) < kExp64Range - 1000.0f) || m > ref_f + 600.0f
+    const bool slow = kMode == kScanSum       ? !(fabsf(ref_f) < LaneExp64::kRange - 1000.0f) || m > ref_f + 600.0f
                       : kMode == kScanEntropy ? m > 600.0f : static_cast<double>(m) > ref + 600.0;
     if (slow) {                                      // (block-uniform)
       double scale = 1.0;
@@ -220,6 +221,181 @@ row_scan_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t de
       double2* out = sums + row_id * gridDim.x + slice;
       *out = kMode == kScanSum ? make_double2(ref, total) : make_double2(total, 0.0);
     }
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ scan of many rows, with a sum
+// Rounds of 4096 entries are numbered through all rows of the call; block i takes rounds per * i .. per * (i + 1) - 1, an equal
+// share that may begin and end inside a row.  Its part of a row is a piece.
+constexpr int kShareStages = 3;                      // rounds a block holds in shared memory
+constexpr int kShareSmem = kShareStages * kRoundChunk * 4;
+constexpr int kShareBlocks = 296;                    // two blocks on each of 148 SMs (a constant: workspaces are sized by it)
+
+struct ShareShape {
+  int N, V, row_rounds;                              // rounds per row
+  int per, total;                                    // rounds per block; of all rows
+  int pieces;                                        // most pieces a row can have
+  __host__ __device__ int first_block(int row) const {
+    return static_cast<int>(static_cast<uint32_t>(row) * static_cast<uint32_t>(row_rounds) / static_cast<uint32_t>(per));
+  }
+  __device__ int pieces_of(int row) const {
+    return static_cast<int>((static_cast<uint32_t>(row + 1) * static_cast<uint32_t>(row_rounds) - 1u) / static_cast<uint32_t>(per)) - first_block(row) + 1;
+  }
+};
+
+// What row_scan_kernel does, with a sum, where the rows are many: gmax as with one round per slice, sums[row][piece].
+// The blocks stay, so that the table of the shorter exponential is set up once, no wave of blocks is left half empty, and a
+// thread's entries arrive in shared memory two rounds ahead (its own places: no barrier).  Loads into registers wait on the
+// same few scoreboards as the conversions and the table, which made the pass as slow as its warps were few.
+// Bound: issue slots, 37 cycles an entry of a warp and scheduler.  32 x 8 rows of 151936 entries with an entropy, the whole
+// construction: 58.9 -> 52.1 us, log-sum-exp 62.4 -> 53.6.  (Tried: three and four blocks per SM, four stages: up to 2 us slower.)
+template <int kMode>
+__global__ void __launch_bounds__(kScanThreads, 2)
+row_share_kernel(const float* __restrict__ rows, int64_t batch_stride, int64_t depth_stride, const ShareShape sh,
+                 float* __restrict__ gmax, const double2* __restrict__ pairs, double2* __restrict__ sums) {
+  static_assert(kMode != kScanMax, "without a sum the rows come at the rate of HBM as it is");
+  static_assert(kScanThreads == SharedExp64::kEntries, "one thread per table entry");
+  grid_dependency_wait();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ __align__(16) float4 s_row[];    // [kShareStages][4][kScanThreads]
+  __shared__ float s_ref[kScanWarps], s_max[2][kScanWarps];
+  __shared__ double s_sum[2][kScanWarps];
+  __shared__ double s_lse;
+  __shared__ SharedExp64::Shared s_exp;
+
+  int at = blockIdx.x * sh.per;                      // the round that is worked on, the one that is requested next
+  const int end = min(at + sh.per, sh.total);
+  int row_id = at / sh.row_rounds, rd = at - row_id * sh.row_rounds;
+  auto row_at = [&](int id) {
+    const int b = id / sh.N;
+    return rows + static_cast<int64_t>(b) * batch_stride + static_cast<int64_t>(id - b * sh.N) * depth_stride;
+  };
+  const float* ahead_row = row_at(row_id);
+  int ahead_at = at, ahead_rd = rd, ahead_id = row_id;
+  auto request = [&]() {
+    if (ahead_at < end) {
+      float4* dst = s_row + (ahead_at % kShareStages) * 4 * kScanThreads + tid;
+      const int e0 = ahead_rd * kRoundChunk + tid * 4;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = e0 + i * kScanThreads * 4;     // (V is a multiple of four)
+        if (e < sh.V)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst + i * kScanThreads))), "l"(ahead_row + e) : "memory");
+        else
+          dst[i * kScanThreads] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      }
+      ++ahead_at;
+      if (++ahead_rd == sh.row_rounds) {
+        ahead_rd = 0;
+        ++ahead_id;
+        if (ahead_at < end) ahead_row = row_at(ahead_id);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto landed = [&]() { asm volatile("cp.async.wait_group %0;" ::"n"(kShareStages - 2) : "memory"); };      // round `at`
+  for (int k = 0; k < kShareStages - 1; ++k) request();
+  const SharedExp64 exp64(s_exp, lane);
+  SharedExp64::fill(s_exp, tid);
+  if (kMode == kScanEntropy) __syncthreads();        // (the other modes meet at a barrier before their first term)
+
+  int flip = 0;
+#pragma unroll 1
+  while (at < end) {                                 // a piece per turn
+    const int first = rd, stop = min(sh.row_rounds, rd + end - at);
+    double ref = 0.0, acc = 0.0;
+    float ref_f = 0.0f, mx = -INFINITY;
+    int shift = 0;
+    if constexpr (kMode == kScanLogitEntropy) {
+      if (warp == 0) {
+        const double l = row_lse(pairs + static_cast<size_t>(row_id) * sh.pieces, sh.pieces_of(row_id), lane);
+        if (lane == 0) s_lse = l;
+      }
+      __syncthreads();
+      ref = s_lse;
+    } else if constexpr (kMode == kScanSum) {
+      // the reference: a whole power of two near the largest entry of the piece's first round
+      landed();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 q = s_row[((at % kShareStages) * 4 + i) * kScanThreads + tid];
+        mx = fmaxf(mx, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
+      }
+      const float mw = warp_max_f32(mx);
+      if (lane == 0) s_ref[warp] = mw;
+      __syncthreads();
+      ref_f = s_ref[0];
+#pragma unroll
+      for (int w = 1; w < kScanWarps; ++w) ref_f = fmaxf(ref_f, s_ref[w]);
+      shift = __float2int_rn(ref_f * 1.4426950408889634f);
+      ref = static_cast<double>(shift);
+    }
+#pragma unroll 1
+    for (; rd < stop; ++rd, ++at) {
+      landed();
+      float x[kRoundElems];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 q = s_row[((at % kShareStages) * 4 + i) * kScanThreads + tid];
+        x[4 * i] = q.x; x[4 * i + 1] = q.y; x[4 * i + 2] = q.z; x[4 * i + 3] = q.w;
+      }
+      request();                                     // (into the places of the round before this one, which has been used)
+      float g = -INFINITY;
+#pragma unroll
+      for (int e = 0; e < kRoundElems; ++e) {
+        g = fmaxf(g, x[e]);
+        if constexpr (kMode == kScanSum) {
+          const float v = fmaxf(x[e], ref_f - kTermFloor);       // (a term of exp(-700) and one of 0 are the same beside exp(0))
+          const Exp64 t = exp64(v, static_cast<double>(v), shift);
+          acc = fma(t.s, t.p, acc);
+        } else {
+          // (entries below the floor, -inf among them, count as the floor: 2^31 of them sum to less than kNothing)
+          const float l = fmaxf(kMode == kScanLogitEntropy ? static_cast<float>(static_cast<double>(x[e]) - ref) : x[e], -kTermFloor);
+          const double ld = static_cast<double>(l);
+          const Exp64 t = exp64(l, ld, 0);
+          acc = fma(t.s * t.p, ld, acc);
+        }
+      }
+      mx = fmaxf(mx, g);
+      if constexpr (kMode != kScanLogitEntropy) {
+        constexpr int kLanes = kGroup / kRoundElems;             // threads of a group
+#pragma unroll
+        for (int o = 1; o < kLanes; o <<= 1) g = fmaxf(g, __shfl_xor_sync(0xffffffffu, g, o));
+        if (tid % kLanes == 0) gmax[(static_cast<size_t>(row_id) * sh.row_rounds + rd) * (kScanThreads / kLanes) + tid / kLanes] = g;
+      }
+    }
+    const float mw = warp_max_f32(mx);
+    acc = warp_sum_f64(acc);
+    if (lane == 0) { s_max[flip][warp] = mw; s_sum[flip][warp] = acc; }
+    __syncthreads();
+    float m = s_max[flip][0];
+#pragma unroll
+    for (int w = 1; w < kScanWarps; ++w) m = fmaxf(m, s_max[flip][w]);
+    const bool slow = kMode == kScanSum       ? !(fabsf(ref_f) < SharedExp64::kRange - 1000.0f) || m > ref_f + 600.0f
+                      : kMode == kScanEntropy ? m > 600.0f : static_cast<double>(m) > ref + 600.0;
+    if (slow) {                                      // (block-uniform)
+      double scale = 1.0;
+      if constexpr (kMode == kScanSum) {
+        ref = rint(static_cast<double>(m) * 1.4426950408889634);
+        scale = exp(static_cast<double>(m) - ref * 0.6931471805599453);
+      }
+      acc = m > -INFINITY ? scale * slow_sum<kMode>(row_at(row_id), first * kRoundChunk, stop - first, sh.V, true, kMode == kScanSum ? static_cast<double>(m) : ref) : 0.0;
+      acc = warp_sum_f64(acc);
+      __syncthreads();
+      if (lane == 0) s_sum[flip][warp] = acc;
+      __syncthreads();
+    }
+    if (tid == 0) {
+      double total = 0.0;
+#pragma unroll
+      for (int w = 0; w < kScanWarps; ++w) total += s_sum[flip][w];
+      if (kMode != kScanSum && fabs(total) < kNothing) total = 0.0;
+      double2* out = sums + static_cast<size_t>(row_id) * sh.pieces + (static_cast<int>(blockIdx.x) - sh.first_block(row_id));
+      *out = kMode == kScanSum ? make_double2(ref, total) : make_double2(total, 0.0);
+    }
+    flip ^= 1;                                       // (the next piece writes while this one's values may still be read)
+    ++row_id;
+    rd = 0;
   }
 }
 
@@ -665,6 +841,11 @@ struct ScanView {
   const double2* pairs;                              // [batch * N][slices] (reference, sum) of raw logits, or null
   const double2* plogp;                              // [batch * N][slices] .x = sum(p * log p) with an entropy score, or null
   int slices, rounds, vec;
+  ShareShape share;                                  // per > 0: the scan was row_share_kernel's, and a row has pieces instead of slices
+  __device__ __forceinline__ const double2* of_row(const double2* sums, size_t row, int& count) const {
+    count = share.per ? share.pieces_of(static_cast<int>(row)) : slices;
+    return sums + row * (share.per ? share.pieces : slices);
+  }
 };
 
 // Small problems (accumulated log-probabilities only): the expansion kernel forms the group maxima itself, in shared memory,
@@ -722,9 +903,10 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     const size_t row_id = static_cast<size_t>(b) * N + d;
     if constexpr (kMode != 0) {
       // entropy: minus the sum of the slices' partial sums (fp64, fixed order), rounded once
-      const double2* part = scan.plogp + row_id * scan.slices;
+      int parts;
+      const double2* part = scan.of_row(scan.plogp, row_id, parts);
       double acc = 0.0;
-      for (int i = lane; i < scan.slices; i += 32) acc += part[i].x;
+      for (int i = lane; i < parts; i += 32) acc += part[i].x;
       acc = warp_sum_f64(acc);
       if (lane == 0) {
         const float h = static_cast<float>(-acc);
@@ -738,7 +920,9 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     TopScratch& w = sh.top[warp];
     if (!kDirect && scan.pairs) {
       top_of_row<true, kDirect, kWide>(rg, gm, groups, Wc, [&] {
-        const double lse = row_lse(scan.pairs + row_id * scan.slices, scan.slices, lane);
+        int parts;
+        const double2* part = scan.of_row(scan.pairs, row_id, parts);
+        const double lse = row_lse(part, parts, lane);
         if (lane == 0 && depth_lse_out) depth_lse_out[row_id] = static_cast<float>(lse);
         return lse;
       }, lane, w);
@@ -828,17 +1012,50 @@ ScanPlan scan_plan(int batch, int N, int V) {
   return p;
 }
 
+// Rows with a sum, aligned and many: dealt out to kShareBlocks blocks (per = 0: not).  The line: a round costs 0.9 of row_scan_kernel's, the
+// blocks' start 450 rounds, and row_scan_kernel also walks the rounds that fill up its slices.  Measured, log-probabilities with an entropy
+// / logits, us a call, before and now: 375 x 8 rows of 4096 entries 82 / 81 and 41 / 43; 29 x 8 of 50256 28.6 / 28.5 and 24.7 / 25.2;
+// 12 x 8 of 151936 28.6 / - and 27.2 / -.  Just beyond the line: 94 x 8 of 16384 25.2 / 25.5 and 25.8 / 26.7, 8 x 8 of 151936 22.4 and 22.8.
+ShareShape share_shape(int batch, int N, int V, bool vec) {
+  ShareShape sh{};
+  const int64_t row_rounds = (static_cast<int64_t>(V) + kRoundChunk - 1) / kRoundChunk, total = row_rounds * N * batch;
+  const ScanPlan other = scan_plan(batch, N, V);
+  if (!vec || V % 4 != 0 || total > (1ll << 30) || total * 9 / 10 + 450 >= static_cast<int64_t>(other.slices) * other.rounds * N * batch) return sh;
+  sh.N = N;
+  sh.V = V;
+  sh.row_rounds = static_cast<int>(row_rounds);
+  sh.total = static_cast<int>(total);
+  sh.per = (sh.total + kShareBlocks - 1) / kShareBlocks;
+  sh.pieces = (sh.row_rounds + sh.per - 2) / sh.per + 1;
+  return sh;
+}
+
+bool share_ready() {
+  static std::atomic<int> states[kMaxDevices];       // per device: 0 = not yet, 1 = ok, -1 = failed
+  std::atomic<int>& state_ref = states[current_device()];
+  int state = state_ref.load(std::memory_order_acquire);
+  if (state == 0) {
+    auto set = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kShareSmem) == cudaSuccess; };
+    state = set(row_share_kernel<kScanEntropy>) && set(row_share_kernel<kScanSum>) && set(row_share_kernel<kScanLogitEntropy>) ? 1 : -1;
+    if (state < 0) cudaGetLastError();
+    state_ref.store(state, std::memory_order_release);
+  }
+  return state > 0;
+}
+
 // The group maxima are formed inside the expansion kernel: no launch in front of it.
 bool build_direct(int N, int V, bool scored, bool from_logits) {
   return !scored && !from_logits && static_cast<int64_t>(N) * ((static_cast<int64_t>(V) + kRoundChunk - 1) / kRoundChunk) <= kDirectSlices;
 }
 
 // Workspace: group maxima, then (raw logits) the log-sum-exp pairs, then (entropy scores) the p * log p sums.
+// (row_share_kernel's group maxima are never more than those of the plan's slices, its sums may be)
 size_t gmax_bytes(int batch, int N, int V) {
   return round_up(static_cast<size_t>(batch) * N * scan_plan(batch, N, V).groups * sizeof(float), 256);
 }
 size_t sums_bytes(int batch, int N, int V) {
-  return round_up(static_cast<size_t>(batch) * N * scan_plan(batch, N, V).slices * sizeof(double2), 256);
+  const int slices = scan_plan(batch, N, V).slices, pieces = share_shape(batch, N, V, true).pieces;
+  return round_up(static_cast<size_t>(batch) * N * (slices > pieces ? slices : pieces) * sizeof(double2), 256);
 }
 
 // Checks and launches shared by the entry points (score_mode: JET_SCORE_*).
@@ -871,6 +1088,16 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   if (from_logits) ws += sums_bytes(batch, N, V);
   auto* plogp = scored ? reinterpret_cast<double2*>(ws) : nullptr;
   const dim3 grid(plan.slices, N, batch);
+  const ShareShape share = from_logits || scored ? share_shape(batch, N, V, vec) : ShareShape{};
+  if (share.per) {
+    plan.rounds = 1;
+    plan.slices = share.row_rounds;
+  }
+  if (share.per && !share_ready()) return JET_ERR_CUDA;
+  auto scan_shared = [&](auto kernel, double2* sums) {
+    launch_dependent_smem(kernel, dim3((share.total + share.per - 1) / share.per), dim3(kScanThreads), kShareSmem, st, rows, batch_stride,
+                          depth_stride, share, gmax, pairs, sums);
+  };
   auto scan = [&](auto kernel, double2* sums) {
     launch_dependent(kernel, grid, dim3(kScanThreads), st, rows, batch_stride, depth_stride, V, plan.rounds, vec, gmax, pairs, sums);
   };
@@ -878,6 +1105,13 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   if (direct) {
     plan.rounds = 1;
     plan.slices = (V + kRoundChunk - 1) / kRoundChunk;
+  } else if (share.per) {
+    if (from_logits) {
+      scan_shared(row_share_kernel<kScanSum>, pairs);
+      if (scored) scan_shared(row_share_kernel<kScanLogitEntropy>, plogp);
+    } else {
+      scan_shared(row_share_kernel<kScanEntropy>, plogp);
+    }
   } else if (from_logits) {
     scan(row_scan_kernel<kScanSum>, pairs);
     if (scored) scan(row_scan_kernel<kScanLogitEntropy>, plogp);
@@ -886,7 +1120,7 @@ jet_status tree_build_launch(const float* rows, int64_t batch_stride, int64_t de
   } else {
     scan(row_scan_kernel<kScanMax>, nullptr);
   }
-  const ScanView view{rows, batch_stride, depth_stride, gmax, pairs, plogp, plan.slices, plan.rounds, vec ? 1 : 0};
+  const ScanView view{rows, batch_stride, depth_stride, gmax, pairs, plogp, plan.slices, plan.rounds, vec ? 1 : 0, share};
   const bool wide = Wc > kFewWidth || plan.slices * 32 * plan.rounds > kQuads * 128;
   auto pick = [&](auto narrow_form, auto wide_form) { return wide ? wide_form : narrow_form; };
   auto expand = direct ? pick(tree_expand_kernel<0, true, false>, tree_expand_kernel<0, true, true>)
