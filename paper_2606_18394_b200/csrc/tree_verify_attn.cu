@@ -18,8 +18,9 @@
 //                 accumulator against a reference fixed after the first tile; if a row overflows that
 //                 reference the CTA repeats the key range in the classic form (own accumulator and
 //                 running maximum per stream, accumulator rescaled when the maximum rises).  With two
-//                 query tiles per CTA each warpgroup owns a tile with the classic bookkeeping, and the
-//                 tiles take turns on one score buffer.  See "the key loop" below.
+//                 query tiles per CTA each warpgroup owns a tile and its accumulator, the reference is fixed
+//                 likewise (and may rise in a repeat), and the tiles take turns on one score buffer.  See "the key
+//                 loop" below.
 //   key slices  = when there are fewer work items than SMs the key range is cut into `nsplit`
 //                 slices.  After the key loop every CTA stages its normalised rows (bf16) and their
 //                 log-sum-exp; the rows' owner CTAs collect them -- by loads from their peers' shared
@@ -136,6 +137,8 @@ struct Cfg {
   __device__ static constexpr int s_buf(int mt, int t) { return t & 1; }
   __device__ static constexpr int s_use(int t) { return t >> 1; }
   static constexpr bool kTurns = MT == 2;
+  // arrivals of a softmax warpgroup: one per warp with two query tiles (1 % of the launch), one per thread otherwise (no difference)
+  static constexpr int kWgArrivals = kTurns ? 4 : 128;
   __device__ static constexpr uint32_t turn_o(int mt) { return mt * 128; }
   __device__ static constexpr uint32_t turn_s() { return 256; }
   __device__ static constexpr uint32_t turn_p(int mt) { return 384 + mt * 64; }
@@ -247,12 +250,11 @@ __device__ __forceinline__ void mask_chunk(uint32_t (&x)[32], uint32_t bits) {
 }
 
 // 32 scores of one row -> probabilities (exp2 of the scaled, shifted score; a score of -inf gives exactly
-// 0), added to the row sum and written as packed bf16 pairs to 16 TMEM columns of the row's lane (the A
+// 0), added to the row sum and packed as bf16 pairs: 16 TMEM columns of the row's lane (the A
 // operand of the P V product).  The stages are kept apart so that the 32 independent exp2 are in flight
 // together.  The scale-and-shift and the row sum take two values per instruction (fma.rn.f32x2 /
 // add.rn.f32x2: the same roundings as the scalar forms, half the issue slots); sum[j & 3] collects column j.
-__device__ __forceinline__ void exp_chunk(const uint32_t (&x)[32], float sl2, float m_ref, float (&sum)[4],
-                                          uint32_t p_tmem) {
+__device__ __forceinline__ void exp_pack(const uint32_t (&x)[32], float sl2, float m_ref, float (&sum)[4], uint32_t (&packed)[16]) {
   using u64 = unsigned long long;
   auto pk2 = [](uint32_t lo, uint32_t hi) { u64 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi)); return r; };
   const u64 s2 = pk2(__float_as_uint(sl2), __float_as_uint(sl2));
@@ -275,9 +277,12 @@ __device__ __forceinline__ void exp_chunk(const uint32_t (&x)[32], float sl2, fl
   }
   asm("mov.b64 {%0, %1}, %2;" : "=f"(sum[0]), "=f"(sum[1]) : "l"(acc0));
   asm("mov.b64 {%0, %1}, %2;" : "=f"(sum[2]), "=f"(sum[3]) : "l"(acc1));
-  uint32_t packed[16];
 #pragma unroll
   for (int j = 0; j < 16; ++j) packed[j] = pack_bf16(e[2 * j], e[2 * j + 1]);
+}
+__device__ __forceinline__ void exp_chunk(const uint32_t (&x)[32], float sl2, float m_ref, float (&sum)[4], uint32_t p_tmem) {
+  uint32_t packed[16];
+  exp_pack(x, sl2, m_ref, sum, packed);
   ptx::tmem_st16(p_tmem, packed);
 }
 
@@ -372,7 +377,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if (lane < Bars::kCount) {
       uint32_t count = 1;
       if (lane >= Bars::kKvEmpty && lane < Bars::kSFull) count = (MT == 1 || C::kTurns) ? 1 : n_mt;   // arrivals per stage
-      else if (lane >= Bars::kSFree && lane < Bars::kODone) count = 128;                // kSFree, kPFull: a softmax warpgroup
+      else if (lane >= Bars::kSFree && lane < Bars::kODone) count = C::kWgArrivals;                     // kSFree, kPFull: a softmax warpgroup
       ptx::mbar_init(bar(lane), count);
       // slice merge: every slice sends this CTA its block of rows of query tile (lane - kRecv)
       if (S > 1 && lane >= Bars::kRecv && lane < Bars::kRecv + MT)
@@ -926,7 +931,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       }
       for (int i = 0; i < 2; ++i) {
         ptx::mbar_init(lbar(Bars::kSFull + i), 1);
-        ptx::mbar_init(lbar(Bars::kPFull + i), 128);
+        ptx::mbar_init(lbar(Bars::kSFree + i), C::kWgArrivals);
+        ptx::mbar_init(lbar(Bars::kPFull + i), C::kWgArrivals);
         ptx::mbar_init(lbar(Bars::kODone + i), 1);
       }
       ptx::fence_mbar_init();
@@ -1329,17 +1335,20 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 
     if constexpr (C::kTurns) {
       // =========================================================== two query tiles per CTA
-      // Each query tile (stream) keeps the classic bookkeeping -- own accumulator, running reference, rescale
-      // when it rises -- but the two tiles take turns on ONE score buffer, which leaves TMEM columns for a P
-      // buffer per tile: a thread releases the score buffer as soon as it has read its row, the other tile's
-      // Q K^T (warp 1) follows at once, and the P V products (warp 3) read P from buffers of their own.  The
-      // chain softmax -> P V -> Q K^T -> softmax of the classic form is gone.
+      // Each query tile (stream) has its own accumulator and reference, but the two tiles take turns on ONE score
+      // buffer, which leaves TMEM columns for a P buffer per tile: a thread releases the score buffer as soon as it has
+      // read its row, the other tile's Q K^T (warp 1) follows at once, and the P V products (warp 3) read P from buffers
+      // of their own.  The chain softmax -> P V -> Q K^T -> softmax of the classic form is gone.  Two passes: the first
+      // against a fixed reference; the second, if a row could not hold it, with the classic bookkeeping (the reference rises, O
+      // is rescaled) on a second set of barriers.
       classic = false;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
       if (has_work) {
         if (warp == 0) {
-          produce(0, std::integral_constant<int, 0>{}, n_early);            // K tiles
+          produce(0, std::integral_constant<int, 0>{}, pass == 0 ? n_early : 0);            // K tiles
         } else if (warp == 2) {
-          produce(0, std::integral_constant<int, 1>{}, n_early);            // V tiles (a paged tile is 16 small copies: two warps request them)
+          produce(0, std::integral_constant<int, 1>{}, pass == 0 ? n_early : 0);            // V tiles (a paged tile is 16 small copies: two warps request them)
         } else if (warp == 1) {
           bool ok = bounded_wait(bar(Bars::kQFull), 0, abort_flag, 4);
           int prev_mt = -1, prev_tl = 0;
@@ -1347,12 +1356,12 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           for (int tl = 0; tl < T && ok; ++tl) {
             const int2 pos = k_pos_split(tl);
             const int stage = pos.x;
-            ok = bounded_wait(bar(Bars::kKvFull + stage), pos.y, abort_flag, 5);
+            ok = bounded_wait(lbar(Bars::kKvFull + stage), pos.y, abort_flag, 5);
             if (!ok) break;
             const uint64_t desc_k = desc_k0 + static_cast<uint64_t>((stage * C::kStageBytes) >> 4);
             for (int mt = 0; mt < n_mt && ok; ++mt) {
               if (prev_mt >= 0) {       // the warpgroup that used the score buffer before has read its scores
-                ok = bounded_wait(bar(Bars::kSFree + prev_mt), prev_tl & 1, abort_flag, 20);
+                ok = bounded_wait(lbar(Bars::kSFree + prev_mt), prev_tl & 1, abort_flag, 20);
                 if (!ok) break;
               }
               ptx::tc_fence_after();
@@ -1364,8 +1373,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                   const uint64_t off = static_cast<uint64_t>(((kd / 4) * kHalfBytes + (kd % 4) * 32) >> 4);
                   ptx::umma_ss(s_tmem, desc_q + off, desc_k + off, idesc_qk, kd > 0 ? 1u : 0u);
                 }
-                ptx::umma_commit(bar(Bars::kSFull + mt));
-                if (mt == n_mt - 1) ptx::umma_commit(bar(Bars::kKvEmpty + stage));    // K tile read
+                ptx::umma_commit(lbar(Bars::kSFull + mt));
+                if (mt == n_mt - 1) ptx::umma_commit(lbar(Bars::kKvEmpty + stage));    // K tile read
               }
               prev_mt = mt;
               prev_tl = tl;
@@ -1377,11 +1386,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           for (int tl = 0; tl < T && ok; ++tl) {
             const int2 pos = v_pos_split(tl);
             const int stage = pos.x;
-            ok = bounded_wait(bar(Bars::kKvFull + stage), pos.y, abort_flag, 7);
+            ok = bounded_wait(lbar(Bars::kKvFull + stage), pos.y, abort_flag, 7);
             if (!ok) break;
             const uint64_t desc_v = desc_v0 + static_cast<uint64_t>((stage * C::kStageBytes) >> 4);
             for (int mt = 0; mt < n_mt && ok; ++mt) {
-              ok = bounded_wait(bar(Bars::kPFull + mt), tl & 1, abort_flag, 8);
+              ok = bounded_wait(lbar(Bars::kPFull + mt), tl & 1, abort_flag, 8);
               if (!ok) break;
               ptx::tc_fence_after();
               const uint32_t p_tmem = tmem_base + C::turn_p(mt);
@@ -1391,12 +1400,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 for (int kk = 0; kk < kBN / 16; ++kk)
                   ptx::umma_ts(o_tmem, p_tmem + kk * 8, desc_v + static_cast<uint64_t>((kk * 2048) >> 4), idesc_pv,
                                (tl == 0 && kk == 0) ? 0u : 1u);
-                ptx::umma_commit(bar(Bars::kODone + mt));
-                if (mt == n_mt - 1) ptx::umma_commit(bar(Bars::kKvEmpty + stage));    // V tile read
+                ptx::umma_commit(lbar(Bars::kODone + mt));
+                if (mt == n_mt - 1) ptx::umma_commit(lbar(Bars::kKvEmpty + stage));    // V tile read
               }
             }
           }
         }
+      }
+      ptx::cta_sync();                                  // every role has left the pass
+      if (pass == 1 || *redo_flag == 0u || *abort_flag != 0u) break;
+      second_barrier_set();
       }
     }
 
@@ -1784,10 +1797,19 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     if constexpr (C::kTurns) {
       classic = false;
       if (has_work && wg < n_mt) {
-        // =========================================================== softmax, one query tile of two
+        // =========================================================== softmax, one query tile of two: fixed reference
+        // As in the shared-accumulator form the row's reference is its maximum over the first key tile, and a row that passes
+        // kSharedSumLimit (or may have lost its keys to underflow) has the CTA repeat its key range, below.  So a thread needs its
+        // scores only once, and its probabilities (64 registers) wait for the P V product of the tile before to leave the P buffer;
+        // while the exponentials themselves waited for it, the chain  exponentials -> P V -> exponentials  was what a key tile
+        // took: 3270 cycles for both query tiles, 2860 now (2048 of tensor work).  Bound: the one score buffer, which each query
+        // tile's Q K^T has to wait for, and L2 -> SM.  Per layer, sustained: 8 sequences of 24001 - 32768 keys, 128 nodes, 32 / 4 heads, two
+        // slices 463 -> 442 us; 32 paged sequences of 1024 - 8192 keys, 64 nodes, 32 / 8 heads 185 -> 183 (power; burst 158 -> 153.5).
+        // (Two or three chunks held instead of four: 2 - 3 % slower; the scores in loads of 64 or 128 columns: 3 - 8 %.)
         bool ok = true;
+        bool saw_key = false;
+        float m_ref = 0.0f;
         const uint32_t tS = t_lane + C::turn_s();
-        const uint32_t tO = t_lane + C::turn_o(mt);
         const uint32_t tP = t_lane + C::turn_p(mt);
         int last_tl = -1;
 #pragma unroll 1
@@ -1800,13 +1822,97 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           uint32_t xa[32], xb[32], xc[32], xd[32];
           uint32_t b0 = 0xFFFFFFFFu, b1 = 0xFFFFFFFFu, b2 = 0xFFFFFFFFu, b3 = 0xFFFFFFFFu;
           if (!full_tile) { b0 = chunk_bits(t, 0); b1 = chunk_bits(t, 1); b2 = chunk_bits(t, 2); b3 = chunk_bits(t, 3); }
+          saw_key = saw_key || (b0 | b1 | b2 | b3) != 0u;
           ptx::tmem_ld32(tS, xa);
           ptx::tmem_ld32(tS + 32, xb);
           ptx::tmem_ld32(tS + 64, xc);
           ptx::tmem_ld32(tS + 96, xd);
           ptx::tmem_wait_ld();
           ptx::tc_fence_before();
-          ptx::mbar_arrive(bar(Bars::kSFree + mt));            // the scores are in registers: the other tile's turn
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar(Bars::kSFree + mt));            // the scores are in registers: the other tile's turn
+          if (!full_tile) {
+            mask_chunk(xa, b0);
+            mask_chunk(xb, b1);
+            mask_chunk(xc, b2);
+            mask_chunk(xd, b3);
+          }
+          if (tl == 0) {
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            max_chunk(xa, mx);
+            max_chunk(xb, mx);
+            max_chunk(xc, mx);
+            max_chunk(xd, mx);
+            const float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            m_used = (m == -INFINITY) ? -0.0f : m;        // -0.0 marks "no reference of its own" (same arithmetic as 0)
+            m_ref = m_used * sl2;
+          }
+          float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          uint32_t pa[16], pb[16], pc[16], pd[16];
+          exp_pack(xa, sl2, m_ref, sum, pa);
+          exp_pack(xb, sl2, m_ref, sum, pb);
+          exp_pack(xc, sl2, m_ref, sum, pc);
+          exp_pack(xd, sl2, m_ref, sum, pd);
+          if (tl > 0) {
+            // the P V product of the tile before has read the P buffer
+            ok = bounded_wait(bar(Bars::kODone + mt), (tl - 1) & 1, abort_flag, 21);
+            if (!ok) break;
+          }
+          ptx::tmem_st16(tP, pa);
+          ptx::tmem_st16(tP + 16, pb);
+          ptx::tmem_st16(tP + 32, pc);
+          ptx::tmem_st16(tP + 48, pd);
+          const float tile_sum = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+          if (row_live && !(tile_sum <= kSharedSumLimit)) *redo_flag = 1u;
+          l += tile_sum;
+          if (!full_tile) {
+            ok = clear_v_tail(t, v_pos_split(tl));
+            if (!ok) break;
+          }
+          ptx::tmem_wait_st();                     // P is in TMEM
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar(Bars::kPFull + mt));
+          last_tl = tl;
+        }
+        if (row_live && saw_key && __float_as_uint(m_used) == 0x80000000u && !(l >= kSharedSumFloor)) *redo_flag = 1u;
+        if (ok && last_tl >= 0) ok = bounded_wait(bar(Bars::kODone + mt), last_tl & 1, abort_flag, 11);
+        if (ok) ptx::tc_fence_after();
+        row_ok = ok;
+      }
+      ptx::cta_sync();                                  // every role has left the pass
+      const bool again = *redo_flag != 0u && *abort_flag == 0u;
+      if (again) {
+        second_barrier_set();
+        m_used = -INFINITY;
+        l = 0.0f;
+        row_ok = has_work;
+      }
+      if (again && has_work && wg < n_mt) {
+        // ----------------------------------------------------------- the same with a reference that may rise
+        bool ok = true;
+        const uint32_t tS = t_lane + C::turn_s();
+        const uint32_t tO = t_lane + C::turn_o(mt);
+        const uint32_t tP = t_lane + C::turn_p(mt);
+        int last_tl = -1;
+#pragma unroll 1
+        for (int tl = 0; tl < T && ok; ++tl) {
+          const int t = t_lo + tl;
+          const bool full_tile = t < TP && (L - t * kBN) >= kBN;      // uniform: every key visible to every row
+          ok = bounded_wait(lbar(Bars::kSFull + mt), tl & 1, abort_flag, 9);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          uint32_t xa[32], xb[32], xc[32], xd[32];
+          uint32_t b0 = 0xFFFFFFFFu, b1 = 0xFFFFFFFFu, b2 = 0xFFFFFFFFu, b3 = 0xFFFFFFFFu;
+          if (!full_tile) { b0 = chunk_bits(t, 0); b1 = chunk_bits(t, 1); b2 = chunk_bits(t, 2); b3 = chunk_bits(t, 3); }
+          ptx::tmem_ld32(tS, xa);
+          ptx::tmem_ld32(tS + 32, xb);
+          ptx::tmem_ld32(tS + 64, xc);
+          ptx::tmem_ld32(tS + 96, xd);
+          ptx::tmem_wait_ld();
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(lbar(Bars::kSFree + mt));            // the scores are in registers: the other tile's turn
           if (!full_tile) {
             mask_chunk(xa, b0);
             mask_chunk(xb, b1);
@@ -1826,7 +1932,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
           if (tl >= 1) {
             // the P V product of the tile before is complete: the P buffer is free and O may be rescaled
-            ok = bounded_wait(bar(Bars::kODone + mt), (tl - 1) & 1, abort_flag, 21);
+            ok = bounded_wait(lbar(Bars::kODone + mt), (tl - 1) & 1, abort_flag, 21);
             if (!ok) break;
             ptx::tc_fence_after();
           }
@@ -1875,14 +1981,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           }
           ptx::tmem_wait_st();                     // P (and a rescaled O) are in TMEM
           ptx::tc_fence_before();
-          ptx::mbar_arrive(bar(Bars::kPFull + mt));
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(lbar(Bars::kPFull + mt));
           last_tl = tl;
         }
         // O is complete once the last P V of this accumulator has been committed
-        if (ok && last_tl >= 0) ok = bounded_wait(bar(Bars::kODone + mt), last_tl & 1, abort_flag, 11);
+        if (ok && last_tl >= 0) ok = bounded_wait(lbar(Bars::kODone + mt), last_tl & 1, abort_flag, 11);
         if (ok) ptx::tc_fence_after();
         row_ok = ok;
       }
+      if (again) ptx::cta_sync();
     }
 
     if (!kPair && !C::kTurns && classic && has_work && (MT == 1 || wg < n_mt)) {
