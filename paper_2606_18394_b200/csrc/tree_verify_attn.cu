@@ -81,6 +81,7 @@ struct AttnParams {
   int npt;            // 128 / G: nodes per query tile
   uint32_t magic_S, magic_G;
   int len_hint;       // the caller's bound on the cached keys (max_seq_len); 0 = none
+  int paced;          // two query tiles: a warpgroup waits for its P V before it exponentiates (see the key loop)
   uint32_t poll_limit;  // workspace merge: polls of the arrival count before the CTA gives up (about a second)
   int stable;         // JET_ATTN_STABLE_PREFIX: lengths, page table and prefix rows may be read before the dependency wait
   int via_global;     // key slices exchange their rows through the workspace instead of a cluster: 1 = inside this
@@ -154,6 +155,12 @@ struct Cfg {
   static constexpr int kBlockBytes = kBM * kRecvPitch;                   // the 128 staged rows of one stream
   static constexpr int kStageOff = 0;
   static constexpr int kRecvOff = (kBlockBytes + 1023) / 1024 * 1024;
+  // Two query tiles per CTA, slices in a cluster: the rows stay in fp32.  These plans take the place of plans without slices, whose
+  // rows are rounded once, and their launches are long: the exchange of twice the bytes is 0.3 % of them.
+  static constexpr bool kWideRows = MT == 2;
+  static constexpr int kWidePitch = D * 4 + 16;
+  static constexpr int kWideRecvOff = (kBM * kWidePitch + 1023) / 1024 * 1024;
+  static_assert(!kWideRows || kWideRecvOff + (kBM + kMaxSplit) * kWidePitch + 4096 <= kTileBytes, "fp32 merge buffers must fit in the tile memory");
   static_assert(kRecvOff + (kBM + kMaxSplit) * kRecvPitch + 4096 <= kTileBytes, "merge buffers must fit in the tile memory");
 };
 
@@ -696,7 +703,8 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
          }
         }
       } else if (kSm && e_wg == mt) {
-        uint8_t* dst = stage + e_r * C::kRecvPitch;
+        const bool wide = C::kWideRows && via_cluster;
+        uint8_t* dst = stage + e_r * (wide ? C::kWidePitch : C::kRecvPitch);
 #pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
@@ -706,16 +714,22 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           }
 #pragma unroll
           for (int q8 = 0; q8 < 4; ++q8) {
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
+            float w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
             if (active) {
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                w[k] = pack_bf16(__uint_as_float(o[q8 * 8 + 2 * k]) * own_inv, __uint_as_float(o[q8 * 8 + 2 * k + 1]) * own_inv);
+              for (int k = 0; k < 8; ++k) w[k] = __uint_as_float(o[q8 * 8 + k]) * own_inv;
             }
-            *reinterpret_cast<uint4*>(dst + (c * 32 + q8 * 8) * 2) = make_uint4(w[0], w[1], w[2], w[3]);
+            if (wide) {
+              float4* d4 = reinterpret_cast<float4*>(dst + (c * 32 + q8 * 8) * 4);
+              d4[0] = make_float4(w[0], w[1], w[2], w[3]);
+              d4[1] = make_float4(w[4], w[5], w[6], w[7]);
+            } else {
+              *reinterpret_cast<uint4*>(dst + (c * 32 + q8 * 8) * 2) =
+                  make_uint4(pack_bf16(w[0], w[1]), pack_bf16(w[2], w[3]), pack_bf16(w[4], w[5]), pack_bf16(w[6], w[7]));
+            }
           }
         }
-        *reinterpret_cast<float*>(dst + D * 2) = own_lse2;
+        *reinterpret_cast<float*>(dst + D * (wide ? 4 : 2)) = own_lse2;
       }
       if (via_cluster) {
         // The slices of the work item form a thread-block cluster: once every CTA has staged its rows (the
@@ -731,24 +745,29 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         if constexpr (kSm) {
           // gather: 16-byte chunk e of this CTA's row block, from slice c, for every (e, c) pair of the thread --
           // at most 16 pairs (fewer slices mean more rows per CTA and the other way round)
-          constexpr int kChunksPerRow = C::kRecvPitch / 16;
+          // (fp32 rows: in two or three rounds of 16)
+          constexpr int kPitch = C::kWideRows ? C::kWidePitch : C::kRecvPitch;
+          constexpr int kChunksPerRow = kPitch / 16;
           const int per_slice = own_n * kChunksPerRow;
           const int pairs = ((per_slice + 255) / 256) * S;
-          const uint32_t local = smem_base + C::kStageOff + static_cast<uint32_t>(own_lo * C::kRecvPitch);
-          uint8_t* recv = smem_gen + C::kRecvOff;
-          uint4 got[16];
+          const uint32_t local = smem_base + C::kStageOff + static_cast<uint32_t>(own_lo * kPitch);
+          uint8_t* recv = smem_gen + (C::kWideRows ? C::kWideRecvOff : C::kRecvOff);
+#pragma unroll 1
+          for (int q0 = 0; q0 < (C::kWideRows ? pairs : 1); q0 += 16) {
+            uint4 got[16];
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            const int j = static_cast<int>(udiv(static_cast<uint32_t>(q), p.magic_S)), c = q - j * S;
-            const int e = tid - 128 + 256 * j;
-            if (q < pairs && e < per_slice) got[q] = ptx::ld_cluster_v4(ptx::map_to_rank(local + static_cast<uint32_t>(e * 16), c));
-          }
+            for (int q = 0; q < 16; ++q) {
+              const int j = static_cast<int>(udiv(static_cast<uint32_t>(q0 + q), p.magic_S)), c = q0 + q - j * S;
+              const int e = tid - 128 + 256 * j;
+              if (q0 + q < pairs && e < per_slice) got[q] = ptx::ld_cluster_v4(ptx::map_to_rank(local + static_cast<uint32_t>(e * 16), c));
+            }
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
-            const int j = static_cast<int>(udiv(static_cast<uint32_t>(q), p.magic_S)), c = q - j * S;
-            const int e = tid - 128 + 256 * j;
-            if (q < pairs && e < per_slice)
-              *reinterpret_cast<uint4*>(recv + static_cast<size_t>(c) * rows_per * C::kRecvPitch + e * 16) = got[q];
+            for (int q = 0; q < 16; ++q) {
+              const int j = static_cast<int>(udiv(static_cast<uint32_t>(q0 + q), p.magic_S)), c = q0 + q - j * S;
+              const int e = tid - 128 + 256 * j;
+              if (q0 + q < pairs && e < per_slice)
+                *reinterpret_cast<uint4*>(recv + static_cast<size_t>(c) * rows_per * kPitch + e * 16) = got[q];
+            }
           }
           ptx::named_sync(2, 256);
         }
@@ -756,7 +775,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       } else {
         ptx::cta_sync();
       }
-      [[maybe_unused]] const uint8_t* src_rows = via_cluster ? smem_gen + C::kRecvOff : stage;         // S == 1: the staged rows themselves
+      [[maybe_unused]] const uint8_t* src_rows = via_cluster ? smem_gen + (C::kWideRows ? C::kWideRecvOff : C::kRecvOff) : stage;         // S == 1: the staged rows themselves
       bool rows_ok = merge_ok;
       if (kTwo || (S > 1 && !via_cluster)) {
         // Exchange through the workspace: publish this CTA's staged rows, count the slices of the unit
@@ -808,7 +827,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           __threadfence();
         }
       }
-      const uint32_t src_stride = rows_per * C::kRecvPitch;     // distance between the blocks of consecutive slices
+      [[maybe_unused]] const bool wide = C::kWideRows && via_cluster;
+      [[maybe_unused]] const uint32_t src_pitch = wide ? C::kWidePitch : C::kRecvPitch;
+      [[maybe_unused]] const uint32_t src_stride = rows_per * src_pitch;     // distance between the blocks of consecutive slices
       // The softmax warpgroups combine the blocks: one item = 8 output values of one row.  A thread first issues
       // every load of its item (the S log-sum-exps of the row and its 16 bytes of every slice), then forms the
       // softmax weights of the slice sums and the weighted sum -- one round trip to shared memory, no chain of
@@ -822,7 +843,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           const int vq = static_cast<int>(udiv(R, p.magic_G));
           const int v = node_lo + vq, h = g * G + (R - vq * G);
           if (v >= p.B) continue;
-          const uint8_t* src = src_rows + rl * C::kRecvPitch;
+          const uint8_t* src = src_rows + rl * src_pitch;
           float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
           float lse2 = -INFINITY;
           if (S == 1) {
@@ -837,6 +858,29 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 acc[2 * q + 1] = __uint_as_float(v4[q] & 0xFFFF0000u);
               }
               lse2 = lc;
+            }
+          } else if (wide) {
+            float mx = -INFINITY, wsum = 0.0f;
+#pragma unroll 1
+            for (int c = 0; c < S; ++c) mx = fmaxf(mx, *reinterpret_cast<const float*>(src + c * src_stride + D * 4));
+            if (v < n && mx > -INFINITY) {
+#pragma unroll 1
+              for (int c = 0; c < S; ++c) {
+                const float lc = *reinterpret_cast<const float*>(src + c * src_stride + D * 4);
+                const float4* x4 = reinterpret_cast<const float4*>(src + c * src_stride + c8 * 32);
+                const float4 x0 = x4[0], x1 = x4[1];
+                // (absent slices get weight 0, and whatever their rows hold is not used)
+                if (lc > -INFINITY) {
+                  const float w = exp2f(lc - mx);
+                  wsum += w;
+                  acc[0] += w * x0.x; acc[1] += w * x0.y; acc[2] += w * x0.z; acc[3] += w * x0.w;
+                  acc[4] += w * x1.x; acc[5] += w * x1.y; acc[6] += w * x1.z; acc[7] += w * x1.w;
+                }
+              }
+              const float inv = 1.0f / wsum;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) acc[k] *= inv;
+              lse2 = mx + log2f(wsum);
             }
           } else {
             // (four slices at a time: their loads are issued together, then used)
@@ -1806,6 +1850,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         // tile's Q K^T has to wait for, and L2 -> SM.  Per layer, sustained: 8 sequences of 24001 - 32768 keys, 128 nodes, 32 / 4 heads, two
         // slices 463 -> 442 us; 32 paged sequences of 1024 - 8192 keys, 64 nodes, 32 / 8 heads 185 -> 183 (power; burst 158 -> 153.5).
         // (Two or three chunks held instead of four: 2 - 3 % slower; the scores in loads of 64 or 128 columns: 3 - 8 %.)
+        // p.paced keeps the wait in front of the exponentials: where every CTA of a single wave streams keys of its own out of HBM (17
+        // paged sequences of 10698 - 14988 keys, 64 nodes: burst 242 against 231.5 us, sustained equal; 3 of 13291 - 25232, 34 nodes,
+        // six slices: 74.5 against 68.8, sustained 82.7 against 79.7) memory is the bound, and evenly spaced requests suit it better.
         bool ok = true;
         bool saw_key = false;
         float m_ref = 0.0f;
@@ -1848,12 +1895,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             m_ref = m_used * sl2;
           }
           float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          if (p.paced && tl > 0) {
+            ok = bounded_wait(bar(Bars::kODone + mt), (tl - 1) & 1, abort_flag, 21);
+            if (!ok) break;
+          }
           uint32_t pa[16], pb[16], pc[16], pd[16];
           exp_pack(xa, sl2, m_ref, sum, pa);
           exp_pack(xb, sl2, m_ref, sum, pb);
           exp_pack(xc, sl2, m_ref, sum, pc);
           exp_pack(xd, sl2, m_ref, sum, pd);
-          if (tl > 0) {
+          if (!p.paced && tl > 0) {
             // the P V product of the tile before has read the P buffer
             ok = bounded_wait(bar(Bars::kODone + mt), (tl - 1) & 1, abort_flag, 21);
             if (!ok) break;
@@ -2363,7 +2414,7 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // Picks the query-tile grouping, the number of key slices and the form of their merge with a cost model, in microseconds
 // of a launch in the steady state of a layer stack:
 //   key tile of a CTA      0.78 + 0.14 f, f = CTAs / SMs (shared L2 and power);
-//                          1.65 (second launch) or 1.75 with two query tiles (two softmax chains share a tensor core)
+//                          1.5 (second launch) or 2.2 (cluster: two rounds of fp32 rows) with two query tiles
 //   fixed, no slices       5.2 + 2.4 f
 //   slices in a cluster    5.7 with four, 6.0 with eight, 7.0 with an odd number, else 6.4, + 2.4 f.  (Four and eight: the
 //                          shape of the row exchange is a power of two.)  Clusters of up to eight CTAs are
@@ -2371,7 +2422,7 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 //   a second launch merges 5.9 + 2.2 f, + 0.5 with the large merge CTAs, + 0.4 when two CTAs have to share a TPC, + 0.7 and 2.0 with
 //                          more than 10 and 12 slices (longer merge code); never below the 4 us of host time that each
 //                          launch costs a caller who issues layer by layer
-// all of the fixed part 1.45 or 1.6 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
+// all of the fixed part 1.35 or 2 times with two query tiles (two merge rounds), and the CTAs run in waves of what the device holds
 // at once.  There is no term for what HBM delivers: where it binds it binds every form alike, and the host knows only the
 // longest sequence.  (A term that charged 1.45 f / g per tile as if all sequences had that length kept ragged batches on
 // fewer slices: three sequences of 4548 - 19896 keys, 15 nodes, 32 / 8 heads, paged: 52.4 us with four slices of 24 work items
@@ -2380,25 +2431,32 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // (budgets 4 - 512, prefixes 64 - 100000, D 64 and 128, contiguous and paged, lengths of a batch spread from 20 to 100 % of
 // the longest): the plans chosen take 1.9 % more than the best form of each shape on average, more than 5 % at 139 of them,
 // 31 % at worst; with the HBM term 2.5 %, 182, 38 %.
-// Beyond it -- more than four sequences or 64 query tiles -- the unit is a key tile out of L2 (0.8 us), a tile costs
-// 1 + 0.75 / g (g = CTAs that read the same tile side by side) and the fixed parts are 6 / 8 / 10 (none, cluster, second
-// launch): with few CTAs per K/V tile this prefers more, shorter CTAs, which even out sequences of different lengths
-// (11 sequences of 13162 - 30066 keys, 13 nodes: three slices in two waves 76 us per layer faster than none in one).  There the
-// plans take 4.2 % more than the best form on average (735 shapes), and waves are whole numbers, so that two forms whose
-// costs are a per cent apart change places by chance.
+// Beyond it -- more than four sequences or 64 query tiles -- the unit is a key tile out of L2 (0.8 us): a tile costs
+// 1 + 0.75 / g (g = CTAs that read the same tile side by side) or 1.7 with two query tiles, the fixed parts are 6 / 8 / 10 (none, cluster,
+// second launch), with two query tiles 9.8 / 15.6 / 16.3; and as the lengths of a batch differ, half of the waves count as
+// they are, not as whole ones.  With two query tiles at 1.7 instead of 2.2 (what a key tile took while the exponentials waited
+// for the P V product before) they are the better form of most long shapes: a K/V tile is read from L2 once for 256 rows.
+// Measured against up to 17 forms of 120 shapes (batches 1 - 32, budgets 10 - 512 of more than 128 rows, prefixes 400 - 32768, ragged, D 64
+// and 128, half of them paged; this range and the other together): the plans chosen take 1.6 % more than the best form on average (4.8 % with the
+// figures before), and 3.7 % less than the launches before.  E.g., us per layer, sustained, before and now: 8 sequences of 24001 - 32768 keys, 128
+// nodes, 32 / 4 heads 474 -> 440 (no slices of one query tile -> two of two); one of 32768, 512 nodes, 32 / 4 heads 260 -> 246; 4 paged
+// ones of 5000 - 8000, 100 nodes, 32 / 8 heads 81 -> 68; one of 16384, 256 nodes, 32 / 8 heads 74 -> 72, paged 88 -> 75 (one query tile per CTA
+// doubles the copies of 16 rows that a paged cache comes in).
 // Not planned, only run where they are asked for: CTA pairs (JET_FORCE_PAIR=1), which need 1.22 times the key-tile time (the
 // hand-overs cross two SMs), and the exchange inside one launch through the workspace (JET_FORCE_SPLIT="<slices>,g"; arrival
 // counters, bounded spin, all CTAs resident at once).  Against a second launch that is 0.2 - 2 us slower at D 128 up to
 // 9000 keys (32 / 8 heads, prefix 4096: 64 nodes 12.5 against 11.8 us, 16 nodes 12.3 against 10.7), within 2 % of it for long
 // sequences, and 0.2 - 0.8 us (2 - 6 %) faster at D 64 or with 18 slices of two query tiles: not enough for kernels that wait
 // for one another.
-double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
+double plan_cost(bool fitted, int batch, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
   if (!fitted) {
-    const double shared = 1.0 + 0.75 / n_mgroups, per_tile = mt == 1 ? shared : (shared > 2.2 ? shared : 2.2);
-    return waves * ((tiles + ns - 1) / ns * per_tile + (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) * (mt == 1 ? 1.0 : 1.6));
+    const double per_tile = mt == 1 ? 1.0 + 0.75 / n_mgroups : 1.7;
+    const double fixed = mt == 1 ? (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) : (ns == 1 ? 9.8 : via == 0 ? 15.6 : 16.3);
+    const double whole = ceil(waves), spread = 0.93 * waves + 0.25;
+    return (batch == 1 ? whole : 0.5 * whole + 0.5 * (spread > 1.0 ? spread : 1.0)) * ((tiles + ns - 1) / ns * per_tile + fixed);
   }
   const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
-  const double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.65 : 1.75;
+  const double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.5 : 2.2;
   double fixed, floor = 4.0;
   if (ns == 1) {
     fixed = 5.2 + 2.4 * f;
@@ -2409,7 +2467,7 @@ double plan_cost(bool fitted, int mt, int ns, int via, double waves, int ctas, i
             (ns > 12 ? 2.0 : ns > 10 ? 0.7 : 0.0);
     floor = 8.0;
   }
-  const double cost = waves * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : via == 2 ? 1.45 : 1.6));
+  const double cost = ceil(waves) * ((tiles + ns - 1) / ns * tile + fixed * (mt == 1 ? 1.0 : via == 2 ? 1.35 : 2.0));
   return cost < floor ? floor - 0.01 * (floor - cost) : cost;      // (still in order below the floor)
 }
 
@@ -2442,7 +2500,7 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
     auto consider = [&](int ns, int via_global, double waves, int pair = 0) {
       if (force_ns && (ns != force_ns || (ns > 1 && via_global != force_via))) return;
       if (pair != (force_pair > 0 && pair_ok ? 1 : 0)) return;
-      const double cost = plan_cost(fitted, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
+      const double cost = plan_cost(fitted, batch, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
       if (best_cost < 0.0 || cost < best_cost) {
         best = pl;
         best.nsplit = ns;
@@ -2455,12 +2513,14 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
     for (int ns = 1; ns <= kMaxSplit && ns <= tiles; ++ns) {
       // (a) the slices of a unit form a thread-block cluster and merge through distributed shared memory
       const int resident = ns <= 8 || force_ns ? max_active_clusters_for(D, mt, ns) : 0;
-      if (resident > 0) consider(ns, 0, static_cast<double>((pl.units + resident - 1) / resident));
+      if (resident > 0) consider(ns, 0, static_cast<double>(pl.units) / resident);
       if (pair_ok && ns == 1) consider(1, 0, static_cast<double>((pl.units + sm_count() - 1) / sm_count()), 1);
       // (b) independent CTAs that merge through the workspace: all of them resident at once (a cluster has to fit into
       //     one GPC, which can leave a third of the SMs idle).  With a second small launch that combines the blocks
       //     once the first has ended nothing waits inside a kernel.
-      if (ns > 1 && static_cast<long>(pl.units) * ns <= sm_count() &&
+      // (With two query tiles per CTA only where one would be sliced as well: the rows travel as bf16.)
+      const bool sliced = mt == 1 || force_mt || 2L * batch * Hkv * ((rows + kBM - 1) / kBM) <= sm_count();
+      if (ns > 1 && sliced && static_cast<long>(pl.units) * ns <= sm_count() &&
           static_cast<size_t>(pl.units) * mt * 2 * sizeof(int) <= kCounterBytes) {
         consider(ns, force_via ? force_via : 2, 1.0);
         if (pair_ok) consider(ns, force_via ? force_via : 1, 1.0, 1);
@@ -2729,6 +2789,7 @@ jet_status attn_call(const void* q, const void* k_cache, const void* v_cache, co
   p.magic_G = udiv_magic(static_cast<uint32_t>(G));
   // (measured: a gain of 3-9 % with one query tile per KV head, none to a small loss with two or more)
   p.len_hint = (!pl.pair && !paged && !tail && batch == 1 && pl.n_mgroups == 1 && max_seq_len > 0 && max_seq_len < (1 << 26)) ? max_seq_len : 0;
+  p.paced = D == 128 && pl.n_mgroups == 1 && static_cast<int64_t>(pl.units) * pl.nsplit <= sm_count() ? 1 : 0;
   p.stable = (flags & JET_ATTN_STABLE_PREFIX) ? 1 : 0;
   // Test hook (read once per process): JET_TEST_POLL_LIMIT shortens the bounded spin of the workspace merge so
   // that a test can make it run out within milliseconds.

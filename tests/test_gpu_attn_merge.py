@@ -31,3 +31,15 @@ def test_second_launch_merge(ns):
     r = subprocess.run([sys.executable, "-c", CHILD, str(ns)], env=env, capture_output=True, text=True, timeout=300,
                        cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("ns", ["2", "3", "5", "8"])
+def test_fp32_rows_through_a_cluster(ns):
+    """Two query tiles per CTA: every number of rounds that the exchange of the fp32 rows takes, ragged paged batches and
+    rows without a key in some slice (the random shapes of test_gpu_attn_random_shapes, in a child process: the
+    library reads the forced plan once)."""
+    env = dict(os.environ, JET_FORCE_MT="2", JET_FORCE_SPLIT=ns)
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(here, "test_gpu_attn_random_shapes.py"), "-m", "gpu", "-x", "-q", "-k",
+                        "random_configurations and 1"], env=env, capture_output=True, text=True, cwd=os.path.dirname(here), timeout=600)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
