@@ -347,6 +347,35 @@ def jet_kv_compact_launches(layers, batch, Hkv, D, N, tail=False) -> int:
     return load().jet_kv_compact_launches(layers, batch, Hkv, D, N, int(tail))
 
 
+def kv_compact_step(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table, max_pages, page_size, path,
+                    accept_len, seq_len, layers, batch, B, Hkv, D, N, tail, arrived):
+    """The commit of a step, copying or (tail) in place, in one launch.  arrived: int32 [batch], zero between calls."""
+    st = native().kv_compact_step(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table, max_pages,
+                                  page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N, tail, arrived, None)
+    if st != JET_OK:
+        _check(st, "jet_kv_compact")
+
+
+def accept_commit_launches(mode, layers, batch, B, V, Hkv, D, N, tail) -> int:
+    """Kernels of a step's acceptance ("greedy", "hidden", "sample") and commit."""
+    if mode == "sample":
+        return 3                                      # scan, path, commit
+    return native().accept_commit_launches(mode == "hidden", layers, batch, B, V, Hkv, D, N, tail)
+
+
+def accept_commit_step(rows, row_stride, lm_head, d, token, parent, depth, anc_mask, n_nodes, batch, B, V, N, tgt, accept_len, path,
+                       out_tokens, device_status, workspace, tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride,
+                       page_table, max_pages, page_size, seq_len, layers, Hkv, D, tail, arrived):
+    """Greedy acceptance (lm_head None: rows are logits, else hidden states) and commit of a step, the path selection fused with the
+    copies.  arrived: int32 [batch], zero between calls."""
+    st = native().accept_commit(rows, row_stride, lm_head, d, token, parent, depth, anc_mask, n_nodes, batch, B, V, N, tgt,
+                                accept_len, path, out_tokens, device_status, workspace, None, tree_k, tree_v, k_cache, v_cache,
+                                cache_layer_stride, kv_batch_stride, page_table, max_pages, page_size, seq_len, layers, Hkv, D,
+                                tail, arrived, None)
+    if st != JET_OK:
+        _check(st, "jet_tree_accept and jet_kv_compact")
+
+
 def jet_kv_compact(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,
                    max_pages_per_seq, page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N,
                    stream=None, check=True):

@@ -1,0 +1,188 @@
+// Commit of the accepted path, the device side: how the rows of every accepted node are copied behind the prefix, or moved in
+// place.  Shared by jet_kv_compact / jet_kv_compact_tail (kv_compact.cu) and by the kernel that selects the path itself
+// (tree_accept.cu).
+#pragma once
+#include "jet_common.cuh"
+#include "sm100_ptx.cuh"
+
+// Not part of the C ABI: see kv_compact.cu.
+extern "C" JET_API jet_status jet_internal_kv_compact_step(
+    const void* tree_k, const void* tree_v, void* k_cache, void* v_cache, int64_t cache_layer_stride, int64_t kv_batch_stride,
+    const int32_t* page_table, int max_pages_per_seq, int page_size, const int32_t* path, const int32_t* accept_len, int32_t* seq_len,
+    int layers, int batch, int B, int Hkv, int D, int N, int tail, int32_t* arrived, void* stream);
+
+namespace jet {
+namespace {
+
+// Threads of a CTA; of one that has its sequence to itself.  (With 1024 the copy spills: 52 rows 0.5 us slower.)
+constexpr int kCommitThreads = 256, kCommitThreadsAlone = 512;
+constexpr int kTailHeld = 16;                        // rows a lane of the in-place form has in flight
+
+struct CommitParams {
+  const uint4 *tree_k, *tree_v;                      // (copying form)
+  uint4 *k_cache, *v_cache;
+  int64_t layer_stride16, batch_stride16;            // in 16-byte pieces
+  const int32_t* page_table;
+  const int32_t* path;                               // (not where the kernel selects the path itself)
+  const int32_t* accept_len;
+  int32_t* seq_len;
+  int* arrived;                                      // one count per sequence, 0 between calls, or null: see finish_commit
+  int max_pages, page_size, layers, batch, B, row16, N;
+  int ctas;                                          // per sequence
+};
+
+// The path of sequence b and where its rows lie: node[i] (-1: not to be copied) and the cache row offsets (within a layer) of
+// position seq_len + i and -- in-place layout -- seq_len + node[i].
+struct CommitTable {
+  int64_t dst[JET_MAX_DEPTH + 1], src[JET_MAX_DEPTH + 1];
+  int node[JET_MAX_DEPTH + 1];
+};
+
+// Offset of a cache position of sequence b; -1: outside the page table (a length beyond it is the caller's error).
+__device__ __forceinline__ int64_t cache_row(const CommitParams& p, int b, int64_t pos) {
+  if (pos < 0) return -1;
+  if (!p.page_table) return b * p.batch_stride16 + pos * p.row16;
+  if (pos / p.page_size >= p.max_pages) return -1;
+  const int page = p.page_table[static_cast<size_t>(b) * p.max_pages + pos / p.page_size];
+  return (static_cast<int64_t>(page) * p.page_size + pos % p.page_size) * p.row16;
+}
+
+// Entry i of the table; dst = cache_row of position len + i.
+template <bool kTail>
+__device__ __forceinline__ void commit_entry(const CommitParams& p, int b, int i, int node, int len, int64_t dst, CommitTable& t) {
+  if (node < 0 || node >= p.B) node = -1;
+  const int64_t src = kTail && node >= 0 ? cache_row(p, b, static_cast<int64_t>(len) + node) : 0;
+  t.node[i] = dst < 0 || src < 0 ? -1 : node;
+  t.dst[i] = dst;
+  t.src[i] = src;
+}
+
+// Advances seq_len of sequence b once every CTA of it has its length; behind a CTA-wide barrier that all threads reached with
+// it.  A CTA alone does so at once.  Several count themselves, and the last one to arrive does it and leaves the count at 0 for the next
+// call: no CTA waits for another.  (Without counts a second launch does it: jet_kv_compact has no memory for them.)
+__device__ __forceinline__ void finish_commit(const CommitParams& p, int b, int next_len) {
+  if (threadIdx.x != 0) return;
+  if (p.ctas == 1) {
+    p.seq_len[b] = next_len;
+  } else if (p.arrived && ptx::atom_add_acq_rel_gpu(p.arrived + b, 1) == p.ctas - 1) {
+    p.arrived[b] = 0;
+    p.seq_len[b] = next_len;
+  }
+}
+
+// The rows of entries 0 .. a, by all CTAs of sequence b.  A warp per row, two rows in flight.  Row r: path entry r mod (a + 1) of
+// (layer, K | V) number r / (a + 1).
+__device__ __forceinline__ void copy_rows(const CommitParams& p, int b, int a, const CommitTable& t) {
+  const int lane = threadIdx.x & 31, warps = p.ctas * (blockDim.x >> 5);
+  const int rows = 2 * p.layers * (a + 1);           // (a below 0: none)
+  for (int r0 = (blockIdx.x % p.ctas) * (blockDim.x >> 5) + (threadIdx.x >> 5); r0 < rows; r0 += 2 * warps) {
+    const uint4* src[2];
+    uint4* dst[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int r = r0 + k * warps, lk = r / (a + 1), i = r - lk * (a + 1), layer = lk >> 1;
+      const int node = r < rows ? t.node[i] : -1;
+      src[k] = node < 0 ? nullptr : ((lk & 1) ? p.tree_v : p.tree_k) + ((static_cast<int64_t>(layer) * p.batch + b) * p.B + node) * p.row16;
+      dst[k] = ((lk & 1) ? p.v_cache : p.k_cache) + layer * p.layer_stride16 + t.dst[i];
+    }
+    for (int e0 = 0; e0 < p.row16; e0 += 128) {
+      uint4 x[2][4];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = e0 + j * 32 + lane;
+          if (src[k] && e < p.row16) x[k][j] = __ldg(src[k] + e);
+        }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = e0 + j * 32 + lane;
+          if (src[k] && e < p.row16) dst[k][e] = x[k][j];
+        }
+    }
+  }
+}
+
+// In place: row seq_len + path[i] moves to seq_len + i for i = 1 .. accept_len (path[i] >= i; the root stays where it is).
+// A unit is (layer, K | V, 32 of the row's 16-byte columns); columns do not meet, so a lane's own order is all that
+// counts: it reads kTailHeld rows of a unit into registers before it writes any, and never writes a row that it still has to
+// read, because rows are taken in increasing i and path[i] >= i, path increasing.  With few rows a warp holds several
+// units at once, if there are more units than warps.
+__device__ __forceinline__ void move_rows(const CommitParams& p, int a, const CommitTable& t) {
+  if (a < 1) return;
+  const int lane = threadIdx.x & 31, warp = (blockIdx.x % p.ctas) * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = p.ctas * (blockDim.x >> 5);
+  const int columns = (p.row16 + 31) / 32, units = 2 * p.layers * columns;
+  const int rows = min(a, kTailHeld);                // of a unit that are held at once
+  const int per = max(1, min(kTailHeld / rows, (units + warps - 1) / warps));
+  for (int first = warp * per; first < units; first += warps * per) {
+    const int lk0 = first / columns, column0 = first - lk0 * columns;
+    for (int i0 = 1; i0 <= a; i0 += kTailHeld) {     // (one pass unless per is 1)
+      auto each = [&](auto&& piece) {
+        int lk = lk0, column = column0, i = i0;
+#pragma unroll
+        for (int k = 0; k < kTailHeld; ++k) {
+          if (k >= rows * per || lk >= 2 * p.layers || i > a) break;      // (warp-uniform)
+          const int e = column * 32 + lane;
+          if (t.node[i] >= 0 && t.node[i] != i && e < p.row16)
+            piece(k, ((lk & 1) ? p.v_cache : p.k_cache) + (lk >> 1) * p.layer_stride16 + e, i);
+          if (++i == i0 + rows && per > 1) {
+            i = 1;
+            if (++column == columns) { column = 0; ++lk; }
+          }
+        }
+      };
+      uint4 held[kTailHeld];
+      each([&](int k, uint4* cache, int i) { held[k] = cache[t.src[i]]; });
+      each([&](int k, uint4* cache, int i) { cache[t.dst[i]] = held[k]; });
+    }
+  }
+}
+
+// Sequences of at most this many rows get one CTA: 8 layers of 9 positions, 144 rows, 7.4 us that way instead of 4.3.
+constexpr int kAloneRows = 64;
+// CTAs of kCommitThreads that an SM holds: more rows than their warps cover are taken in turns, not in waves.
+constexpr int kCopyResident = 3, kTailResident = 2;
+
+struct CommitPlan {
+  int ctas, threads;                                 // per sequence; of a CTA
+  int launches() const { return ctas > 1 ? 2 : 1; }
+};
+
+// A warp per row of every layer, or, in place, per unit; threads: of a CTA that shares its sequence.
+CommitPlan commit_plan(int layers, int batch, int row16, int N, bool tail, int threads = kCommitThreads) {
+  const int64_t rows = static_cast<int64_t>(2 * layers) * (N + 1);
+  if (rows <= kAloneRows) return {1, kCommitThreadsAlone};
+  const int64_t work = tail ? static_cast<int64_t>(2 * layers) * ((row16 + 31) / 32) : rows;
+  const int64_t fill = (work + threads / 32 - 1) / (threads / 32);
+  const int64_t spread = static_cast<int64_t>(tail ? kTailResident : kCopyResident) * kCommitThreads / threads * sm_count() / batch;
+  return {static_cast<int>(fill < spread ? fill : spread > 1 ? spread : 1), threads};
+}
+
+// What the arguments of jet_kv_compact (tail: jet_kv_compact_tail) come to; path, accept_len and batch are checked by the caller.
+inline jet_status commit_params(const void* tree_k, const void* tree_v, void* k_cache, void* v_cache, int64_t cache_layer_stride,
+                                int64_t kv_batch_stride, const int32_t* page_table, int max_pages_per_seq, int page_size,
+                                const int32_t* path, const int32_t* accept_len, int32_t* seq_len, int layers, int batch, int B,
+                                int Hkv, int D, int N, bool tail, CommitParams* out) {
+  if ((!tail && (!tree_k || !tree_v)) || !k_cache || !v_cache || !path || !accept_len || !seq_len) return JET_ERR_INVALID_ARG;
+  if (layers < 1 || layers > 65535 || batch < 1 || (!tail && batch > 65535) || B < 1 || B > JET_MAX_NODES || Hkv < 1 || D < 1 ||
+      N < 1 || N > JET_MAX_DEPTH)
+    return JET_ERR_INVALID_ARG;
+  const int64_t row_elems = static_cast<int64_t>(Hkv) * D;
+  if (row_elems % 8 != 0 || cache_layer_stride % 8 != 0) return JET_ERR_INVALID_ARG;   // 16-byte rows
+  if ((!tail && (!aligned(tree_k, 16) || !aligned(tree_v, 16))) || !aligned(k_cache, 16) || !aligned(v_cache, 16))
+    return JET_ERR_INVALID_ARG;
+  if (page_table) {
+    if (page_size < 1 || max_pages_per_seq < 1) return JET_ERR_INVALID_ARG;
+  } else if (kv_batch_stride % 8 != 0 || kv_batch_stride < 0) {
+    return JET_ERR_INVALID_ARG;
+  }
+  *out = {static_cast<const uint4*>(tree_k), static_cast<const uint4*>(tree_v), static_cast<uint4*>(k_cache),
+          static_cast<uint4*>(v_cache), cache_layer_stride / 8, kv_batch_stride / 8, page_table, path, accept_len, seq_len, nullptr,
+          max_pages_per_seq, page_size, layers, batch, B, static_cast<int>(row_elems / 8), N, 1};
+  return JET_OK;
+}
+
+}  // namespace
+}  // namespace jet

@@ -23,6 +23,18 @@ extern "C" jet_status jet_internal_tree_build_step(
     const int32_t* node_budget, int score_mode, float alpha, int32_t* parent, int32_t* depth, int32_t* token, float* score,
     uint32_t* anc_mask, int32_t* n_nodes, float* depth_entropy, float* depth_lse, int from_logits, const int32_t* len_src,
     int32_t* len_dst, void* workspace, size_t workspace_bytes, void* stream);
+extern "C" jet_status jet_internal_kv_compact_step(
+    const void* tree_k, const void* tree_v, void* k_cache, void* v_cache, int64_t cache_layer_stride, int64_t kv_batch_stride,
+    const int32_t* page_table, int max_pages_per_seq, int page_size, const int32_t* path, const int32_t* accept_len, int32_t* seq_len,
+    int layers, int batch, int B, int Hkv, int D, int N, int tail, int32_t* arrived, void* stream);
+extern "C" jet_status jet_internal_accept_commit(
+    const void* rows, int64_t row_stride, const void* lm_head_weight, int d, const int32_t* token, const int32_t* parent,
+    const int32_t* depth, const uint32_t* anc_mask, const int32_t* n_nodes, int batch, int B, int V, int N, int32_t* tgt_argmax,
+    int32_t* accept_len, int32_t* path, int32_t* out_tokens, int32_t* device_status, void* workspace, size_t workspace_bytes,
+    const void* tree_k, const void* tree_v, void* k_cache, void* v_cache, int64_t cache_layer_stride, int64_t kv_batch_stride,
+    const int32_t* page_table, int max_pages_per_seq, int page_size, int32_t* seq_len, int layers, int Hkv, int D, int tail,
+    int32_t* arrived, void* stream);
+extern "C" int jet_internal_accept_commit_launches(int hidden, int layers, int batch, int B, int V, int Hkv, int D, int N, int tail);
 
 namespace {
 
@@ -398,10 +410,79 @@ PyObject* kv_compact(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
                                  D, N, st));
 }
 
+// (tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table, max_pages, page_size, path, accept_len,
+//  seq_len, layers, batch, B, Hkv, D, N, tail, arrived, stream)
+PyObject* kv_compact_step(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
+  Args a(argv, argc, 21);
+  const void* tk = a.ptr();
+  const void* tv = a.ptr();
+  void* k = a.ptr();
+  void* v = a.ptr();
+  const int64_t ls = a.i64(), bs = a.i64();
+  const int32_t* table = in<int32_t>(a.ptr());
+  const int max_pages = a.i32(), page_size = a.i32();
+  const int32_t* path = in<int32_t>(a.ptr());
+  const int32_t* len = in<int32_t>(a.ptr());
+  int32_t* seq_len = out<int32_t>(a.ptr());
+  const int layers = a.i32(), batch = a.i32(), B = a.i32(), Hkv = a.i32(), D = a.i32(), N = a.i32(), tail = a.i32();
+  int32_t* arrived = out<int32_t>(a.ptr());
+  void* st = a.stream();
+  JET_CALL(jet_internal_kv_compact_step(tk, tv, k, v, ls, bs, table, max_pages, page_size, path, len, seq_len, layers, batch, B, Hkv,
+                                        D, N, tail, arrived, st));
+}
+
+// (rows, row_stride, lm_head_weight, d, token, parent, depth, anc_mask, n_nodes, batch, B, V, N, tgt_argmax, accept_len, path,
+//  out_tokens, device_status, workspace, workspace_bytes, tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride,
+//  page_table, max_pages, page_size, seq_len, layers, Hkv, D, tail, arrived, stream).  lm_head_weight None: rows are logits.
+PyObject* accept_commit(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
+  Args a(argv, argc, 36);
+  const void* rows = a.ptr();
+  const int64_t stride = a.i64();
+  const void* weight = a.ptr();
+  const int d = a.i32();
+  const int32_t* token = in<int32_t>(a.ptr());
+  const int32_t* parent = in<int32_t>(a.ptr());
+  const int32_t* depth = in<int32_t>(a.ptr());
+  const uint32_t* anc = in<uint32_t>(a.ptr());
+  const int32_t* n_nodes = in<int32_t>(a.ptr());
+  const int batch = a.i32(), B = a.i32(), V = a.i32(), N = a.i32();
+  int32_t* tgt = out<int32_t>(a.ptr());
+  int32_t* len = out<int32_t>(a.ptr());
+  int32_t* path = out<int32_t>(a.ptr());
+  int32_t* toks = out<int32_t>(a.ptr());
+  int32_t* dev_status = out<int32_t>(a.ptr());
+  size_t wb = 0;
+  void* ws = a.workspace(&wb);
+  const void* tk = a.ptr();
+  const void* tv = a.ptr();
+  void* k = a.ptr();
+  void* v = a.ptr();
+  const int64_t ls = a.i64(), bs = a.i64();
+  const int32_t* table = in<int32_t>(a.ptr());
+  const int max_pages = a.i32(), page_size = a.i32();
+  int32_t* seq_len = out<int32_t>(a.ptr());
+  const int layers = a.i32(), Hkv = a.i32(), D = a.i32(), tail = a.i32();
+  int32_t* arrived = out<int32_t>(a.ptr());
+  void* st = a.stream();
+  JET_CALL(jet_internal_accept_commit(rows, stride, weight, d, token, parent, depth, anc, n_nodes, batch, B, V, N, tgt, len, path, toks,
+                                      dev_status, ws, wb, tk, tv, k, v, ls, bs, table, max_pages, page_size, seq_len, layers, Hkv, D,
+                                      tail, arrived, st));
+}
+
+// (hidden, layers, batch, B, V, Hkv, D, N, tail)
+PyObject* accept_commit_launches(PyObject*, PyObject* const* argv, Py_ssize_t argc) {
+  Args a(argv, argc, 9);
+  const int hidden = a.i32(), layers = a.i32(), batch = a.i32(), B = a.i32(), V = a.i32(), Hkv = a.i32(), D = a.i32(), N = a.i32(),
+            tail = a.i32();
+  if (a.bad()) return nullptr;
+  return PyLong_FromLong(jet_internal_accept_commit_launches(hidden, layers, batch, B, V, Hkv, D, N, tail));
+}
+
 #define JET_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {JET_METHOD(tree_build),         JET_METHOD(tree_build_scored),  JET_METHOD(tree_verify_attn),
                          JET_METHOD(tree_accept),        JET_METHOD(tree_accept_hidden), JET_METHOD(tree_accept_sample),
-                         JET_METHOD(kv_compact),         {nullptr, nullptr, 0, nullptr}};
+                         JET_METHOD(kv_compact),         JET_METHOD(kv_compact_step),    JET_METHOD(accept_commit),
+                         JET_METHOD(accept_commit_launches), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_jetcall", "argument marshalling of libjet.so", -1, methods,
                           nullptr, nullptr, nullptr, nullptr};
 

@@ -10,6 +10,7 @@
 //                          against it, picks the deepest accepted node and writes the
 //                          path and the output tokens.
 #include <atomic>
+#include "commit_rows.cuh"
 #include "jet_common.cuh"
 #include "sm100_ptx.cuh"
 #include "tma_host.cuh"
@@ -21,9 +22,17 @@ constexpr int kArgThreads = 256;
 constexpr int kArgElems = 32;
 constexpr int kArgChunk = kArgThreads * kArgElems;
 
+// Where the key of (row v, slice c) of a sequence lies.  A row's keys lie together; for more than 128 nodes the rows of a slice do:
+// a thread of the reader then has few companions in its row, and its loads would not coalesce (512 nodes of 151936 logits, acceptance
+// 49.9 -> 47.6 us; but 64 nodes 7.1 -> 7.3, acceptance and commit 10.0 -> 11.6).
+struct KeyLayout {
+  int row, slice;
+};
+inline KeyLayout key_layout(int B, int nchunks) { return B > 128 ? KeyLayout{1, B} : KeyLayout{nchunks, 1}; }
+
 __global__ void __launch_bounds__(kArgThreads)
 argmax_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int V, int B,
-                      const int32_t* __restrict__ n_nodes, int nchunks, bool vec_ok,
+                      const int32_t* __restrict__ n_nodes, int nchunks, bool vec_ok, KeyLayout at,
                       unsigned long long* __restrict__ partial) {
   grid_dependency_wait();
   const int chunk = blockIdx.x;
@@ -91,7 +100,7 @@ argmax_partial_kernel(const float* __restrict__ logits, int64_t row_stride, int 
   if (tid < 32) {
     unsigned long long w = tid < kArgThreads / 32 ? warp_best[tid] : 0ull;
     w = warp_max_u64(w);
-    if (tid == 0) partial[static_cast<size_t>(row) * nchunks + chunk] = w;
+    if (tid == 0) partial[static_cast<size_t>(b) * nchunks * B + static_cast<size_t>(v) * at.row + static_cast<size_t>(chunk) * at.slice] = w;
   }
 }
 
@@ -104,79 +113,161 @@ struct TreeView {
   int32_t *tgt_out, *accept_len, *path, *out_tokens;
 };
 
-// Path selection of sequence b by one CTA of at least B threads, one per node: tgt = the target's arg-max at this thread's
-// node (-1 for padding).
-__device__ __forceinline__ void select_path(const TreeView& t, int b, int32_t tgt) {
-  __shared__ int32_t s_tgt[JET_MAX_NODES];
-  __shared__ uint32_t s_match[JET_MAX_NODES / 32];
-  __shared__ uint32_t s_best[JET_MAX_NODES / 32];
-  __shared__ uint32_t s_end_row[JET_MAX_NODES / 32];
-  __shared__ int s_end;
+// One node of a tree, held by the thread of its number.
+struct NodeView {
+  int n;                                             // nodes of the tree
+  bool live;
+  int parent, depth, token;
+  uint32_t mask[JET_MAX_NODES / 32];                 // ancestors and itself
+};
 
+__device__ __forceinline__ NodeView load_node(const TreeView& t, int b) {
+  NodeView x;
+  const int v = threadIdx.x, words = (t.B + 31) / 32;
+  const size_t o = static_cast<size_t>(b) * t.B + v;
+  x.n = min(__ldcg(t.n_nodes + b), t.B);
+  x.live = v < x.n;
+  x.parent = x.depth = x.token = -1;
+  if (v < t.B) {                                     // (padding rows are read too: nothing here waits for the tree's size)
+    x.parent = __ldcg(t.parent + o);
+    x.depth = __ldcg(t.depth + o);
+    x.token = __ldcg(t.token + o);
+  }
+#pragma unroll
+  for (int w = 0; w < JET_MAX_NODES / 32; ++w) x.mask[w] = v < t.B && w < words ? __ldcg(t.anc_mask + o * words + w) : 0u;
+  if (!x.live) x.parent = x.depth = x.token = -1;
+  return x;
+}
+
+struct PathScratch {
+  int32_t tgt[JET_MAX_NODES];                        // the target's arg-max at every node (-1 for padding)
+  uint32_t match[JET_MAX_NODES / 32], best[JET_MAX_NODES / 32], end_row[JET_MAX_NODES / 32];
+  int32_t path[JET_MAX_DEPTH + 1];                   // node of every depth up to a, -1 behind
+  int a;
+};
+
+// Path selection of sequence b by one CTA of at least B threads, one per node; s.tgt is filled.  Returns a: entries 0 .. a of s.path
+// are the accepted path.  write: the results are stored too.
+__device__ __forceinline__ int select_path(const TreeView& t, int b, const NodeView& x, PathScratch& s, bool write) {
   const int v = threadIdx.x, lane = v & 31, warp = v >> 5;
-  const int B = t.B, N = t.N, n = min(t.n_nodes[b], B);
-  const int words = (B + 31) / 32;
-  const size_t o = static_cast<size_t>(b) * B;
-  const bool live = v < n;              // blockDim.x >= B, n <= B
-  int my_parent = -1, my_depth = -1, my_token = -1;
-  if (live) { my_parent = t.parent[o + v]; my_depth = t.depth[o + v]; my_token = t.token[o + v]; }
-  s_tgt[v] = tgt;
-  if (v < B) t.tgt_out[o + v] = tgt;
+  const int N = t.N, words = (t.B + 31) / 32;
+  if (v <= N) s.path[v] = -1;
   __syncthreads();
+  if (write && v < t.B) t.tgt_out[static_cast<size_t>(b) * t.B + v] = s.tgt[v];
 
   // match[v]: the root always matches; other nodes iff token == target prediction at the parent
-  const bool match = live && (v == 0 || (my_parent >= 0 && my_parent < n && my_token == s_tgt[my_parent]));
+  const bool match = x.live && (v == 0 || (x.parent >= 0 && x.parent < x.n && x.token == s.tgt[x.parent]));
   const uint32_t mbits = __ballot_sync(0xffffffffu, match);
-  if (lane == 0) s_match[warp] = mbits;
+  if (lane == 0) s.match[warp] = mbits;
   __syncthreads();
 
   // accepted iff every node of Anc(v)+{v} matches
-  bool acc = live;
-  if (live) {
-    const uint32_t* row = t.anc_mask + (o + v) * words;
-    for (int w = 0; w < words; ++w) acc = acc && ((row[w] & ~s_match[w]) == 0u);
-  }
+  bool acc = x.live;
+#pragma unroll
+  for (int w = 0; w < JET_MAX_NODES / 32; ++w)
+    if (w < words) acc = acc && ((x.mask[w] & ~s.match[w]) == 0u);      // (words <= the CTA's warps: all written)
   // deepest accepted node, ties -> lowest index
-  uint32_t key = acc ? ((static_cast<uint32_t>(my_depth) << 16) | (0xFFFFu - v)) : 0u;
+  uint32_t key = acc ? ((static_cast<uint32_t>(x.depth) << 16) | (0xFFFFu - v)) : 0u;
   key = __reduce_max_sync(0xffffffffu, key);
-  if (lane == 0) s_best[warp] = key;
+  if (lane == 0) s.best[warp] = key;
   __syncthreads();
-  if (warp == 0) {
-    uint32_t k = lane < blockDim.x / 32 ? s_best[lane] : 0u;
-    k = __reduce_max_sync(0xffffffffu, k);
-    if (lane == 0) s_end = k ? static_cast<int>(0xFFFFu - (k & 0xFFFFu)) : 0;
+  // (every warp works the end out: no barrier for it)
+  const uint32_t k = __reduce_max_sync(0xffffffffu, lane < static_cast<int>(blockDim.x / 32) ? s.best[lane] : 0u);
+  const int end = k ? static_cast<int>(0xFFFFu - (k & 0xFFFFu)) : 0;
+  if (v == end) {
+    // (clamped: the arrays of a tree are the caller's and are not validated; a depth outside 0 .. N must not turn
+    //  into a store outside the N + 1 entries of this sequence's outputs)
+    s.a = s.tgt[end] >= 0 ? min(max(x.depth, 0), N) : 0;
+#pragma unroll
+    for (int w = 0; w < JET_MAX_NODES / 32; ++w)
+      if (w < words) s.end_row[w] = x.mask[w];
   }
-  __syncthreads();
-  const int end = s_end;
-  if (v < words) s_end_row[v] = t.anc_mask[(o + end) * words + v];
   __syncthreads();
 
-  // (clamped: the arrays of a tree are the caller's and are not validated; a depth outside 0 .. N must not turn
-  //  into a store outside the N + 1 entries of this sequence's outputs)
-  const int a = s_tgt[end] >= 0 ? min(max(t.depth[o + end], 0), N) : 0;
+  const int a = s.a;
   int32_t* my_path = t.path + static_cast<size_t>(b) * (N + 1);
   int32_t* my_tok = t.out_tokens + static_cast<size_t>(b) * (N + 1);
-  for (int i = v; i <= N; i += blockDim.x)
-    if (i > a) { my_path[i] = -1; my_tok[i] = -1; }
-  if (live && ((s_end_row[v >> 5] >> (v & 31)) & 1u) && my_depth >= 0 && my_depth <= N) {
-    my_path[my_depth] = v;
-    if (my_depth >= 1) my_tok[my_depth - 1] = my_token;
+  if (x.live && ((s.end_row[v >> 5] >> (v & 31)) & 1u) && x.depth >= 0 && x.depth <= N) {
+    s.path[x.depth] = v;
+    if (write) {
+      if (x.depth <= a) my_path[x.depth] = v;
+      if (x.depth >= 1 && x.depth <= a) my_tok[x.depth - 1] = x.token;
+    }
   }
-  if (v == 0) { t.accept_len[b] = a; my_tok[a] = s_tgt[end]; }
+  if (write) {
+    if (v > a && v <= N) { my_path[v] = -1; my_tok[v] = -1; }
+    if (v == 0) { t.accept_len[b] = a; my_tok[a] = s.tgt[end]; }
+  }
+  return a;
 }
 
-__global__ void __launch_bounds__(JET_MAX_NODES)
-accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks, const TreeView t) {
-  grid_dependency_wait();
-  const int b = blockIdx.x, v = threadIdx.x;
-  int32_t tgt = -1;
-  if (v < min(t.n_nodes[b], t.B)) {
-    unsigned long long k = 0ull;
-    const unsigned long long* pr = partial + (static_cast<size_t>(b) * t.B + v) * nchunks;
-    for (int c = 0; c < nchunks; ++c) { const unsigned long long x = pr[c]; k = x > k ? x : k; }
-    tgt = static_cast<int32_t>(key_index(k));
+// Threads of a CTA that selects a path: a node each, and two or more per row where the rows' keys are fetched.
+int path_threads(int B) { return B <= 128 ? 256 : JET_MAX_NODES; }
+
+// The best of every row's keys, into s.tgt: `per` neighbouring threads share a row, eight loads each in flight (a thread per row took
+// 19 keys of 151936 logits in five round trips to L2).
+__device__ __forceinline__ void finish_rows(const unsigned long long* __restrict__ partial, int nchunks, KeyLayout at, int b, int B, int n,
+                                            PathScratch& s) {
+  int shift = 0;
+  while (shift < 5 && (((B + 31) & ~31) << (shift + 1)) <= static_cast<int>(blockDim.x)) ++shift;
+  const int per = 1 << shift, row = static_cast<int>(threadIdx.x) >> shift;
+  unsigned long long k = 0ull;
+  if (row < n) {
+    const unsigned long long* pr = partial + static_cast<size_t>(b) * nchunks * B + static_cast<size_t>(row) * at.row;
+    for (int c0 = static_cast<int>(threadIdx.x) & (per - 1); c0 < nchunks; c0 += 8 * per) {
+      unsigned long long x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = c0 + j * per < nchunks ? __ldcg(pr + static_cast<size_t>(c0 + j * per) * at.slice) : 0ull;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) k = x[j] > k ? x[j] : k;
+    }
   }
-  select_path(t, b, tgt);
+  for (int o = per >> 1; o > 0; o >>= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
+    k = other > k ? other : k;
+  }
+  if ((threadIdx.x & (per - 1)) == 0 && row < B) s.tgt[row] = row < n ? static_cast<int32_t>(key_index(k)) : -1;
+}
+
+// (The tree is older than the keys' kernel, which this one follows in the stream: it is read before the wait.)
+__global__ void __launch_bounds__(JET_MAX_NODES)
+accept_path_kernel(const unsigned long long* __restrict__ partial, int nchunks, KeyLayout at, const TreeView t) {
+  __shared__ PathScratch s;
+  const int b = blockIdx.x;
+  const NodeView x = load_node(t, b);
+  grid_dependency_wait();
+  finish_rows(partial, nchunks, at, b, t.B, x.n, s);
+  select_path(t, b, x, s, true);
+}
+
+// Keys of a sequence up to which every copying CTA reads them all (48 KB out of L2): 64 nodes of 151936 logits and 36 layers 11.0 us for
+// acceptance and commit apart, 10.0 in one; 256 nodes 28.0 and 26.3; 512 nodes, 9728 keys, 52.0 and 52.5.
+constexpr int kFusedKeys = 6144;
+
+// Acceptance and commit in one launch: every CTA that copies rows of a sequence selects its path too, the first one writes it.
+// Bound: latency.  Two launches fewer per step (path selection, lengths), and of the chain  keys, tree -> path | path, lengths -> page
+// table -> rows | lengths  only  keys -> path -> rows  is left behind the wait for the scan.  us for acceptance and commit in a captured
+// stream, apart and in one: 64 nodes, 151936 logits, 36 layers 10.8 -> 10.1, in place 11.0 -> 10.1, one layer 10.3 -> 9.2; 256 nodes 28.0 ->
+// 26.3; 32 sequences of 64 nodes, 8 layers, paged 177 -> 174.5; 16 nodes of 1024 logits, one layer (the small form below) 5.7 -> 4.9.
+// (At most one CTA of 512 threads per SM is asked for: held to 64 registers the copies wait for one another, 1.7 us.)
+template <bool kTail>
+__global__ void __launch_bounds__(JET_MAX_NODES, 1)
+accept_commit_kernel(const unsigned long long* __restrict__ partial, int nchunks, KeyLayout at, const TreeView t, const CommitParams p) {
+  __shared__ PathScratch s;
+  __shared__ CommitTable table;
+  const int b = blockIdx.x / p.ctas, i = threadIdx.x;
+  const NodeView x = load_node(t, b);
+  const int len = __ldcg(p.seq_len + b);
+  const int64_t dst = i <= t.N ? cache_row(p, b, static_cast<int64_t>(len) + i) : 0;
+  grid_dependency_wait();
+  finish_rows(partial, nchunks, at, b, t.B, x.n, s);
+  const int a = select_path(t, b, x, s, blockIdx.x % p.ctas == 0);
+  __syncthreads();
+  if (i <= a) commit_entry<kTail>(p, b, i, s.path[i], len, dst, table);
+  __syncthreads();
+  finish_commit(p, b, len + a + 1);
+  if constexpr (kTail) move_rows(p, a, table);
+  else copy_rows(p, b, a, table);
 }
 
 // Both parts in one launch for small problems: a CTA per sequence, a warp per row of logits.  One turn of its 16 warps takes
@@ -191,14 +282,11 @@ bool accept_is_small(int batch, int B, int V) {
   return V <= kSmallRow && ((B <= kSmallThreads / 32 && logits <= kSmallLogits) || (batch >= kSmallBatch && logits <= kSmallBatchLogits));
 }
 
-__global__ void __launch_bounds__(kSmallThreads)
-accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t) {
-  grid_dependency_wait();
-  __shared__ int32_t s_row[JET_MAX_NODES];
-  const int b = blockIdx.x, lane = threadIdx.x & 31;
-  const int n = min(t.n_nodes[b], t.B);
+__device__ __forceinline__ void small_rows(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, int b, int B, int n,
+                                           PathScratch& s) {
+  const int lane = threadIdx.x & 31;
   for (int v = threadIdx.x >> 5; v < n; v += kSmallThreads / 32) {
-    const float* p = logits + (static_cast<int64_t>(b) * t.B + v) * row_stride;
+    const float* p = logits + (static_cast<int64_t>(b) * B + v) * row_stride;
     float best = 0.0f;
     uint32_t best_idx = 0xFFFFFFFFu;                 // none yet
     auto take = [&](float x, int idx) {              // (called with ascending indices)
@@ -229,11 +317,40 @@ accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V,
       }
     }
     const unsigned long long key = warp_max_u64(best_idx == 0xFFFFFFFFu ? 0ull : make_key(best, best_idx));
-    if (lane == 0) s_row[v] = static_cast<int32_t>(key_index(key));
+    if (lane == 0) s.tgt[v] = static_cast<int32_t>(key_index(key));
   }
+  if (static_cast<int>(threadIdx.x) >= n && static_cast<int>(threadIdx.x) < B) s.tgt[threadIdx.x] = -1;
+}
+
+__global__ void __launch_bounds__(kSmallThreads)
+accept_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t) {
+  __shared__ PathScratch s;
+  const int b = blockIdx.x;
+  grid_dependency_wait();
+  const NodeView x = load_node(t, b);
+  small_rows(logits, row_stride, V, vec_ok, b, t.B, x.n, s);
+  select_path(t, b, x, s, true);
+}
+
+// The same and the commit, one CTA per sequence, where that many rows are committed (kAloneRows).
+template <bool kTail>
+__global__ void __launch_bounds__(kSmallThreads)
+accept_commit_small_kernel(const float* __restrict__ logits, int64_t row_stride, int V, bool vec_ok, const TreeView t, const CommitParams p) {
+  __shared__ PathScratch s;
+  __shared__ CommitTable table;
+  const int b = blockIdx.x, i = threadIdx.x;
+  grid_dependency_wait();
+  const NodeView x = load_node(t, b);
+  const int len = __ldcg(p.seq_len + b);
+  const int64_t dst = i <= t.N ? cache_row(p, b, static_cast<int64_t>(len) + i) : 0;
+  small_rows(logits, row_stride, V, vec_ok, b, t.B, x.n, s);
+  const int a = select_path(t, b, x, s, true);
   __syncthreads();
-  const int v = threadIdx.x;
-  select_path(t, b, v < n ? s_row[v] : -1);
+  if (i <= a) commit_entry<kTail>(p, b, i, s.path[i], len, dst, table);
+  __syncthreads();
+  finish_commit(p, b, len + a + 1);
+  if constexpr (kTail) move_rows(p, a, table);
+  else copy_rows(p, b, a, table);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -650,6 +767,82 @@ static __device__ __align__(256) unsigned long long g_accept_scratch[kStaticKeys
 }  // namespace
 }  // namespace jet
 
+namespace jet {
+namespace {
+
+// Path selection behind a kernel that leaves `nchunks` keys per row, and the commit where there is one.
+jet_status finish_accept(const unsigned long long* keys, int nchunks, const TreeView& tree, int batch, CommitParams* commit, bool tail,
+                         cudaStream_t st) {
+  const KeyLayout at = key_layout(tree.B, nchunks);
+  if (!commit) {
+    launch_dependent(accept_path_kernel, dim3(batch), dim3(path_threads(tree.B)), st, keys, nchunks, at, tree);
+    return launch_status();
+  }
+  const CommitPlan plan = commit_plan(commit->layers, batch, commit->row16, commit->N, tail, path_threads(tree.B));
+  commit->ctas = plan.ctas;
+  launch_dependent(tail ? accept_commit_kernel<true> : accept_commit_kernel<false>, dim3(static_cast<unsigned>(plan.ctas) * batch),
+                   dim3(plan.threads), st, keys, nchunks, at, tree, *commit);
+  return launch_status();
+}
+
+// Greedy acceptance from logits, arguments checked; with commit, behind it the commit of the path (commit->arrived given).
+jet_status accept_logits(const float* logits, int64_t row_stride, int V, const TreeView& tree, int batch, void* workspace,
+                         CommitParams* commit, bool tail, cudaStream_t st) {
+  const int nchunks = chunks_for(V), B = tree.B;
+  const bool vec_ok = aligned(logits, 16) && row_stride % 4 == 0;
+  auto* partial = static_cast<unsigned long long*>(workspace);
+  if (accept_is_small(batch, B, V)) {
+    if (!commit)
+      launch_dependent(accept_small_kernel, dim3(batch), dim3(kSmallThreads), st, logits, row_stride, V, vec_ok, tree);
+    else
+      launch_dependent(tail ? accept_commit_small_kernel<true> : accept_commit_small_kernel<false>, dim3(batch), dim3(kSmallThreads), st,
+                       logits, row_stride, V, vec_ok, tree, *commit);
+    return launch_status();
+  }
+  launch_dependent(argmax_partial_kernel, dim3(nchunks, batch * B), dim3(kArgThreads), st, logits, row_stride, V, B, tree.n_nodes, nchunks,
+                   vec_ok, key_layout(B, nchunks), partial);
+  return finish_accept(partial, nchunks, tree, batch, commit, tail, st);
+}
+
+// Greedy acceptance from hidden states, arguments checked; with commit, behind it the commit of the path (commit->arrived given).
+jet_status accept_hidden(const void* hidden, const void* lm_head_weight, int d, int V, const TreeView& tree, int batch, void* workspace,
+                         int32_t* device_status, CommitParams* commit, bool tail, cudaStream_t st) {
+  const int rows = batch * tree.B;
+  CUtensorMap tx;
+  {
+    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(rows)};
+    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
+    const uint32_t box[2] = {64, 128};
+    if (!tma_make_map_bf16(&tx, hidden, 2, dims, str, box)) return JET_ERR_CUDA;
+  }
+  auto* keys = static_cast<unsigned long long*>(workspace);
+  // every row's key starts as "no entry" (0 is below any valid key)
+  if (cudaMemsetAsync(keys, 0, static_cast<size_t>(rows) * sizeof(unsigned long long), st) != cudaSuccess) {
+    cudaGetLastError();
+    return JET_ERR_CUDA;
+  }
+  // Up to 128 rows the call is a weight stream and one 128-row CTA per weight tile keeps HBM busy; above, it is bound by the
+  // tensor cores and runs on CTA pairs (the weights cross HBM once per 512 rows).
+  jet_status r;
+  if (rows <= kLmBM) {
+    CUtensorMap tw;
+    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(V)};
+    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
+    const uint32_t box[2] = {64, 128};
+    if (!tma_make_map_bf16(&tw, lm_head_weight, 2, dims, str, box)) return JET_ERR_CUDA;
+    r = launch_lm_head(tx, tw, rows, V, d, keys, device_status, st);
+  } else if (rows <= 2 * kLmBM) {
+    r = launch_lm_head_pair<false>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
+  } else {
+    r = launch_lm_head_pair<true>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
+  }
+  if (r != JET_OK) return r;
+  return finish_accept(keys, 1, tree, batch, commit, tail, st);
+}
+
+}  // namespace
+}  // namespace jet
+
 extern "C" size_t jet_tree_accept_workspace_bytes(int batch, int B, int V) {
   if (batch < 1 || B < 1 || V < 1) return 0;
   return jet::round_up(static_cast<size_t>(batch) * B * jet::chunks_for(V) * sizeof(unsigned long long), 256);
@@ -678,20 +871,8 @@ extern "C" jet_status jet_tree_accept(const float* logits, int64_t logits_row_st
   const size_t need = jet_tree_accept_workspace_bytes(batch, B, V);
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
 
-  const int nchunks = chunks_for(V);
-  const bool vec_ok = aligned(logits, 16) && logits_row_stride % 4 == 0;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  auto* partial = static_cast<unsigned long long*>(workspace);
   const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
-  if (accept_is_small(batch, B, V)) {
-    launch_dependent(accept_small_kernel, dim3(batch), dim3(kSmallThreads), st, logits, logits_row_stride, V, vec_ok, tree);
-    return launch_status();
-  }
-  launch_dependent(argmax_partial_kernel, dim3(nchunks, batch * B), dim3(kArgThreads), st,
-      logits, logits_row_stride, V, B, n_nodes, nchunks, vec_ok, partial);
-  const int threads = (B + 31) / 32 * 32;
-  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, partial, nchunks, tree);
-  return launch_status();
+  return accept_logits(logits, logits_row_stride, V, tree, batch, workspace, nullptr, false, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" jet_status jet_tree_accept_static(const float* logits, int64_t logits_row_stride,
@@ -751,39 +932,61 @@ extern "C" jet_status jet_tree_accept_hidden(const void* hidden, const void* lm_
   if (!aligned(hidden, 16) || !aligned(lm_head_weight, 16)) return JET_ERR_INVALID_ARG;
   const size_t need = jet_tree_accept_hidden_workspace_bytes(batch, B);
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
-  const int rows = batch * B;
-  CUtensorMap tx;
-  {
-    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(rows)};
-    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
-    const uint32_t box[2] = {64, 128};
-    if (!tma_make_map_bf16(&tx, hidden, 2, dims, str, box)) return JET_ERR_CUDA;
-  }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  auto* keys = static_cast<unsigned long long*>(workspace);
-  // every row's key starts as "no entry" (0 is below any valid key)
-  if (cudaMemsetAsync(keys, 0, static_cast<size_t>(rows) * sizeof(unsigned long long), st) != cudaSuccess) {
-    cudaGetLastError();
-    return JET_ERR_CUDA;
-  }
-  // Up to 128 rows the call is a weight stream and one 128-row CTA per weight tile keeps HBM busy; above, it is bound by the
-  // tensor cores and runs on CTA pairs (the weights cross HBM once per 512 rows).
-  jet_status r;
-  if (rows <= kLmBM) {
-    CUtensorMap tw;
-    const uint64_t dims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(V)};
-    const uint64_t str[1] = {static_cast<uint64_t>(d) * 2};
-    const uint32_t box[2] = {64, 128};
-    if (!tma_make_map_bf16(&tw, lm_head_weight, 2, dims, str, box)) return JET_ERR_CUDA;
-    r = launch_lm_head(tx, tw, rows, V, d, keys, device_status, st);
-  } else if (rows <= 2 * kLmBM) {
-    r = launch_lm_head_pair<false>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
-  } else {
-    r = launch_lm_head_pair<true>(tx, lm_head_weight, rows, V, d, keys, device_status, st);
-  }
-  if (r != JET_OK) return r;
-  const int threads = (B + 31) / 32 * 32;
   const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
-  launch_dependent(accept_path_kernel, dim3(batch), dim3(threads), st, keys, 1, tree);
-  return launch_status();
+  return accept_hidden(hidden, lm_head_weight, d, V, tree, batch, workspace, device_status, nullptr, false, static_cast<cudaStream_t>(stream));
+}
+
+namespace jet {
+namespace {
+
+// Path selection apart from the copies: every CTA that copies would scan the logits, or read that many keys, again.
+bool path_apart(bool hidden, int layers, int batch, int B, int V, int row16, int N, bool tail) {
+  return !hidden && (accept_is_small(batch, B, V) || B * chunks_for(V) > kFusedKeys) && commit_plan(layers, batch, row16, N, tail).ctas > 1;
+}
+
+}  // namespace
+}  // namespace jet
+
+// Not part of the C ABI: kernels that jet_internal_accept_commit launches.
+extern "C" JET_API int jet_internal_accept_commit_launches(int hidden, int layers, int batch, int B, int V, int Hkv, int D, int N, int tail) {
+  using namespace jet;
+  const bool apart = path_apart(hidden != 0, layers, batch, B, V, static_cast<int>(static_cast<int64_t>(Hkv) * D / 8), N, tail != 0);
+  return (!hidden && accept_is_small(batch, B, V) ? 1 : 2) + (apart ? 1 : 0);
+}
+
+// Not part of the C ABI: what VerifyStep calls -- jet_tree_accept (lm_head_weight null: rows are logits) or jet_tree_accept_hidden, and
+// behind it jet_kv_compact or (tail) jet_kv_compact_tail of the path, in two launches or one.  The arguments are theirs, checked before
+// anything is launched; arrived: one int per sequence, 0 between calls.
+extern "C" JET_API jet_status jet_internal_accept_commit(
+    const void* rows, int64_t row_stride, const void* lm_head_weight, int d, const int32_t* token, const int32_t* parent,
+    const int32_t* depth, const uint32_t* anc_mask, const int32_t* n_nodes, int batch, int B, int V, int N, int32_t* tgt_argmax,
+    int32_t* accept_len, int32_t* path, int32_t* out_tokens, int32_t* device_status, void* workspace, size_t workspace_bytes,
+    const void* tree_k, const void* tree_v, void* k_cache, void* v_cache, int64_t cache_layer_stride, int64_t kv_batch_stride,
+    const int32_t* page_table, int max_pages_per_seq, int page_size, int32_t* seq_len, int layers, int Hkv, int D, int tail,
+    int32_t* arrived, void* stream) {
+  using namespace jet;
+  if (!rows || !token || !parent || !depth || !anc_mask || !n_nodes || !tgt_argmax || !accept_len || !path || !out_tokens || !arrived)
+    return JET_ERR_INVALID_ARG;
+  if (batch < 1 || B < 1 || B > JET_MAX_NODES || V < 1 || N < 1 || N > JET_MAX_DEPTH || static_cast<int64_t>(batch) * B > 65535)
+    return JET_ERR_INVALID_ARG;
+  if (lm_head_weight ? d < 64 : row_stride < V) return JET_ERR_INVALID_ARG;
+  if (lm_head_weight && d % 64 != 0) return JET_ERR_UNSUPPORTED;
+  if (lm_head_weight ? !aligned(rows, 16) || !aligned(lm_head_weight, 16) : !aligned(rows, 4)) return JET_ERR_INVALID_ARG;
+  const size_t need = lm_head_weight ? jet_tree_accept_hidden_workspace_bytes(batch, B) : jet_tree_accept_workspace_bytes(batch, B, V);
+  if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return JET_ERR_WORKSPACE;
+  CommitParams p;
+  const jet_status r = commit_params(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,
+                                     max_pages_per_seq, page_size, path, accept_len, seq_len, layers, batch, B, Hkv, D, N, tail != 0, &p);
+  if (r != JET_OK) return r;
+  p.arrived = arrived;
+  const TreeView tree{token, parent, depth, anc_mask, n_nodes, B, N, tgt_argmax, accept_len, path, out_tokens};
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (path_apart(lm_head_weight != nullptr, layers, batch, B, V, p.row16, N, tail != 0)) {
+    const jet_status a = accept_logits(static_cast<const float*>(rows), row_stride, V, tree, batch, workspace, nullptr, false, st);
+    return a != JET_OK ? a : jet_internal_kv_compact_step(tree_k, tree_v, k_cache, v_cache, cache_layer_stride, kv_batch_stride, page_table,
+                                                          max_pages_per_seq, page_size, path, accept_len, seq_len, layers, batch, B, Hkv,
+                                                          D, N, tail, arrived, stream);
+  }
+  return lm_head_weight ? accept_hidden(rows, lm_head_weight, d, V, tree, batch, workspace, device_status, &p, tail != 0, st)
+                        : accept_logits(static_cast<const float*>(rows), row_stride, V, tree, batch, workspace, &p, tail != 0, st);
 }

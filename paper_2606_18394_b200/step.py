@@ -63,6 +63,7 @@ class VerifyStep:
         self.tgt = torch.zeros((batch, B), **i32)
         self.accept_len = torch.zeros(batch, **i32)
         self.path = torch.zeros((batch, N + 1), **i32)
+        self.arrived = torch.zeros(batch, **i32)      # CTAs that have got to the commit (zero between steps)
         self.out_tokens = torch.zeros((batch, N + 1), **i32)
         # ---- workspaces
         def ws(nbytes):
@@ -210,13 +211,21 @@ class VerifyStep:
 
     def run_back(self):
         """Acceptance against the target logits and the commit."""
+        tail = self.tail
+        rows = (None, None) if tail else (self.tree_k, self.tree_v)
         if self.accept_mode == "sample":
             self.tree_accept_sample()
-        elif self.accept_mode == "hidden":
-            self.tree_accept_hidden()
-        else:
-            self.tree_accept()
-        self.kv_compact()
+            jet.kv_compact_step(*rows, self.k_cache, self.v_cache, self.cache_layer_stride, self.kv_batch_stride, self.page_table,
+                                self.max_pages, self.page_size, self.path, self.accept_len, self.seq_len, self.layers, self.batch,
+                                self.B, self.Hkv, self.D, self.N, tail, self.arrived)
+            return
+        hidden = self.accept_mode == "hidden"
+        jet.accept_commit_step(self.hidden if hidden else self.logits, self.V, self.lm_head if hidden else None,
+                               self.d_model if hidden else 0, self.token, self.parent, self.depth, self.anc_mask, self.n_nodes,
+                               self.batch, self.B, self.V, self.N, self.tgt, self.accept_len, self.path, self.out_tokens, self.status,
+                               self.ws_accept_hidden if hidden else self.ws_accept, *rows, self.k_cache, self.v_cache,
+                               self.cache_layer_stride, self.kv_batch_stride, self.page_table, self.max_pages, self.page_size,
+                               self.seq_len, self.layers, self.Hkv, self.D, tail, self.arrived)
 
     def run(self):
         """The whole hot path once, on the current stream."""
@@ -228,8 +237,8 @@ class VerifyStep:
         """Kernel launches of a step's tree construction, acceptance and commit (small ones take fewer)."""
         mode = {"accum_logp": 0, "entropy": 1, "hybrid": 2}[self.score_mode]
         build = jet.jet_tree_build_launches(self.N, self.V, mode, self.draft_logits)
-        accept = jet.jet_tree_accept_launches(self.batch, self.B, self.V) if self.accept_mode == "greedy" else 2
-        return build + accept + jet.jet_kv_compact_launches(self.layers, self.batch, self.Hkv, self.D, self.N, self.tail)
+        return build + jet.accept_commit_launches(self.accept_mode, self.layers, self.batch, self.B, self.V, self.Hkv, self.D,
+                                                  self.N, self.tail)
 
     def launches_per_step(self, attn_launches_per_layer=None):
         if attn_launches_per_layer is None:       # what the library says one attention call of this shape enqueues
