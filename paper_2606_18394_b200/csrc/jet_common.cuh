@@ -28,9 +28,8 @@ inline int current_device() {
   return dev;
 }
 
-inline int sm_count() {
+inline int sm_count(int dev) {
   static std::atomic<int> cache[kMaxDevices];
-  const int dev = current_device();
   int n = cache[dev].load(std::memory_order_relaxed);
   if (n == 0) {
     int v = 0;
@@ -43,6 +42,7 @@ inline int sm_count() {
   }
   return n;
 }
+inline int sm_count() { return sm_count(current_device()); }
 
 // Launch with programmatic stream serialization: the grid may be scheduled while the preceding kernel of the
 // stream drains, so its launch latency is hidden.  Every kernel launched this way executes grid_dependency_wait()

@@ -2370,12 +2370,12 @@ bool configure_kernel() {
 }
 
 // How many clusters of `cluster` CTAs of this kernel the device can hold at once (one CTA per SM, and a
-// cluster must fit inside one GPC).  Asked of the driver once per cluster size and cached.
+// cluster must fit inside one GPC).  Asked of the driver once per cluster size and cached; dev is the current device.
 template <int D, int MT>
-int max_active_clusters(int cluster) {
+int max_active_clusters(int cluster, int dev) {
   static std::atomic<int> caches[kMaxDevices][kMaxSplit + 1];      // per device: 0 = unknown, -1 = none
   if (cluster < 1 || cluster > kMaxCluster) return 0;       // (the occupancy query does not refuse larger ones)
-  std::atomic<int>* cache = caches[current_device()];
+  std::atomic<int>* cache = caches[dev];
   if (cache[cluster].load(std::memory_order_relaxed) == 0) {
     int n = 0;
     if (configure_kernel<D, MT>()) {
@@ -2401,14 +2401,14 @@ int max_active_clusters(int cluster) {
   return have > 0 ? have : 0;
 }
 
-int max_active_clusters_for(int D, int mt, int cluster) {
-  if (D == 128) return mt == 1 ? max_active_clusters<128, 1>(cluster) : max_active_clusters<128, 2>(cluster);
-  return mt == 1 ? max_active_clusters<64, 1>(cluster) : max_active_clusters<64, 2>(cluster);
+int max_active_clusters_for(int D, int mt, int cluster, int dev) {
+  if (D == 128) return mt == 1 ? max_active_clusters<128, 1>(cluster, dev) : max_active_clusters<128, 2>(cluster, dev);
+  return mt == 1 ? max_active_clusters<64, 1>(cluster, dev) : max_active_clusters<64, 2>(cluster, dev);
 }
 
 // Small merge CTAs where one wave of them covers the rows and their registers hold the slices.
-bool merge_is_small(int query_tiles, int ns, int D) {
-  return ns <= kMergeSmallSlices && query_tiles * kBM <= sm_count() * (kMergeSmall / (D / 8));
+bool merge_is_small(int query_tiles, int ns, int D, int sms) {
+  return ns <= kMergeSmallSlices && query_tiles * kBM <= sms * (kMergeSmall / (D / 8));
 }
 
 // Picks the query-tile grouping, the number of key slices and the form of their merge with a cost model, in microseconds
@@ -2448,14 +2448,15 @@ bool merge_is_small(int query_tiles, int ns, int D) {
 // 9000 keys (32 / 8 heads, prefix 4096: 64 nodes 12.5 against 11.8 us, 16 nodes 12.3 against 10.7), within 2 % of it for long
 // sequences, and 0.2 - 0.8 us (2 - 6 %) faster at D 64 or with 18 slices of two query tiles: not enough for kernels that wait
 // for one another.
-double plan_cost(bool fitted, int batch, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D) {
+double plan_cost(bool fitted, int batch, int mt, int ns, int via, double waves, int ctas, int units, int n_mgroups, int tiles, int D,
+                 int sms) {
   if (!fitted) {
     const double per_tile = mt == 1 ? 1.0 + 0.75 / n_mgroups : 1.7;
     const double fixed = mt == 1 ? (ns == 1 ? 6.0 : via == 0 ? 8.0 : 10.0) : (ns == 1 ? 9.8 : via == 0 ? 15.6 : 16.3);
     const double whole = ceil(waves), spread = 0.93 * waves + 0.25;
     return (batch == 1 ? whole : 0.5 * whole + 0.5 * (spread > 1.0 ? spread : 1.0)) * ((tiles + ns - 1) / ns * per_tile + fixed);
   }
-  const double f = ctas >= sm_count() ? 1.0 : static_cast<double>(ctas) / sm_count();
+  const double f = ctas >= sms ? 1.0 : static_cast<double>(ctas) / sms;
   const double tile = mt == 1 ? 0.78 + 0.14 * f : via == 2 ? 1.5 : 2.2;
   double fixed, floor = 4.0;
   if (ns == 1) {
@@ -2463,7 +2464,7 @@ double plan_cost(bool fitted, int batch, int mt, int ns, int via, double waves, 
   } else if (via == 0) {
     fixed = (ns == 4 ? 5.7 : ns == 8 ? 6.0 : ns % 2 ? 7.0 : 6.4) + 2.4 * f;
   } else {
-    fixed = 5.9 + 2.2 * f + (merge_is_small(units * mt, ns, D) ? 0.0 : 0.5) + (2 * ctas > sm_count() ? 0.4 : 0.0) +
+    fixed = 5.9 + 2.2 * f + (merge_is_small(units * mt, ns, D, sms) ? 0.0 : 0.5) + (2 * ctas > sms ? 0.4 : 0.0) +
             (ns > 12 ? 2.0 : ns > 10 ? 0.7 : 0.0);
     floor = 8.0;
   }
@@ -2476,6 +2477,8 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
   const int rows = B * G;
   const int tiles = (max_seq_len + kBN - 1) / kBN + (B + kBN - 1) / kBN;
   const bool fitted = batch <= 4 && batch * Hkv * ((rows + kBM - 1) / kBM) <= 64;      // (see plan_cost)
+  // (asked once: every call plans, and asking the runtime for the device at every use made a plan cost 2 - 6 us of host time)
+  const int dev = current_device(), sms = sm_count(dev);
   Plan best{};
   double best_cost = -1.0;
   // Test hooks (read once per process): JET_FORCE_MT = query tiles per CTA, JET_FORCE_SPLIT = "slices" or
@@ -2500,7 +2503,7 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
     auto consider = [&](int ns, int via_global, double waves, int pair = 0) {
       if (force_ns && (ns != force_ns || (ns > 1 && via_global != force_via))) return;
       if (pair != (force_pair > 0 && pair_ok ? 1 : 0)) return;
-      const double cost = plan_cost(fitted, batch, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D);
+      const double cost = plan_cost(fitted, batch, mt, ns, via_global, waves, pl.units * ns, pl.units, pl.n_mgroups, tiles, D, sms);
       if (best_cost < 0.0 || cost < best_cost) {
         best = pl;
         best.nsplit = ns;
@@ -2512,15 +2515,15 @@ Plan make_plan(int batch, int B, int Hq, int Hkv, int D, int max_seq_len) {
 
     for (int ns = 1; ns <= kMaxSplit && ns <= tiles; ++ns) {
       // (a) the slices of a unit form a thread-block cluster and merge through distributed shared memory
-      const int resident = ns <= 8 || force_ns ? max_active_clusters_for(D, mt, ns) : 0;
+      const int resident = ns <= 8 || force_ns ? max_active_clusters_for(D, mt, ns, dev) : 0;
       if (resident > 0) consider(ns, 0, static_cast<double>(pl.units) / resident);
-      if (pair_ok && ns == 1) consider(1, 0, static_cast<double>((pl.units + sm_count() - 1) / sm_count()), 1);
+      if (pair_ok && ns == 1) consider(1, 0, static_cast<double>((pl.units + sms - 1) / sms), 1);
       // (b) independent CTAs that merge through the workspace: all of them resident at once (a cluster has to fit into
       //     one GPC, which can leave a third of the SMs idle).  With a second small launch that combines the blocks
       //     once the first has ended nothing waits inside a kernel.
       // (With two query tiles per CTA only where one would be sliced as well: the rows travel as bf16.)
-      const bool sliced = mt == 1 || force_mt || 2L * batch * Hkv * ((rows + kBM - 1) / kBM) <= sm_count();
-      if (ns > 1 && sliced && static_cast<long>(pl.units) * ns <= sm_count() &&
+      const bool sliced = mt == 1 || force_mt || 2L * batch * Hkv * ((rows + kBM - 1) / kBM) <= sms;
+      if (ns > 1 && sliced && static_cast<long>(pl.units) * ns <= sms &&
           static_cast<size_t>(pl.units) * mt * 2 * sizeof(int) <= kCounterBytes) {
         consider(ns, force_via ? force_via : 2, 1.0);
         if (pair_ok) consider(ns, force_via ? force_via : 1, 1.0, 1);
@@ -2576,7 +2579,7 @@ bool launch_merge(const MergeParams& m, cudaStream_t st) {
     const int per = threads / (D / 8);
     return dim3(static_cast<unsigned>((rows + per - 1) / per));
   };
-  const bool is_small = merge_is_small(m.tiles, m.S, D);
+  const bool is_small = merge_is_small(m.tiles, m.S, D, sm_count());
   launch_dependent_smem(is_small ? small[which] : large[which], is_small ? grid(kMergeSmall) : grid(kMergeLarge),
                         dim3(is_small ? kMergeSmall : kMergeLarge), is_small ? 0 : kMergeLargeSmem, st, m);
   return true;
