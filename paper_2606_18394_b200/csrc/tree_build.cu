@@ -18,6 +18,8 @@
 //                        sequential pop/expand loop in one warp with the pending queue in
 //                        registers and emits parent / depth / token / score / ancestor mask.
 //                        (Small problems: it forms the group maxima itself, one launch.)
+#include <type_traits>
+
 #include "fp64_exp.cuh"
 #include "jet_common.cuh"
 
@@ -63,19 +65,30 @@ __device__ __forceinline__ double warp_sum_f64(double x) {
 
 // The row's log-sum-exp from the slices' (m, z = sum exp(x) * 2^-m), m a whole number: M = the largest m, lse = M ln2 +
 // log(sum z * 2^(m - M)), fp64, one warp, fixed order (every caller gets the same bits).
+// (Up to 128 slices are read once, all of a lane's loads in flight; 38 slices in two passes of dependent loads took 1.9 us.)
 __device__ __forceinline__ double row_lse(const double2* __restrict__ part, int slices, int lane) {
+  constexpr int kHeld = 4;
+  double2 held[kHeld];
+#pragma unroll
+  for (int j = 0; j < kHeld; ++j) held[j] = j * 32 + lane < slices ? part[j * 32 + lane] : make_double2(0.0, 0.0);
   double M = -INFINITY;                              // this lane's largest m with a finite entry
-  for (int i = lane; i < slices; i += 32) M = fmax(M, part[i].y > 0.0 ? part[i].x : -INFINITY);
+#pragma unroll
+  for (int j = 0; j < kHeld; ++j) M = fmax(M, held[j].y > 0.0 ? held[j].x : -INFINITY);
+#pragma unroll 1
+  for (int i = kHeld * 32 + lane; i < slices; i += 32) M = fmax(M, part[i].y > 0.0 ? part[i].x : -INFINITY);
   const uint32_t order = f32_order(static_cast<float>(M));
   const int holder = __ffs(__ballot_sync(0xffffffffu, order == __reduce_max_sync(0xffffffffu, order))) - 1;
   M = __shfl_sync(0xffffffffu, M, holder);           // (the largest, up to the rounding of a float: any m near it will do)
   double Z = 0.0;
-  for (int i = lane; i < slices; i += 32) {
-    const double2 mz = part[i];
+  auto add = [&](const double2 mz) {
     const double shift = mz.x - M;                   // beyond -1000 the slice is nothing beside the largest
     if (mz.y > 0.0 && shift > -1000.0)
       Z += mz.y * __hiloint2double((1023 + static_cast<int>(shift)) << 20, 0);
-  }
+  };
+#pragma unroll
+  for (int j = 0; j < kHeld; ++j) add(held[j]);
+#pragma unroll 1
+  for (int i = kHeld * 32 + lane; i < slices; i += 32) add(part[i]);
   Z = warp_sum_f64(Z);
   return fma(M, 0.6931471805599453, log(Z));
 }
@@ -730,15 +743,110 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
 // of them instead of B), kept in registers -- entry i by lane i % 32 in register i / 32 as a key of two words, (priority,
 // ~index : depth), largest first.  A pop is two warp reductions; the entry then moves on to the next sibling.  The loop
 // only records the nodes it expands; their children are written out by the whole CTA afterwards (child j of expansion e is
-// node 1 + e * Wc + j).  It is one warp's dependent chain, so its length in instructions is its time: about 250 cycles a
-// pop (650 with the children written inside the loop and 64-bit keys; 900 with a queue indexed through local memory).
+// node 1 + e * Wc + j).  It is one warp's dependent chain.
+//  * expand_scores: the priority is the accumulated log-probability (the key's value is the node's score).  The body is one
+//    block without branches, with the siblings' keys formed under the reductions: 300 cycles a pop, where the form below takes
+//    460 (one sequence of raw logits, 256 nodes: 21.1 -> 17.6 us a call; 512 nodes, W 7 / 3 / 2 30.7 / 76 / 106 -> 24.2 / 66 / 91).
+//  * expand_tree: kMode 1 = priority is the entropy of the node's depth, 2 = score + alpha * that entropy, formed as two rounded
+//    float operations.  (As one block it was slower there: 32 sequences, 64 nodes 0.3 us a call.)  depth_h[d] = entropy of the
+//    distribution the tokens of depth d + 1 were drawn from.
+// Tried: a queue kept in order over the lanes, whose new keys are placed by comparing with the neighbours', no reductions: 460 cycles a
+// pop; children written inside the loop and 64-bit keys 650; a queue indexed through local memory 900.
 // kSlots = registers per lane.
-// kMode: 0 = priority is the accumulated log-probability (the key's value is the node's score); 1 = priority
-// is the entropy of the node's depth; 2 = score + alpha * that entropy, formed as two rounded float operations.
-// depth_h[d] = entropy of the distribution the tokens of depth d + 1 were drawn from.
 struct Expansion { uint32_t lo; float score; };      // the expanded node: (~index : depth) as in the keys, its score
 
+// f32_order of an accumulated score.  Scores start at +0 and a rounded sum is -0 only of two -0, so none is -0.
+__device__ __forceinline__ uint32_t score_order(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
+}
+
 __device__ __forceinline__ int key_node(uint32_t lo) { return static_cast<int>(0xFFFFFFu - (lo >> 8)); }
+
+template <int kSlots>
+__device__ __forceinline__ int expand_scores(int lane, int N, int Wc, int B, const float (*top_lp)[JET_MAX_WIDTH], Expansion* made) {
+  uint32_t hi[kSlots], lo[kSlots];                   // the entry's best pending child; both 0: none
+  float ps[kSlots];                                  // its parent's score
+  int tl[kSlots];                                    // where the sibling behind it is in the table of log-probabilities (its
+                                                     // rank in the low bits; 0: past the last rank the table has room for)
+#pragma unroll
+  for (int i = 0; i < kSlots; ++i) {
+    hi[i] = lo[i] = 0u;
+    ps[i] = 0.0f;
+    tl[i] = 0;
+  }
+  const float* table = top_lp[0];
+  // the priority of the sibling behind every entry's child is formed while the reductions run (with many registers only the moved
+  // entry's is worth forming, on the chain)
+  constexpr bool kAhead = kSlots <= 4;
+  const int last = (B - 2) / Wc;                     // the expansion that fills the tree
+  uint32_t node = 0xFFFFFFu << 8;                    // (~index : depth) of the node taken, the root first
+  float score = 0.0f;
+  int e = 0;                                         // expansions before this one, and the entry of this one's children
+  for (;; ++e) {
+    // the node taken gets its children (its depth is below N: see below)
+    const int d = static_cast<int>(node & 0xFFu);
+    const float first_lp = table[d * JET_MAX_WIDTH];
+    made[e] = {node, score};                         // (every lane, the same: no branch)
+    if (e == last) break;
+    const bool fresh = d + 1 < N;                    // children at depth N are never expanded: taking one would only drop it
+    // (every lane forms the new entry and its keeper selects it: no indexed register array, which would live in local memory)
+    const uint32_t h = fresh ? score_order(__fadd_rn(score, first_lp)) : 0u;
+    const uint32_t l = fresh ? ((0xFFFFFEu - static_cast<uint32_t>(e * Wc)) << 8) + static_cast<uint32_t>(d + 1) : 0u;
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) {
+      const bool here = e - i * 32 == lane;
+      hi[i] = here ? h : hi[i];
+      lo[i] = here ? l : lo[i];
+      ps[i] = here ? score : ps[i];
+      tl[i] = here ? d * JET_MAX_WIDTH + 1 : tl[i];
+    }
+    float behind_lp[kAhead ? kSlots : 1];
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int i = 0; i < kSlots; ++i) behind_lp[i] = table[tl[i]];
+    }
+    uint32_t bh = hi[0], bl = lo[0];
+#pragma unroll
+    for (int i = 1; i < kSlots; ++i) {
+      const bool more = hi[i] > bh || (hi[i] == bh && lo[i] > bl);
+      bh = more ? hi[i] : bh;
+      bl = more ? lo[i] : bl;
+    }
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, bh);
+    uint32_t ahead[kAhead ? kSlots : 1], next[kSlots];
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) {
+      const int rank = tl[i] & (JET_MAX_WIDTH - 1);
+      const bool more = rank != 0 && rank < Wc;
+      next[i] = more ? lo[i] - 256u : 0u;
+      if constexpr (kAhead) ahead[i] = more ? score_order(__fadd_rn(ps[i], behind_lp[i])) : 0u;
+    }
+    node = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
+    if (node == 0u) break;                           // nothing pending
+    float parent_score = 0.0f;
+    int at = 0;
+    if constexpr (!kAhead) {
+#pragma unroll
+      for (int i = 0; i < kSlots; ++i) {
+        const bool hit = lo[i] == node;              // (a node is in one entry only)
+        parent_score = hit ? ps[i] : parent_score;
+        at = hit ? tl[i] : at;
+      }
+    }
+    score = __uint_as_float((mh & 0x80000000u) ? (mh & 0x7FFFFFFFu) : ~mh);
+    // its entry moves on to the next sibling
+    if constexpr (!kAhead) ahead[0] = score_order(__fadd_rn(parent_score, table[at]));
+#pragma unroll
+    for (int i = 0; i < kSlots; ++i) {
+      const bool hit = lo[i] == node;
+      hi[i] = hit ? (kAhead ? ahead[i] : next[i] != 0u ? ahead[0] : 0u) : hi[i];
+      lo[i] = hit ? next[i] : lo[i];
+      tl[i] += hit ? 1 : 0;
+    }
+  }
+  return min(1 + (e + 1) * Wc, B);
+}
 
 template <int kSlots, int kMode>
 __device__ __forceinline__ int expand_tree(int lane, int N, int Wc, int B, const float (*top_lp)[JET_MAX_WIDTH],
@@ -756,8 +864,7 @@ __device__ __forceinline__ int expand_tree(int lane, int N, int Wc, int B, const
   const float* table = top_lp[0];
   auto priority = [&](float score, int dep) -> uint32_t {      // of a node of depth dep >= 1
     if constexpr (kMode == 1) return f32_order(depth_h[dep - 1]);
-    if constexpr (kMode == 2) return f32_order(__fadd_rn(score, __fmul_rn(alpha, depth_h[dep - 1])));
-    return f32_order(score);
+    else return f32_order(__fadd_rn(score, __fmul_rn(alpha, depth_h[dep - 1])));
   };
   auto depth_of = [](uint32_t node) { return max(static_cast<int>(node & 0xFFu), 1); };
   int n = 1, entries = 0;
@@ -804,20 +911,14 @@ __device__ __forceinline__ int expand_tree(int lane, int N, int Wc, int B, const
     if (node == 0u) break;                           // nothing pending
     float parent_score = 0.0f;
     int at = 0;
-    if constexpr (kMode != 0 || !kAhead) {
 #pragma unroll
-      for (int i = 0; i < kSlots; ++i) {
-        const bool hit = lo[i] == node;              // (a node is in one entry only)
-        parent_score = hit ? ps[i] : parent_score;
-        at = hit ? tl[i] : at;
-      }
+    for (int i = 0; i < kSlots; ++i) {
+      const bool hit = lo[i] == node;                // (a node is in one entry only)
+      parent_score = hit ? ps[i] : parent_score;
+      at = hit ? tl[i] : at;
     }
-    if constexpr (kMode == 0) {
-      score = __uint_as_float((mh & 0x80000000u) ? (mh & 0x7FFFFFFFu) : ~mh);
-    } else {
-      const float own = __fadd_rn(parent_score, table[max(at - 1, 0)]);
-      score = __shfl_sync(0xffffffffu, own, __ffs(__ballot_sync(0xffffffffu, bl == node)) - 1);
-    }
+    const float own = __fadd_rn(parent_score, table[max(at - 1, 0)]);
+    score = __shfl_sync(0xffffffffu, own, __ffs(__ballot_sync(0xffffffffu, bl == node)) - 1);
     // its entry moves on to the next sibling
     if constexpr (!kAhead) ahead[0] = priority(__fadd_rn(parent_score, table[at]), depth_of(node));
 #pragma unroll
@@ -946,11 +1047,16 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     const int slots = ((Wc == 1 ? min(Bb - 1, N) : (Bb - 1 + Wc - 1) / Wc) + 31) / 32;
     Expansion* made = sh.tree.made;
     int n;
-    if (slots <= 1) n = expand_tree<1, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
-    else if (slots <= 2) n = expand_tree<2, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
-    else if (slots <= 4) n = expand_tree<4, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
-    else if (slots <= 8) n = expand_tree<8, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
-    else n = expand_tree<JET_MAX_NODES / 32, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    auto expand = [&](auto registers) {
+      constexpr int kSlots = decltype(registers)::value;
+      if constexpr (kMode == 0) return expand_scores<kSlots>(lane, N, Wc, Bb, s_top_lp, made);
+      else return expand_tree<kSlots, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
+    };
+    if (slots <= 1) n = expand(std::integral_constant<int, 1>{});
+    else if (slots <= 2) n = expand(std::integral_constant<int, 2>{});
+    else if (slots <= 4) n = expand(std::integral_constant<int, 4>{});
+    else if (slots <= 8) n = expand(std::integral_constant<int, 8>{});
+    else n = expand(std::integral_constant<int, JET_MAX_NODES / 32>{});
     if (lane == 0) s_n = n;
   }
   __syncthreads();
