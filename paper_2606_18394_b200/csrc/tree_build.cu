@@ -746,11 +746,7 @@ __device__ __forceinline__ void top_of_row(const RowGroups& rg, const float* __r
 // node 1 + e * Wc + j).  It is one warp's dependent chain.
 //  * expand_scores: the priority is the accumulated log-probability (the key's value is the node's score).  The body is one
 //    block without branches, with the siblings' keys formed under the reductions: 300 cycles a pop, where the form below takes
-//    460 (one sequence of raw logits, 256 nodes: 21.1 -> 17.6 us a call).
-//  * expand_many: the same for more than 64 expansions.  The keys of the best child and of the next sibling are formed once, by every
-//    lane alike, and not per register, and an entry is its key alone.  512 nodes, us a call of expand_tree, expand_scores and this:
-//    W 7 (four registers) 30.7, 24.5, 23.7; W 3 (eight) 76, 66, 53; W 2, 500 nodes 106, 91, 71.  With one or two registers it is the slower:
-//    64 nodes 8.0 and 8.1, 449 nodes 18.0 and 18.35.  (A function of its own: the usual forms stay short.)
+//    460 (one sequence of raw logits, 256 nodes: 21.1 -> 17.6 us a call; 512 nodes, W 7 / 3 / 2 30.7 / 76 / 106 -> 24.2 / 66 / 91).
 //  * expand_tree: kMode 1 = priority is the entropy of the node's depth, 2 = score + alpha * that entropy, formed as two rounded
 //    float operations.  (As one block it was slower there: 32 sequences, 64 nodes 0.3 us a call.)  depth_h[d] = entropy of the
 //    distribution the tokens of depth d + 1 were drawn from.
@@ -780,6 +776,9 @@ __device__ __forceinline__ int expand_scores(int lane, int N, int Wc, int B, con
     tl[i] = 0;
   }
   const float* table = top_lp[0];
+  // the priority of the sibling behind every entry's child is formed while the reductions run (with many registers only the moved
+  // entry's is worth forming, on the chain)
+  constexpr bool kAhead = kSlots <= 4;
   const int last = (B - 2) / Wc;                     // the expansion that fills the tree
   uint32_t node = 0xFFFFFFu << 8;                    // (~index : depth) of the node taken, the root first
   float score = 0.0f;
@@ -802,9 +801,11 @@ __device__ __forceinline__ int expand_scores(int lane, int N, int Wc, int B, con
       ps[i] = here ? score : ps[i];
       tl[i] = here ? d * JET_MAX_WIDTH + 1 : tl[i];
     }
-    float behind_lp[kSlots];
+    float behind_lp[kAhead ? kSlots : 1];
+    if constexpr (kAhead) {
 #pragma unroll
-    for (int i = 0; i < kSlots; ++i) behind_lp[i] = table[tl[i]];
+      for (int i = 0; i < kSlots; ++i) behind_lp[i] = table[tl[i]];
+    }
     uint32_t bh = hi[0], bl = lo[0];
 #pragma unroll
     for (int i = 1; i < kSlots; ++i) {
@@ -813,74 +814,36 @@ __device__ __forceinline__ int expand_scores(int lane, int N, int Wc, int B, con
       bl = more ? lo[i] : bl;
     }
     const uint32_t mh = __reduce_max_sync(0xffffffffu, bh);
-    // the key of the sibling behind every entry's child is formed while the reductions run
-    uint32_t ahead[kSlots], next[kSlots];
+    uint32_t ahead[kAhead ? kSlots : 1], next[kSlots];
 #pragma unroll
     for (int i = 0; i < kSlots; ++i) {
       const int rank = tl[i] & (JET_MAX_WIDTH - 1);
       const bool more = rank != 0 && rank < Wc;
       next[i] = more ? lo[i] - 256u : 0u;
-      ahead[i] = more ? score_order(__fadd_rn(ps[i], behind_lp[i])) : 0u;
+      if constexpr (kAhead) ahead[i] = more ? score_order(__fadd_rn(ps[i], behind_lp[i])) : 0u;
     }
     node = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
     if (node == 0u) break;                           // nothing pending
+    float parent_score = 0.0f;
+    int at = 0;
+    if constexpr (!kAhead) {
+#pragma unroll
+      for (int i = 0; i < kSlots; ++i) {
+        const bool hit = lo[i] == node;              // (a node is in one entry only)
+        parent_score = hit ? ps[i] : parent_score;
+        at = hit ? tl[i] : at;
+      }
+    }
     score = __uint_as_float((mh & 0x80000000u) ? (mh & 0x7FFFFFFFu) : ~mh);
     // its entry moves on to the next sibling
+    if constexpr (!kAhead) ahead[0] = score_order(__fadd_rn(parent_score, table[at]));
 #pragma unroll
     for (int i = 0; i < kSlots; ++i) {
       const bool hit = lo[i] == node;
-      hi[i] = hit ? ahead[i] : hi[i];
+      hi[i] = hit ? (kAhead ? ahead[i] : next[i] != 0u ? ahead[0] : 0u) : hi[i];
       lo[i] = hit ? next[i] : lo[i];
       tl[i] += hit ? 1 : 0;
     }
-  }
-  return min(1 + (e + 1) * Wc, B);
-}
-
-// Low word of a key: ~index (10 bits), depth (7), rank among its siblings (6), expansion that made it (9).
-template <int kSlots>
-__device__ __noinline__ int expand_many(int lane, int N, int Wc, int B, const float (*top_lp)[JET_MAX_WIDTH], Expansion* made) {
-  static_assert(JET_MAX_NODES + JET_MAX_WIDTH < 1023 && JET_MAX_DEPTH < 128 && JET_MAX_WIDTH < 64 && JET_MAX_NODES <= 512, "fields of a key");
-  uint32_t hi[kSlots], lo[kSlots];                   // the entry's best pending child; hi 0: none
-#pragma unroll
-  for (int i = 0; i < kSlots; ++i) hi[i] = lo[i] = 0u;
-  const float* table = top_lp[0];
-  const int last = (B - 2) / Wc;                     // the expansion that fills the tree
-  uint32_t node = 1023u << 22;                       // low word of the node taken, the root first
-  float score = 0.0f;
-  int e = 0;                                         // expansions before this one, and the entry of this one's children
-  for (;; ++e) {
-    // the node taken gets its children (its depth is below N: see below), and its entry moves on to the next sibling
-    const int d = static_cast<int>(node >> 15) & 127, rank = static_cast<int>(node >> 9) & 63;
-    const float child_lp = table[d * JET_MAX_WIDTH];
-    const float next_lp = table[max(d - 1, 0) * JET_MAX_WIDTH + rank + 1];
-    const float parent_score = made[node & 511u].score;         // (the root's is not used)
-    made[e] = {((0xFFFC00u + (node >> 22)) << 8) + static_cast<uint32_t>(d), score};      // (every lane, the same: no branch)
-    if (e == last) break;
-    const uint32_t ch = d + 1 < N ? score_order(__fadd_rn(score, child_lp)) : 0u;      // (children at depth N are never expanded)
-    const uint32_t cl = ((1022u - static_cast<uint32_t>(e * Wc)) << 22) + (static_cast<uint32_t>(d + 1) << 15) + static_cast<uint32_t>(e);
-    const uint32_t sh = rank + 1 < Wc ? score_order(__fadd_rn(parent_score, next_lp)) : 0u;
-    const uint32_t sl = node - (1u << 22) + (1u << 9);
-#pragma unroll
-    for (int i = 0; i < kSlots; ++i) {
-      const bool hit = lo[i] == node;                // (a node is in one entry only; the root in none)
-      hi[i] = hit ? sh : hi[i];
-      lo[i] = hit ? sl : lo[i];
-      const bool here = e - i * 32 == lane;
-      hi[i] = here ? ch : hi[i];
-      lo[i] = here ? cl : lo[i];
-    }
-    uint32_t bh = hi[0], bl = lo[0];
-#pragma unroll
-    for (int i = 1; i < kSlots; ++i) {
-      const bool more = hi[i] > bh || (hi[i] == bh && lo[i] > bl);
-      bh = more ? hi[i] : bh;
-      bl = more ? lo[i] : bl;
-    }
-    const uint32_t mh = __reduce_max_sync(0xffffffffu, bh);
-    node = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
-    if (mh == 0u) break;                             // nothing pending
-    score = __uint_as_float((mh & 0x80000000u) ? (mh & 0x7FFFFFFFu) : ~mh);
   }
   return min(1 + (e + 1) * Wc, B);
 }
@@ -991,7 +954,7 @@ struct ScanView {
 constexpr int kDirectSlices = 6;
 
 template <int kMode, bool kDirect, bool kWide>
-__global__ void __launch_bounds__(kExpThreads, 1)      // (held to 64 registers one form spills: 16 nodes of 1024 logits 5.45 -> 5.65 us)
+__global__ void __launch_bounds__(kExpThreads)
 tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, int N, int V, int Wc, int B, float alpha,
                    int32_t* __restrict__ parent_out, int32_t* __restrict__ depth_out,
                    int32_t* __restrict__ token_out, float* __restrict__ score_out,
@@ -1086,8 +1049,7 @@ tree_expand_kernel(const ScanView scan, const int32_t* __restrict__ root_token, 
     int n;
     auto expand = [&](auto registers) {
       constexpr int kSlots = decltype(registers)::value;
-      if constexpr (kMode == 0 && kSlots <= 2) return expand_scores<kSlots>(lane, N, Wc, Bb, s_top_lp, made);
-      else if constexpr (kMode == 0) return expand_many<kSlots>(lane, N, Wc, Bb, s_top_lp, made);
+      if constexpr (kMode == 0) return expand_scores<kSlots>(lane, N, Wc, Bb, s_top_lp, made);
       else return expand_tree<kSlots, kMode>(lane, N, Wc, Bb, s_top_lp, made, s_depth_h, alpha);
     };
     if (slots <= 1) n = expand(std::integral_constant<int, 1>{});
